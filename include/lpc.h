@@ -238,8 +238,8 @@ int lpc_scheme_bits(int scheme, int64_t d, int32_t b, int32_t N, uint64_t* bits_
  *   huffman_bits_out  host, N * nseg, nullable: sum_c count_c * len_c under Huffman's code for that histogram (one
  *                     bit per coordinate when a message holds a single value).
  * Neither count includes the code table or the 32-bit scale; compare with the raw b * len of Section 3.2.
- * With both host outputs NULL the call only enqueues the histogram; otherwise it waits for the stream and does the
- * two sums on the host.  Errors: LPC_ERR_UNSUPPORTED unless 1 <= b <= 8.
+ * With both host outputs NULL the call only enqueues the histogram; otherwise both sums are formed on
+ * the device and the call waits for the stream.  Errors: LPC_ERR_UNSUPPORTED unless 1 <= b <= 8.
  */
 int lpc_message_entropy(lpc_ctx* ctx, const uint32_t* codes, int64_t len, const int64_t* seg_offsets, int32_t nseg,
                         unsigned long long* hist_dev, double* entropy_bits_out, uint64_t* huffman_bits_out);

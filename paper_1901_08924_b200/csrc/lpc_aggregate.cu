@@ -6,6 +6,8 @@
 // A thread owns 8 consecutive coordinates per sweep: per worker it loads the 8*b bits that hold
 // their codes (b whole bytes, naturally aligned when b is 1, 2, 4, 8 or 16), and accumulates
 // delta_i * index in worker order, every operation a separate fp32 round-to-nearest operation.
+#include <algorithm>
+
 #include "lpc_device.cuh"
 #include "lpc_kernels.h"
 
@@ -488,8 +490,6 @@ __global__ void __launch_bounds__(AT, 4) server_reduce4_kernel(ServerArgs a) {
     if ((j >> 5) * OW + i < so.pad_words) o[i] = out[i];
 }
 
-constexpr int HRUN = 32;  // tiles per CTA: the counts reach the message's histogram (a few hot addresses) once per run and segment
-
 // Histogram of a message's code values, the input of the entropy-coding count (Section 5.1: the experiments pass the
 // codes through Huffman's code).
 //
@@ -536,10 +536,10 @@ __device__ __forceinline__ void count_unit(uint4 q, uint32_t* cnt) {
 }
 
 template <int BITS>  // 1, 2, 4
-__global__ void __launch_bounds__(AT) code_histogram_swar_kernel(HistArgs a) {
+__global__ void __launch_bounds__(AT) code_histogram_swar_kernel(HistArgs a, int run) {
   constexpr int BINS = 1 << BITS, CPU = 128 / BITS;  // codes per 16-byte unit
   const int worker = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-  const int tile0 = blockIdx.x * HRUN, tile1 = min(tile0 + HRUN, a.ntiles);
+  const int tile0 = blockIdx.x * run, tile1 = min(tile0 + run, a.ntiles);
   __shared__ unsigned int total[BINS];
   if (tid < BINS) total[tid] = 0u;
   __syncthreads();
@@ -583,131 +583,180 @@ __global__ void __launch_bounds__(AT) code_histogram_swar_kernel(HistArgs a) {
   }
 }
 
-// Widths without a bit-sliced count (8 bits, and the odd widths): every thread counts the 32 codes it reads in counters
-// of its own in shared memory -- one byte per code value, four values to a 32-bit word, word[value / 4][thread] -- so
-// that counting needs no atomic operation however skewed the codes are and a warp's accesses fall on 32 different banks.
-// The block then adds the columns up with warp reductions and sends the tile's count of every value to the message's
-// histogram with one atomic addition each.
-template <int BITS>  // 1, 2, 4, 8: code width known at compile time; 0: b in 1..8 from the arguments
-__global__ void __launch_bounds__(AT) code_histogram_kernel(HistArgs a) {
-  const int worker = blockIdx.y;
-  const int tile0 = blockIdx.x * HRUN, tile1 = min(tile0 + HRUN, a.ntiles);
-  const int tid = threadIdx.x;
-  const int b = BITS ? BITS : a.b, bins = 1 << b;
-  const int rows = (bins + 3) / 4;  // words per thread and copy
-  // Narrow codes keep NCH copies of the counters, one per coordinate position modulo NCH: the eight increments of a
-  // group then form NCH independent chains of read-modify-writes instead of one (they may hit the same counter, so
-  // the chain of one copy cannot be reordered)
-  constexpr int NCH = (BITS >= 1 && BITS <= 4) ? 4 : 1;
-  extern __shared__ __align__(16) uint32_t cw[];  // NCH x rows x AT words
-  uint8_t* mine = reinterpret_cast<uint8_t*>(cw + tid);  // this thread's counter of value c in copy q: mine[((q * rows + c / 4) * AT) * 4 + c % 4]
-  __shared__ unsigned int total[256];
-  for (int c = tid; c < bins; c += AT) total[c] = 0u;
-  int cur_seg = -1;
-  auto flush = [&]() {  // the counts gathered for segment cur_seg go to its histogram (all threads call this)
-    __syncthreads();
-    if (cur_seg >= 0)
-      for (int c = tid; c < bins; c += AT) {
-        if (total[c]) atomicAdd(&a.hist[((int64_t)worker * a.nseg + cur_seg) * bins + c], (unsigned long long)total[c]);
-        total[c] = 0u;
-      }
-    __syncthreads();
-  };
-#pragma unroll 1
-  for (int tile = tile0; tile < tile1; ++tile) {
+// Widths without a bit-sliced count (3 and 5 to 8 bits): one 32-bit counter per code value and LANE in shared memory,
+// tab[value][lane], added to by atomic operations that return nothing.  A warp's 32 additions fall on 32 different banks
+// and addresses however skewed the codes are (heavy-tailed gradients without clipping put nearly all codes on three
+// values), no addition waits for the one before it, and all warps of the CTA share one 32 KB table, so a CTA adds its
+// columns up and clears them once per run and segment instead of once per tile.  Bound by the shared-memory atomics
+// (about 11 additions per clock and SM).  8 x 2^24 8-bit codes: 46 us, against 530 us for byte counters of every thread
+// that were read, changed, written back and added up tile by tile.
+template <int BITS>
+__device__ __forceinline__ void count_codes(uint32_t* col, const uint32_t* w, int first, int count) {
+  constexpr uint32_t MASK = (1u << BITS) - 1u;
+#pragma unroll
+  for (int e = 0; e < count; ++e) {
+    const int pos = (first + e) * BITS, i = pos >> 5, sh = pos & 31;
+    const uint32_t code = (sh + BITS <= 32 ? w[i] >> sh : __funnelshift_r(w[i], w[i + 1], sh)) & MASK;
+    atomicAdd(col + code * 32, 1u);
+  }
+}
+
+constexpr int HT = 512;
+template <int BITS>  // 3, 5, 6, 7, 8
+__global__ void __launch_bounds__(HT) code_histogram_kernel(HistArgs a, int run) {
+  constexpr int BINS = 1 << BITS;
+  constexpr int UW = BITS == 8 ? 4 : BITS;   // words of a thread's unit: 16 bytes, or the shortest whole number of words
+  constexpr int UC = UW * 32 / BITS;         // codes in it
+  const int worker = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tile0 = blockIdx.x * run, tile1 = min(tile0 + run, a.ntiles);
+  __shared__ uint32_t tab[BINS * 32];
+  for (int i = tid; i < BINS * 32; i += HT) tab[i] = 0u;
+  __syncthreads();
+  uint32_t* col = tab + lane;
+  int tile = tile0;
+  while (tile < tile1) {  // one pass per tensor segment that the run touches
     const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
-    if (seg != cur_seg) {
-      flush();
-      cur_seg = seg;
-    }
     const SegInfo s = a.segs[seg];
-    const int64_t tstart = (int64_t)(tile - s.tile_first) * TILE;
-    for (int i = tid; i < NCH * rows * AT; i += AT) cw[i] = 0u;  // a thread clears and uses its own column only
-    const uint32_t* w = a.codes + (int64_t)worker * a.stride_words + s.word_off;
-    if constexpr (BITS != 0) {
-      // fixed widths: which thread counts which code does not matter, so a thread takes whole words of the tile's
-      // stream, BITS of them, AT words apart (coalesced), all requested before the first is used
-      constexpr int CPW = 32 / BITS;  // codes per word
-      const int64_t nvalid_tile = min((int64_t)TILE, s.len - tstart);
-      const uint32_t* wt = w + (tstart >> 5) * BITS;
-      uint32_t cwords[BITS];
-#pragma unroll
-      for (int i = 0; i < BITS; ++i) {
-        const int wi = i * AT + tid;
-        cwords[i] = ((int64_t)wi * CPW < nvalid_tile) ? __ldcs(wt + wi) : 0u;
+    const int tend = min(tile1, s.tile_first + s.tile_count);
+    const int64_t j0 = (int64_t)(tile - s.tile_first) * TILE;
+    const int n = (int)(min(s.len, (int64_t)(tend - s.tile_first) * TILE) - j0);  // codes to count (run * TILE at most)
+    const uint32_t* w = a.codes + (int64_t)worker * a.stride_words + s.word_off + (j0 >> 5) * BITS;  // 16-byte aligned
+    const int units = n / UC;
+    if constexpr (BITS == 8) {
+      const uint4* wu = reinterpret_cast<const uint4*>(w);
+      int u = tid;
+      for (; u + HT < units; u += 2 * HT) {
+        const uint4 q0 = __ldcs(wu + u), q1 = __ldcs(wu + u + HT);
+        const uint32_t v0[4] = {q0.x, q0.y, q0.z, q0.w}, v1[4] = {q1.x, q1.y, q1.z, q1.w};
+        count_codes<8>(col, v0, 0, 16);
+        count_codes<8>(col, v1, 0, 16);
       }
-#pragma unroll
-      for (int i = 0; i < BITS; ++i) {
-        const int wi = i * AT + tid;
-        const int64_t left = nvalid_tile - (int64_t)wi * CPW;  // codes of this word that exist
-        if (left >= CPW) {
-#pragma unroll
-          for (int e = 0; e < CPW; ++e) {
-            const uint32_t code = (cwords[i] >> (e * BITS)) & (uint32_t)(bins - 1);
-            mine[((((e % NCH) * rows + (code >> 2)) * (AT * 4))) | (code & 3u)] += 1;
-          }
-        } else {
-          for (int e = 0; e < (int)left; ++e) {
-            const uint32_t code = (cwords[i] >> (e * BITS)) & (uint32_t)(bins - 1);
-            mine[((((e % NCH) * rows + (code >> 2)) * (AT * 4))) | (code & 3u)] += 1;
-          }
-        }
+      if (u < units) {
+        const uint4 q0 = __ldcs(wu + u);
+        const uint32_t v0[4] = {q0.x, q0.y, q0.z, q0.w};
+        count_codes<8>(col, v0, 0, 16);
       }
     } else {
-#pragma unroll 1
-      for (int it = 0; it < AITER; ++it) {  // a thread sees at most AITER * 8 = 32 codes: a byte counter cannot overflow
-        const int64_t j = tstart + (int64_t)it * AGROUP + tid * 8;
-        if (j >= s.len) break;
-        const int nvalid = (int)min((int64_t)8, s.len - j);
-        uint64_t lo, hi;
-        load_chunk<0>(w, j >> 3, b, s.pad_words, lo, hi);  // 8 * b <= 64 bits: all in lo
+      for (int u = tid; u < units; u += HT) {
+        uint32_t v[UW];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          if (e < nvalid) {
-            const uint32_t code = (uint32_t)(lo >> (e * b)) & (uint32_t)(bins - 1);
-            mine[((code >> 2) * (AT * 4)) | (code & 3u)] += 1;
-          }
-        }
+        for (int i = 0; i < UW; ++i) v[i] = w[(int64_t)u * UW + i];
+        count_codes<BITS>(col, v, 0, UC);
       }
     }
-    // the tile's columns add up: a word's four byte counters (each <= 32) widen to two words of 16-bit lanes, a warp
-    // adds them with one integer reduction each (32 lanes * 32 fits 16 bits), lane 0 adds the sums to the run's totals
-    for (int r = 0; r < rows; ++r) {
-      uint32_t v = cw[r * AT + tid];
+    for (int j = units * UC + tid; j < n; j += HT) {  // the ragged end, code by code
+      const int64_t pos = (int64_t)j * BITS;
+      const uint32_t sh = (uint32_t)(pos & 31);
+      uint32_t code = w[pos >> 5] >> sh;
+      if (sh + BITS > 32) code |= w[(pos >> 5) + 1] << (32 - sh);
+      atomicAdd(col + (code & (uint32_t)(BINS - 1)) * 32, 1u);
+    }
+    // a warp adds the 32 columns of a value; one addition per value, run and segment reaches the message's histogram
+    __syncthreads();
+    for (int v = warp; v < BINS; v += HT / 32) {
+      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, col[v * 32]);
+      col[v * 32] = 0u;
+      if (lane == 0 && sum) atomicAdd(&a.hist[((int64_t)worker * a.nseg + seg) * BINS + v], (unsigned long long)sum);
+    }
+    __syncthreads();
+    tile = tend;
+  }
+}
+
+// Entropy bound and Huffman length of every message from its histogram, one CTA per message (Section 5.1).
+//   entropy   -sum_c count_c log2(count_c / n) in double precision
+//   Huffman   the sum of the weights of all merged nodes.  The counts are sorted by rank counting (256 threads, every
+//             thread compares its count with all others), then one thread merges them with the two-queue method: merged
+//             weights come out in ascending order, so the two smallest of all nodes are among the first two of either
+//             queue, and a step is three additions, two comparisons and two shared-memory reads.
+// A serial chain of up to 255 steps, but of all messages at the same time: 8 messages of 256 values take about 20 us
+// with the wait for the stream, against 50 us on the host, which took them one after the other.
+__global__ void __launch_bounds__(256) coded_size_kernel(const unsigned long long* __restrict__ hist, int bins,
+                                                         double* __restrict__ entropy_out, unsigned long long* __restrict__ huffman_out) {
+  constexpr unsigned long long NONE = 1ull << 62;  // larger than any sum of counts
+  __shared__ unsigned long long cnt[256], leaf[256 + 2], node[256 + 2];
+  __shared__ unsigned long long wsum[8];
+  __shared__ double wbits[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned long long h = (tid < bins) ? hist[(int64_t)blockIdx.x * bins + tid] : 0ull;
+  cnt[tid] = h;
+  for (int i = tid; i < 258; i += 256) leaf[i] = node[i] = NONE;
+  unsigned long long n = h;
 #pragma unroll
-      for (int q = 1; q < NCH; ++q) v += cw[(q * rows + r) * AT + tid];  // byte lanes: at most 32 in all, no carry
-      const uint32_t even = __reduce_add_sync(0xFFFFFFFFu, v & 0x00FF00FFu);         // values 4r, 4r+2
-      const uint32_t odd = __reduce_add_sync(0xFFFFFFFFu, (v >> 8) & 0x00FF00FFu);   // values 4r+1, 4r+3
-      if ((tid & 31) == 0) {
-        if (even & 0xFFFFu) atomicAdd(&total[4 * r], even & 0xFFFFu);
-        if (even >> 16) atomicAdd(&total[4 * r + 2], even >> 16);
-        if (odd & 0xFFFFu) atomicAdd(&total[4 * r + 1], odd & 0xFFFFu);
-        if (odd >> 16) atomicAdd(&total[4 * r + 3], odd >> 16);
-      }
+  for (int m = 16; m >= 1; m >>= 1) n += __shfl_xor_sync(0xFFFFFFFFu, n, m);
+  if (lane == 0) wsum[warp] = n;
+  const int used = __syncthreads_count(h != 0ull);
+  n = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) n += wsum[w];
+  double bits = h ? -(double)h * log2((double)h / (double)n) : 0.0;
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) bits += __shfl_xor_sync(0xFFFFFFFFu, bits, m);
+  if (lane == 0) wbits[warp] = bits;
+  if (h) {
+    int rank = 0;
+    for (int c = 0; c < bins; ++c) {
+      const unsigned long long o = cnt[c];
+      rank += (o != 0ull && (o < h || (o == h && c < tid))) ? 1 : 0;
+    }
+    leaf[rank] = h;
+  }
+  __syncthreads();
+  if (tid != 0) return;
+  bits = 0.0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) bits += wbits[w];
+  entropy_out[blockIdx.x] = bits;
+  unsigned long long total = 0;
+  if (used == 1) {
+    total = n;  // a code word cannot be empty: one bit per coordinate
+  } else {
+    int il = 0, in = 0;
+    unsigned long long l0 = leaf[0], l1 = leaf[1], m0 = NONE, m1 = NONE;
+    for (int k = 0; k + 1 < used; ++k) {
+      const unsigned long long ll = l0 + l1, lm = l0 + m0, mm = m0 + m1;
+      unsigned long long sum = ll;
+      int dl = 2;
+      if (lm < sum) { sum = lm; dl = 1; }
+      if (mm < sum) { sum = mm; dl = 0; }
+      node[k] = sum;
+      total += sum;
+      il += dl;
+      in += 2 - dl;
+      l0 = leaf[il]; l1 = leaf[il + 1];
+      m0 = node[in]; m1 = node[in + 1];
     }
   }
-  flush();
+  huffman_out[blockIdx.x] = total;
 }
 
 }  // namespace
 
-cudaError_t launch_code_histogram(const HistArgs& a, cudaStream_t st) {
+cudaError_t launch_code_histogram(const HistArgs& a, int sm_count, cudaStream_t st) {
   if (a.ntiles <= 0 || a.N <= 0) return cudaSuccess;
-  const size_t sh = (size_t)(a.b <= 4 && (a.b == 1 || a.b == 2 || a.b == 4) ? 4 : 1) * (size_t)(((1 << a.b) + 3) / 4) * AT * sizeof(uint32_t);
-  const dim3 grid((unsigned)((a.ntiles + HRUN - 1) / HRUN), (unsigned)a.N);
-  auto go = [&](auto kernel) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    if (e != cudaSuccess) return e;
-    kernel<<<grid, AT, sh, st>>>(a);
-    return cudaGetLastError();
-  };
+  // Tiles per CTA (a run): the counts reach the message's histogram, a few hot addresses, once per run and segment, so
+  // runs are as long as about four CTAs per SM allow, 32 tiles at most.
+  const int64_t all = (int64_t)a.ntiles * a.N;
+  const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, all / (4 * (int64_t)sm_count)));
+  const dim3 grid((unsigned)((a.ntiles + run - 1) / run), (unsigned)a.N);
   switch (a.b) {
-    case 1: code_histogram_swar_kernel<1><<<grid, AT, 0, st>>>(a); return cudaGetLastError();
-    case 2: code_histogram_swar_kernel<2><<<grid, AT, 0, st>>>(a); return cudaGetLastError();
-    case 4: code_histogram_swar_kernel<4><<<grid, AT, 0, st>>>(a); return cudaGetLastError();
-    case 8: return go(code_histogram_kernel<8>);
-    default: return go(code_histogram_kernel<0>);
+    case 1: code_histogram_swar_kernel<1><<<grid, AT, 0, st>>>(a, run); break;
+    case 2: code_histogram_swar_kernel<2><<<grid, AT, 0, st>>>(a, run); break;
+    case 3: code_histogram_kernel<3><<<grid, HT, 0, st>>>(a, run); break;
+    case 4: code_histogram_swar_kernel<4><<<grid, AT, 0, st>>>(a, run); break;
+    case 5: code_histogram_kernel<5><<<grid, HT, 0, st>>>(a, run); break;
+    case 6: code_histogram_kernel<6><<<grid, HT, 0, st>>>(a, run); break;
+    case 7: code_histogram_kernel<7><<<grid, HT, 0, st>>>(a, run); break;
+    default: code_histogram_kernel<8><<<grid, HT, 0, st>>>(a, run); break;
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_coded_size(const unsigned long long* hist, int messages, int b, double* entropy_out,
+                              unsigned long long* huffman_out, cudaStream_t st) {
+  if (messages <= 0) return cudaSuccess;
+  coded_size_kernel<<<(unsigned)messages, 256, 0, st>>>(hist, 1 << b, entropy_out, huffman_out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_server_reduce(const ServerArgs& a, cudaStream_t st) {

@@ -3,13 +3,11 @@
 // bits.  All arithmetic of the method runs in the kernels of the other files.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <queue>
-#include <functional>
-#include <cmath>
 #include <vector>
 
 #include "../../include/lpc.h"
@@ -119,6 +117,8 @@ struct lpc_ctx {
   uint64_t q_done_version = ~0ull;
   unsigned int q_epoch = 0;
   int last_one_launch = 0;
+  unsigned long long* coded_host = nullptr;  // pinned: entropy (double) and Huffman length of coded_cap messages each
+  size_t coded_cap = 0;
   // graph replay
   cudaGraphExec_t graph = nullptr;
   cudaStream_t cap_stream = nullptr;  // used only to capture the graph
@@ -617,6 +617,7 @@ int lpc_destroy(lpc_ctx* c) {
                   c->partial_mu, c->partial_f, c->flags, c->ll, c->ll_vhat, c->q_pmax, c->q_ps1, c->q_ps2, c->q_scales, c->q_clip, c->q_done};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (c->coded_host) cudaFreeHost(c->coded_host);
   free_plan(c->inner_seg);
   free_plan(c->seg);
   free_plan(c->seg_out);
@@ -928,35 +929,6 @@ int lpc_scheme_bits(int scheme, int64_t d, int32_t b, int32_t N, uint64_t* bits_
   }
 }
 
-namespace {
-// n * H in bits for a histogram.
-double entropy_of(const unsigned long long* h, int bins) {
-  unsigned long long n = 0;
-  for (int c = 0; c < bins; ++c) n += h[c];
-  double bits = 0.0;
-  for (int c = 0; c < bins; ++c)
-    if (h[c]) bits -= (double)h[c] * std::log2((double)h[c] / (double)n);
-  return bits;
-}
-// Length of the message under Huffman's code for its own histogram: the sum of the weights of all merged nodes.
-uint64_t huffman_of(const unsigned long long* h, int bins) {
-  std::vector<unsigned long long> w;
-  for (int c = 0; c < bins; ++c)
-    if (h[c]) w.push_back(h[c]);
-  if (w.empty()) return 0;
-  if (w.size() == 1) return w[0];  // a code word cannot be empty: one bit per coordinate
-  std::priority_queue<unsigned long long, std::vector<unsigned long long>, std::greater<unsigned long long>> q(w.begin(), w.end());
-  uint64_t total = 0;
-  while (q.size() > 1) {
-    const unsigned long long x = q.top(); q.pop();
-    const unsigned long long y = q.top(); q.pop();
-    total += x + y;
-    q.push(x + y);
-  }
-  return total;
-}
-}  // namespace
-
 int lpc_message_entropy(lpc_ctx* c, const uint32_t* codes, int64_t len, const int64_t* seg_offsets, int32_t nseg,
                         unsigned long long* hist_dev, double* entropy_bits_out, uint64_t* huffman_bits_out) {
   if (!c) return LPC_ERR_INVALID_ARG;
@@ -971,15 +943,22 @@ int lpc_message_entropy(lpc_ctx* c, const uint32_t* codes, int64_t len, const in
   HistArgs a;
   a.codes = codes; a.stride_words = c->seg.stride_words; a.N = c->N; a.b = c->b; a.segs = c->seg.d_segs;
   a.tile_seg = c->seg.d_tile_seg; a.nseg = nseg; a.ntiles = c->seg.ntiles; a.hist = hist_dev;
-  { ProfScope ps_(c, LPC_KERNEL_OTHER); CU(c, launch_code_histogram(a, c->stream)); }
+  { ProfScope ps_(c, LPC_KERNEL_OTHER); CU(c, launch_code_histogram(a, c->sm_count, c->stream)); }
   if (!entropy_bits_out && !huffman_bits_out) return LPC_OK;  // histogram only: stays asynchronous
-  std::vector<unsigned long long> h(count);
-  CU(c, cudaMemcpyAsync(h.data(), hist_dev, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-  CU(c, cudaStreamSynchronize(c->stream));
-  for (size_t m = 0; m < (size_t)c->N * (size_t)nseg; ++m) {
-    if (entropy_bits_out) entropy_bits_out[m] = entropy_of(h.data() + m * bins, bins);
-    if (huffman_bits_out) huffman_bits_out[m] = huffman_of(h.data() + m * bins, bins);
+  // both sums on the device; the results land in pinned host memory that the context keeps
+  const size_t messages = (size_t)c->N * (size_t)nseg;
+  if (messages > c->coded_cap) {
+    CU(c, cudaStreamSynchronize(c->stream));
+    if (c->coded_host) { cudaFreeHost(c->coded_host); c->coded_host = nullptr; c->coded_cap = 0; }
+    CU(c, cudaHostAlloc(reinterpret_cast<void**>(&c->coded_host), messages * 16, cudaHostAllocDefault));
+    c->coded_cap = messages;
   }
+  double* ent = reinterpret_cast<double*>(c->coded_host);
+  unsigned long long* huf = c->coded_host + messages;
+  { ProfScope ps_(c, LPC_KERNEL_OTHER); CU(c, launch_coded_size(hist_dev, (int)messages, c->b, ent, huf, c->stream)); }
+  CU(c, cudaStreamSynchronize(c->stream));
+  if (entropy_bits_out) std::memcpy(entropy_bits_out, ent, messages * sizeof(double));
+  if (huffman_bits_out) std::memcpy(huffman_bits_out, huf, messages * sizeof(uint64_t));
   return LPC_OK;
 }
 

@@ -134,7 +134,10 @@ struct HistArgs {
   int ntiles;
   unsigned long long* hist;  // N * nseg * 2^b counts, added to (the caller clears them)
 };
-cudaError_t launch_code_histogram(const HistArgs& a, cudaStream_t st);
+cudaError_t launch_code_histogram(const HistArgs& a, int sm_count, cudaStream_t st);
+// Entropy bound and Huffman length of `messages` histograms of 2^b counts each; the outputs may be pinned host memory.
+cudaError_t launch_coded_size(const unsigned long long* hist, int messages, int b, double* entropy_out,
+                              unsigned long long* huffman_out, cudaStream_t st);
 
 }  // namespace lpc
 

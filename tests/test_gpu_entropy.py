@@ -41,6 +41,14 @@ def test_histogram_and_counts_match_oracle(b, N, length):
     _check(N, length, b, "gauss")
 
 
+@pytest.mark.parametrize("b", [3, 5, 6, 7, 8])
+@pytest.mark.parametrize("length", [15, 16 * 512 - 1, 8192 * 33 + 31])
+def test_lane_counter_widths(b, length):
+    """The table-of-lanes histogram: lengths around its units (16 bytes or 32 codes), runs and the ragged end; heavy tails
+    without clipping, so that nearly all codes have the same value."""
+    _check(3, length, b, "student_t3", offs=[0, min(9, length), length])
+
+
 def test_segments_heavy_tails_and_known_streams():
     _check(4, 30000, 4, "student_t3", offs=[0, 7, 7, 9000, 30000])
     # a stream built on the CPU with a known histogram: every code value c appears c + 1 times per 136 coordinates
