@@ -33,6 +33,8 @@ struct SegPlan {
   int32_t* d_tile_seg = nullptr;    // nullptr when nseg == 1
   uint64_t msg_bits = 0;            // sum over segments of 32 + b*len_s
   uint64_t version = 0;             // changes whenever the tables are rebuilt
+  int longest_tiles = 0;            // of one segment
+  int64_t whole_runs = 0;           // runs of 8 tiles that consist of whole tiles of one segment whose offset keeps 16-byte alignment
 };
 
 struct GraphKey {
@@ -230,6 +232,13 @@ int make_plan(lpc_ctx* c, SegPlan& p, int64_t len, int b, const int64_t* seg_off
   p.offsets[nseg] = len;
   p.segs = segs;
   p.tile_seg = tile_seg;
+  for (const SegInfo& g : segs) p.longest_tiles = std::max(p.longest_tiles, g.tile_count);
+  const int run = quantize_run_tiles();
+  for (int t0 = 0; t0 < p.ntiles; t0 += run) {
+    const int t1 = std::min(t0 + run, p.ntiles) - 1;
+    const SegInfo& g = p.segs[p.tile_seg[t0]];
+    if (p.tile_seg[t0] == p.tile_seg[t1] && g.off % 4 == 0 && (int64_t)(t1 + 1 - g.tile_first) * TILE <= g.len) p.whole_runs += 1;
+  }
   CU(c, cudaMalloc(&p.d_segs, sizeof(SegInfo) * nseg));
   CU(c, cudaMemcpyAsync(p.d_segs, p.segs.data(), sizeof(SegInfo) * nseg, cudaMemcpyHostToDevice, c->stream));
   if (nseg > 1 && p.ntiles > 0) {
@@ -865,25 +874,14 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   a.codes = codes_out; a.stride_words = p.stride_words; a.delta_out = delta_out;
   a.clipped_out = clipped_out ? clipped_out : c->q_clip; a.count_clipped = clipped_out ? 1 : 0; a.dev_status = c->dev_status;
   a.shared_scale = c->shared_scale;
-  {  // runs of the second pass that consist of whole tiles of one segment of 16-byte aligned vectors (per worker)
-    const int run = quantize_run_tiles();
-    const bool vec = aligned16(U) && (!U_sub || aligned16(U_sub)) && (ld % 4 == 0);
-    int64_t runs = 0;
-    const bool fixed_width = (c->b == 1 || c->b == 2 || c->b == 3 || c->b == 4 || c->b == 8);  // the other widths go tile by tile
-    for (int t0 = 0; vec && fixed_width && t0 < p.ntiles; t0 += run) {
-      const int t1 = std::min(t0 + run, p.ntiles) - 1;
-      const SegInfo& g = p.segs[p.tile_seg[t0]];
-      if (p.tile_seg[t0] == p.tile_seg[t1] && g.off % 4 == 0 && (int64_t)(t1 + 1 - g.tile_first) * TILE <= g.len) ++runs;
-    }
-    c->last_pipelined_runs = runs;
-  }
+  const bool vec = aligned16(U) && (!U_sub || aligned16(U_sub)) && (ld % 4 == 0);
+  const bool fixed_width = (c->b == 1 || c->b == 2 || c->b == 3 || c->b == 4 || c->b == 8);  // the other widths go tile by tile
+  c->last_pipelined_runs = vec && fixed_width ? p.whole_runs : 0;
   // one cooperative launch when the vectors stay in L2 between the statistics and the codes
   c->last_one_launch = 0;
   if (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
       (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) {
-    int max_tiles = 1;
-    for (const SegInfo& g : p.segs) max_tiles = std::max(max_tiles, g.tile_count);
-    if (c->q_done_version != p.version || ((uint64_t)c->q_epoch + 2) * (uint64_t)max_tiles >= 0x7FFFFFFFull) {
+    if (c->q_done_version != p.version || ((uint64_t)c->q_epoch + 2) * (uint64_t)std::max(p.longest_tiles, 1) >= 0x7FFFFFFFull) {
       CU(c, cudaMemsetAsync(c->q_done, 0, recs * 4, c->stream));
       c->q_done_version = p.version;
       c->q_epoch = 0;
@@ -899,7 +897,7 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
     }
   }
   if (c->last_one_launch) c->last_pipelined_runs = 0;
-  else CU(c, launch_quantize_pack(a, c->stream, c->profile ? prof_hook : nullptr, c));
+  else CU(c, launch_quantize_pack(a, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
   if (!c->shared_scale) c->step2_bits += p.msg_bits * (uint64_t)c->N * (uint64_t)(c->N - 1);  // scheme (a); the server schemes count in lpc_server_reduce
   return LPC_OK;
 }

@@ -21,8 +21,9 @@ struct SegInfo {
 
 struct ScaleRec {  // result of the scale rule for one (worker, segment)
   float delta, rdelta, T, lower;
-  uint32_t flags, pad0, pad1, pad2;
+  uint32_t flags, pad0, pad1, pad2;  // flags: bit 0 degenerate, bit 1 non-finite input, SCALE_NONE_OUTSIDE
 };
+constexpr uint32_t SCALE_NONE_OUTSIDE = 4u;  // the threshold is the largest magnitude: no coordinate is outside the hull
 
 struct QuantArgs {
   const float* U;
@@ -58,7 +59,7 @@ typedef void (*LaunchHook)(void* user, int kind, int begin);
 // Tiles per CTA of the second pass, and whether the run of tiles that starts at tile0 consists of whole tiles of one
 // segment (the condition, besides 16-byte aligned vectors and a non-degenerate scale, for its pipelined loop).
 int quantize_run_tiles();
-cudaError_t launch_quantize_pack(const QuantArgs& a, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
+cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
 // The same work in one cooperative launch, for vectors short enough to stay in L2 between the statistics and the codes
 // (b in 1..16, own scales).  done: N * nseg arrival counters, zero before the first call with a layout; epoch: calls
 // made with that layout since.

@@ -6,6 +6,8 @@
 // worker; a thread owns groups of 8 consecutive coordinates (two 128-bit loads, one Philox block,
 // 8*b packed bits).  All sums follow the balanced binary tree over the coordinate index, so the
 // scale -- and with it every code -- does not depend on the tiling.
+#include <type_traits>
+
 #include "lpc_device.cuh"
 #include "lpc_kernels.h"
 
@@ -39,9 +41,73 @@ __device__ __forceinline__ void load8(const float* __restrict__ p, const float* 
   }
 }
 
+// The launches of a call overlap (programmatic dependent launch): the next one's CTAs come in as this one's leave and wait
+// here until it has completed, which hides launch latency and the filling of the machine, about 2 us each.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+__device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
+// Eight whole values as four pairs: one 32-byte load where the alignment allows it, two 16-byte loads through L1
+// otherwise (without L1 each of them would fetch the whole sector).  LAST: nobody reads them again, L2 may drop them.
+template <bool LAST>
+__device__ __forceinline__ void load8v(const float* p, bool al32, f32x2* v) {
+  if (al32) {
+    if constexpr (LAST)
+      asm volatile("ld.global.L1::no_allocate.L2::evict_first.v4.b64 {%0, %1, %2, %3}, [%4];"
+                   : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+    else
+      asm volatile("ld.global.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];"
+                   : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+  } else {
+    asm volatile("ld.global.v2.b64 {%0, %1}, [%4];\n\tld.global.v2.b64 {%2, %3}, [%4+16];"
+                 : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+  }
+}
 
 // ---- pass 1: per-tile partial (max |u| as bit pattern, tree sums of u and u^2) ---------------------------
+__device__ __forceinline__ float max3_abs(float m, float a, float b) {
+  float r;  // a NaN among the operands comes out as NaN, whose bit pattern is above infinity's
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+  return r;
+}
+
+// max |u| into mx; with SUMS the tree sums of the eight values and of their squares, as one pair.
+template <bool SUMS>
+__device__ __forceinline__ f32x2 stats_group8(const f32x2* v, float& mx) {
+  f32x2 pr[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    float v0, v1;
+    unpack2(v[h], v0, v1);
+    mx = max3_abs(mx, v0, v1);
+    if constexpr (SUMS) {
+      float s0, s1;
+      unpack2(mul2_rn(v[h], v[h]), s0, s1);
+      pr[h] = pack2(add_rn(v0, v1), add_rn(s0, s1));
+    }
+  }
+  if constexpr (SUMS) return add2_rn(add2_rn(pr[0], pr[1]), add2_rn(pr[2], pr[3]));
+  else return 0ull;
+}
+
+// The warp's tree sums of its four sweeps, by recursive halving (9 shuffles instead of 40): afterwards lane l < 8 holds
+// S1 (bit 2 clear) or S2 of sweep 2 * bit 0 + bit 1.
+__device__ __forceinline__ float warp_sums4(const f32x2* pr, int lane) {
+  const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4;
+  const f32x2 k0 = add2_rn(u0 ? pr[2] : pr[0], __shfl_xor_sync(0xFFFFFFFFu, u0 ? pr[0] : pr[2], 1));
+  const f32x2 k1 = add2_rn(u0 ? pr[3] : pr[1], __shfl_xor_sync(0xFFFFFFFFu, u0 ? pr[1] : pr[3], 1));
+  const f32x2 k = add2_rn(u1 ? k1 : k0, __shfl_xor_sync(0xFFFFFFFFu, u1 ? k0 : k1, 2));
+  float a, b;
+  unpack2(k, a, b);
+  float r = add_rn(u2 ? b : a, __shfl_xor_sync(0xFFFFFFFFu, u2 ? a : b, 4));
+  r = add_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, 8));
+  return add_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, 16));
+}
+
+// Bound by memory: all of a thread's loads of a tile are under way before the first is used, and the sums of the four
+// sweeps share their shuffles.
 template <bool NEED_SUMS>
 __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int worker, float* sh1, float* sh2, uint32_t* shm) {
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
@@ -49,90 +115,141 @@ __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int wor
   const int64_t tstart = (int64_t)(tile - s.tile_first) * TILE;
   const float* p = a.U + (int64_t)worker * a.ld + s.off;
   const float* q = a.U_sub ? a.U_sub + (int64_t)worker * a.ld + s.off : nullptr;
-  const bool vec = aligned16(p) && (!q || aligned16(q));
+  const bool vec = aligned16(p) && (!q || aligned16(q)), al32 = aligned32(p) && (!q || aligned32(q));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  uint32_t mx = 0;
+  float mx = 0.f;
+  f32x2 pr[QITER];
+  if (vec && tstart + TILE <= s.len) {
+    const float* pt = p + tstart + tid * 8;
+    if (!q) {
+      f32x2 v[QITER][4];
 #pragma unroll
-  for (int it = 0; it < QITER; ++it) {
-    const int64_t j = tstart + (int64_t)it * QGROUP + tid * 8;
-    float v[8];
-    if (j < s.len) {
-      load8(p, q, j, s.len, vec, v);
+      for (int it = 0; it < QITER; ++it) load8v<false>(pt + it * QGROUP, al32, v[it]);
+#pragma unroll
+      for (int it = 0; it < QITER; ++it) pr[it] = stats_group8<NEED_SUMS>(v[it], mx);
     } else {
+      const float* qt = q + tstart + tid * 8;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = 0.f;
+      for (int half = 0; half < QITER; half += 2) {
+        f32x2 v[2][4], w[2][4];
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+          load8v<false>(pt + (half + it) * QGROUP, al32, v[it]);
+          load8v<false>(qt + (half + it) * QGROUP, al32, w[it]);
+        }
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+#pragma unroll
+          for (int h = 0; h < 4; ++h) v[it][h] = sub2_rn(v[it][h], w[it][h]);
+          pr[half + it] = stats_group8<NEED_SUMS>(v[it], mx);
+        }
+      }
     }
+  } else {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) mx = max(mx, __float_as_uint(fabsf(v[e])));
-    if (NEED_SUMS) {
-      float sq[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) sq[e] = mul_rn(v[e], v[e]);
-      const float s1 = warp_tree_sum(tree8(v));
-      const float s2 = warp_tree_sum(tree8(sq));
-      if (lane == 0) { sh1[it * 8 + warp] = s1; sh2[it * 8 + warp] = s2; }
+    for (int it = 0; it < QITER; ++it) {
+      float u[8];
+      load8(p, q, tstart + (int64_t)it * QGROUP + tid * 8, s.len, vec, u);
+      const f32x2 u2[4] = {pack2(u[0], u[1]), pack2(u[2], u[3]), pack2(u[4], u[5]), pack2(u[6], u[7])};
+      pr[it] = stats_group8<NEED_SUMS>(u2, mx);
     }
   }
-  mx = warp_max_u32(mx);
-  if (lane == 0) shm[warp] = mx;
+  const uint32_t wm = warp_max_u32(__float_as_uint(mx) & 0x7FFFFFFFu);
+  if (lane == 0) shm[warp] = wm;
+  if (NEED_SUMS) {
+    const float r = warp_sums4(pr, lane);
+    const int j = (((lane & 1) * 2) + ((lane >> 1) & 1)) * 8 + warp;
+    if (lane < 4) sh1[j] = r;
+    else if (lane < 8) sh2[j] = r;
+  }
   __syncthreads();
-  if (tid == 0) {
-    uint32_t m = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) m = max(m, shm[w]);
-    const int64_t o = (int64_t)worker * a.ntiles + tile;
-    a.pmax[o] = m;
-    if (NEED_SUMS) {
-      a.ps1[o] = smem_tree_sum(sh1, QITER * 8);
-      a.ps2[o] = smem_tree_sum(sh2, QITER * 8);
+  const int64_t o = (int64_t)worker * a.ntiles + tile;
+  if (warp == 0) {
+    const uint32_t m = warp_max_u32(shm[lane & 7]);
+    const float r = NEED_SUMS ? warp_tree_sum(sh1[lane]) : 0.f;
+    if (lane == 0) {
+      a.pmax[o] = m;
+      if (NEED_SUMS) a.ps1[o] = r;
     }
+  } else if (NEED_SUMS && warp == 1) {
+    const float r = warp_tree_sum(sh2[lane]);
+    if (lane == 0) a.ps2[o] = r;
   }
 }
 
 template <bool NEED_SUMS>
 __global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a) {
+  launch_dependents();
   __shared__ float sh1[QITER * 8], sh2[QITER * 8];
   __shared__ uint32_t shm[8];
   stats_tile<NEED_SUMS>(a, blockIdx.x, blockIdx.y, sh1, sh2, shm);
 }
 
-// Tree sum over `count` tile partials by one CTA of QT threads (leaf order = tile order).
-__device__ float block_tree_sum(const float* __restrict__ v, int count, float* sh8) {
-  int64_t P = 1;
+// Tree sums over `count` tile partials of both kinds by one CTA of QT threads (leaf order = tile order): a thread owns a
+// power-of-two stretch of leaves, eight loads of either array in flight.
+__device__ __forceinline__ void block_tree_sums(const float* __restrict__ v1, const float* __restrict__ v2, int count,
+                                                float* sh16, float& S1, float& S2) {
+  int P = 1;
   while (P < count) P <<= 1;
-  const int chunk = (P >= QT) ? (int)(P / QT) : 1;
+  const int chunk = (P >= QT) ? P / QT : 1;
   const int lo = threadIdx.x * chunk;
-  float stack[32];
-  int top = 0;
-  for (int i = 0; i < chunk; ++i) {
-    float cur = (lo + i < count) ? __ldcg(v + lo + i) : 0.f;  // written by other CTAs: read where they wrote it
-    int idx = i;
-    while (idx & 1) { cur = add_rn(stack[--top], cur); idx >>= 1; }
-    stack[top++] = cur;
+  float a = 0.f, b = 0.f;
+  if (chunk < 8) {
+    float x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // written by other CTAs: read where they wrote it
+      const bool in = i < chunk && lo + i < count;
+      x[i] = in ? __ldcg(v1 + lo + i) : 0.f;
+      y[i] = in ? __ldcg(v2 + lo + i) : 0.f;
+    }
+    if (chunk == 1) { a = x[0]; b = y[0]; }
+    else if (chunk == 2) { a = add_rn(x[0], x[1]); b = add_rn(y[0], y[1]); }
+    else { a = tree4(x[0], x[1], x[2], x[3]); b = tree4(y[0], y[1], y[2], y[3]); }
+  } else {
+    float st1[24], st2[24];  // one pending sum per level
+    int top = 0;
+    for (int i = 0; i < chunk; i += 8) {
+      float x[8], y[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const bool in = lo + i + e < count;
+        x[e] = in ? __ldcg(v1 + lo + i + e) : 0.f;
+        y[e] = in ? __ldcg(v2 + lo + i + e) : 0.f;
+      }
+      a = tree8(x);
+      b = tree8(y);
+      for (int idx = i >> 3; idx & 1; idx >>= 1) {
+        --top;
+        a = add_rn(st1[top], a);
+        b = add_rn(st2[top], b);
+      }
+      st1[top] = a;
+      st2[top] = b;
+      ++top;
+    }
   }
-  const float w = warp_tree_sum(stack[0]);
+  a = warp_tree_sum(a);
+  b = warp_tree_sum(b);
+  if ((threadIdx.x & 31) == 0) { sh16[threadIdx.x >> 5] = a; sh16[8 + (threadIdx.x >> 5)] = b; }
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) sh8[threadIdx.x >> 5] = w;
-  __syncthreads();
-  return tree8(sh8);
+  S1 = tree8(sh16);
+  S2 = tree8(sh16 + 8);
 }
 
 // ---- between the passes: one CTA per (segment, worker) finishes the reductions and applies Eq. 2 -------
 // The scale record of (segment, worker) from its tile partials, by all threads of the CTA; valid in thread 0.
-__device__ __forceinline__ ScaleRec finish_segment(const QuantArgs& a, int seg, int worker, float* sh8, uint32_t* shm) {
+__device__ __forceinline__ ScaleRec finish_segment(const QuantArgs& a, int seg, int worker, float* sh16, uint32_t* shm) {
   const SegInfo s = a.segs[seg];
   const int64_t base = (int64_t)worker * a.ntiles + s.tile_first;
   uint32_t mx = 0;
+#pragma unroll 8
   for (int t = threadIdx.x; t < s.tile_count; t += QT) mx = max(mx, __ldcg(a.pmax + base + t));
   mx = warp_max_u32(mx);
   if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = mx;
   float S1 = 0.f, S2 = 0.f;
-  if (a.clip_mode == CLIP_STD) {
-    S1 = block_tree_sum(a.ps1 + base, s.tile_count, sh8);
-    S2 = block_tree_sum(a.ps2 + base, s.tile_count, sh8);
-  }
-  __syncthreads();
+  if (a.clip_mode == CLIP_STD) block_tree_sums(a.ps1 + base, a.ps2 + base, s.tile_count, sh16, S1, S2);
+  else __syncthreads();
   ScaleRec r;
   r.delta = r.rdelta = r.T = r.lower = 0.f;
   r.flags = r.pad0 = r.pad1 = r.pad2 = 0;
@@ -142,15 +259,19 @@ __device__ __forceinline__ ScaleRec finish_segment(const QuantArgs& a, int seg, 
     for (int w = 0; w < 8; ++w) m = max(m, shm[w]);
     const Scale sc = make_scale(m, S1, S2, s.len, a.b, a.clip_mode, a.clip_value);
     r.delta = sc.delta; r.rdelta = sc.rdelta; r.T = sc.T; r.lower = sc.lower; r.flags = sc.flags;
+    // the threshold is the largest magnitude: nothing can lie outside the hull, and nothing has to be counted
+    if (sc.T >= __uint_as_float(m) && (!a.shared_scale || a.clip_mode == CLIP_NONE)) r.flags |= SCALE_NONE_OUTSIDE;
   }
   return r;
 }
 
 __global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
+  launch_dependents();
+  wait_for_launch_before();
   const int seg = blockIdx.x, worker = blockIdx.y;
-  __shared__ float sh8[8];
+  __shared__ float sh16[16];
   __shared__ uint32_t shm[8];
-  const ScaleRec r = finish_segment(a, seg, worker, sh8, shm);
+  const ScaleRec r = finish_segment(a, seg, worker, sh16, shm);
   if (threadIdx.x == 0) {
     const int64_t o = (int64_t)worker * a.nseg + seg;
     a.scales[o] = r;
@@ -191,10 +312,11 @@ __global__ void __launch_bounds__(32) share_scale_kernel(QuantArgs a) {
 // BITS = 1, 2, 3, 4, 8: register/shuffle packing with direct coalesced stores.
 // BITS = 0: any b in 1..16 read from the arguments; each thread's 8*b bits are b whole bytes, staged
 //           through shared memory and written out as words.
-// A CTA takes a run of QRUN consecutive tiles of one worker.  Runs that consist of whole tiles of one segment of
-// 16-byte aligned vectors (all but a segment's last tiles) go through a software-pipelined loop: the loads of the
-// next sweeps are in flight while the current ones are quantized, nothing is tested per group and every index is a
-// small offset from the run's base.  Everything else goes tile by tile through the general code.
+// A CTA takes a run of up to QRUN consecutive tiles of one worker.  Runs that consist of whole tiles of one segment of
+// 16-byte aligned vectors (all but a segment's last tiles) go through a software-pipelined loop: nothing is tested per
+// group and every index is a small offset from the run's base.  Everything else goes tile by tile through the general code.
+// Runs are handed out from the last worker's last tile back: the values that the first pass read last (up to some 80 MB)
+// are still in L2.
 constexpr int QRUN = 8;
 
 template <int BITS>
@@ -221,51 +343,44 @@ __device__ __forceinline__ void store_group(uint32_t* __restrict__ ot, int g, in
   }
 }
 
-// `nsweeps` sweeps of QGROUP coordinates from pt/qt (this thread's first group); HAS_Q: u = p - q.
-// A step covers SW sweeps (2 without a subtrahend, 1 with), i.e. four 16-byte loads per thread; the loads of step
-// i + 1 are issued before step i is quantized.
+// `nsweeps` sweeps (a multiple of 4) of QGROUP coordinates from pt/qt (this thread's first group); HAS_Q: u = p - q.
+// 64 bytes per thread are in flight while a group is quantized: a group's registers are loaded again as soon as its
+// values have been scaled and counted.
 template <int BITS, bool COUNT, bool HAS_Q>
 __device__ __forceinline__ void quantize_run(const QuantArgs& a, const ScaleRec& sc, const float* __restrict__ pt,
-                                             const float* __restrict__ qt, uint32_t block0, uint32_t* __restrict__ ot,
-                                             int nsweeps, int worker, int tid, int lane, float& fclip) {
-  constexpr int SW = HAS_Q ? 1 : 2;
-  const int nsteps = nsweeps / SW;  // a tile has QITER = 4 sweeps, so this is exact
-  float4 cur[4], nxt[4];
-  auto load = [&](float4* dst, int step) {
-#pragma unroll
-    for (int w = 0; w < SW; ++w) {
-      const int off = (step * SW + w) * QGROUP;
-      dst[2 * w] = __ldcs(reinterpret_cast<const float4*>(pt + off));
-      dst[2 * w + 1] = __ldcs(reinterpret_cast<const float4*>(pt + off + 4));
-      if (HAS_Q) {
-        dst[2] = __ldcs(reinterpret_cast<const float4*>(qt + off));
-        dst[3] = __ldcs(reinterpret_cast<const float4*>(qt + off + 4));
-      }
-    }
+                                             const float* __restrict__ qt, bool al32, uint32_t block0,
+                                             uint32_t* __restrict__ ot, int nsweeps, int worker, int tid, int lane, float& fclip) {
+  float s[8];
+  f32x2 v0[4], v1[4];
+  auto finish = [&](int sweep) {
+    const int g = sweep * (QGROUP / 8) + tid;  // coordinate group inside the run
+    const U4 r = stream_block(a.seed, TAG_ROUND, (uint32_t)worker, a.k, block0 + (uint32_t)g);
+    store_group<BITS>(ot, g, lane, quantize_scaled8<BITS>(s, r));
   };
-  auto work = [&](const float4* src, int step) {
-#pragma unroll
-    for (int w = 0; w < SW; ++w) {
-      float v[8] = {src[2 * w].x, src[2 * w].y, src[2 * w].z, src[2 * w].w,
-                    src[2 * w + 1].x, src[2 * w + 1].y, src[2 * w + 1].z, src[2 * w + 1].w};
-      if (HAS_Q) {
-        v[0] = __fsub_rn(v[0], src[2].x); v[1] = __fsub_rn(v[1], src[2].y); v[2] = __fsub_rn(v[2], src[2].z);
-        v[3] = __fsub_rn(v[3], src[2].w); v[4] = __fsub_rn(v[4], src[3].x); v[5] = __fsub_rn(v[5], src[3].y);
-        v[6] = __fsub_rn(v[6], src[3].z); v[7] = __fsub_rn(v[7], src[3].w);
-      }
-      const int g = (step * SW + w) * (QGROUP / 8) + tid;  // coordinate group inside the run
-      const U4 r = stream_block(a.seed, TAG_ROUND, (uint32_t)worker, a.k, block0 + (uint32_t)g);
-      const uint64_t lo = quantize_group8<BITS, COUNT>(v, sc.rdelta, r, sc.T, sc.lower, fclip);
-      store_group<BITS>(ot, g, lane, lo);
-    }
-  };
-  load(cur, 0);
+  load8v<true>(pt, al32, v0);
+  load8v<true>(HAS_Q ? qt : pt + QGROUP, al32, v1);
+  if constexpr (HAS_Q) {
 #pragma unroll 1
-  for (int step = 0; step < nsteps; step += 2) {  // nsteps is even: a tile is 2 or 4 steps
-    load(nxt, step + 1);
-    work(cur, step);
-    if (step + 2 < nsteps) load(cur, step + 2);
-    work(nxt, step + 1);
+    for (int sweep = 0; sweep < nsweeps; ++sweep) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) v0[h] = sub2_rn(v0[h], v1[h]);
+      scale_group8<COUNT>(v0, sc.rdelta, sc.T, sc.lower, fclip, s);
+      if (sweep + 1 < nsweeps) {
+        load8v<true>(pt + (sweep + 1) * QGROUP, al32, v0);
+        load8v<true>(qt + (sweep + 1) * QGROUP, al32, v1);
+      }
+      finish(sweep);
+    }
+  } else {
+#pragma unroll 1
+    for (int sweep = 0; sweep < nsweeps; sweep += 2) {
+      scale_group8<COUNT>(v0, sc.rdelta, sc.T, sc.lower, fclip, s);
+      if (sweep + 2 < nsweeps) load8v<true>(pt + (sweep + 2) * QGROUP, al32, v0);
+      finish(sweep);
+      scale_group8<COUNT>(v1, sc.rdelta, sc.T, sc.lower, fclip, s);
+      if (sweep + 2 < nsweeps) load8v<true>(pt + (sweep + 3) * QGROUP, al32, v1);
+      finish(sweep + 1);
+    }
   }
 }
 
@@ -369,34 +484,50 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, int tile, int 
   if (COUNT && lane == 0 && nclip) atomicAdd(&a.clipped_out[(int64_t)worker * a.nseg + seg], nclip);
 }
 
+// The run [tile, tile + whole) of whole tiles of one segment, by all threads of the CTA.
 template <int BITS, bool COUNT>
-__global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a) {
-  const int worker = blockIdx.y;
-  const int tile0 = blockIdx.x * QRUN;
-  const int ntl = min(QRUN, a.ntiles - tile0);
+__device__ __forceinline__ void quantize_whole_tiles(const QuantArgs& a, const SegInfo& s, const ScaleRec& sc, const float* p, const float* q,
+                                                     int tile, int whole, int seg, int worker) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t tstart = (int64_t)(tile - s.tile_first) * TILE;
+  const uint32_t block0 = s.block_base + (uint32_t)(tstart >> 3);
+  uint32_t* ot = a.codes + (int64_t)worker * a.stride_words + s.word_off + (tstart >> 5) * BITS;
+  const bool al32 = aligned32(p) && (!q || aligned32(q));
+  const float* pt = p + tstart + tid * 8;
+  float fclip = 0.f;
+  if (q) {
+    const float* qt = q + tstart + tid * 8;
+    if (COUNT && !(sc.flags & SCALE_NONE_OUTSIDE))
+      quantize_run<BITS, true, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+    else
+      quantize_run<BITS, false, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+  } else {
+    if (COUNT && !(sc.flags & SCALE_NONE_OUTSIDE))
+      quantize_run<BITS, true, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+    else
+      quantize_run<BITS, false, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+  }
+  const uint32_t nclip = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)fclip);
+  if (COUNT && lane == 0 && nclip) atomicAdd(&a.clipped_out[(int64_t)worker * a.nseg + seg], nclip);
+}
+
+template <int BITS, bool COUNT>
+__global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
+  wait_for_launch_before();
+  const int worker = (int)(gridDim.y - 1 - blockIdx.y);
+  const int tile0 = (int)(gridDim.x - 1 - blockIdx.x) * run;
+  const int ntl = min(run, a.ntiles - tile0);
   __shared__ __align__(16) uint8_t stage[BITS == 0 ? QT * 16 : 16];
   if constexpr (BITS != 0) {
     const int seg = a.tile_seg ? a.tile_seg[tile0] : 0;
     const int seg_last = a.tile_seg ? a.tile_seg[tile0 + ntl - 1] : 0;  // tiles are numbered segment by segment
     if (seg == seg_last) {
       const SegInfo s = a.segs[seg];
-      const int64_t tstart = (int64_t)(tile0 - s.tile_first) * TILE;
       const float* p = a.U + (int64_t)worker * a.ld + s.off;
       const float* q = a.U_sub ? a.U_sub + (int64_t)worker * a.ld + s.off : nullptr;
       const ScaleRec sc = a.scales[(int64_t)worker * a.nseg + seg];
-      if (aligned16(p) && (!q || aligned16(q)) && !(sc.flags & 1u) && tstart + (int64_t)ntl * TILE <= s.len) {
-        const int tid = threadIdx.x, lane = tid & 31;
-        const uint32_t block0 = s.block_base + (uint32_t)(tstart >> 3);
-        uint32_t* ot = a.codes + (int64_t)worker * a.stride_words + s.word_off + (tstart >> 5) * BITS;
-        float fclip = 0.f;
-        if (q)
-          quantize_run<BITS ? BITS : 1, COUNT, true>(a, sc, p + tstart + tid * 8, q + tstart + tid * 8, block0, ot,
-                                                     ntl * QITER, worker, tid, lane, fclip);
-        else
-          quantize_run<BITS ? BITS : 1, COUNT, false>(a, sc, p + tstart + tid * 8, nullptr, block0, ot, ntl * QITER,
-                                                      worker, tid, lane, fclip);
-        const uint32_t nclip = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)fclip);
-        if (COUNT && lane == 0 && nclip) atomicAdd(&a.clipped_out[(int64_t)worker * a.nseg + seg], nclip);
+      if (aligned16(p) && (!q || aligned16(q)) && !(sc.flags & 1u) && (int64_t)(tile0 + ntl - s.tile_first) * TILE <= s.len) {
+        quantize_whole_tiles<BITS ? BITS : 1, COUNT>(a, s, sc, p, q, tile0, ntl, seg, worker);
         return;
       }
     }
@@ -417,7 +548,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a) {
 // `epoch` waits for (epoch + 1) * tile_count arrivals.  A wait that runs out records a timeout and goes on.
 template <int BITS, bool COUNT, bool NEED_SUMS>
 __global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsigned int* done, unsigned int epoch, int cpw) {
-  __shared__ float sh1[QITER * 8], sh2[QITER * 8], sh8[8];
+  __shared__ float sh1[QITER * 8], sh2[QITER * 8], sh16[16];
   __shared__ uint32_t shm[8];
   __shared__ ScaleRec srec;
   __shared__ __align__(16) uint8_t stage[BITS == 0 ? QT * 16 : 16];
@@ -441,7 +572,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsi
     const int w = o / a.nseg, seg = o % a.nseg;
     if (a.segs[seg].tile_count != 0) continue;
     __syncthreads();
-    const ScaleRec r = finish_segment(a, seg, w, sh8, shm);
+    const ScaleRec r = finish_segment(a, seg, w, sh16, shm);
     if (tid == 0) { a.scales[o] = r; a.delta_out[o] = r.delta; a.clipped_out[o] = 0; }
   }
   int tile = t0;
@@ -465,7 +596,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsi
       }
     }
     __syncthreads();
-    const ScaleRec r = finish_segment(a, seg, worker, sh8, shm);
+    const ScaleRec r = finish_segment(a, seg, worker, sh16, shm);
     if (tid == 0) {
       srec = r;
       if (tile == s.tile_first) {  // one CTA leaves the record and the scale for the caller
@@ -485,20 +616,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsi
         const int64_t full_tiles = s.len / TILE;  // tiles of the segment without a ragged end
         whole = (int)max((int64_t)0, min((int64_t)(tend - s.tile_first), full_tiles) - (tile - s.tile_first));
       }
-      if (whole > 0) {
-        const int64_t tstart = (int64_t)(tile - s.tile_first) * TILE;
-        const uint32_t block0 = s.block_base + (uint32_t)(tstart >> 3);
-        uint32_t* ot = a.codes + (int64_t)worker * a.stride_words + s.word_off + (tstart >> 5) * BITS;
-        float fclip = 0.f;
-        if (q)
-          quantize_run<BITS ? BITS : 1, COUNT, true>(a, sc, p + tstart + tid * 8, q + tstart + tid * 8, block0, ot, whole * QITER,
-                                                     worker, tid, lane, fclip);
-        else
-          quantize_run<BITS ? BITS : 1, COUNT, false>(a, sc, p + tstart + tid * 8, nullptr, block0, ot, whole * QITER, worker,
-                                                      tid, lane, fclip);
-        const uint32_t nclip = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)fclip);
-        if (COUNT && lane == 0 && nclip) atomicAdd(&a.clipped_out[o], nclip);
-      }
+      if (whole > 0) quantize_whole_tiles<BITS ? BITS : 1, COUNT>(a, s, sc, p, q, tile, whole, seg, worker);
     }
     for (int t = tile + whole; t < tend; ++t) {
       if (BITS == 0 && t > tile) __syncthreads();  // the staging buffer is reused from tile to tile
@@ -549,6 +667,7 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
 }
 
 __global__ void __launch_bounds__(QT) bypass_kernel(QuantArgs a) {
+  wait_for_launch_before();
   const int tile = blockIdx.x, worker = blockIdx.y;
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
   bypass_tile(a, tile, worker, a.scales[(int64_t)worker * a.nseg + seg]);
@@ -602,51 +721,63 @@ cudaError_t launch_quantize_fused(const QuantArgs& a, unsigned int* done, unsign
 
 int quantize_run_tiles() { return QRUN; }
 
-cudaError_t launch_quantize_pack(const QuantArgs& a, cudaStream_t st, LaunchHook hook, void* user) {
+cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
   if (a.N <= 0 || a.nseg <= 0) return cudaSuccess;
   const dim3 grid((unsigned)(a.ntiles > 0 ? a.ntiles : 1), (unsigned)a.N), block(QT);
+  bool first = true;  // the call's first launch waits for everything before it, the others overlap with the one before
+  auto launch = [&](auto kernel, dim3 g, auto... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = first ? 0 : 1;
+    first = false;
+    return cudaLaunchKernelEx(&cfg, kernel, a, args...);
+  };
+  cudaError_t e = cudaSuccess;
   if (a.ntiles > 0) {
     if (hook) hook(user, 3 /* LPC_KERNEL_QUANT_STATS */, 1);
-    if (a.clip_mode == CLIP_STD)
-      stats_kernel<true><<<grid, block, 0, st>>>(a);
-    else
-      stats_kernel<false><<<grid, block, 0, st>>>(a);
+    e = a.clip_mode == CLIP_STD ? launch(stats_kernel<true>, grid) : launch(stats_kernel<false>, grid);
     if (hook) hook(user, 3, 0);
+    if (e != cudaSuccess) return e;
   }
   if (hook) hook(user, 5 /* LPC_KERNEL_OTHER */, 1);
-  finish_kernel<<<dim3((unsigned)a.nseg, (unsigned)a.N), block, 0, st>>>(a);  // also covers empty segments
+  e = launch(finish_kernel, dim3((unsigned)a.nseg, (unsigned)a.N));  // also covers empty segments
   if (hook) hook(user, 5, 0);
-  if (a.shared_scale) share_scale_kernel<<<(unsigned)a.nseg, 32, 0, st>>>(a);
-  if (a.ntiles <= 0) return cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (a.shared_scale) {
+    share_scale_kernel<<<(unsigned)a.nseg, 32, 0, st>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    first = true;
+  }
+  if (a.ntiles <= 0) return cudaSuccess;
   struct Close {  // closes the timing scope of the second pass on every return path
     LaunchHook h; void* u;
     ~Close() { if (h) h(u, 4, 0); }
   } close_{hook, user};
   if (hook) hook(user, 4 /* LPC_KERNEL_QUANT_PACK */, 1);
-  const dim3 grid_tiles = grid;  // one tile per CTA: the statistics pass and the full-precision bypass
-  const dim3 grid_runs((unsigned)((a.ntiles + QRUN - 1) / QRUN), (unsigned)a.N);  // QRUN tiles per CTA
-  if (a.count_clipped) {
-    switch (a.b) {
-      case 1: quantize_kernel<1, true><<<grid_runs, block, 0, st>>>(a); break;
-      case 2: quantize_kernel<2, true><<<grid_runs, block, 0, st>>>(a); break;
-      case 3: quantize_kernel<3, true><<<grid_runs, block, 0, st>>>(a); break;
-      case 4: quantize_kernel<4, true><<<grid_runs, block, 0, st>>>(a); break;
-      case 8: quantize_kernel<8, true><<<grid_runs, block, 0, st>>>(a); break;
-      case 32: bypass_kernel<<<grid_tiles, block, 0, st>>>(a); break;
-      default: quantize_kernel<0, true><<<grid_runs, block, 0, st>>>(a); break;
-    }
-  } else {
-    switch (a.b) {
-      case 1: quantize_kernel<1, false><<<grid_runs, block, 0, st>>>(a); break;
-      case 2: quantize_kernel<2, false><<<grid_runs, block, 0, st>>>(a); break;
-      case 3: quantize_kernel<3, false><<<grid_runs, block, 0, st>>>(a); break;
-      case 4: quantize_kernel<4, false><<<grid_runs, block, 0, st>>>(a); break;
-      case 8: quantize_kernel<8, false><<<grid_runs, block, 0, st>>>(a); break;
-      case 32: bypass_kernel<<<grid_tiles, block, 0, st>>>(a); break;
-      default: quantize_kernel<0, false><<<grid_runs, block, 0, st>>>(a); break;
-    }
+  // Tiles per CTA: long runs read ahead better, but the last wave of CTAs (four to an SM) should be a small part of all:
+  // eight tiles from 8 waves on (8 x 2^24: 3.5 waves of eight cost 10 % against 7 of four), fewer below.
+  int run = QRUN;
+  while (run > 1 && (int64_t)a.ntiles * a.N < 8ll * run * 4 * sm_count) run >>= 1;
+  const dim3 runs((unsigned)((a.ntiles + run - 1) / run), (unsigned)a.N);
+  auto pack = [&](auto width) {
+    constexpr int B = decltype(width)::value;
+    return a.count_clipped ? launch(quantize_kernel<B, true>, runs, run) : launch(quantize_kernel<B, false>, runs, run);
+  };
+  switch (a.b) {
+    case 1: return pack(std::integral_constant<int, 1>());
+    case 2: return pack(std::integral_constant<int, 2>());
+    case 3: return pack(std::integral_constant<int, 3>());
+    case 4: return pack(std::integral_constant<int, 4>());
+    case 8: return pack(std::integral_constant<int, 8>());
+    case 32: return launch(bypass_kernel, grid);
+    default: return pack(std::integral_constant<int, 0>());
   }
-  return cudaGetLastError();
 }
 
 }  // namespace lpc

@@ -7,6 +7,7 @@ import of a symbol fails loudly.
 import ctypes as C
 import os
 
+import numpy as np
 import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -91,8 +92,8 @@ class LpcError(RuntimeError):
         self.code = code
 
 
-def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+def _ptr(t):  # a c_void_p argument also takes the plain integer
+    return None if t is None else t.data_ptr()
 
 
 def _seg(seg_offsets):
@@ -154,6 +155,8 @@ class Context:
             self.device = torch.device("cuda", torch.cuda.current_device())
         self.n, self.d, self.N, self.B, self.b = n, d, N, B, b
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        self._lib = lib()
+        self._layouts = {}  # (length, bits) -> (seg_offsets, C array, segments, stride in words) of the last call
         rc = lib().lpc_init(C.byref(self._h), _ptr(X), _ptr(y), n, d, loss, lambda_l1, N, B, b, clip_mode, clip_value,
                             seed, C.c_void_p(self.stream.cuda_stream))
         if rc != OK:
@@ -165,6 +168,19 @@ class Context:
     def _ck(self, rc):
         if rc != OK:
             raise LpcError(rc, lib().lpc_last_error(self._h).decode())
+
+    def _layout(self, length, bits, seg_offsets):
+        """C array of the offsets, segment count and stride in words; the last layout of a width is kept, because a training
+        loop asks for the same one in every round."""
+        hit = self._layouts.get((length, bits))
+        if hit is not None and hit[0] == seg_offsets:
+            return hit[1:]
+        arr, nseg = _seg(seg_offsets)
+        _, stride = packed_layout(length, bits, seg_offsets)
+        if len(self._layouts) >= 16:
+            self._layouts.clear()
+        self._layouts[(length, bits)] = (None if seg_offsets is None else list(seg_offsets), arr, nseg, stride)
+        return arr, nseg, stride
 
     def close(self):
         if self._h:
@@ -225,48 +241,51 @@ class Context:
 
     def quantize_pack(self, U, k, U_sub=None, seg_offsets=None, codes_out=None, delta_out=None, clipped_out=None):
         """U: (N, len) fp32 CUDA tensor (row stride = U.stride(0)).  Returns (codes, delta, clipped)."""
-        assert U.is_cuda and U.dtype == torch.float32 and U.dim() == 2 and U.shape[0] == self.N and U.stride(1) == 1
-        length, ld = U.shape[1], (U.stride(0) if U.shape[0] > 1 else max(U.shape[1], 1))
+        shape, strides = U.shape, U.stride()
+        assert U.is_cuda and U.dtype == torch.float32 and len(shape) == 2 and shape[0] == self.N and strides[1] == 1
+        length = shape[1]
+        ld = strides[0] if shape[0] > 1 else max(length, 1)
         if U_sub is not None:
-            assert U_sub.shape == U.shape and U_sub.stride() == U.stride() and U_sub.dtype == torch.float32
-        arr, nseg = _seg(seg_offsets)
-        _, stride = packed_layout(length, self.b, seg_offsets)
+            assert U_sub.shape == shape and U_sub.stride() == strides and U_sub.dtype == torch.float32
+        arr, nseg, stride = self._layout(length, self.b, seg_offsets)
         if codes_out is None:
             codes_out = torch.empty((self.N, stride), dtype=torch.int32, device=U.device)
         if delta_out is None:
             delta_out = torch.empty((self.N, nseg), dtype=torch.float32, device=U.device)
         if clipped_out is None:
             clipped_out = torch.empty((self.N, nseg), dtype=torch.int32, device=U.device)
-        self._ck(lib().lpc_quantize_pack(self._h, _ptr(U), _ptr(U_sub), length, ld, arr, nseg, k, _ptr(codes_out),
-                                         _ptr(delta_out), _ptr(clipped_out)))
+        rc = self._lib.lpc_quantize_pack(self._h, U.data_ptr(), _ptr(U_sub), length, ld, arr, nseg, k, codes_out.data_ptr(),
+                                         delta_out.data_ptr(), clipped_out.data_ptr())
+        if rc != OK:
+            self._ck(rc)
         return codes_out, delta_out, clipped_out
 
     def unpack_average_prox(self, codes, delta, length, x, eta, lambda_l1, mu=None, seg_offsets=None, v_out=None):
-        arr, nseg = _seg(seg_offsets)
-        self._ck(lib().lpc_unpack_average_prox(self._h, _ptr(codes), _ptr(delta), length, arr, nseg, _ptr(mu), _ptr(x),
-                                               eta, lambda_l1, _ptr(v_out)))
+        arr, nseg, _ = self._layout(length, self.b, seg_offsets)
+        rc = self._lib.lpc_unpack_average_prox(self._h, _ptr(codes), _ptr(delta), length, arr, nseg, _ptr(mu), _ptr(x),
+                                               eta, lambda_l1, _ptr(v_out))
+        if rc != OK:
+            self._ck(rc)
         return x
 
     def message_entropy(self, codes, length, seg_offsets=None, hist_out=None, host_counts=True):
         """Histogram of every (worker, segment) message and, on the host, its entropy bound and Huffman length in bits.
         Returns (hist (N, nseg, 2^b) int64 CUDA tensor, entropy (N, nseg) or None, huffman (N, nseg) or None)."""
-        arr, nseg = _seg(seg_offsets)
+        arr, nseg, _ = self._layout(length, self.b, seg_offsets)
         if hist_out is None:
             hist_out = torch.empty((self.N, nseg, 1 << self.b), dtype=torch.int64, device=codes.device)
-        ent = (C.c_double * (self.N * nseg))() if host_counts else None
-        huf = (C.c_uint64 * (self.N * nseg))() if host_counts else None
-        self._ck(lib().lpc_message_entropy(self._h, _ptr(codes), length, arr, nseg, _ptr(hist_out), ent, huf))
         if not host_counts:
+            self._ck(self._lib.lpc_message_entropy(self._h, _ptr(codes), length, arr, nseg, _ptr(hist_out), None, None))
             return hist_out, None, None
-        import numpy as np
-        return (hist_out, np.array(ent[:], dtype=np.float64).reshape(self.N, nseg),
-                np.array(huf[:], dtype=np.uint64).reshape(self.N, nseg))
+        ent, huf = np.empty((self.N, nseg), dtype=np.float64), np.empty((self.N, nseg), dtype=np.uint64)
+        self._ck(self._lib.lpc_message_entropy(self._h, _ptr(codes), length, arr, nseg, _ptr(hist_out),
+                                               C.cast(ent.ctypes.data, _f64p), C.cast(huf.ctypes.data, _u64p)))
+        return hist_out, ent, huf
 
     def server_reduce(self, codes, length, scheme, k, seg_offsets=None, codes_out=None):
         """The server of scheme (b) or (c): N streams of b bits in, one stream out.  Returns (codes_out, bits_out)."""
-        arr, nseg = _seg(seg_offsets)
         bo = sum_bits(self.b, self.N) if scheme == SCHEME_SERVER_SUM else self.b
-        _, stride = packed_layout(length, bo, seg_offsets)
+        arr, nseg, stride = self._layout(length, bo, seg_offsets)
         if codes_out is None:
             codes_out = torch.empty((1, stride), dtype=torch.int32, device=codes.device)
         self._ck(lib().lpc_server_reduce(self._h, _ptr(codes), length, arr, nseg, scheme, k, _ptr(codes_out)))
