@@ -93,6 +93,8 @@ __global__ void __launch_bounds__(AT) unpack_average_prox_kernel(AggArgs a) {
   const int tid = threadIdx.x;
   const int b = (BITS == 0) ? a.b : BITS;
 
+  launch_dependents();
+  wait_for_launch_before();
   extern __shared__ float sdelta[];
   for (int i = tid; i < a.N; i += AT) sdelta[i] = a.delta[(int64_t)i * a.nseg + seg];
   __syncthreads();
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(AT) unpack_average_prox_kernel(AggArgs a) {
       store8f(a.ysum + s.off, j, s.len, vec, sv);
     }
   }
-  if (a.k_counter && blockIdx.x == 0 && tid == 0) *a.k_counter += 1;
+  if (a.k_counter && blockIdx.x == 0 && tid == 0) *a.k_counter += a.k_step;
 }
 
 // The server of schemes (b) and (c) (Section 3.2).  A thread owns 8 consecutive coordinates per sweep: it adds the
@@ -793,15 +795,14 @@ cudaError_t launch_unpack_average_prox(const AggArgs& a, cudaStream_t st) {
   const dim3 grid((unsigned)(a.ntiles * a.split)), block(AT);
   const size_t sh = (size_t)a.N * sizeof(float);
   switch (a.b) {
-    case 1: unpack_average_prox_kernel<1><<<grid, block, sh, st>>>(a); break;
-    case 2: unpack_average_prox_kernel<2><<<grid, block, sh, st>>>(a); break;
-    case 3: unpack_average_prox_kernel<3><<<grid, block, sh, st>>>(a); break;
-    case 4: unpack_average_prox_kernel<4><<<grid, block, sh, st>>>(a); break;
-    case 8: unpack_average_prox_kernel<8><<<grid, block, sh, st>>>(a); break;
-    case 32: unpack_average_prox_kernel<32><<<grid, block, sh, st>>>(a); break;
-    default: unpack_average_prox_kernel<0><<<grid, block, sh, st>>>(a); break;
+    case 1: return launch_overlapped(unpack_average_prox_kernel<1>, grid, block, sh, st, a);
+    case 2: return launch_overlapped(unpack_average_prox_kernel<2>, grid, block, sh, st, a);
+    case 3: return launch_overlapped(unpack_average_prox_kernel<3>, grid, block, sh, st, a);
+    case 4: return launch_overlapped(unpack_average_prox_kernel<4>, grid, block, sh, st, a);
+    case 8: return launch_overlapped(unpack_average_prox_kernel<8>, grid, block, sh, st, a);
+    case 32: return launch_overlapped(unpack_average_prox_kernel<32>, grid, block, sh, st, a);
+    default: return launch_overlapped(unpack_average_prox_kernel<0>, grid, block, sh, st, a);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace lpc

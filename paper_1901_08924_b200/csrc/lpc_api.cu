@@ -325,7 +325,7 @@ InnerArgs inner_args(lpc_ctx* c, uint64_t k_base, const uint64_t* k_dev, int has
   a.codes = c->codes; a.stride_words = c->inner_seg.stride_words; a.pad_words = c->inner_seg.stride_words;
   a.delta = c->delta; a.clipped_part = c->clipped_part;
   a.idx_tap = c->idx_tap; a.coef_tap = c->coef_tap; a.u_tap = c->tap_u ? c->u_tap : nullptr;
-  a.dev_status = c->dev_status; a.CS = c->CS; a.SL = c->SL; a.stream_stages = c->innerStages;
+  a.dev_status = c->dev_status; a.CS = c->CS; a.SL = c->SL; a.stream_stages = c->innerStages; a.overlapped = 0;
   return a;
 }
 
@@ -337,7 +337,7 @@ AggArgs agg_args(lpc_ctx* c, const SegPlan& p, const uint32_t* codes, const floa
   a.divisor = divisor;
   a.split = aggregate_split(p.ntiles, c->sm_count);
   a.segs = p.d_segs; a.tile_seg = p.d_tile_seg; a.nseg = p.nseg; a.ntiles = p.ntiles;
-  a.mu = mu; a.x = x; a.eta = eta; a.lambda_l1 = lambda_l1; a.v_out = v_out; a.k_counter = nullptr;
+  a.mu = mu; a.x = x; a.eta = eta; a.lambda_l1 = lambda_l1; a.v_out = v_out; a.k_counter = nullptr; a.k_step = 0;
   a.mode = 0; a.y = nullptr; a.z = nullptr; a.ysum = nullptr; a.vhat = nullptr; a.alpha = 0.f; a.inv4L = 0.f;
   a.cy = 1.f; a.cz = 1.f; a.wy = 1.f;
   return a;
@@ -357,25 +357,30 @@ int replan_inner(lpc_ctx* c) {
   return LPC_OK;
 }
 
+constexpr int GRAPH_STEPS = 128;  // inner steps per captured graph
+
 // One LPC inner step enqueued on the stream (Algorithm 1 steps 6-10).
-int enqueue_lpc_step(lpc_ctx* c, float eta, uint64_t k_base, const uint64_t* k_dev, uint64_t* k_counter) {
+// `overlapped`: the step before it was enqueued just now, so that only the iterate has to be waited for.
+int enqueue_lpc_step(lpc_ctx* c, float eta, uint64_t k_base, const uint64_t* k_dev, uint64_t* k_counter, bool overlapped) {
   InnerArgs ia = inner_args(c, k_base, k_dev, 0);
+  ia.overlapped = overlapped ? 1 : 0;
   { ProfScope ps_(c, LPC_KERNEL_WORKER); CU(c, launch_inner(ia, c->innerSmem, c->stream)); }
   // the training loops always average over the context's N workers (Eq. 3); LPC_OPT_AVERAGE_DIVISOR does not apply
   AggArgs ag = agg_args(c, c->inner_seg, c->codes, c->delta, c->mu, c->x, eta, c->lambda_l1, c->tap_u ? c->v_tap : nullptr, c->N);
-  ag.k_counter = k_counter;
+  ag.k_counter = k_counter; ag.k_step = GRAPH_STEPS;
   { ProfScope ps_(c, LPC_KERNEL_AGGREGATE); CU(c, launch_unpack_average_prox(ag, c->stream)); }
   return LPC_OK;
 }
 
 // One ALPC step enqueued on the stream (Algorithm 2 steps 6-13).
 int enqueue_alpc_step(lpc_ctx* c, float tau1, float tau2, float alpha, float inv4L, uint64_t k_base,
-                      const uint64_t* k_dev, uint64_t* k_counter) {
+                      const uint64_t* k_dev, uint64_t* k_counter, bool overlapped) {
   { ProfScope ps_(c, LPC_KERNEL_OTHER); CU(c, launch_coupling(c->zv, c->xt, c->yv, tau1, tau2, c->d, c->x, c->stream)); }
   InnerArgs ia = inner_args(c, k_base, k_dev, 1);
+  ia.overlapped = overlapped ? 1 : 0;
   { ProfScope ps_(c, LPC_KERNEL_WORKER); CU(c, launch_inner(ia, c->innerSmem, c->stream)); }
   AggArgs ag = agg_args(c, c->inner_seg, c->codes, c->delta, c->mu, c->x, 0.f, c->lambda_l1, c->tap_u ? c->v_tap : nullptr, c->N);
-  ag.k_counter = k_counter;
+  ag.k_counter = k_counter; ag.k_step = GRAPH_STEPS;
   ag.mode = 1; ag.y = c->yv; ag.z = c->zv; ag.ysum = c->ysum; ag.vhat = c->vhat; ag.alpha = alpha; ag.inv4L = inv4L;
   if (c->sigma > 0.f) {  // each product and sum below is one fp32 operation, as on the device
     volatile float t1 = c->sigma * inv4L, t2 = alpha * c->sigma;
@@ -392,13 +397,11 @@ int enqueue_alpc_step(lpc_ctx* c, float tau1, float tau2, float alpha, float inv
   return LPC_OK;
 }
 
-constexpr int GRAPH_STEPS = 128;  // inner steps per captured graph
-
 int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) {
   if (count < 0) return fail(c, LPC_ERR_INVALID_ARG, "count < 0");
   if (!has_model(c) || !c->inner_ok) return fail(c, LPC_ERR_UNSUPPORTED, "no linear model or d too large for the fused step");
-  auto one = [&](uint64_t kb, const uint64_t* kd, uint64_t* kc) {
-    return kind == 0 ? enqueue_lpc_step(c, p[0], kb, kd, kc) : enqueue_alpc_step(c, p[0], p[1], p[2], p[3], kb, kd, kc);
+  auto one = [&](uint64_t kb, const uint64_t* kd, uint64_t* kc, bool overlapped) {
+    return kind == 0 ? enqueue_lpc_step(c, p[0], kb, kd, kc, overlapped) : enqueue_alpc_step(c, p[0], p[1], p[2], p[3], kb, kd, kc, overlapped);
   };
   int64_t done = 0;
   const bool loop_ok = (kind == 0) ? c->persist_ok : c->apersist_ok;
@@ -464,7 +467,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
       CU(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
       c->stream = c->cap_stream;
       int rc = LPC_OK;
-      for (int i = 0; i < GRAPH_STEPS && rc == LPC_OK; ++i) rc = one(0, c->k_dev, c->k_dev);
+      for (int i = 0; i < GRAPH_STEPS && rc == LPC_OK; ++i) rc = one((uint64_t)i, c->k_dev, i == GRAPH_STEPS - 1 ? c->k_dev : nullptr, i > 0);
       c->stream = user;
       cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
       if (rc != LPC_OK) { if (g) cudaGraphDestroy(g); return rc; }
@@ -481,7 +484,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
       done += GRAPH_STEPS;
     }
   }
-  for (; done < count; ++done) TRY(one(k0 + (uint64_t)done, nullptr, nullptr));
+  for (int64_t i = 0; done < count; ++done, ++i) TRY(one(k0 + (uint64_t)done, nullptr, nullptr, i > 0));
   const uint64_t per_step = (32ull + (uint64_t)c->b * (uint64_t)c->d) * (uint64_t)c->N * (uint64_t)(c->N - 1);
   c->step2_bits += per_step * (uint64_t)count;
   return LPC_OK;

@@ -22,10 +22,13 @@
 // coordinates of u and add the rows -- still in shared memory -- into u, then hand the stage back; one refills
 // the stages.  Every hand-over is an mbarrier phase, so waiting warps sleep in hardware and take no issue slots or
 // shared-memory bandwidth from the working ones.  Each row is read from HBM once.
+#include <atomic>
+
 #include <cooperative_groups.h>
 
 #include "lpc_device.cuh"
 #include "lpc_inner.h"
+#include "lpc_kernels.h"
 
 namespace cg = cooperative_groups;
 
@@ -108,6 +111,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
   unsigned char* dyn = smem_raw + ((sizeof(Smem) + 15) & ~(size_t)15);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  launch_dependents();
   LPC_PHASE_MARK(0);
   constexpr int NT = STREAM ? SNT : IT;  // the streaming path runs more warps, specialised by role
   const int rank = (int)cluster.block_rank();
@@ -204,9 +208,12 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
   }
 
   // ---- this thread's coordinates and the iterate at them ---------------------------------------------------
+  // Sampling, the barriers and the first copies of rows above need nothing of the step before and run while its last kernel
+  // is leaving; the iterate does.  (Streaming: the margin warps wait, everything that is written comes after them.)
+  if constexpr (!STREAM) wait_for_launch_before();
   float xr[MAXP][8];
 #pragma unroll
-  for (int p = 0; p < MAXP; ++p) {
+  for (int p = 0; !STREAM && p < MAXP; ++p) {
     const int off = p * IGROUP + tid * 8;  // offset inside the slice
 #pragma unroll
     for (int e = 0; e < 8; ++e) xr[p][e] = 0.f;
@@ -312,6 +319,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       constexpr int SMW = 4, QB = NBK / SMW;  // warps per side; blocks per warp
       static_assert(SDW == 2 * SMW && QB * SG == 16, "one 16-value recursive-halving reduction per group");
       const int wq = warp % SMW;
+      wait_for_launch_before();
       float4 xs[QB];
 #pragma unroll
       for (int q = 0; q < QB; ++q) {
@@ -348,12 +356,12 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
               sv[(h + j) * QB + q] = tree4(mul_rn(v[j][q].x, xs[q].x), mul_rn(v[j][q].y, xs[q].y), mul_rn(v[j][q].z, xs[q].z),
                                            mul_rn(v[j][q].w, xs[q].w));
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.ebar[g % R]);  // this warp has read its quarter of the stage
         WarpHalving<SG * QB, 0>::run(sv, lane);  // lane holds the 32-lane tree sum of (row, block) halving_index<4>(lane)
         float part = sv[0];
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 8));  // blocks 2k, 2k+1 of the row
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 4));
+        // this warp has read, and used, its quarter of the stage
+        mbar_arrive_after(&sm.ebar[g % R], __any_sync(0xFFFFFFFFu, __float_as_uint(part) == 0x7FFFFFFFu), lane == 0);
         if ((lane >> 2) < CS && myrow < cnt)
           st_async_cluster(&sm.parts[g % SSLOTS][(myrow * MAXCS + rank) * SMW + wq], &sm.pbar[g % SSLOTS],
                            (uint32_t)(lane >> 2), __float_as_uint(part));
@@ -380,8 +388,14 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
 #pragma unroll
             for (int q = 0; q < UC; ++q) v[j][q] = row4(s * SG + j, q * (IGROUP / UC) + t * 4);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.ebar[s]);  // release: the loads above are performed before the arrival counts
+        // The stage may be overwritten once everybody has arrived, and an arrival can overtake shared-memory reads whose
+        // results nobody has used yet: the vote uses one word of each of them.
+        uint32_t x = 0;
+#pragma unroll
+        for (int j = 0; j < SG; ++j)
+#pragma unroll
+          for (int q = 0; q < UC; ++q) x ^= __float_as_uint(v[j][q].x);
+        mbar_arrive_after(&sm.ebar[s], __any_sync(0xFFFFFFFFu, x == 0x7FFFFFFFu), lane == 0);
       };
       auto add = [&](int g, const float4 (&v)[SG][UC]) {
         const int cnt = min(SG, B - g * SG);
@@ -744,20 +758,30 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
 
 template <int BITS, bool STREAM>
 cudaError_t launch_t(const InnerArgs& a, size_t smem, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(inner_kernel<BITS, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the attribute is raised to what a launch needs once per device, not on every step
+  static std::atomic<size_t> allowed[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || allowed[dev].load(std::memory_order_relaxed) < smem) {
+    e = cudaFuncSetAttribute(inner_kernel<BITS, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) allowed[dev].store(smem, std::memory_order_relaxed);
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.CS, (unsigned)(a.N + (a.has_J ? 1 : 0)), 1);
   cfg.blockDim = dim3(STREAM ? SNT : IT, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)a.CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = a.overlapped ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, inner_kernel<BITS, STREAM>, a);
 }
 
@@ -773,6 +797,8 @@ __global__ void clipped_sum_kernel(const uint32_t* __restrict__ part, int N, uin
 // x = tau1*z + tau2*x~ + (1 - tau1 - tau2)*y  (Algorithm 2 step 6), evaluated as ((tau1*z)+(tau2*x~))+(tau3*y).
 __global__ void coupling_kernel(const float* __restrict__ z, const float* __restrict__ xt, const float* __restrict__ y,
                                 float tau1, float tau2, int d, float* __restrict__ x) {
+  launch_dependents();
+  wait_for_launch_before();
   const float tau3 = __fsub_rn(__fsub_rn(1.0f, tau1), tau2);
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < d) x[j] = add_rn(add_rn(mul_rn(tau1, z[j]), mul_rn(tau2, xt[j])), mul_rn(tau3, y[j]));
@@ -860,8 +886,7 @@ cudaError_t launch_clipped_sum(const uint32_t* part, int N, uint32_t* out, cudaS
 
 cudaError_t launch_coupling(const float* z, const float* xt, const float* y, float tau1, float tau2, int d, float* x,
                             cudaStream_t st) {
-  coupling_kernel<<<(d + 255) / 256, 256, 0, st>>>(z, xt, y, tau1, tau2, d, x);
-  return cudaGetLastError();
+  return launch_overlapped(coupling_kernel, dim3((unsigned)((d + 255) / 256)), dim3(256), 0, st, z, xt, y, tau1, tau2, d, x);
 }
 
 cudaError_t launch_mean_y(float* ysum, float inv_m, int d, float* x, cudaStream_t st) {

@@ -34,6 +34,7 @@ struct InnerArgs {
   unsigned int* dev_status;
   int CS;                  // CTAs per cluster
   int SL;                  // coordinates per CTA slice
+  int overlapped;          // 1: may come in while earlier kernels are leaving that write nothing but this step's point
   int stream_stages;       // 0: the B rows are resident in shared memory; > 0: they stream through that many ring stages
 };
 

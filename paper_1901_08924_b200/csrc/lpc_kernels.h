@@ -7,6 +7,22 @@ namespace lpc {
 
 constexpr int TILE = 8192;  // coordinates per CTA tile of the standalone quantizer / aggregator kernels
 
+// Launches a kernel that calls wait_for_launch_before, so that it overlaps with the tail of the kernel before it.
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // One tensor segment of a (segmented) vector.
 struct SegInfo {
   int64_t off;         // first element in the vector
@@ -81,7 +97,8 @@ struct AggArgs {
   float eta;
   float lambda_l1;
   float* v_out;     // nullable
-  uint64_t* k_counter;  // nullable: incremented by one when the kernel finishes (graph replay)
+  uint64_t* k_counter;  // nullable: incremented by k_step when the kernel finishes (graph replay)
+  uint64_t k_step;
   // mode 1 (Algorithm 2, steps 12-13): x is read only (the coupled point x_{k+1}) and instead of the
   // proximal step on x the kernel updates  y = soft(x - inv4L*v, inv4L*lambda_l1),
   // z = soft(z - alpha*vhat, alpha*lambda_l1),  ysum += y.

@@ -41,11 +41,6 @@ __device__ __forceinline__ void load8(const float* __restrict__ p, const float* 
   }
 }
 
-// The launches of a call overlap (programmatic dependent launch): the next one's CTAs come in as this one's leave and wait
-// here until it has completed, which hides launch latency and the filling of the machine, about 2 us each.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 __device__ __forceinline__ bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
@@ -181,6 +176,7 @@ __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int wor
 template <bool NEED_SUMS>
 __global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a) {
   launch_dependents();
+  wait_for_launch_before();
   __shared__ float sh1[QITER * 8], sh2[QITER * 8];
   __shared__ uint32_t shm[8];
   stats_tile<NEED_SUMS>(a, blockIdx.x, blockIdx.y, sh1, sh2, shm);
@@ -286,6 +282,8 @@ __global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
 // record of the segment.  Workers whose own vector is zero then send zeros on the shared grid; when every worker
 // is degenerate nothing changes.  One warp per segment.
 __global__ void __launch_bounds__(32) share_scale_kernel(QuantArgs a) {
+  launch_dependents();
+  wait_for_launch_before();
   const int seg = blockIdx.x, lane = threadIdx.x;
   float bestT = -1.f;
   int best = -1;
@@ -513,6 +511,7 @@ __device__ __forceinline__ void quantize_whole_tiles(const QuantArgs& a, const S
 
 template <int BITS, bool COUNT>
 __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
+  launch_dependents();
   wait_for_launch_before();
   const int worker = (int)(gridDim.y - 1 - blockIdx.y);
   const int tile0 = (int)(gridDim.x - 1 - blockIdx.x) * run;
@@ -548,6 +547,8 @@ __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
 // `epoch` waits for (epoch + 1) * tile_count arrivals.  A wait that runs out records a timeout and goes on.
 template <int BITS, bool COUNT, bool NEED_SUMS>
 __global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsigned int* done, unsigned int epoch, int cpw) {
+  launch_dependents();
+  wait_for_launch_before();
   __shared__ float sh1[QITER * 8], sh2[QITER * 8], sh16[16];
   __shared__ uint32_t shm[8];
   __shared__ ScaleRec srec;
@@ -667,6 +668,7 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
 }
 
 __global__ void __launch_bounds__(QT) bypass_kernel(QuantArgs a) {
+  launch_dependents();
   wait_for_launch_before();
   const int tile = blockIdx.x, worker = blockIdx.y;
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
@@ -711,11 +713,13 @@ cudaError_t launch_quantize_fused(const QuantArgs& a, unsigned int* done, unsign
   cfg.blockDim = dim3(QT, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident or the launch fails: they wait on one another
   attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k, a, done, epoch, (int)cpw);
 }
 
@@ -724,20 +728,7 @@ int quantize_run_tiles() { return QRUN; }
 cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
   if (a.N <= 0 || a.nseg <= 0) return cudaSuccess;
   const dim3 grid((unsigned)(a.ntiles > 0 ? a.ntiles : 1), (unsigned)a.N), block(QT);
-  bool first = true;  // the call's first launch waits for everything before it, the others overlap with the one before
-  auto launch = [&](auto kernel, dim3 g, auto... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = g;
-    cfg.blockDim = block;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = first ? 0 : 1;
-    first = false;
-    return cudaLaunchKernelEx(&cfg, kernel, a, args...);
-  };
+  auto launch = [&](auto kernel, dim3 g, auto... args) { return launch_overlapped(kernel, g, block, 0, st, a, args...); };
   cudaError_t e = cudaSuccess;
   if (a.ntiles > 0) {
     if (hook) hook(user, 3 /* LPC_KERNEL_QUANT_STATS */, 1);
@@ -750,9 +741,7 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
   if (hook) hook(user, 5, 0);
   if (e != cudaSuccess) return e;
   if (a.shared_scale) {
-    share_scale_kernel<<<(unsigned)a.nseg, 32, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    first = true;
+    if ((e = launch_overlapped(share_scale_kernel, dim3((unsigned)a.nseg), dim3(32), 0, st, a)) != cudaSuccess) return e;
   }
   if (a.ntiles <= 0) return cudaSuccess;
   struct Close {  // closes the timing scope of the second pass on every return path
@@ -761,9 +750,9 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
   } close_{hook, user};
   if (hook) hook(user, 4 /* LPC_KERNEL_QUANT_PACK */, 1);
   // Tiles per CTA: long runs read ahead better, but the last wave of CTAs (four to an SM) should be a small part of all:
-  // eight tiles from 8 waves on (8 x 2^24: 3.5 waves of eight cost 10 % against 7 of four), fewer below.
+  // as long as there are three waves (8 x 2^23: 103 us with two tiles, 119 with one; 8 x 2^24: 187 us with four, 195 with two).
   int run = QRUN;
-  while (run > 1 && (int64_t)a.ntiles * a.N < 8ll * run * 4 * sm_count) run >>= 1;
+  while (run > 1 && (int64_t)a.ntiles * a.N < 3ll * run * 4 * sm_count) run >>= 1;
   const dim3 runs((unsigned)((a.ntiles + run - 1) / run), (unsigned)a.N);
   auto pack = [&](auto width) {
     constexpr int B = decltype(width)::value;
