@@ -882,7 +882,10 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   c->last_pipelined_runs = vec && fixed_width ? p.whole_runs : 0;
   // one cooperative launch when the vectors stay in L2 between the statistics and the codes
   c->last_one_launch = 0;
-  if (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
+  if (c->one_launch && quantize_fits_cluster(a, c->sm_count)) {
+    { ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED); CU(c, launch_quantize_cluster(a, c->stream)); }
+    c->last_one_launch = 1;
+  } else if (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
       (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) {
     if (c->q_done_version != p.version || ((uint64_t)c->q_epoch + 2) * (uint64_t)std::max(p.longest_tiles, 1) >= 0x7FFFFFFFull) {
       CU(c, cudaMemsetAsync(c->q_done, 0, recs * 4, c->stream));

@@ -81,6 +81,10 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
 // made with that layout since.
 cudaError_t launch_quantize_fused(const QuantArgs& a, unsigned int* done, unsigned int epoch, int sm_count, cudaStream_t st);
 
+// The same for short vectors, one cluster per worker and nothing looked at twice.
+bool quantize_fits_cluster(const QuantArgs& a, int sm_count);
+cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st);
+
 struct AggArgs {
   const uint32_t* codes;
   int64_t stride_words;

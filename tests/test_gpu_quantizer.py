@@ -200,3 +200,33 @@ def test_bit_counters_follow_table1():
     s1, s2 = ctx.comm_bits()
     assert s1 == 0 and s2 == 2 * orc.broadcast_bits(length, b, N) == 2 * 24384
     ctx.close()
+
+
+@pytest.mark.parametrize("b", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("length", [127, 2049, 2 * 8192 + 1, 5 * 8192 - 3, 65535, 65536])
+def test_cluster_per_worker_matches_the_three_launches(b, length):
+    """Vectors of at most eight tiles: one cluster per worker (1, 2, 4 or 8 CTAs), ragged and full, with a subtrahend, a row
+    stride off 32-byte boundaries and a zero vector among the workers; bit for bit what the other path gives, and the
+    oracle's for one worker."""
+    N, seed, k = 5, 99, 3
+    g = torch.Generator().manual_seed(b * 1000 + length)
+    ld = (length + 3) // 4 * 4 + 4
+    base, sub = torch.randn(N, ld, generator=g), torch.randn(N, ld, generator=g)
+    base[2] = sub[2]  # a zero difference: degenerate scale
+    U, S = base.to(DEV)[:, :length], sub.to(DEV)[:, :length]
+    for clip, value in ((orc.CLIP_STD, 1.5), (orc.CLIP_NONE, 1.0)):
+        for subtrahend in (None, S):
+            got = {}
+            for one in (1, 0):
+                ctx = _ctx(N, b, clip, value, seed)
+                ctx.set_option(lpc.OPT_ONE_LAUNCH_QUANTIZE, one)
+                got[one] = [t.clone() for t in ctx.quantize_pack(U, k, U_sub=subtrahend)]
+                ctx.sync_status()
+                assert ctx.query(lpc.INFO_QUANT_ONE_LAUNCH) == one
+                ctx.close()
+            W = orc.packed_words(length, b)
+            assert torch.equal(got[1][0][:, :W], got[0][0][:, :W])
+            assert torch.equal(got[1][1].view(torch.int32), got[0][1].view(torch.int32)) and torch.equal(got[1][2], got[0][2])
+    u = (base[3, :length] - sub[3, :length]).numpy()  # the last combination: no clipping, with the subtrahend
+    w, dl, _ = orc.quantize_pack(u, b, orc.CLIP_NONE, 1.0, seed, 3, k)
+    assert (_u32(got[1][0])[3, : w.size] == w).all() and got[1][1][3, 0].item() == dl
