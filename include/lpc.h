@@ -85,7 +85,7 @@ typedef struct lpc_ctx lpc_ctx;
 #define LPC_OPT_SHARED_SCALE 6  /* 1: lpc_quantize_pack gives every worker the unified scale delta_t = max_i delta_t^i of the parameter-server schemes (b), (c) of Section 3.2; needs b in 2..16 */
 #define LPC_OPT_AVERAGE_DIVISOR 7 /* lpc_unpack_average_prox (and only it: the training loops always average over N) divides the decoded sum by this count instead of the context's N (0 = N): the worker count behind a server's sum stream */
 #define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits */
-#define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack uses one launch for inputs of at most LPC_ONE_LAUNCH_BYTES */
+#define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack may take its short-vector path (one launch where a vector fits a cluster) for inputs of at most LPC_ONE_LAUNCH_BYTES */
 #define LPC_ONE_LAUNCH_BYTES (48ll << 20)
 #define LPC_OPT_LOOP_COOPERATIVE 9 /* 1 (default): the one-launch loops are cooperative launches (the driver guarantees that all their CTAs are resident together, which they rely on).  0: a plain cluster launch of the same grid, for profilers that cannot replay a cooperative cluster launch; use it only on a GPU that runs nothing else (the launch plan has checked that all clusters fit, and every wait in the kernel is bounded, so a grid that is not resident together ends with LPC_ERR_TIMEOUT instead of hanging) */
 
@@ -180,10 +180,10 @@ int lpc_packed_words(int64_t len, int32_t b, int64_t* words_out); /* ceil(len*b/
  *   codes_out  N * stride_words words, stride from lpc_packed_layout
  *   delta_out  N * nseg floats
  *   clipped_out nullable, N * nseg counts of coordinates outside the hull
- * Vectors longer than L2 are read twice (once for ||u||_inf and the variance, once to quantize) by three launches;
- * when all N vectors together take at most LPC_ONE_LAUNCH_BYTES the call is ONE launch: for vectors of at most 65,536
- * values in one segment a cluster per worker that keeps the values in registers, else a cooperative launch whose second
- * look at the values is served by L2 (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches both off).  Same codes either way.
+ * Vectors longer than L2 are read twice (once for ||u||_inf and the variance, once to quantize) by three launches that overlap;
+ * when all N vectors together take at most LPC_ONE_LAUNCH_BYTES the second look is served by L2, and vectors of at most
+ * 65,536 values in one segment take ONE launch, a cluster per worker that keeps the values in registers
+ * (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches that off).  Same codes either way.
  * N, b and the clip rule come from the context.
  */
 int lpc_quantize_pack(lpc_ctx* ctx, const float* U, const float* U_sub, int64_t len, int64_t ld,
@@ -294,7 +294,7 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
 #define LPC_INFO_STEP_RING_STAGES 8        /* per-step kernel: 0 = minibatch rows resident on chip, else ring stages they stream through */
 #define LPC_INFO_LOOP_COORDS_PER_THREAD 11  /* one-launch loop: consecutive coordinates a thread owns (8, 4 or 2; 0: not available) */
 #define LPC_INFO_ALPC_LOOP_COORDS_PER_THREAD 12
-#define LPC_INFO_QUANT_ONE_LAUNCH 13        /* last lpc_quantize_pack: 1 when it ran as one launch */
+#define LPC_INFO_QUANT_ONE_LAUNCH 13        /* last lpc_quantize_pack: 1 when the input was short enough (LPC_ONE_LAUNCH_BYTES) for the short-vector path and LPC_OPT_ONE_LAUNCH_QUANTIZE allowed it */
 #define LPC_INFO_AGGREGATE_SPLIT 9         /* last lpc_unpack_average_prox: CTAs that shared one tile of 8192 coordinates (1, 2 or 4) */
 #define LPC_INFO_QUANT_PIPELINED_RUNS 10   /* last lpc_quantize_pack: runs of 8 tiles per worker that were whole tiles of one segment and
                                               so took the second pass's software-pipelined loop (unless that worker's scale was

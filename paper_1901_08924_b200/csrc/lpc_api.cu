@@ -32,8 +32,6 @@ struct SegPlan {
   SegInfo* d_segs = nullptr;
   int32_t* d_tile_seg = nullptr;    // nullptr when nseg == 1
   uint64_t msg_bits = 0;            // sum over segments of 32 + b*len_s
-  uint64_t version = 0;             // changes whenever the tables are rebuilt
-  int longest_tiles = 0;            // of one segment
   int64_t whole_runs = 0;           // runs of 8 tiles that consist of whole tiles of one segment whose offset keeps 16-byte alignment
 };
 
@@ -112,12 +110,8 @@ struct lpc_ctx {
   ScaleRec* q_scales = nullptr;
   uint32_t* q_clip = nullptr;
   size_t q_scale_cap = 0;
-  // one-launch quantizer: arrival counters per (worker, segment), valid for one layout; calls made with it so far
   int loop_cooperative = 1;       // LPC_OPT_LOOP_COOPERATIVE
   int one_launch = 1;             // LPC_OPT_ONE_LAUNCH_QUANTIZE
-  unsigned int* q_done = nullptr;
-  uint64_t q_done_version = ~0ull;
-  unsigned int q_epoch = 0;
   int last_one_launch = 0;
   unsigned long long* coded_host = nullptr;  // pinned: entropy (double) and Huffman length of coded_cap messages each
   size_t coded_cap = 0;
@@ -222,9 +216,7 @@ int make_plan(lpc_ctx* c, SegPlan& p, int64_t len, int b, const int64_t* seg_off
   const int rc = layout(len, b, seg_offsets, nseg, segs, tile_seg, &stride, &bits);
   if (rc != LPC_OK) return fail(c, rc, "invalid segment layout");
   CU(c, cudaStreamSynchronize(c->stream));  // the old tables may still be in use
-  const uint64_t version = p.version + 1;
   free_plan(p);
-  p.version = version;
   p.len = len; p.b = b; p.nseg = nseg; p.stride_words = stride; p.msg_bits = bits;
   p.ntiles = (int)tile_seg.size();
   p.offsets.resize(nseg + 1);
@@ -232,7 +224,6 @@ int make_plan(lpc_ctx* c, SegPlan& p, int64_t len, int b, const int64_t* seg_off
   p.offsets[nseg] = len;
   p.segs = segs;
   p.tile_seg = tile_seg;
-  for (const SegInfo& g : segs) p.longest_tiles = std::max(p.longest_tiles, g.tile_count);
   const int run = quantize_run_tiles();
   for (int t0 = 0; t0 < p.ntiles; t0 += run) {
     const int t1 = std::min(t0 + run, p.ntiles) - 1;
@@ -626,7 +617,7 @@ int lpc_destroy(lpc_ctx* c) {
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   void* ptrs[] = {c->x, c->xt, c->mu, c->margins, c->yv, c->zv, c->ysum, c->vhat, c->v_tap, c->u_tap, c->codes,
                   c->delta, c->clipped_part, c->clipped, c->idx_tap, c->coef_tap, c->k_dev, c->dev_status, c->f_dev,
-                  c->partial_mu, c->partial_f, c->flags, c->ll, c->ll_vhat, c->q_pmax, c->q_ps1, c->q_ps2, c->q_scales, c->q_clip, c->q_done};
+                  c->partial_mu, c->partial_f, c->flags, c->ll, c->ll_vhat, c->q_pmax, c->q_ps1, c->q_ps2, c->q_scales, c->q_clip};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->coded_host) cudaFreeHost(c->coded_host);
@@ -863,12 +854,10 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   const size_t recs = (size_t)c->N * (size_t)nseg;
   if (recs > c->q_scale_cap) {
     CU(c, cudaStreamSynchronize(c->stream));
-    if (c->q_scales) { cudaFree(c->q_scales); cudaFree(c->q_clip); cudaFree(c->q_done); c->q_scales = nullptr; c->q_clip = nullptr; c->q_done = nullptr; }
+    if (c->q_scales) { cudaFree(c->q_scales); cudaFree(c->q_clip); c->q_scales = nullptr; c->q_clip = nullptr; }
     c->q_scale_cap = 0;
     CU(c, cudaMalloc(&c->q_scales, recs * sizeof(ScaleRec))); CU(c, cudaMalloc(&c->q_clip, recs * 4));
-    CU(c, cudaMalloc(&c->q_done, recs * 4));
     c->q_scale_cap = recs;
-    c->q_done_version = ~0ull;
   }
   QuantArgs a;
   a.U = U; a.U_sub = U_sub; a.ld = ld; a.N = c->N; a.b = c->b; a.clip_mode = c->clip_mode; a.clip_value = c->clip_value;
@@ -880,30 +869,15 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   const bool vec = aligned16(U) && (!U_sub || aligned16(U_sub)) && (ld % 4 == 0);
   const bool fixed_width = (c->b == 1 || c->b == 2 || c->b == 3 || c->b == 4 || c->b == 8);  // the other widths go tile by tile
   c->last_pipelined_runs = vec && fixed_width ? p.whole_runs : 0;
-  // one cooperative launch when the vectors stay in L2 between the statistics and the codes
-  c->last_one_launch = 0;
-  if (c->one_launch && quantize_fits_cluster(a, c->sm_count)) {
-    { ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED); CU(c, launch_quantize_cluster(a, c->stream)); }
-    c->last_one_launch = 1;
-  } else if (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
-      (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) {
-    if (c->q_done_version != p.version || ((uint64_t)c->q_epoch + 2) * (uint64_t)std::max(p.longest_tiles, 1) >= 0x7FFFFFFFull) {
-      CU(c, cudaMemsetAsync(c->q_done, 0, recs * 4, c->stream));
-      c->q_done_version = p.version;
-      c->q_epoch = 0;
-    }
-    cudaError_t e;
-    { ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED); e = launch_quantize_fused(a, c->q_done, c->q_epoch, c->sm_count, c->stream); }
-    if (e == cudaSuccess) {
-      c->q_epoch += 1;
-      c->last_one_launch = 1;
-    } else {
-      cudaGetLastError();  // the launch was refused: nothing ran, use the three launches
-      c->one_launch = 0;
-    }
-  }
+  c->last_one_launch = (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
+                        (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) ? 1 : 0;
   if (c->last_one_launch) c->last_pipelined_runs = 0;
-  else CU(c, launch_quantize_pack(a, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
+  if (c->last_one_launch && quantize_fits_cluster(a, c->sm_count)) {
+    ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
+    CU(c, launch_quantize_cluster(a, c->stream));
+  } else {
+    CU(c, launch_quantize_pack(a, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
+  }
   if (!c->shared_scale) c->step2_bits += p.msg_bits * (uint64_t)c->N * (uint64_t)(c->N - 1);  // scheme (a); the server schemes count in lpc_server_reduce
   return LPC_OK;
 }

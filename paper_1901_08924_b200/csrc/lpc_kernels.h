@@ -64,7 +64,7 @@ struct QuantArgs {
   uint32_t* codes;
   int64_t stride_words;
   float* delta_out;       // N * nseg
-  uint32_t* clipped_out;  // N * nseg, cleared by the finish kernel (never null: internal scratch when the caller gives none)
+  uint32_t* clipped_out;  // N * nseg, cleared with the scale (never null: internal scratch when the caller gives none)
   int count_clipped;      // 0: skip counting the coordinates outside the hull (the counts stay zero)
   int shared_scale;       // 1: every worker quantizes with delta_t = max_i delta_t^i (schemes (b), (c) of Section 3.2)
   unsigned int* dev_status;
@@ -76,11 +76,6 @@ typedef void (*LaunchHook)(void* user, int kind, int begin);
 // segment (the condition, besides 16-byte aligned vectors and a non-degenerate scale, for its pipelined loop).
 int quantize_run_tiles();
 cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
-// The same work in one cooperative launch, for vectors short enough to stay in L2 between the statistics and the codes
-// (b in 1..16, own scales).  done: N * nseg arrival counters, zero before the first call with a layout; epoch: calls
-// made with that layout since.
-cudaError_t launch_quantize_fused(const QuantArgs& a, unsigned int* done, unsigned int epoch, int sm_count, cudaStream_t st);
-
 // The same for short vectors, one cluster per worker and nothing looked at twice.
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count);
 cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st);

@@ -8,7 +8,6 @@
 // scale -- and with it every code -- does not depend on the tiling.
 #include <cooperative_groups.h>
 
-#include <atomic>
 #include <type_traits>
 
 #include "lpc_device.cuh"
@@ -236,9 +235,29 @@ __device__ __forceinline__ void block_tree_sums(const float* __restrict__ v1, co
   S2 = tree8(sh16 + 8);
 }
 
-// ---- between the passes: one CTA per (segment, worker) finishes the reductions and applies Eq. 2 -------
-// The scale record of (segment, worker) from its tile partials, by all threads of the CTA; valid in thread 0.
-__device__ __forceinline__ ScaleRec finish_segment(const QuantArgs& a, int seg, int worker, float* sh16, uint32_t* shm) {
+// ---- between the passes: Eq. 2 from the tile partials --------------------------------------------------------------
+// The scale record of (segment, worker), the scale for the caller and the cleared count; one thread.
+__device__ __forceinline__ void write_scale(const QuantArgs& a, const SegInfo& s, int seg, int worker, uint32_t m, float S1, float S2) {
+  const Scale sc = make_scale(m, S1, S2, s.len, a.b, a.clip_mode, a.clip_value);
+  ScaleRec r;
+  r.delta = sc.delta; r.rdelta = sc.rdelta; r.T = sc.T; r.lower = sc.lower; r.flags = sc.flags;
+  r.pad0 = r.pad1 = r.pad2 = 0;
+  // the threshold is the largest magnitude: nothing can lie outside the hull, and nothing has to be counted
+  if (sc.T >= __uint_as_float(m) && (!a.shared_scale || a.clip_mode == CLIP_NONE)) r.flags |= SCALE_NONE_OUTSIDE;
+  const int64_t o = (int64_t)worker * a.nseg + seg;
+  a.scales[o] = r;
+  a.delta_out[o] = r.delta;
+  a.clipped_out[o] = 0;
+  if (r.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
+}
+
+// One CTA per (segment, worker); also covers segments without a single coordinate.
+__global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
+  launch_dependents();
+  wait_for_launch_before();
+  __shared__ float sh16[16];
+  __shared__ uint32_t shm[8];
+  const int seg = blockIdx.x, worker = blockIdx.y;
   const SegInfo s = a.segs[seg];
   const int64_t base = (int64_t)worker * a.ntiles + s.tile_first;
   uint32_t mx = 0;
@@ -249,34 +268,11 @@ __device__ __forceinline__ ScaleRec finish_segment(const QuantArgs& a, int seg, 
   float S1 = 0.f, S2 = 0.f;
   if (a.clip_mode == CLIP_STD) block_tree_sums(a.ps1 + base, a.ps2 + base, s.tile_count, sh16, S1, S2);
   else __syncthreads();
-  ScaleRec r;
-  r.delta = r.rdelta = r.T = r.lower = 0.f;
-  r.flags = r.pad0 = r.pad1 = r.pad2 = 0;
   if (threadIdx.x == 0) {
     uint32_t m = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) m = max(m, shm[w]);
-    const Scale sc = make_scale(m, S1, S2, s.len, a.b, a.clip_mode, a.clip_value);
-    r.delta = sc.delta; r.rdelta = sc.rdelta; r.T = sc.T; r.lower = sc.lower; r.flags = sc.flags;
-    // the threshold is the largest magnitude: nothing can lie outside the hull, and nothing has to be counted
-    if (sc.T >= __uint_as_float(m) && (!a.shared_scale || a.clip_mode == CLIP_NONE)) r.flags |= SCALE_NONE_OUTSIDE;
-  }
-  return r;
-}
-
-__global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
-  launch_dependents();
-  wait_for_launch_before();
-  const int seg = blockIdx.x, worker = blockIdx.y;
-  __shared__ float sh16[16];
-  __shared__ uint32_t shm[8];
-  const ScaleRec r = finish_segment(a, seg, worker, sh16, shm);
-  if (threadIdx.x == 0) {
-    const int64_t o = (int64_t)worker * a.nseg + seg;
-    a.scales[o] = r;
-    a.delta_out[o] = r.delta;
-    a.clipped_out[o] = 0;
-    if (r.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
+    write_scale(a, s, seg, worker, m, S1, S2);
   }
 }
 
@@ -541,96 +537,6 @@ __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
   }
 }
 
-// ---- one launch for vectors that stay in L2 between the two passes ------------------------------------------------
-// The grid is resident as a whole (cooperative launch) and every CTA takes the (worker, tile) pairs item, item + grid,
-// ...: first their statistics, then -- once all tiles of a pair's (worker, segment) have reported, which a counter per
-// (worker, segment) says -- the scale from the tile partials (every CTA that needs it forms it itself: same partials,
-// same tree, same bits) and the codes of its tiles, whose values come from L2 this time.  Two kernel boundaries and the
-// separate scale kernel are gone, which is most of the cost of a short vector.  The counters only grow: call number
-// `epoch` waits for (epoch + 1) * tile_count arrivals.  A wait that runs out records a timeout and goes on.
-template <int BITS, bool COUNT, bool NEED_SUMS>
-__global__ void __launch_bounds__(QT, 4) quantize_fused_kernel(QuantArgs a, unsigned int* done, unsigned int epoch, int cpw) {
-  launch_dependents();
-  wait_for_launch_before();
-  __shared__ float sh1[QITER * 8], sh2[QITER * 8], sh16[16];
-  __shared__ uint32_t shm[8];
-  __shared__ ScaleRec srec;
-  __shared__ __align__(16) uint8_t stage[BITS == 0 ? QT * 16 : 16];
-  const int tid = threadIdx.x, lane = tid & 31;
-  // CTA (chunk, worker) takes the tiles [t0, t1) of its worker: cpw chunks of consecutive tiles per worker
-  const int worker = blockIdx.x / cpw, chunk = blockIdx.x % cpw;
-  const int t0 = (int)((int64_t)a.ntiles * chunk / cpw), t1 = (int)((int64_t)a.ntiles * (chunk + 1) / cpw);
-  for (int tile = t0; tile < t1; ++tile) {
-    const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
-    if (tile != t0) __syncthreads();  // the reduction buffers are reused from tile to tile
-    stats_tile<NEED_SUMS>(a, tile, worker, sh1, sh2, shm);
-    if (tid == 0) {
-      const int64_t o = (int64_t)worker * a.nseg + seg;
-      if (tile == a.segs[seg].tile_first) a.clipped_out[o] = 0;
-      __threadfence();  // the partials (and the cleared count) before the arrival
-      atomicAdd(&done[o], 1u);
-    }
-  }
-  // segments without a single coordinate have no tile: their records are written here
-  for (int o = blockIdx.x; o < a.N * a.nseg; o += gridDim.x) {
-    const int w = o / a.nseg, seg = o % a.nseg;
-    if (a.segs[seg].tile_count != 0) continue;
-    __syncthreads();
-    const ScaleRec r = finish_segment(a, seg, w, sh16, shm);
-    if (tid == 0) { a.scales[o] = r; a.delta_out[o] = r.delta; a.clipped_out[o] = 0; }
-  }
-  int tile = t0;
-  while (tile < t1) {  // one pass per tensor segment that the chunk touches
-    const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
-    const SegInfo s = a.segs[seg];
-    const int tend = min(t1, s.tile_first + s.tile_count);
-    const int o = worker * a.nseg + seg;
-    if (tid == 0) {
-      const unsigned int want = (epoch + 1u) * (unsigned int)s.tile_count;
-      uint64_t t0ns = 0;
-      for (uint32_t it = 0;; ++it) {
-        unsigned int seen;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(done + o) : "memory");
-        if (seen >= want) break;
-        if ((it & 63u) == 63u) {
-          const uint64_t now = global_ns();
-          if (t0ns == 0) t0ns = now;
-          else if (now - t0ns > 2000000000ull) { atomicOr(a.dev_status, DEV_TIMEOUT); break; }
-        }
-      }
-    }
-    __syncthreads();
-    const ScaleRec r = finish_segment(a, seg, worker, sh16, shm);
-    if (tid == 0) {
-      srec = r;
-      if (tile == s.tile_first) {  // one CTA leaves the record and the scale for the caller
-        a.scales[o] = r;
-        a.delta_out[o] = r.delta;
-        if (r.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
-      }
-    }
-    __syncthreads();
-    const ScaleRec sc = srec;
-    // whole tiles of aligned vectors go through the pipelined loop, the rest tile by tile
-    const float* p = a.U + (int64_t)worker * a.ld + s.off;
-    const float* q = a.U_sub ? a.U_sub + (int64_t)worker * a.ld + s.off : nullptr;
-    int whole = 0;
-    if constexpr (BITS != 0) {
-      if (aligned16(p) && (!q || aligned16(q)) && !(sc.flags & 1u)) {
-        const int64_t full_tiles = s.len / TILE;  // tiles of the segment without a ragged end
-        whole = (int)max((int64_t)0, min((int64_t)(tend - s.tile_first), full_tiles) - (tile - s.tile_first));
-      }
-      if (whole > 0) quantize_whole_tiles<BITS ? BITS : 1, COUNT>(a, s, sc, p, q, tile, whole, seg, worker);
-    }
-    for (int t = tile + whole; t < tend; ++t) {
-      if (BITS == 0 && t > tile) __syncthreads();  // the staging buffer is reused from tile to tile
-      quantize_tile<BITS, COUNT>(a, t, worker, stage, sc);
-    }
-    tile = tend;
-    if (tile < t1) __syncthreads();  // srec and the reduction buffers are reused for the next segment
-  }
-}
-
 // ---- one cluster per worker for vectors of at most 8 tiles ----------------------------------------------------------
 // A CTA holds its tile in registers from the statistics to the codes; the tile partials go to all CTAs of the cluster
 // through distributed shared memory and every CTA forms the scale itself (same partials, same tree, same bits).  Nothing
@@ -829,17 +735,8 @@ __global__ void __launch_bounds__(QT) bypass_kernel(QuantArgs a) {
   bypass_tile(a, tile, worker, a.scales[(int64_t)worker * a.nseg + seg]);
 }
 
-using FusedKernel = void (*)(QuantArgs, unsigned int*, unsigned int, int);
-template <int BITS>
-FusedKernel pick_fused(bool count, bool sums) {
-  if (count) return sums ? quantize_fused_kernel<BITS, true, true> : quantize_fused_kernel<BITS, true, false>;
-  return sums ? quantize_fused_kernel<BITS, false, true> : quantize_fused_kernel<BITS, false, false>;
-}
-
 }  // namespace
 
-// The one-launch path (see quantize_fused_kernel): `done` holds N * nseg arrival counters that have seen `epoch` calls
-// with this layout.  Returns cudaErrorCooperativeLaunchTooLarge when no CTA of the kernel fits on the device.
 // One cluster per worker: vectors of one segment and at most CTILES tiles, the fixed widths.  Up to about four CTAs per SM
 // the clusters run side by side; with more of them the two passes over L2 of the other paths are as good.
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count) {
@@ -875,49 +772,6 @@ cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 
-cudaError_t launch_quantize_fused(const QuantArgs& a, unsigned int* done, unsigned int epoch, int sm_count, cudaStream_t st) {
-  if (a.N <= 0 || a.nseg <= 0) return cudaSuccess;
-  FusedKernel k;
-  const bool sums = a.clip_mode == CLIP_STD, count = a.count_clipped != 0;
-  switch (a.b) {
-    case 1: k = pick_fused<1>(count, sums); break;
-    case 2: k = pick_fused<2>(count, sums); break;
-    case 3: k = pick_fused<3>(count, sums); break;
-    case 4: k = pick_fused<4>(count, sums); break;
-    case 8: k = pick_fused<8>(count, sums); break;
-    default: k = pick_fused<0>(count, sums); break;
-  }
-  // asked for once per kernel (the devices of a process are alike)
-  static std::atomic<int> resident_of[6 * 4];
-  std::atomic<int>& known = resident_of[(a.b <= 4 ? a.b : a.b == 8 ? 5 : 0) * 4 + (count ? 2 : 0) + (sums ? 1 : 0)];
-  int per_sm = known.load(std::memory_order_relaxed);
-  if (per_sm == 0) {
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, QT, 0);
-    if (e != cudaSuccess) return e;
-    known.store(per_sm, std::memory_order_relaxed);
-  }
-  if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-  const long long resident = (long long)per_sm * sm_count;
-  if (resident < a.N) return cudaErrorCooperativeLaunchTooLarge;
-  // chunks of consecutive tiles per worker: as many as fit the resident grid, at most one per tile
-  long long cpw = resident / a.N;
-  if (cpw > a.ntiles) cpw = a.ntiles;
-  if (cpw < 1) cpw = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(cpw * a.N), 1, 1);
-  cfg.blockDim = dim3(QT, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs co-resident or the launch fails: they wait on one another
-  attr[0].val.cooperative = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k, a, done, epoch, (int)cpw);
-}
-
 int quantize_run_tiles() { return QRUN; }
 
 cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
@@ -932,7 +786,7 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
     if (e != cudaSuccess) return e;
   }
   if (hook) hook(user, 5 /* LPC_KERNEL_OTHER */, 1);
-  e = launch(finish_kernel, dim3((unsigned)a.nseg, (unsigned)a.N));  // also covers empty segments
+  e = launch(finish_kernel, dim3((unsigned)a.nseg, (unsigned)a.N));
   if (hook) hook(user, 5, 0);
   if (e != cudaSuccess) return e;
   if (a.shared_scale) {
