@@ -251,15 +251,16 @@ __device__ __forceinline__ uint32_t quantize_code(float u, float rdelta, uint32_
   }
 }
 
-// Any b in 1..16 (64-bit fixed point).
+// Any b in 1..16.  A = ceil(s 65536 - 1/2) in one rounding: where floats are coarser than that the product is a whole
+// number already, and A is at least -2^31 (s = -2^15).  The sum below lies in [0, 2^32).
 __device__ __forceinline__ uint32_t quantize_code_rt(float u, float rdelta, uint32_t r16, int b) {
   if (b == 1) return quantize_code<1>(u, rdelta, r16);
   const float lo = -(float)(1 << (b - 1));
   const float hi = (float)((1 << (b - 1)) - 1);
   float s = mul_rn(u, rdelta);
   s = fminf(fmaxf(s, lo), hi);
-  const long long A = __float2ll_ru(mul_rn(s, 131072.f)) >> 1;
-  return (uint32_t)((A + (65535ll + (65536ll << (b - 1))) - (long long)r16) >> 16);
+  const uint32_t A = (uint32_t)__float2int_ru(__fmaf_ru(s, 65536.f, -0.5f));
+  return (A + (65535u + (65536u << (b - 1))) - r16) >> 16;
 }
 
 // Exact float value of the signed codebook index of a stored code (code < 2^16).

@@ -316,6 +316,36 @@ __global__ void __launch_bounds__(32) share_scale_kernel(QuantArgs a) {
 // are still in L2.
 constexpr int QRUN = 8;
 
+__device__ __forceinline__ void push_code(uint64_t& lo, uint64_t& hi, uint32_t code, int b) {  // (hi, lo) = (hi, lo) << b | code
+  const uint32_t w0 = (uint32_t)lo, w1 = (uint32_t)(lo >> 32), w2 = (uint32_t)hi, w3 = (uint32_t)(hi >> 32);
+  hi = (uint64_t)__funnelshift_l(w1, w2, b) | ((uint64_t)__funnelshift_l(w2, w3, b) << 32);
+  lo = (uint64_t)((w0 << b) | code) | ((uint64_t)__funnelshift_l(w0, w1, b) << 32);
+}
+
+// The b bytes of every thread's group to their place in a sweep's 64 b words, of which `words` exist.  16 bits are
+// whole words of a thread's own; the others are put together per warp in shared memory (a warp's 32 groups are 8 b whole
+// words), two bytes at a time where b is even.
+__device__ __forceinline__ void store_any_width(uint32_t* __restrict__ out, int words, uint64_t lo, uint64_t hi, int b, int tid, int lane,
+                                                uint8_t* stage) {
+  if (b == 16) {
+    if (tid * 4 < words) *reinterpret_cast<uint4*>(out + tid * 4) = make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+    return;
+  }
+  const int warp = tid >> 5;
+  uint8_t* mine = stage + warp * 512 + lane * b;
+  __syncwarp();  // the words of the sweep before have been read
+  if ((b & 1) == 0) {
+    uint16_t* m2 = reinterpret_cast<uint16_t*>(mine);
+    for (int i = 0; i < b / 2; ++i) m2[i] = (uint16_t)((i < 4) ? (lo >> (16 * i)) : (hi >> (16 * (i - 4))));
+  } else {
+    for (int i = 0; i < b; ++i) mine[i] = (uint8_t)((i < 8) ? (lo >> (8 * i)) : (hi >> (8 * (i - 8))));
+  }
+  __syncwarp();
+  const uint32_t* st = reinterpret_cast<const uint32_t*>(stage + warp * 512);
+  for (int w = lane; w < 8 * b; w += 32)
+    if (warp * 8 * b + w < words) out[warp * 8 * b + w] = st[w];
+}
+
 template <int BITS>
 __device__ __forceinline__ void store_group(uint32_t* __restrict__ ot, int g, int lane, uint64_t lo) {
   if (BITS == 8) {
@@ -415,18 +445,11 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, int tile, int 
           if (nvalid < 8) lo &= (1ull << (nvalid * BITS)) - 1ull;
         } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (e < nvalid) {
-              const uint32_t code = quantize_code_rt(v[e], sc.rdelta, lane16(r, e), b);
-              if (COUNT) nclip += (v[e] > sc.T || v[e] < sc.lower) ? 1u : 0u;
-              const int pos = e * b;
-              if (pos < 64) {
-                lo |= (uint64_t)code << pos;
-                if (pos + b > 64) hi |= (uint64_t)code >> (64 - pos);
-              } else {
-                hi |= (uint64_t)code << (pos - 64);
-              }
-            }
+          for (int e = 7; e >= 0; --e) {  // from the last code down, everything so far moves up by one code
+            uint32_t code = quantize_code_rt(v[e], sc.rdelta, lane16(r, e), b);
+            if (e >= nvalid) code = 0u;
+            else if (COUNT) nclip += (v[e] > sc.T || v[e] < sc.lower) ? 1u : 0u;
+            push_code(lo, hi, code, b);
           }
         }
       } else {
@@ -466,15 +489,7 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, int tile, int 
       const int64_t w = 3 * (j >> 5) + i;
       if (i < 3 && w < s.pad_words) out[w] = (mine >> (8 * i)) | (next << (24 - 8 * i));
     } else {
-      // generic: b bytes per thread at byte tid*b of the sweep's 256*b-byte block
-      if (it > 0) __syncthreads();
-      for (int i = 0; i < b; ++i)
-        stage[tid * b + i] = (uint8_t)((i < 8) ? (lo >> (8 * i)) : (hi >> (8 * (i - 8))));
-      __syncthreads();
-      const int64_t w0 = (sweep0 >> 5) * b;  // sweep0 is a multiple of 2048, so this is exact
-      const uint32_t* st = reinterpret_cast<const uint32_t*>(stage);
-      for (int w = tid; w < (QGROUP / 32) * b; w += QT)
-        if (w0 + w < s.pad_words) out[w0 + w] = st[w];
+      store_any_width(out + (sweep0 >> 5) * b, (int)min((int64_t)(QGROUP / 32) * b, s.pad_words - (sweep0 >> 5) * b), lo, hi, b, tid, lane, stage);
     }
   }
   nclip = __reduce_add_sync(0xFFFFFFFFu, nclip + (uint32_t)fclip);
@@ -699,17 +714,14 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
   const int tid = threadIdx.x, lane = tid & 31;
   uint32_t* out = a.codes + (int64_t)worker * a.stride_words + s.word_off;
   uint32_t nclip = 0;
+  float u[QITER][8];  // all loads before the first store
+#pragma unroll
+  for (int it = 0; it < QITER; ++it) load8(p, q, tstart + (int64_t)it * QGROUP + tid * 8, s.len, vec, u[it]);
 #pragma unroll
   for (int it = 0; it < QITER; ++it) {
     const int64_t j = tstart + (int64_t)it * QGROUP + tid * 8;
     if (j >= s.pad_words) continue;
-    float v[8];
-    if (j < s.len) {
-      load8(p, q, j, s.len, vec, v);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = 0.f;
-    }
+    float* v = u[it];
     if (a.clip_mode != CLIP_NONE) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -719,9 +731,14 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
         }
       }
     }
+    if (j + 8 <= s.len) {  // the stream starts on a 16-byte boundary
+      *reinterpret_cast<float4*>(out + j) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<float4*>(out + j + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
 #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (j + e < s.pad_words) out[j + e] = (j + e < s.len) ? __float_as_uint(v[e]) : 0u;
+      for (int e = 0; e < 8; ++e)
+        if (j + e < s.pad_words) out[j + e] = (j + e < s.len) ? __float_as_uint(v[e]) : 0u;
+    }
   }
   nclip = __reduce_add_sync(0xFFFFFFFFu, nclip);
   if (lane == 0 && nclip) atomicAdd(&a.clipped_out[(int64_t)worker * a.nseg + seg], nclip);
@@ -730,7 +747,7 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
 __global__ void __launch_bounds__(QT) bypass_kernel(QuantArgs a) {
   launch_dependents();
   wait_for_launch_before();
-  const int tile = blockIdx.x, worker = blockIdx.y;
+  const int tile = (int)(gridDim.x - 1 - blockIdx.x), worker = (int)(gridDim.y - 1 - blockIdx.y);  // from the end, as quantize_kernel
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
   bypass_tile(a, tile, worker, a.scales[(int64_t)worker * a.nseg + seg]);
 }
