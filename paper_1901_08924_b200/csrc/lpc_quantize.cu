@@ -316,10 +316,53 @@ __global__ void __launch_bounds__(32) share_scale_kernel(QuantArgs a) {
 // are still in L2.
 constexpr int QRUN = 8;
 
+// One atomic addition per CTA to a message's count (all threads call this with their own part).  With one per warp and tile,
+// 131,072 additions to eight neighbouring words took 8 x 2^24 values at b = 32 from 240 to 378 us.
+__device__ __forceinline__ void add_count(uint32_t n, uint32_t* dst) {
+  __shared__ uint32_t part[QT / 32];
+  n = __reduce_add_sync(0xFFFFFFFFu, n);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+#pragma unroll
+    for (int w = 0; w < QT / 32; ++w) t += part[w];
+    if (t) atomicAdd(dst, t);
+  }
+}
+
 __device__ __forceinline__ void push_code(uint64_t& lo, uint64_t& hi, uint32_t code, int b) {  // (hi, lo) = (hi, lo) << b | code
   const uint32_t w0 = (uint32_t)lo, w1 = (uint32_t)(lo >> 32), w2 = (uint32_t)hi, w3 = (uint32_t)(hi >> 32);
   hi = (uint64_t)__funnelshift_l(w1, w2, b) | ((uint64_t)__funnelshift_l(w2, w3, b) << 32);
   lo = (uint64_t)((w0 << b) | code) | ((uint64_t)__funnelshift_l(w0, w1, b) << 32);
+}
+
+// The packed bits of a group at a width known at run time, from its scaled values; 2 to 7 bits by the rule of
+// quantize_scaled8, wider codes by conversion to an integer.
+__device__ __forceinline__ void quantize_scaled8_rt(const float* s, const U4& r, int b, uint64_t& lo, uint64_t& hi) {
+  const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
+  lo = hi = 0;
+  if (b <= 7) {
+    const float SC = __int_as_float((127 - b) << 23), HS = (float)((1 << (b - 1)) - 1) * SC;  // 2^-b and hi 2^-b, exact
+    const float C = 1.0f - SC - SC / 131072.f, UP = (float)(1 << (16 + b));
+#pragma unroll
+    for (int h = 3; h >= 0; --h) {
+      const float q0 = fma_ru_sat(fma_rd_sat(s[2 * h], -SC, HS), -1.f, C), q1 = fma_ru_sat(fma_rd_sat(s[2 * h + 1], -SC, HS), -1.f, C);
+      float t0, t1;
+      unpack2(fma2_ru(pack2(q0, q1), pack2(UP, UP), pack2(8388608.f, 8388608.f)), t0, t1);
+      const uint32_t x0 = __dp2a_lo(~rw[h], 0x0001u, __float_as_uint(t0)), x1 = __dp2a_lo(~rw[h], 0x0100u, __float_as_uint(t1));
+      const uint32_t two = ((x0 >> 16) & 0xFFu) | (((x1 >> 16) & 0xFFu) << b);
+      hi = 0;
+      lo = (lo << (2 * b)) | two;
+    }
+  } else {
+    const float l = -(float)(1 << (b - 1)), u = (float)((1 << (b - 1)) - 1);
+#pragma unroll
+    for (int e = 7; e >= 0; --e) {
+      const uint32_t A = (uint32_t)__float2int_ru(__fmaf_ru(fminf(fmaxf(s[e], l), u), 65536.f, -0.5f));
+      push_code(lo, hi, (A + (65535u + (65536u << (b - 1))) - lane16(r, e)) >> 16, b);
+    }
+  }
 }
 
 // The b bytes of every thread's group to their place in a sweep's 64 b words, of which `words` exist.  16 bits are
@@ -376,13 +419,20 @@ __device__ __forceinline__ void store_group(uint32_t* __restrict__ ot, int g, in
 template <int BITS, bool COUNT, bool HAS_Q>
 __device__ __forceinline__ void quantize_run(const QuantArgs& a, const ScaleRec& sc, const float* __restrict__ pt,
                                              const float* __restrict__ qt, bool al32, uint32_t block0,
-                                             uint32_t* __restrict__ ot, int nsweeps, int worker, int tid, int lane, float& fclip) {
+                                             uint32_t* __restrict__ ot, int nsweeps, int worker, int tid, int lane, float& fclip,
+                                             uint8_t* stage) {
   float s[8];
   f32x2 v0[4], v1[4];
   auto finish = [&](int sweep) {
     const int g = sweep * (QGROUP / 8) + tid;  // coordinate group inside the run
     const U4 r = stream_block(a.seed, TAG_ROUND, (uint32_t)worker, a.k, block0 + (uint32_t)g);
-    store_group<BITS>(ot, g, lane, quantize_scaled8<BITS>(s, r));
+    if constexpr (BITS != 0) {
+      store_group<BITS>(ot, g, lane, quantize_scaled8<BITS ? BITS : 1>(s, r));
+    } else {
+      uint64_t lo, hi;
+      quantize_scaled8_rt(s, r, a.b, lo, hi);
+      store_any_width(ot + (int64_t)sweep * (QGROUP / 32) * a.b, (QGROUP / 32) * a.b, lo, hi, a.b, tid, lane, stage);
+    }
   };
   load8v<true>(pt, al32, v0);
   load8v<true>(HAS_Q ? qt : pt + QGROUP, al32, v1);
@@ -499,28 +549,27 @@ __device__ __forceinline__ void quantize_tile(const QuantArgs& a, int tile, int 
 // The run [tile, tile + whole) of whole tiles of one segment, by all threads of the CTA.
 template <int BITS, bool COUNT>
 __device__ __forceinline__ void quantize_whole_tiles(const QuantArgs& a, const SegInfo& s, const ScaleRec& sc, const float* p, const float* q,
-                                                     int tile, int whole, int seg, int worker) {
+                                                     int tile, int whole, int seg, int worker, uint8_t* stage) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t tstart = (int64_t)(tile - s.tile_first) * TILE;
   const uint32_t block0 = s.block_base + (uint32_t)(tstart >> 3);
-  uint32_t* ot = a.codes + (int64_t)worker * a.stride_words + s.word_off + (tstart >> 5) * BITS;
+  uint32_t* ot = a.codes + (int64_t)worker * a.stride_words + s.word_off + (tstart >> 5) * (BITS ? BITS : a.b);
   const bool al32 = aligned32(p) && (!q || aligned32(q));
   const float* pt = p + tstart + tid * 8;
   float fclip = 0.f;
   if (q) {
     const float* qt = q + tstart + tid * 8;
     if (COUNT && !(sc.flags & SCALE_NONE_OUTSIDE))
-      quantize_run<BITS, true, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+      quantize_run<BITS, true, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip, stage);
     else
-      quantize_run<BITS, false, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+      quantize_run<BITS, false, true>(a, sc, pt, qt, al32, block0, ot, whole * QITER, worker, tid, lane, fclip, stage);
   } else {
     if (COUNT && !(sc.flags & SCALE_NONE_OUTSIDE))
-      quantize_run<BITS, true, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+      quantize_run<BITS, true, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip, stage);
     else
-      quantize_run<BITS, false, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip);
+      quantize_run<BITS, false, false>(a, sc, pt, nullptr, al32, block0, ot, whole * QITER, worker, tid, lane, fclip, stage);
   }
-  const uint32_t nclip = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)fclip);
-  if (COUNT && lane == 0 && nclip) atomicAdd(&a.clipped_out[(int64_t)worker * a.nseg + seg], nclip);
+  if (COUNT && !(sc.flags & SCALE_NONE_OUTSIDE)) add_count((uint32_t)fclip, &a.clipped_out[(int64_t)worker * a.nseg + seg]);
 }
 
 template <int BITS, bool COUNT>
@@ -531,7 +580,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
   const int tile0 = (int)(gridDim.x - 1 - blockIdx.x) * run;
   const int ntl = min(run, a.ntiles - tile0);
   __shared__ __align__(16) uint8_t stage[BITS == 0 ? QT * 16 : 16];
-  if constexpr (BITS != 0) {
+  {
     const int seg = a.tile_seg ? a.tile_seg[tile0] : 0;
     const int seg_last = a.tile_seg ? a.tile_seg[tile0 + ntl - 1] : 0;  // tiles are numbered segment by segment
     if (seg == seg_last) {
@@ -540,7 +589,7 @@ __global__ void __launch_bounds__(QT, 4) quantize_kernel(QuantArgs a, int run) {
       const float* q = a.U_sub ? a.U_sub + (int64_t)worker * a.ld + s.off : nullptr;
       const ScaleRec sc = a.scales[(int64_t)worker * a.nseg + seg];
       if (aligned16(p) && (!q || aligned16(q)) && !(sc.flags & 1u) && (int64_t)(tile0 + ntl - s.tile_first) * TILE <= s.len) {
-        quantize_whole_tiles<BITS ? BITS : 1, COUNT>(a, s, sc, p, q, tile0, ntl, seg, worker);
+        quantize_whole_tiles<BITS, COUNT>(a, s, sc, p, q, tile0, ntl, seg, worker, stage);
         return;
       }
     }
@@ -714,6 +763,30 @@ __device__ __forceinline__ void bypass_tile(const QuantArgs& a, int tile, int wo
   const int tid = threadIdx.x, lane = tid & 31;
   uint32_t* out = a.codes + (int64_t)worker * a.stride_words + s.word_off;
   uint32_t nclip = 0;
+  if (vec && tstart + TILE <= s.len) {  // four values per thread and access: neighbouring lanes fill whole lines
+    const float *pt = p + tstart + tid * 4, *qt = q ? q + tstart + tid * 4 : nullptr;
+    float4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldcs(reinterpret_cast<const float4*>(pt + i * QT * 4));
+    if (qt) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 w = __ldcs(reinterpret_cast<const float4*>(qt + i * QT * 4));
+        v[i] = make_float4(__fsub_rn(v[i].x, w.x), __fsub_rn(v[i].y, w.y), __fsub_rn(v[i].z, w.z), __fsub_rn(v[i].w, w.w));
+      }
+    }
+    auto clamp = [&](float& x) {
+      if (x > sc.T) { x = sc.T; ++nclip; }
+      if (x < -sc.T) { x = -sc.T; ++nclip; }
+    };
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (a.clip_mode != CLIP_NONE) { clamp(v[i].x); clamp(v[i].y); clamp(v[i].z); clamp(v[i].w); }
+      *reinterpret_cast<float4*>(out + tstart + tid * 4 + i * QT * 4) = v[i];
+    }
+    if (a.clip_mode != CLIP_NONE) add_count(nclip, &a.clipped_out[(int64_t)worker * a.nseg + seg]);
+    return;
+  }
   float u[QITER][8];  // all loads before the first store
 #pragma unroll
   for (int it = 0; it < QITER; ++it) load8(p, q, tstart + (int64_t)it * QGROUP + tid * 8, s.len, vec, u[it]);
