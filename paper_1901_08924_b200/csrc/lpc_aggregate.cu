@@ -281,6 +281,8 @@ __device__ __forceinline__ void sum_codes8x2(const uint32_t* __restrict__ w, int
 // is 4 or 8, else staged through shared memory and written out as words.
 template <int BITS>  // input width: 2, 4, 8 fixed; 0: b in 2..16 from the arguments
 __global__ void __launch_bounds__(AT, 4) server_reduce_kernel(ServerArgs a) {
+  launch_dependents();
+  wait_for_launch_before();
   const int tile = blockIdx.x;
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
   const SegInfo s = a.segs[seg];
@@ -406,6 +408,8 @@ __global__ void __launch_bounds__(AT, 4) server_reduce_kernel(ServerArgs a) {
 // constant powers of two (the low part of the product is the shifted value, the high part its spill into the next word).
 template <int BO, bool REQ>
 __global__ void __launch_bounds__(AT, 4) server_reduce4_kernel(ServerArgs a) {
+  launch_dependents();
+  wait_for_launch_before();
   constexpr int OW = REQ ? 4 : BO;  // output words per thread
   const int tile = blockIdx.x, tid = threadIdx.x;
   const int seg = a.tile_seg ? a.tile_seg[tile] : 0;
@@ -549,6 +553,8 @@ __device__ __forceinline__ void count_unit(uint4 q, uint32_t* cnt) {
 
 template <int BITS>  // 1, 2, 4
 __global__ void __launch_bounds__(AT) code_histogram_swar_kernel(HistArgs a, int run) {
+  launch_dependents();
+  wait_for_launch_before();
   constexpr int BINS = 1 << BITS, CPU = 128 / BITS;  // codes per 16-byte unit
   const int worker = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
   const int tile0 = blockIdx.x * run, tile1 = min(tile0 + run, a.ntiles);
@@ -616,6 +622,8 @@ __device__ __forceinline__ void count_codes(uint32_t* col, const uint32_t* w, in
 constexpr int HT = 512;
 template <int BITS>  // 3, 5, 6, 7, 8
 __global__ void __launch_bounds__(HT) code_histogram_kernel(HistArgs a, int run) {
+  launch_dependents();
+  wait_for_launch_before();
   constexpr int BINS = 1 << BITS;
   constexpr int UW = BITS == 8 ? 4 : BITS;   // words of a thread's unit: 16 bytes, or the shortest whole number of words
   constexpr int UC = UW * 32 / BITS;         // codes in it
@@ -685,6 +693,8 @@ __global__ void __launch_bounds__(HT) code_histogram_kernel(HistArgs a, int run)
 // with the wait for the stream, against 50 us on the host, which took them one after the other.
 __global__ void __launch_bounds__(256) coded_size_kernel(const unsigned long long* __restrict__ hist, int bins,
                                                          double* __restrict__ entropy_out, unsigned long long* __restrict__ huffman_out) {
+  launch_dependents();
+  wait_for_launch_before();
   constexpr unsigned long long NONE = 1ull << 62;  // larger than any sum of counts
   __shared__ unsigned long long cnt[256], leaf[256 + 2], node[256 + 2];
   __shared__ unsigned long long wsum[8];
@@ -752,46 +762,43 @@ cudaError_t launch_code_histogram(const HistArgs& a, int sm_count, cudaStream_t 
   const int run = (int)std::min<int64_t>(32, std::max<int64_t>(1, all / (4 * (int64_t)sm_count)));
   const dim3 grid((unsigned)((a.ntiles + run - 1) / run), (unsigned)a.N);
   switch (a.b) {
-    case 1: code_histogram_swar_kernel<1><<<grid, AT, 0, st>>>(a, run); break;
-    case 2: code_histogram_swar_kernel<2><<<grid, AT, 0, st>>>(a, run); break;
-    case 3: code_histogram_kernel<3><<<grid, HT, 0, st>>>(a, run); break;
-    case 4: code_histogram_swar_kernel<4><<<grid, AT, 0, st>>>(a, run); break;
-    case 5: code_histogram_kernel<5><<<grid, HT, 0, st>>>(a, run); break;
-    case 6: code_histogram_kernel<6><<<grid, HT, 0, st>>>(a, run); break;
-    case 7: code_histogram_kernel<7><<<grid, HT, 0, st>>>(a, run); break;
-    default: code_histogram_kernel<8><<<grid, HT, 0, st>>>(a, run); break;
+    case 1: return launch_overlapped(code_histogram_swar_kernel<1>, grid, dim3(AT), 0, st, a, run);
+    case 2: return launch_overlapped(code_histogram_swar_kernel<2>, grid, dim3(AT), 0, st, a, run);
+    case 3: return launch_overlapped(code_histogram_kernel<3>, grid, dim3(HT), 0, st, a, run);
+    case 4: return launch_overlapped(code_histogram_swar_kernel<4>, grid, dim3(AT), 0, st, a, run);
+    case 5: return launch_overlapped(code_histogram_kernel<5>, grid, dim3(HT), 0, st, a, run);
+    case 6: return launch_overlapped(code_histogram_kernel<6>, grid, dim3(HT), 0, st, a, run);
+    case 7: return launch_overlapped(code_histogram_kernel<7>, grid, dim3(HT), 0, st, a, run);
+    default: return launch_overlapped(code_histogram_kernel<8>, grid, dim3(HT), 0, st, a, run);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_coded_size(const unsigned long long* hist, int messages, int b, double* entropy_out,
                               unsigned long long* huffman_out, cudaStream_t st) {
   if (messages <= 0) return cudaSuccess;
-  coded_size_kernel<<<(unsigned)messages, 256, 0, st>>>(hist, 1 << b, entropy_out, huffman_out);
-  return cudaGetLastError();
+  return launch_overlapped(coded_size_kernel, dim3((unsigned)messages), dim3(256), 0, st, hist, 1 << b, entropy_out, huffman_out);
 }
 
 cudaError_t launch_server_reduce(const ServerArgs& a, cudaStream_t st) {
   if (a.ntiles <= 0) return cudaSuccess;
   const dim3 grid((unsigned)a.ntiles), block(AT);
   if (a.b == 4 && a.N <= 16) {  // sums of at most 8 bits: whole words per thread
-    if (a.requantize) { server_reduce4_kernel<4, true><<<grid, block, 0, st>>>(a); return cudaGetLastError(); }
+    if (a.requantize) return launch_overlapped(server_reduce4_kernel<4, true>, grid, block, 0, st, a);
     switch (a.b_out) {
-      case 4: server_reduce4_kernel<4, false><<<grid, block, 0, st>>>(a); return cudaGetLastError();
-      case 5: server_reduce4_kernel<5, false><<<grid, block, 0, st>>>(a); return cudaGetLastError();
-      case 6: server_reduce4_kernel<6, false><<<grid, block, 0, st>>>(a); return cudaGetLastError();
-      case 7: server_reduce4_kernel<7, false><<<grid, block, 0, st>>>(a); return cudaGetLastError();
-      case 8: server_reduce4_kernel<8, false><<<grid, block, 0, st>>>(a); return cudaGetLastError();
+      case 4: return launch_overlapped(server_reduce4_kernel<4, false>, grid, block, 0, st, a);
+      case 5: return launch_overlapped(server_reduce4_kernel<5, false>, grid, block, 0, st, a);
+      case 6: return launch_overlapped(server_reduce4_kernel<6, false>, grid, block, 0, st, a);
+      case 7: return launch_overlapped(server_reduce4_kernel<7, false>, grid, block, 0, st, a);
+      case 8: return launch_overlapped(server_reduce4_kernel<8, false>, grid, block, 0, st, a);
       default: break;
     }
   }
   switch (a.b) {
-    case 2: server_reduce_kernel<2><<<grid, block, 0, st>>>(a); break;
-    case 4: server_reduce_kernel<4><<<grid, block, 0, st>>>(a); break;
-    case 8: server_reduce_kernel<8><<<grid, block, 0, st>>>(a); break;
-    default: server_reduce_kernel<0><<<grid, block, 0, st>>>(a); break;
+    case 2: return launch_overlapped(server_reduce_kernel<2>, grid, block, 0, st, a);
+    case 4: return launch_overlapped(server_reduce_kernel<4>, grid, block, 0, st, a);
+    case 8: return launch_overlapped(server_reduce_kernel<8>, grid, block, 0, st, a);
+    default: return launch_overlapped(server_reduce_kernel<0>, grid, block, 0, st, a);
   }
-  return cudaGetLastError();
 }
 
 int aggregate_split(int ntiles, int sm_count) {
