@@ -425,7 +425,7 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
     # the floor of a timed launch: the same calls on 8 x 2^10 values, where there is next to nothing to do
     r0 = qa_point(dev, peak, U[:, : 1 << 10], 4, 2.0, reps=20)
     res["launch_floor_us"] = {"workload": "N=8, len 2^10, b=4 (an event pair around a launch that has next to nothing to do)",
-                              "quantize_fused_kernel (cooperative launch, one grid-wide hand-over)": round(r0["quantize_pack"]["one_launch_ms"] * 1e3, 2),
+                              "quantize_cluster_kernel (one cluster per worker)": round(r0["quantize_pack"]["one_launch_ms"] * 1e3, 2),
                               "unpack_average_prox_kernel (plain launch)": round(r0["unpack_average_prox"]["ms"] * 1e3, 2)}
     lens = [l for l in (16, 20, 24, 26, 28) if l <= top]
     for l2 in lens:
@@ -433,7 +433,7 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
         wl = "sweep N=8, len 2^%d, N(0,1), b=4, clip 2 std" % l2
         qp, ua = r["quantize_pack"], r["unpack_average_prox"]
         resident = r["l2_resident_input"]
-        name = ("quantize_fused_kernel<4> (quantize+pack in one cooperative launch)" if qp["one_launch_ms"] > 0 else
+        name = ("quantize_cluster_kernel<4> (quantize+pack, one cluster per worker)" if qp["one_launch_ms"] > 0 else
                 "quantize+pack (stats_kernel + finish_kernel + quantize_kernel<4>)")
         roof.append(roofline_entry(name, wl, qp["ms"] * 1e3, qp["bytes"], peak,
                                    note="input stays in L2 between the two looks at it: bound 4 + b/8 B per element; launch-bound at "
@@ -576,7 +576,7 @@ def kernel_pass(dev, log2_len):
     short = min(length, 1 << 20)
     q = lpc.Context(None, None, lpc.LOGISTIC, 0.0, N, 1, 4, lpc.CLIP_STD, 2.0, 0)
     for k in range(2):
-        q.quantize_pack(U[:, :short], k)                             # quantize_fused_kernel<4> (one cooperative launch)
+        q.quantize_pack(U[:, :short], k)                             # the short-vector path
     q.sync_status()
     one = q.query(lpc.INFO_QUANT_ONE_LAUNCH)
     q.close()
