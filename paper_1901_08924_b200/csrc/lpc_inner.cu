@@ -356,12 +356,15 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
               sv[(h + j) * QB + q] = tree4(mul_rn(v[j][q].x, xs[q].x), mul_rn(v[j][q].y, xs[q].y), mul_rn(v[j][q].z, xs[q].z),
                                            mul_rn(v[j][q].w, xs[q].w));
         }
+        // this warp has read, and used, its quarter of the stage (every partial product sum needs one of the reads)
+        uint32_t seen = 0;
+#pragma unroll
+        for (int i = 0; i < SG * QB; ++i) seen ^= __float_as_uint(sv[i]);
+        mbar_arrive_after(&sm.ebar[g % R], __any_sync(0xFFFFFFFFu, seen == 0x7FFFFFFFu), lane == 0);
         WarpHalving<SG * QB, 0>::run(sv, lane);  // lane holds the 32-lane tree sum of (row, block) halving_index<4>(lane)
         float part = sv[0];
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 8));  // blocks 2k, 2k+1 of the row
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 4));
-        // this warp has read, and used, its quarter of the stage
-        mbar_arrive_after(&sm.ebar[g % R], __any_sync(0xFFFFFFFFu, __float_as_uint(part) == 0x7FFFFFFFu), lane == 0);
         if ((lane >> 2) < CS && myrow < cnt)
           st_async_cluster(&sm.parts[g % SSLOTS][(myrow * MAXCS + rank) * SMW + wq], &sm.pbar[g % SSLOTS],
                            (uint32_t)(lane >> 2), __float_as_uint(part));

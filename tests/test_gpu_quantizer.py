@@ -230,3 +230,29 @@ def test_cluster_per_worker_matches_the_three_launches(b, length):
     u = (base[3, :length] - sub[3, :length]).numpy()  # the last combination: no clipping, with the subtrahend
     w, dl, _ = orc.quantize_pack(u, b, orc.CLIP_NONE, 1.0, seed, 3, k)
     assert (_u32(got[1][0])[3, : w.size] == w).all() and got[1][1][3, 0].item() == dl
+
+
+@pytest.mark.parametrize("b", [5, 6, 7, 9, 14, 16, 32])
+def test_run_time_widths_whole_tiles_and_decode(b):
+    """Widths without a fixed-width path, and 32-bit messages: runs of whole tiles with a ragged tail, rows on 16-byte
+    boundaries, a subtrahend; codes, counts and the decoded step against the oracle."""
+    N, seed, k, length = 2, 17, 9, 3 * 8192 + 37
+    rng = np.random.default_rng(b)
+    ld = (length + 3) // 4 * 4
+    U, S = (rng.standard_normal((N, ld)).astype(np.float32) for _ in range(2))
+    x0 = rng.standard_normal(length).astype(np.float32)
+    for sub in (False, True):
+        V = (U - S if sub else U)[:, :length]
+        ctx = _ctx(N, b, orc.CLIP_STD, 1.5, seed)
+        dev = [torch.from_numpy(a).to(DEV)[:, :length] for a in (U, S)]
+        codes, delta, clipped = ctx.quantize_pack(dev[0], k, U_sub=dev[1] if sub else None)
+        x = torch.from_numpy(x0).to(DEV)
+        ctx.unpack_average_prox(codes, delta, length, x, 0.1, 1e-3)
+        ctx.sync_status()
+        rc, rd, rcl = _oracle_quantize(np.ascontiguousarray(V), b, orc.CLIP_STD, 1.5, seed, k)
+        W = orc.packed_words(length, b)
+        assert (_u32(codes)[:, :W] == rc[:, :W]).all() and (delta.cpu().numpy() == rd).all()
+        assert (clipped.cpu().numpy() == rcl).all()
+        xr = orc.unpack_average_prox(np.ascontiguousarray(rc[:, :W]), rd.reshape(-1), length, b, None, x0, 0.1, 1e-3)
+        assert (x.cpu().numpy().view(np.uint32) == xr.view(np.uint32)).all()
+        ctx.close()
