@@ -135,6 +135,9 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
   const int passes = (SL + IGROUP - 1) / IGROUP;
   const int c0 = rank * SL;                         // first coordinate of this CTA's slice
   const int width = max(0, min(SL, d - c0));        // coordinates of the slice that exist
+  // CTAs of the cluster that have a column: d is rounded up to a power of two, so the last ones can be empty (one of four for
+  // d in 4,097..6,144; one to three of eight for d in 8,193..14,336)
+  const int CSW = (d + SL - 1) / SL;
 
   // ---- sampling (Algorithm 1 step 6): slot a uses word 0 of block a of the batch stream -----------------
   auto sample_slot = [&](int slot) -> int64_t {
@@ -292,9 +295,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
         gave_up = true;
       }
     };
-    auto wait_stage = [&](int g) {
-      if (width > 0) wait_on(&sm.sbar[g % R], (uint32_t)((g / R) & 1), false);
-    };
+    auto wait_stage = [&](int g) { wait_on(&sm.sbar[g % R], (uint32_t)((g / R) & 1), false); };
     // Shared-memory reads are laid out so that a warp's 16-byte loads touch consecutive addresses (no bank
     // conflicts): the ring is read twice per row and written once, and that traffic is what bounds a group.
     constexpr int NBK = IGROUP / 128;    // blocks of 128 coordinates per slice: 16; a lane takes 4 coordinates of each
@@ -309,12 +310,17 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     auto row4 = [&](int r, int off) {  // four row values of the slice (zero outside the existing columns)
       return (off < width) ? *reinterpret_cast<const float4*>(rows + (size_t)r * SL + off) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
-    if (warp < SDW) {
+    if (width == 0) {
+      // A CTA without a column takes no part in the ring or in the margins: it has no stage to wait for, and that wait is what
+      // keeps a CTA's partial sums within reach of its peers' exchange slots.  Its peers count and add the CSW others
+      // only; it meets them again at the scale.
+      wait_for_launch_before();
+    } else if (warp < SDW) {
       // -- margins: the SMW = 4 warps of a side share a group, warp w of them taking the blocks 4 w .. 4 w + 3 (a quarter
       // of the slice) of all rows of the group; the two sides alternate groups.  Lane l holds x for the coordinates
       // 128 q + 4 l .. + 3 of its blocks q.  The leaves of the tree in coordinate order: four products per lane
       // (tree4), then the tree over the 32 lanes of a block, then the tree over the four blocks; the quarter sums go to
-      // every CTA of the cluster as stores that count on that CTA's barrier of the group, and are combined there.
+      // every CTA with columns as stores that count on that CTA's barrier of the group, and are combined there.
       // Sixteen independent 16-byte loads and one reduction per group keep a warp's dependent chains short.
       constexpr int SMW = 4, QB = NBK / SMW;  // warps per side; blocks per warp
       static_assert(SDW == 2 * SMW && QB * SG == 16, "one 16-value recursive-halving reduction per group");
@@ -365,7 +371,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
         float part = sv[0];
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 8));  // blocks 2k, 2k+1 of the row
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 4));
-        if ((lane >> 2) < CS && myrow < cnt)
+        if ((lane >> 2) < CSW && myrow < cnt)
           st_async_cluster(&sm.parts[g % SSLOTS][(myrow * MAXCS + rank) * SMW + wq], &sm.pbar[g % SSLOTS],
                            (uint32_t)(lane >> 2), __float_as_uint(part));
       }
@@ -436,16 +442,16 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       for (int g = warp - (SDW + SUW); g < ngroups; g += SCW) {
         const int cnt = min(SG, B - g * SG);
         const int sl = g % SSLOTS;
-        if (lane == 0) mbar_expect_tx(&sm.pbar[sl], (uint32_t)(CS * cnt * 16));  // this phase: one arrival and the bytes of 4 quarter sums per row and CTA
+        if (lane == 0) mbar_expect_tx(&sm.pbar[sl], (uint32_t)(CSW * cnt * 16));  // this phase: one arrival and the bytes of 4 quarter sums per row and CTA with columns
         __syncwarp();
         wait_on(&sm.mbar_meta[(g * SG) / 32], 0u, false);
         wait_on(&sm.pbar[sl], (uint32_t)((g / SSLOTS) & 1), true);
         // lane (j, q) = (lane / MAXCS, lane % MAXCS): the tree over the four quarter sums of CTA q's slice for row j, then
-        // the tree over the CTAs by shuffles; lane (j, 0) ends with the margin of row j
+        // the tree over the CTAs by shuffles (an empty slice adds zero); lane (j, 0) ends with the margin of row j
         {
           const int j = lane / MAXCS, q = lane % MAXCS;
           float mq = 0.f;
-          if (q < CS) {
+          if (q < CSW) {
             const float4 pq = *reinterpret_cast<const float4*>(&sm.parts[sl][(j * MAXCS + q) * 4]);
             mq = tree4(pq.x, pq.y, pq.z, pq.w);
           }
@@ -476,7 +482,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
         const int h = g - R;
         wait_on(&sm.ebar[h % R], (uint32_t)((h / R) & 1), false);
         if (gave_up) break;
-        if (width > 0 && lane < SG) issue(g, lane);
+        if (lane < SG) issue(g, lane);
         __syncwarp();
       }
     } else {
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     }
     __syncthreads();  // both sides are done with the ring: it now carries u to the usual owner of each coordinate
     if (sm.stream_fail) {  // a wait ran out: give the copies still in flight a bounded chance to land before the ring is reused
-      if (tid == 0 && width > 0)
+      if (tid == 0)
         for (int g = max(0, sm.issued - R); g < sm.issued; ++g) mbar_wait(&sm.sbar[g % R], (uint32_t)((g / R) & 1), 100000000ull);
       __syncthreads();
     }

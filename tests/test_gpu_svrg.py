@@ -125,6 +125,24 @@ def test_inner_step_chain_of_custody(loss, cfg):
     ctx.close()
 
 
+@pytest.mark.parametrize("loss", ["least_squares", "logistic"])
+@pytest.mark.parametrize("cfg", [
+    dict(n=512, d=5000, N=2, B=100, b=4), dict(n=512, d=6144, N=2, B=256, b=2), dict(n=256, d=8196, N=2, B=70, b=4),
+    dict(n=512, d=9000, N=2, B=256, b=8), dict(n=510, d=12288, N=3, B=129, b=3), dict(n=512, d=13000, N=2, B=256, b=4),
+])
+def test_streaming_step_with_empty_slices(loss, cfg):
+    # d is rounded up to a power of two and split over 4 or 8 CTAs: one CTA of four, or one to three of eight, have no
+    # column and take no part in the margins; more than 64 rows, so that the exchange slots of the ring are used again
+    c = dict(cfg)
+    n, d = c.pop("n"), c.pop("d")
+    P, ctx = _setup(n, d, loss, **c)
+    cs = ctx.query(lpc.INFO_STEP_CLUSTER_SIZE)
+    width = max(32, 1 << (d - 1).bit_length()) // cs
+    assert ctx.query(lpc.INFO_STEP_RING_STAGES) > 0 and (cs - 1) * width >= d  # streamed, and the last CTA is empty
+    ctx.close()
+    test_inner_step_chain_of_custody(loss, cfg)
+
+
 @pytest.mark.parametrize("cs", [1, 2, 4, 8])
 @pytest.mark.parametrize("clip", [(orc.CLIP_NONE, 1.0), (orc.CLIP_LAMBDA, 0.9), (orc.CLIP_STD, 2.0)])
 def test_inner_step_cluster_sizes_and_clip_rules(cs, clip):
@@ -324,6 +342,13 @@ def test_alpc_step_chain_of_custody(loss, cfg):
                 assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref) + 1e-7
         y, z, ysum = yn, zn, sn
     ctx.close()
+
+
+@pytest.mark.parametrize("loss", ["least_squares", "logistic"])
+@pytest.mark.parametrize("cfg", [dict(n=512, d=5000, N=2, B=100, b=4), dict(n=512, d=9000, N=2, B=70, b=2),
+                                 dict(n=512, d=13000, N=2, B=256, b=4)])
+def test_alpc_streaming_step_with_empty_slices(loss, cfg):
+    test_alpc_step_chain_of_custody(loss, cfg)  # the cluster of the shared batch J has CTAs without a column too
 
 
 def test_alpc_epochs_follow_algorithm3():
