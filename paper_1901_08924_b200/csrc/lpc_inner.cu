@@ -77,7 +77,7 @@ struct Smem {
   uint64_t mbar_meta[SMAXB / 32]; // labels and snapshot-side derivatives of 32 sampled rows are in place (used once each)
   __align__(16) float parts[SSLOTS][SG * MAXCS * 4];  // quarter-slice partial sums of the groups in flight (written by all CTAs of the cluster)
   __align__(16) float coefs[SSLOTS][SG];
-  int stream_fail;                // a bounded wait ran out somewhere in this CTA
+  int failed;                     // a bounded wait ran out somewhere in this CTA
   int issued;                     // groups whose bulk copies have been issued
 };
 
@@ -192,13 +192,14 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     if (tid == 0) {
       mbar_init(&sm.bar, 1);
       mbar_init(&sm.xbar, 1);
-      sm.stream_fail = 0;
+      sm.failed = 0;
     }
     if (tid < 64) mbar_fence_init();
   } else if (tid == 0) {
     mbar_init(&sm.bar, 1);
     mbar_init(&sm.xbar, 1);
     mbar_fence_init();
+    sm.failed = 0;
   }
   // Every CTA of the cluster announces that it is running (its barriers exist); peers wait for this before their
   // first store into this CTA's shared memory.
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       const bool ok = from_cluster ? mbar_wait_cluster(bar, parity) : mbar_wait(bar, parity);
       if (!ok) {
         atomicOr(a.dev_status, DEV_TIMEOUT);
-        sm.stream_fail = 1;
+        sm.failed = 1;
         gave_up = true;
       }
     };
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       }
     }
     __syncthreads();  // both sides are done with the ring: it now carries u to the usual owner of each coordinate
-    if (sm.stream_fail) {  // a wait ran out: give the copies still in flight a bounded chance to land before the ring is reused
+    if (sm.failed) {  // a wait ran out: give the copies still in flight a bounded chance to land before the ring is reused
       if (tid == 0)
         for (int g = max(0, sm.issued - R); g < sm.issued; ++g) mbar_wait(&sm.sbar[g % R], (uint32_t)((g / R) & 1), 100000000ull);
       __syncthreads();
@@ -591,6 +592,24 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
 
   }
 
+  // Leaving.  A CTA whose waits all ended well has received every store that its peers make into its shared memory, because each
+  // of them counts on a phase it waited for.  One that gave up has not, and a peer that is late would store into memory that
+  // another CTA may own by then.  So no CTA leaves before all of its cluster have made their last store into a peer (every wait
+  // before that is bounded, so all arrive here), and one that gave up stays another millisecond for stores on their way.
+  // The arrival comes with the last store, the wait at the very end: nobody waits there unless a peer is late.
+  auto last_store_made = [] {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  };
+  auto wait_to_leave = [&] {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (tid == 0 && sm.failed) {
+      const uint64_t t0 = global_ns();
+      while (global_ns() - t0 < 1000000ull) __nanosleep(1000);
+    }
+  };
+
   if (is_J) {  // double sampling: v^ = u_J + mu in full precision, nothing quantized
 #pragma unroll
     for (int p = 0; p < MAXP; ++p) {
@@ -601,7 +620,9 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
           if (off + e < width) a.vhat[c0 + off + e] = add_rn(u[p][e], a.mu[c0 + off + e]);
       }
     }
-    return;  // the whole cluster leaves together: no further cluster barrier on this path
+    last_store_made();
+    wait_to_leave();
+    return;  // the whole cluster takes this path
   }
   if (a.u_tap) {
 #pragma unroll
@@ -659,7 +680,10 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       st_async_cluster(&sm.s1part[rank], &sm.xbar, (uint32_t)q, __float_as_uint(s1));
       st_async_cluster(&sm.s2part[rank], &sm.xbar, (uint32_t)q, __float_as_uint(s2));
     }
-    if (!mbar_wait_cluster(&sm.xbar, 0)) atomicOr(a.dev_status, DEV_TIMEOUT);
+    if (!mbar_wait_cluster(&sm.xbar, 0)) {
+      atomicOr(a.dev_status, DEV_TIMEOUT);
+      sm.failed = 1;
+    }
   }
   if (tid == 0) {
     uint32_t m = 0;
@@ -673,6 +697,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     }
   }
   __syncthreads();
+  last_store_made();
   LPC_PHASE_MARK(6);
   const Scale sc = sm.scale;
   const bool degenerate = (sc.flags & 1u) != 0;
@@ -763,6 +788,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     a.clipped_part[worker * MAXCS + rank] = t;
   }
   LPC_PHASE_MARK(7);
+  wait_to_leave();
 }
 
 template <int BITS, bool STREAM>
