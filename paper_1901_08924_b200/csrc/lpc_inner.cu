@@ -318,7 +318,10 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       wait_for_launch_before();
     } else if (warp < SDW) {
       // -- margins: the SMW = 4 warps of a side share a group, warp w of them taking the blocks 4 w .. 4 w + 3 (a quarter
-      // of the slice) of all rows of the group; the two sides alternate groups.  Lane l holds x for the coordinates
+      // of the slice) of all rows of the group.  One side takes the groups of the even stages of the ring, the other those of the odd
+      // ones: a stage's barrier is waited for by parity, so a side has to see every phase of the stages it reads.  (With
+      // the sides alternating groups and an odd ring, a side met a stage in every second phase only and could pass with the
+      // rows of two phases ago while the copies of the phase between were on their way.)  Lane l holds x for the coordinates
       // 128 q + 4 l .. + 3 of its blocks q.  The leaves of the tree in coordinate order: four products per lane
       // (tree4), then the tree over the 32 lanes of a block, then the tree over the four blocks; the quarter sums go to
       // every CTA with columns as stores that count on that CTA's barrier of the group, and are combined there.
@@ -336,7 +339,8 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
       // after the reduction lane l holds the sum of row halving_index<2>(l & 3); lane l sends it to CTA l >> 2
       const int myrow = ((lane & 1) << 1) | ((lane >> 1) & 1);
 #pragma unroll 1
-      for (int g = warp / SMW; g < ngroups; g += SDW / SMW) {
+      for (int g = 0, s = 0; g < ngroups; ++g, s = (s + 1 == R) ? 0 : s + 1) {  // s = g % R
+        if ((s & 1) != warp / SMW) continue;
         const int cnt = min(SG, B - g * SG);
         wait_stage(g);
         // two rows at a time (eight loads in flight): the sixteen partial sums of the group are all that stays
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
         for (int h = 0; h < SG; h += 2) {
           float4 v[2][QB];
           if (full) {
-            const float* src = rows + (size_t)((g % R) * SG + h) * SL + wq * QB * 128 + lane * 4;
+            const float* src = rows + (size_t)(s * SG + h) * SL + wq * QB * 128 + lane * 4;
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
-              for (int q = 0; q < QB; ++q) v[j][q] = row4((g % R) * SG + h + j, (wq * QB + q) * 128 + lane * 4);
+              for (int q = 0; q < QB; ++q) v[j][q] = row4(s * SG + h + j, (wq * QB + q) * 128 + lane * 4);
           }
 #pragma unroll
           for (int j = 0; j < 2; ++j)
@@ -367,7 +371,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
         uint32_t seen = 0;
 #pragma unroll
         for (int i = 0; i < SG * QB; ++i) seen ^= __float_as_uint(sv[i]);
-        mbar_arrive_after(&sm.ebar[g % R], __any_sync(0xFFFFFFFFu, seen == 0x7FFFFFFFu), lane == 0);
+        mbar_arrive_after(&sm.ebar[s], __any_sync(0xFFFFFFFFu, seen == 0x7FFFFFFFu), lane == 0);
         WarpHalving<SG * QB, 0>::run(sv, lane);  // lane holds the 32-lane tree sum of (row, block) halving_index<4>(lane)
         float part = sv[0];
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 8));  // blocks 2k, 2k+1 of the row

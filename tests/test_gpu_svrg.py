@@ -143,6 +143,17 @@ def test_streaming_step_with_empty_slices(loss, cfg):
     test_inner_step_chain_of_custody(loss, cfg)
 
 
+@pytest.mark.parametrize("loss", ["least_squares", "logistic"])
+@pytest.mark.parametrize("cfg", [dict(n=2048, d=2048, N=2, B=1021, b=4), dict(n=2048, d=5000, N=2, B=1024, b=2)])
+def test_streaming_step_with_an_odd_ring(loss, cfg):
+    # five stages: the two margin sides own stages, not every second group, so that each sees every phase of its stages
+    c = dict(cfg)
+    P, ctx = _setup(c.pop("n"), c.pop("d"), loss, **c)
+    assert ctx.query(lpc.INFO_STEP_RING_STAGES) % 2 == 1
+    ctx.close()
+    test_inner_step_chain_of_custody(loss, cfg)
+
+
 @pytest.mark.parametrize("cs", [1, 2, 4, 8])
 @pytest.mark.parametrize("clip", [(orc.CLIP_NONE, 1.0), (orc.CLIP_LAMBDA, 0.9), (orc.CLIP_STD, 2.0)])
 def test_inner_step_cluster_sizes_and_clip_rules(cs, clip):
