@@ -22,6 +22,7 @@
 // coordinates of u and add the rows -- still in shared memory -- into u, then hand the stage back; one refills
 // the stages.  Every hand-over is an mbarrier phase, so waiting warps sleep in hardware and take no issue slots or
 // shared-memory bandwidth from the working ones.  Each row is read from HBM once.
+#include <algorithm>
 #include <atomic>
 
 #include <cooperative_groups.h>
@@ -42,8 +43,20 @@ constexpr int MAXB = 64;          // minibatch rows
 constexpr int MAXCS = 8;
 // streaming path
 constexpr int SG = 4;             // rows per ring stage
-constexpr int SSLOTS = 16;        // exchange slots (a peer's margins run at most 2 * SMAXR - 2 groups ahead of this CTA's u)
+constexpr int SSLOTS = 16;        // exchange slots
 constexpr int SMAXR = 8;          // ring stages at most
+// How far the ring may run with SSLOTS slots.  A slot of group h may be written again when the u of group h - SSLOTS is done
+// everywhere.  The margins of group h need its rows, so the refill of its stage, so all update warps of that CTA to have taken
+// group h - R, which they do after adding group h - R - 2: of its own u, a CTA is at most R + 1 groups ahead.  Adding group
+// h - R - 2 took the margins of all peers for it, whose update warps had by the same chain added group h - 2 R - 4: of a peer's u,
+// a CTA is at most 2 R + 3 groups ahead.
+constexpr int groups_ahead(int R, int CS) { return CS > 1 ? 2 * R + 3 : R + 1; }
+constexpr int stream_stages_limit(int CS) {
+  int R = SMAXR;
+  while (groups_ahead(R, CS) >= SSLOTS) --R;
+  return R;
+}
+static_assert(stream_stages_limit(1) == SMAXR && stream_stages_limit(2) >= 6, "the slots cover rings of the usual slices");
 constexpr int SMAXB = 1024;       // rows per worker at most
 constexpr int SDW = 8;            // warps that take margin partial sums: SDW / SG groups in flight on that side
 constexpr int SUW = 8;            // warps that own the coordinates of u
@@ -890,7 +903,7 @@ bool inner_plan(int d, int B, int want_cs, int max_smem, int* CS_out, int* SL_ou
     const size_t stage = (size_t)SG * SL * 4;
     if (fixed + meta + 3 * stage > (size_t)max_smem) continue;
     int R = (int)(((size_t)max_smem - fixed - meta) / stage);
-    if (R > SMAXR) R = SMAXR;
+    R = std::min(R, stream_stages_limit(cs));  // slices of at most 1,024 columns in clusters: 6, not 8
     *CS_out = cs; *SL_out = SL; *smem_out = fixed + meta + (size_t)R * stage; *stages_out = R;
     return true;
   }

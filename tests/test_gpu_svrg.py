@@ -155,6 +155,27 @@ def test_streaming_step_with_an_odd_ring(loss, cfg):
 
 
 @pytest.mark.parametrize("cs", [1, 2, 4, 8])
+def test_streaming_ring_stays_within_the_exchange_slots(cs):
+    # slices narrow enough for eight stages: with peers a CTA's margins run up to 2 R + 3 groups ahead of a peer's u, and
+    # there are 16 exchange slots, so clusters get at most six stages
+    cfg = dict(n=1024, d=1000, N=2, B=301, b=4)
+    c = dict(cfg)
+    P, ctx = _setup(c.pop("n"), c.pop("d"), "least_squares", **c)
+    ctx.set_option(lpc.OPT_CLUSTER_SIZE, cs)
+    assert ctx.query(lpc.INFO_STEP_CLUSTER_SIZE) == cs
+    R = ctx.query(lpc.INFO_STEP_RING_STAGES)
+    assert R == (8 if cs == 1 else 6)
+    ctx.set_option(lpc.OPT_TAP_U, 1)
+    rng = np.random.default_rng(cs)
+    xs = (rng.standard_normal(P.d) * 0.3).astype(np.float32)
+    x = (xs + rng.standard_normal(P.d).astype(np.float32) * 0.05).astype(np.float32)
+    mu = _inject_snapshot(ctx, P, xs)
+    for k in (0, 5):
+        x = _check_step(P, ctx, k, 0.05, x, xs, mu)
+    ctx.close()
+
+
+@pytest.mark.parametrize("cs", [1, 2, 4, 8])
 @pytest.mark.parametrize("clip", [(orc.CLIP_NONE, 1.0), (orc.CLIP_LAMBDA, 0.9), (orc.CLIP_STD, 2.0)])
 def test_inner_step_cluster_sizes_and_clip_rules(cs, clip):
     P, ctx = _setup(128, 4096, "least_squares", N=4, B=4, b=4, clip=clip)
