@@ -500,12 +500,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// The same arrival either way, but not before `seen` is known (two forms of the instruction, so that the choice stays).
-__device__ __forceinline__ void mbar_arrive_after(uint64_t* bar, bool seen, bool leader) {
-  if (!leader) return;
-  if (seen) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-  else mbar_arrive(bar);
-}
 // Non-blocking look at a phase: true when the phase with this parity has completed.
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;

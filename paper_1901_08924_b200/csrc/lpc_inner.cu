@@ -380,11 +380,8 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
               sv[(h + j) * QB + q] = tree4(mul_rn(v[j][q].x, xs[q].x), mul_rn(v[j][q].y, xs[q].y), mul_rn(v[j][q].z, xs[q].z),
                                            mul_rn(v[j][q].w, xs[q].w));
         }
-        // this warp has read, and used, its quarter of the stage (every partial product sum needs one of the reads)
-        uint32_t seen = 0;
-#pragma unroll
-        for (int i = 0; i < SG * QB; ++i) seen ^= __float_as_uint(sv[i]);
-        mbar_arrive_after(&sm.ebar[s], __any_sync(0xFFFFFFFFu, seen == 0x7FFFFFFFu), lane == 0);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.ebar[s]);  // this warp has read its quarter of the stage
         WarpHalving<SG * QB, 0>::run(sv, lane);  // lane holds the 32-lane tree sum of (row, block) halving_index<4>(lane)
         float part = sv[0];
         part = add_rn(part, __shfl_xor_sync(0xFFFFFFFFu, part, 8));  // blocks 2k, 2k+1 of the row
@@ -415,14 +412,10 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
 #pragma unroll
             for (int q = 0; q < UC; ++q) v[j][q] = row4(s * SG + j, q * (IGROUP / UC) + t * 4);
         }
-        // The stage may be overwritten once everybody has arrived, and an arrival can overtake shared-memory reads whose
-        // results nobody has used yet: the vote uses one word of each of them.
-        uint32_t x = 0;
-#pragma unroll
-        for (int j = 0; j < SG; ++j)
-#pragma unroll
-          for (int q = 0; q < UC; ++q) x ^= __float_as_uint(v[j][q].x);
-        mbar_arrive_after(&sm.ebar[s], __any_sync(0xFFFFFFFFu, x == 0x7FFFFFFFu), lane == 0);
+        // The stage may be overwritten once everybody has arrived.  The lanes meet in __syncwarp and the arrival is a release, so
+        // the loads above are performed before it counts, whether or not their results have been used.
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.ebar[s]);
       };
       auto add = [&](int g, const float4 (&v)[SG][UC]) {
         const int cnt = min(SG, B - g * SG);
