@@ -342,6 +342,48 @@ def test_multi_step_paths_equal_single_launches(cfg, mode):
     ref.close()
 
 
+@pytest.mark.parametrize("cfg", [
+    dict(n=2048, d=1000, N=4, B=301, b=2), dict(n=1024, d=2048, N=2, B=1021, b=4), dict(n=2048, d=8192, N=8, B=256, b=8),
+    dict(n=512, d=5000, N=2, B=100, b=4), dict(n=512, d=13000, N=2, B=129, b=3),
+])
+@pytest.mark.parametrize("method", ["lpc", "alpc"])
+def test_streaming_steps_in_graphs_and_overlapped_equal_single_launches(cfg, method):
+    # minibatches that stream: consecutive steps of one call overlap (programmatic launches), 128 of them inside a captured
+    # graph; 131 steps with graphs, without them (plain overlapped launches) and one launch at a time must give the same bits
+    c = dict(cfg)
+    P, ctx = _setup(c.pop("n"), c.pop("d"), "logistic", **c)
+    x0 = (np.random.default_rng(9).standard_normal(P.d) * 0.1).astype(np.float32)
+    count, got = 131, {}
+    for mode in ("graph", "plain", "single"):
+        cx = lpc.Context(ctx.X, ctx.y, P.loss, P.lambda_l1, P.N, P.B, P.b, P.clip_mode, P.clip_value, P.seed)
+        assert cx.query(lpc.INFO_STEP_RING_STAGES) > 0
+        cx.set_option(lpc.OPT_TAP_U, 1)
+        cx.set_option(lpc.OPT_USE_GRAPH, 1 if mode == "graph" else 0)
+        cx.set_iterate(torch.from_numpy(x0).to(DEV))
+        cx.alpc_begin()
+        cx.snapshot_full_grad()
+        many = cx.inner_steps if method == "lpc" else cx.alpc_double_sample_steps
+        one = cx.inner_step if method == "lpc" else cx.alpc_double_sample_step
+        par = (0.05,) if method == "lpc" else (0.4, 0.5, 0.3, 0.2)
+        one(*par, 0)
+        if mode == "single":
+            for k in range(1, 1 + count):
+                one(*par, k)
+        else:
+            many(*par, 1, count)
+        cx.sync_status()
+        assert cx.query(lpc.INFO_LOOP_LAUNCHES) == 0
+        which = (lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_CLIPPED, lpc.BUF_U, lpc.BUF_V, lpc.BUF_BATCH_IDX, lpc.BUF_COEF)
+        which += (lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_VHAT) if method == "alpc" else ()
+        got[mode] = [cx.get_buffer(w).cpu().numpy() for w in which]
+        if method == "lpc":  # the last row of the sampled rows and coefficients belongs to Algorithm 2's shared batch
+            got[mode][6], got[mode][7] = got[mode][6][: P.N], got[mode][7][: P.N]
+        cx.close()
+    for w, a, b2, s in zip(which, got["graph"], got["plain"], got["single"]):
+        assert _same(a, s) and _same(b2, s), w
+    ctx.close()
+
+
 @pytest.mark.parametrize("loss", ["least_squares", "logistic"])
 @pytest.mark.parametrize("cfg", [dict(n=128, d=1000, N=4, B=2, b=2), dict(n=128, d=8192, N=4, B=16, b=8),
                                  dict(n=64, d=4096, N=2, B=4, b=4), dict(n=1024, d=2048, N=2, B=130, b=4)])
