@@ -172,6 +172,8 @@ class Context:
     def _layout(self, length, bits, seg_offsets):
         """C array of the offsets, segment count and stride in words; the last layout of a width is kept, because a training
         loop asks for the same one in every round."""
+        if seg_offsets is not None and type(seg_offsets) is not list:  # arrays, tensors and tuples compare as lists of integers
+            seg_offsets = [int(v) for v in seg_offsets]
         hit = self._layouts.get((length, bits))
         if hit is not None and hit[0] == seg_offsets:
             return hit[1:]

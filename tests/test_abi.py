@@ -68,3 +68,23 @@ def test_init_rejects_bad_arguments_before_touching_the_device(lpc):
         assert not h.value
     assert L.lpc_destroy(None) == lpc.OK
     assert L.lpc_inner_step(None, 0.1, 0) == lpc.ERR_INVALID_ARG
+
+
+def test_offsets_of_a_call_may_be_a_list_a_tuple_an_array_or_a_tensor(lpc):
+    # the binding keeps the last layout of a length and width; a second call with the same length must compare the offsets
+    # whatever holds them
+    import numpy as np
+    import torch
+
+    ctx = lpc.Context.__new__(lpc.Context)  # the layout cache needs no device
+    ctx._h, ctx._layouts = C.c_void_p(None), {}
+    want = [0, 10, 10, 33, 100]
+    for offs in (want, tuple(want), np.array(want), np.array(want, np.int32), torch.tensor(want)):
+        for _ in range(2):
+            arr, nseg, stride = ctx._layout(100, 4, offs)
+            assert list(arr) == want and nseg == 4 and stride == 20
+    offs = np.array(want)
+    offs[1] = 9  # changed in place between two calls
+    assert list(ctx._layout(100, 4, offs)[0]) == [0, 9, 10, 33, 100]
+    assert ctx._layout(100, 4, None)[:2] == (None, 1)
+    assert list(ctx._layout(100, 4, np.array([0, 100]))[0]) == [0, 100]
