@@ -578,9 +578,9 @@ def kernel_pass(dev, log2_len):
     for k in range(2):
         q.quantize_pack(U[:, :short], k)                             # the short-vector path
     q.sync_status()
-    one = q.query(lpc.INFO_QUANT_ONE_LAUNCH)
+    launches = q.query(lpc.INFO_QUANT_LAUNCHES)
     q.close()
-    return {"kernel_pass": "8 x 2^%d" % log2_len, "widths": done, "one_launch_on_2^20": one}
+    return {"kernel_pass": "8 x 2^%d" % log2_len, "widths": done, "launches_on_2^20": launches}
 
 
 def tiny_logistic_bench(dev):

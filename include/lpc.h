@@ -182,8 +182,9 @@ int lpc_packed_words(int64_t len, int32_t b, int64_t* words_out); /* ceil(len*b/
  *   clipped_out nullable, N * nseg counts of coordinates outside the hull
  * Vectors longer than L2 are read twice (once for ||u||_inf and the variance, once to quantize) by three launches that overlap;
  * when all N vectors together take at most LPC_ONE_LAUNCH_BYTES the second look is served by L2, and vectors of at most
- * 65,536 values in one segment take ONE launch, a cluster per worker that keeps the values in registers
- * (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches that off).  Same codes either way.
+ * 65,536 values in one segment, with b in {1, 2, 3, 4, 8}, own scales and at most four CTAs per SM in all, take ONE launch, a
+ * cluster per worker that keeps the values in registers (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches that off).  Same codes
+ * either way; LPC_INFO_QUANT_LAUNCHES says which it was.
  * N, b and the clip rule come from the context.
  */
 int lpc_quantize_pack(lpc_ctx* ctx, const float* U, const float* U_sub, int64_t len, int64_t ld,
@@ -298,7 +299,10 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
 #define LPC_INFO_AGGREGATE_SPLIT 9         /* last lpc_unpack_average_prox: CTAs that shared one tile of 8192 coordinates (1, 2 or 4) */
 #define LPC_INFO_QUANT_PIPELINED_RUNS 10   /* last lpc_quantize_pack: runs of 8 tiles per worker that were whole tiles of one segment and
                                               so took the second pass's software-pipelined loop (unless that worker's scale was
-                                              degenerate); 0 unless every worker's vector starts on a 16-byte boundary (ld % 4 == 0) */
+                                              degenerate; short vectors take it in shorter runs); 0 unless every worker's vector starts
+                                              on a 16-byte boundary (ld % 4 == 0), for b = 32, and when the call was one launch */
+#define LPC_INFO_QUANT_LAUNCHES 14         /* last lpc_quantize_pack: kernels it launched.  1: a cluster per worker (or an empty vector);
+                                              3: statistics, scale, codes; 4: the same and the unified scale */
 int lpc_query(const lpc_ctx* ctx, int what, int64_t* out);
 
 /* Per-kernel device time measured with CUDA events on the context's stream while LPC_OPT_PROFILE is

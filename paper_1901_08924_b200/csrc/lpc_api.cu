@@ -114,7 +114,7 @@ struct lpc_ctx {
   size_t q_scale_cap = 0;
   int loop_cooperative = 1;       // LPC_OPT_LOOP_COOPERATIVE
   int one_launch = 1;             // LPC_OPT_ONE_LAUNCH_QUANTIZE
-  int last_one_launch = 0;
+  int last_one_launch = 0, last_quant_launches = 0;
   unsigned long long* coded_host = nullptr;  // pinned: entropy (double) and Huffman length of coded_cap messages each
   size_t coded_cap = 0;
   // graph replay
@@ -820,6 +820,7 @@ int lpc_query(const lpc_ctx* c, int what, int64_t* out) {
     case LPC_INFO_SNAPSHOT_ROWS_PER_TILE: *out = c->snapR; return LPC_OK;
     case LPC_INFO_SNAPSHOT_STAGES: *out = c->snapStages; return LPC_OK;
     case LPC_INFO_QUANT_ONE_LAUNCH: *out = c->last_one_launch; return LPC_OK;
+    case LPC_INFO_QUANT_LAUNCHES: *out = c->last_quant_launches; return LPC_OK;
     case LPC_INFO_AGGREGATE_SPLIT: *out = c->last_split; return LPC_OK;
     case LPC_INFO_QUANT_PIPELINED_RUNS: *out = c->last_pipelined_runs; return LPC_OK;
     default: return LPC_ERR_INVALID_ARG;
@@ -875,12 +876,12 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   a.clipped_out = clipped_out ? clipped_out : c->q_clip; a.count_clipped = clipped_out ? 1 : 0; a.dev_status = c->dev_status;
   a.shared_scale = c->shared_scale;
   const bool vec = aligned16(U) && (!U_sub || aligned16(U_sub)) && (ld % 4 == 0);
-  const bool fixed_width = (c->b == 1 || c->b == 2 || c->b == 3 || c->b == 4 || c->b == 8);  // the other widths go tile by tile
-  c->last_pipelined_runs = vec && fixed_width ? p.whole_runs : 0;
   c->last_one_launch = (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
                         (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) ? 1 : 0;
-  if (c->last_one_launch) c->last_pipelined_runs = 0;
-  if (c->last_one_launch && quantize_fits_cluster(a, c->sm_count)) {
+  const bool cluster = c->last_one_launch && quantize_fits_cluster(a, c->sm_count);
+  c->last_pipelined_runs = vec && c->b != 32 && !cluster ? p.whole_runs : 0;
+  c->last_quant_launches = cluster ? 1 : quantize_pack_launches(a);
+  if (cluster) {
     ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
     CU(c, launch_quantize_cluster(a, c->stream));
   } else {

@@ -75,6 +75,7 @@ typedef void (*LaunchHook)(void* user, int kind, int begin);
 // Tiles per CTA of the second pass, and whether the run of tiles that starts at tile0 consists of whole tiles of one
 // segment (the condition, besides 16-byte aligned vectors and a non-degenerate scale, for its pipelined loop).
 int quantize_run_tiles();
+int quantize_pack_launches(const QuantArgs& a);  // kernels that launch_quantize_pack launches
 cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
 // The same for short vectors, one cluster per worker and nothing looked at twice.
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count);

@@ -864,6 +864,11 @@ cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st) {
 
 int quantize_run_tiles() { return QRUN; }
 
+int quantize_pack_launches(const QuantArgs& a) {
+  if (a.N <= 0 || a.nseg <= 0) return 0;
+  return (a.ntiles > 0 ? 3 : 1) + (a.shared_scale ? 1 : 0);  // statistics, scale, codes; nothing but the scale of an empty vector
+}
+
 cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
   if (a.N <= 0 || a.nseg <= 0) return cudaSuccess;
   const dim3 grid((unsigned)(a.ntiles > 0 ? a.ntiles : 1), (unsigned)a.N), block(QT);

@@ -185,9 +185,9 @@ def test_three_level_codes_full_length_windows(b):
 @pytest.mark.parametrize("b", [1, 2, 3, 4, 8, 16])
 @pytest.mark.parametrize("log2_len", [16, 20])
 def test_one_launch_quantizer_short_vectors_bit_exact(b, log2_len):
-    # the sweep's short vectors (8 x 2^16, 8 x 2^20) stay in L2 between the statistics and the codes: one cooperative
-    # launch; at 2^20 the 1,024 tiles exceed the resident CTAs, so a CTA takes several tiles of different workers.
-    # Twice in a row: the arrival counters carry over from call to call.
+    # the sweep's short vectors: 8 x 2^16 takes one launch, a cluster of eight CTAs per worker, where the width is a fixed
+    # one; 8 x 2^20 (and b = 16) takes three launches that overlap, the second look at the values from L2.  Twice in a row:
+    # the scratch and the clipped counts of a call must not leak into the next.
     N, seed = 8, 71
     length = 1 << log2_len
     U = synth.gradient_vectors(N, length, "student_t3", seed=b + log2_len)
@@ -197,15 +197,17 @@ def test_one_launch_quantizer_short_vectors_bit_exact(b, log2_len):
         codes, delta, clipped = q.quantize_pack(Ud, k)
         q.sync_status()
         assert q.query(lpc.INFO_QUANT_ONE_LAUNCH) == 1
+        one = log2_len == 16 and b != 16
+        assert q.query(lpc.INFO_QUANT_LAUNCHES) == (1 if one else 3)
         W = orc.packed_words(length, b)
         for i in range(N):
             w, dl, cl = orc.quantize_pack(U[i].numpy(), b, orc.CLIP_STD, 2.0, seed, i, k)
             assert (_u32(codes)[i, :W] == w).all(), (k, i)
             assert _bits(np.float32(dl).reshape(1))[0] == _u32(delta)[i, 0] and int(_u32(clipped)[i, 0]) == cl
-    # the three-launch path on the same input gives the same bits
+    # the three-launch path on the same input gives the same bits (where the calls above took it too, the same call again)
     q.set_option(lpc.OPT_ONE_LAUNCH_QUANTIZE, 0)
     c2, d2, cl2 = q.quantize_pack(Ud, 4)
     q.sync_status()
-    assert q.query(lpc.INFO_QUANT_ONE_LAUNCH) == 0
+    assert q.query(lpc.INFO_QUANT_ONE_LAUNCH) == 0 and q.query(lpc.INFO_QUANT_LAUNCHES) == 3
     assert torch.equal(c2, codes) and torch.equal(d2.view(torch.int32), delta.view(torch.int32)) and torch.equal(cl2, clipped)
     q.close()

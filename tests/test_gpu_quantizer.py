@@ -54,7 +54,8 @@ def test_philox_streams_match_oracle_bitwise():
 @pytest.mark.parametrize("clip", [(orc.CLIP_NONE, 1.0), (orc.CLIP_LAMBDA, 0.85), (orc.CLIP_STD, 2.5)])
 @pytest.mark.parametrize("one_launch", [1, 0])
 def test_quantize_pack_bit_exact(b, clip, one_launch):
-    # one_launch = 1: the single cooperative launch that short vectors take (b = 32 always takes three launches)
+    # one_launch = 1: the cluster per worker that short vectors of the fixed widths take; the other widths, and b = 32, take
+    # three launches whatever the option says
     N, seed, k = 3, 1234, 7
     rng = np.random.default_rng(b * 10 + clip[0])
     for length in (1, 7, 8, 9, 31, 33, 257, 2047, 8191, 8192, 8193, 3 * 8192 + 1001):
@@ -65,6 +66,7 @@ def test_quantize_pack_bit_exact(b, clip, one_launch):
         codes, delta, clipped = ctx.quantize_pack(torch.from_numpy(U).to(DEV), k)
         ctx.sync_status()
         assert ctx.query(lpc.INFO_QUANT_ONE_LAUNCH) == (1 if one_launch and b != 32 else 0)
+        assert ctx.query(lpc.INFO_QUANT_LAUNCHES) == (1 if one_launch and b in (1, 2, 3, 4, 8) else 3)
         rc, rd, rcl = _oracle_quantize(U, b, clip[0], clip[1], seed, k)
         assert (delta.cpu().numpy() == rd).all(), (length, delta, rd)
         assert (_u32(codes) == rc).all(), length
@@ -223,6 +225,7 @@ def test_cluster_per_worker_matches_the_three_launches(b, length):
                 got[one] = [t.clone() for t in ctx.quantize_pack(U, k, U_sub=subtrahend)]
                 ctx.sync_status()
                 assert ctx.query(lpc.INFO_QUANT_ONE_LAUNCH) == one
+                assert ctx.query(lpc.INFO_QUANT_LAUNCHES) == (1 if one else 3)
                 ctx.close()
             W = orc.packed_words(length, b)
             assert torch.equal(got[1][0][:, :W], got[0][0][:, :W])
@@ -256,3 +259,24 @@ def test_run_time_widths_whole_tiles_and_decode(b):
         xr = orc.unpack_average_prox(np.ascontiguousarray(rc[:, :W]), rd.reshape(-1), length, b, None, x0, 0.1, 1e-3)
         assert (x.cpu().numpy().view(np.uint32) == xr.view(np.uint32)).all()
         ctx.close()
+
+
+@pytest.mark.parametrize("length,b,offs,option,shared,launches,runs", [
+    (65536, 4, None, 1, 0, 1, 0),                      # a cluster per worker
+    (65536, 4, None, 0, 0, 3, 1),                      # the same vector with that path switched off
+    (65536, 5, None, 1, 0, 3, 1),                      # a width known at run time: three launches, the pipelined loop
+    (9 * 8192, 4, None, 1, 0, 3, 2),                   # nine whole tiles, a run of eight and one of one: too long for a cluster
+    (65536, 4, [0, 32768, 65536], 1, 0, 3, 0),         # two tensors: three launches, no run of eight tiles of one of them
+    (65536, 4, None, 1, 1, 4, 1),                      # unified scale
+    (65536, 32, None, 1, 0, 3, 0),                     # full precision
+    (0, 4, None, 1, 0, 1, 0),
+])
+def test_queries_say_what_the_last_call_ran(length, b, offs, option, shared, launches, runs):
+    ctx = _ctx(2, b, orc.CLIP_STD, 2.0, 1)
+    ctx.set_option(lpc.OPT_ONE_LAUNCH_QUANTIZE, option)
+    ctx.set_option(lpc.OPT_SHARED_SCALE, shared)
+    ctx.quantize_pack(torch.randn((2, length), device=DEV), 0, seg_offsets=offs)
+    ctx.sync_status()
+    assert ctx.query(lpc.INFO_QUANT_LAUNCHES) == launches
+    assert ctx.query(lpc.INFO_QUANT_PIPELINED_RUNS) == runs
+    ctx.close()
