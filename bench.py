@@ -241,7 +241,7 @@ def run_ours(args):
         if "snapshot" in kernels:
             ks = kernels["snapshot"]
             roofline["kernels"].append(roofline_entry("snapshot_kernel", args.workload, ks["avg_us"], ks["bytes_per_launch"], peak,
-                                                      "snapshot_kernel", n * d))
+                                                      "snapshot_kernel", n * d, short="snapshot"))
     launches_per_epoch = 2 + sum(kernels[k]["launches_per_step"] for k in kernels if k != "snapshot")
 
     out = {
@@ -287,8 +287,33 @@ def run_ours(args):
     ctx.close()
     dist_util.barrier()
     if rank == 0:
-        print(json.dumps(out))
+        detail = json.dumps(out)
+        if args.detail_out:
+            with open(args.detail_out, "w") as f:
+                f.write(detail + "\n")
+        else:
+            print(detail, file=sys.stderr, flush=True)
+        print(json.dumps(headline(out)))
     dist_util.shutdown()
+
+
+def headline(out):
+    """The line for standard output: every key of the measurement itself and microseconds and fraction of the copy rate of
+    each kernel that the extra legs time, short enough (three thousand characters) to be kept whole by whoever records it.
+    The legs in full go to standard error, or to the file of --detail-out."""
+    head = {k: v for k, v in out.items() if k not in ("kernels", "quantize_aggregate", "alpc", "fused_large_batch", "tiny_logistic",
+                                                      "launch_plan", "wall_s", "objective_end")}
+    if out.get("roofline"):
+        r = dict(out["roofline"])
+        r.pop("traffic_source", None)
+        r["note"] = "latency-bound: a strict step-to-step dependency; kernels: [us, fraction of the copy rate]"
+        r["kernels"] = {e["short"]: [round(e["avg_us"], 1), round(e["frac"], 3)] for e in r["kernels"] if "short" in e}
+        head["roofline"] = r
+    if out.get("tiny_logistic"):
+        head["tiny_logistic_step_us"] = out["tiny_logistic"]["step_us"]
+    if out.get("alpc"):
+        head["alpc_step_us"] = {b: out["alpc"][b]["step_us"] for b in ("b2", "b8") if b in out["alpc"]}
+    return head
 
 
 NOMINAL_HBM_GBS = 8000.0   # the vendor's round figure for the part's HBM3e, for context beside the measured copy rate
@@ -320,7 +345,7 @@ def traffic_of(name, units):
     return round(bytes_ * units / cap_units), "%s, scaled by %g" % (src, units / cap_units)
 
 
-def roofline_entry(kernel, workload, avg_us, alg_bytes, peak, traffic_name=None, units=None, note=None):
+def roofline_entry(kernel, workload, avg_us, alg_bytes, peak, traffic_name=None, units=None, note=None, short=None):
     gbs = alg_bytes / avg_us * 1e-3
     tr, src = traffic_of(traffic_name, units) if traffic_name else (None, None)
     e = {"kernel": kernel, "workload": workload, "avg_us": round(avg_us, 3), "algorithmic_bytes": int(alg_bytes),
@@ -330,6 +355,8 @@ def roofline_entry(kernel, workload, avg_us, alg_bytes, peak, traffic_name=None,
         e["traffic_source"] = src
     if note:
         e["note"] = note
+    if short:
+        e["short"] = short  # its name in the headline
     return e
 
 
@@ -438,24 +465,26 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
         roof.append(roofline_entry(name, wl, qp["ms"] * 1e3, qp["bytes"], peak,
                                    note="input stays in L2 between the two looks at it: bound 4 + b/8 B per element; launch-bound at "
                                         "this size (see quantize_aggregate.launch_floor_us)" if resident else
-                                   "two passes: 8 + b/8 B per element"))
+                                   "two passes: 8 + b/8 B per element", short="quantize 2^%d" % l2))
         if not resident and qp["stats_ms"] > 0:
             roof.append(roofline_entry("stats_kernel", wl, qp["stats_ms"] * 1e3, N * (1 << l2) * 4, peak, "stats_kernel", N * (1 << l2)))
             roof.append(roofline_entry("quantize_kernel<4>", wl, qp["pack_ms"] * 1e3, N * (1 << l2) * 4.5, peak, "quantize_kernel<4>", N * (1 << l2)))
         roof.append(roofline_entry("unpack_average_prox_kernel<4>", wl, ua["ms"] * 1e3, ua["bytes"], peak,
                                    None if resident else "unpack_average_prox_kernel<4>", 1 << l2,
-                                   note="launch-bound at this size" if resident else None))
+                                   note="launch-bound at this size" if resident else None, short="aggregate 2^%d" % l2))
     mid = min(26, top)
     Um = U[:, : 1 << mid]
     for b in (1, 2, 3, 8):
         r = point("gauss_len2^%d_b%d_clip2" % (mid, b), Um, b, 2.0)
         wl = "sweep N=8, len 2^%d, N(0,1), b=%d, clip 2 std" % (mid, b)
-        roof.append(roofline_entry("quantize+pack, b=%d" % b, wl, r["quantize_pack"]["ms"] * 1e3, r["quantize_pack"]["bytes"], peak))
+        roof.append(roofline_entry("quantize+pack, b=%d" % b, wl, r["quantize_pack"]["ms"] * 1e3, r["quantize_pack"]["bytes"], peak,
+                                   short="quantize b%d" % b))
         if b == 3 and r["quantize_pack"]["pack_ms"] > 0:  # (a short vector goes through the one-launch path instead)
             roof.append(roofline_entry("quantize_kernel<3>", wl, r["quantize_pack"]["pack_ms"] * 1e3, N * (1 << mid) * (4 + 3 / 8), peak,
                                        "quantize_kernel<3>", N * (1 << mid)))
         roof.append(roofline_entry("unpack_average_prox_kernel<%d>" % b, wl, r["unpack_average_prox"]["ms"] * 1e3,
-                                   r["unpack_average_prox"]["bytes"], peak, "unpack_average_prox_kernel<3>" if b == 3 else None, 1 << mid))
+                                   r["unpack_average_prox"]["bytes"], peak, "unpack_average_prox_kernel<3>" if b == 3 else None, 1 << mid,
+                                   short="aggregate b%d" % b))
     if full:
         for clip in (1.0, 4.0):
             point("gauss_len2^%d_b4_clip%g" % (mid, clip), Um, 4, clip)
@@ -484,7 +513,7 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
         "bits_per_coordinate": {"raw": b, "entropy_bound": round(float(ent.mean()) / length, 4),
                                 "huffman": round(float(huf.astype("float64").mean()) / length, 4)}}
     roof.append(roofline_entry("code_histogram_swar_kernel<4>", "8 x 2^%d 4-bit codes" % mid, th * 1e3, bh, peak,
-                               "code_histogram_swar_kernel<4>", N * length))
+                               "code_histogram_swar_kernel<4>", N * length, short="histogram"))
     q.set_option(lpc.OPT_SHARED_SCALE, 1)
     tqs = _kernel_ms(q, lambda i: q.quantize_pack(Um, i, codes_out=codes, delta_out=delta, clipped_out=clipped), 4,
                      ("quant_stats", "other", "quant_pack", "quant_fused"))
@@ -507,7 +536,8 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
                     "worker_decode_prox": {"ms": round(tw, 4), "bytes": bw, "gbs": round(bw / tw * 1e-6, 1),
                                            "frac": round(bw / tw * 1e-6 / peak, 4)}}
         roof.append(roofline_entry("server_reduce4_kernel (%s)" % name, "8 x 2^%d 4-bit codes in, %d-bit stream out" % (mid, bo),
-                                   ts * 1e3, bs, peak, "server_reduce4_kernel<7, sum>" if scheme == lpc.SCHEME_SERVER_SUM else None, length))
+                                   ts * 1e3, bs, peak, "server_reduce4_kernel<7, sum>" if scheme == lpc.SCHEME_SERVER_SUM else None, length,
+                                   short="server sum" if scheme == lpc.SCHEME_SERVER_SUM else "server requantize"))
         del x2
     q.sync_status()
     res["parameter_server_N8_len2^%d_b4" % mid] = ps
@@ -541,8 +571,8 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
         "unpack_average_prox": {"ms": round(ta, 4), "bytes": ba, "gbs": round(ba / ta * 1e-6, 1), "frac": round(ba / ta * 1e-6 / peak, 4)},
         "combined_gbs": round((bq + ba) / (tq + ta) * 1e-6, 1)}
     wl = "62 tensors of an 18-layer residual network, 11.7M parameters, N=16, b=4, clip 2.5 std per tensor"
-    roof.append(roofline_entry("quantize+pack with u = cur - snap (3 launches)", wl, tq * 1e3, bq, peak))
-    roof.append(roofline_entry("unpack_average_prox_kernel<4> (+ mu)", wl, ta * 1e3, ba, peak))
+    roof.append(roofline_entry("quantize+pack with u = cur - snap (3 launches)", wl, tq * 1e3, bq, peak, short="quantize 62 tensors"))
+    roof.append(roofline_entry("unpack_average_prox_kernel<4> (+ mu)", wl, ta * 1e3, ba, peak, short="aggregate 62 tensors"))
     q.close()
     res["roofline_kernels"] = roof
     return res
@@ -646,7 +676,7 @@ def fused_large_batch_bench(dev, peak, n=65536, steps=30):
             out["roofline_kernels"].append(roofline_entry(
                 "inner_kernel<%d, stream> (fused sampling + SVRG difference + scale + quantize + pack)" % b,
                 "logistic %d x 8192, N=32 workers, B=%d rows per worker, b=%d" % (n, B, b), tw * 1e3, bw, peak,
-                "inner_kernel<2, stream>" if b == 2 else None, N * B))
+                "inner_kernel<2, stream>" if b == 2 else None, N * B, short="stream B%d b%d" % (B, b)))
             ctx.close()
     return out
 
@@ -691,10 +721,10 @@ def alpc_bench(dev, peak):
         out["roofline_kernels"].append(roofline_entry(
             "persist_kernel<%d, alpc> (one launch = %d steps of Algorithm 2)" % (b, m), out["workload"] + ", b=%d" % b,
             loop * 1e3, m * step_bytes, peak, note="latency chain per step: rows of N+1 minibatches, tagged code words "
-            "written and read, second-estimator words"))
+            "written and read, second-estimator words", short="alpc loop b%d" % b))
         if b == 2:
             out["roofline_kernels"].append(roofline_entry("snapshot_kernel", out["workload"], snap * 1e3, n * d * 4 + 8 * n + 4 * d,
-                                                          peak, "snapshot_kernel (logistic)", n * d))
+                                                          peak, "snapshot_kernel (logistic)", n * d, short="snapshot logistic"))
         ctx.close()
     # the strongly convex case (Algorithm 2, elastic net with sigma = L/1000, Theorem 3's tau1 and alpha)
     b, sigma = 2, L / 1000.0
@@ -824,6 +854,7 @@ def main():
     ap.add_argument("--fused-large-batch-only", type=int, default=0, metavar="ROWS",
                     help="run only the large-minibatch leg of the fused worker kernel on a ROWS x 8192 matrix "
                          "(a small case for profiler captures)")
+    ap.add_argument("--detail-out", default="", metavar="FILE", help="write the measurement with all its legs here (default: standard error)")
     args = ap.parse_args()
     if args.kernel_pass:
         import torch
