@@ -326,15 +326,15 @@ L2_BYTES = 126e6
 TRAFFIC = {
     "snapshot_kernel": (268.56e6 + 4.25e6, 16384 * 4096, "profiles/snapshot_kernel_ls_16384x4096.md"),
     "snapshot_kernel (logistic)": (537.00e6 + 4.16e6, 16384 * 8192, "profiles/snapshot_kernel_logistic_16384x8192.md"),
-    "stats_kernel": (536.96e6 + 4.20e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
-    "quantize_kernel<4>": (536.95e6 + 14.21e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
-    "quantize_kernel<3>": (536.92e6 + 8.00e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
-    "unpack_average_prox_kernel<4>": (134.25e6 + 25.20e6, 1 << 24, "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
-    "unpack_average_prox_kernel<3>": (117.47e6 + 21.75e6, 1 << 24, "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
+    "stats_kernel": (536.90e6 + 0.29e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
+    "quantize_kernel<4>": (536.96e6 + 10.59e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
+    "quantize_kernel<3>": (536.97e6 + 6.38e6, 8 * (1 << 24), "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
+    "unpack_average_prox_kernel<4>": (134.27e6 + 24.19e6, 1 << 24, "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
+    "unpack_average_prox_kernel<3>": (117.47e6 + 20.07e6, 1 << 24, "profiles/quantize_aggregate_N8_len2p24_b4_b3.md"),
     "code_histogram_swar_kernel<4>": (67.13e6 + 0.26e6, 8 * (1 << 24), "profiles/server_reduce4_and_code_histogram_N8_len2p24_b4.md"),
     "server_reduce4_kernel<7, sum>": (67.12e6 + 1.84e6, 1 << 24, "profiles/server_reduce4_and_code_histogram_N8_len2p24_b4.md"),
     "inner_kernel<4> (per step)": (2.220e6, 1, "profiles/inner_step_kernels_ls_16384x4096_N16_B8_b4.md"),
-    "inner_kernel<2, stream>": (234.3e6 + 4.8e6, 32 * 256, "profiles/streaming_worker_kernel_logistic_16384x8192_N32_B256_b2.md"),
+    "inner_kernel<2, stream>": (234.0e6 + 3.6e6, 32 * 256, "profiles/streaming_worker_kernel_logistic_16384x8192_N32_B256_b2.md"),
 }
 
 
@@ -479,7 +479,7 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
         wl = "sweep N=8, len 2^%d, N(0,1), b=%d, clip 2 std" % (mid, b)
         roof.append(roofline_entry("quantize+pack, b=%d" % b, wl, r["quantize_pack"]["ms"] * 1e3, r["quantize_pack"]["bytes"], peak,
                                    short="quantize b%d" % b))
-        if b == 3 and r["quantize_pack"]["pack_ms"] > 0:  # (a short vector goes through the one-launch path instead)
+        if b == 3 and r["quantize_pack"]["pack_ms"] > 0:  # (a short vector takes a cluster per worker instead)
             roof.append(roofline_entry("quantize_kernel<3>", wl, r["quantize_pack"]["pack_ms"] * 1e3, N * (1 << mid) * (4 + 3 / 8), peak,
                                        "quantize_kernel<3>", N * (1 << mid)))
         roof.append(roofline_entry("unpack_average_prox_kernel<%d>" % b, wl, r["unpack_average_prox"]["ms"] * 1e3,

@@ -21,7 +21,9 @@
 // count on the receiver's mbarrier of that group; two turn the complete margins into coefficients; eight own the
 // coordinates of u and add the rows -- still in shared memory -- into u, then hand the stage back; one refills
 // the stages.  Every hand-over is an mbarrier phase, so waiting warps sleep in hardware and take no issue slots or
-// shared-memory bandwidth from the working ones.  Each row is read from HBM once.
+// shared-memory bandwidth from the working ones.  Each row is read from HBM once.  What bounds it is the chain of hand-overs of a
+// group of four rows, 0.61 us whatever their bytes, and at 128 CTAs memory as well: 32 workers with rows of 8,192 take 53 us for
+// 256 rows each (5.0 TB/s) and 170 us for 1,024 (6.3 TB/s) under an event pair, of which 6 us are the floor of the launch.
 #include <algorithm>
 #include <atomic>
 
@@ -412,7 +414,8 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
             for (int q = 0; q < UC; ++q) v[j][q] = row4(s * SG + j, q * (IGROUP / UC) + t * 4);
         }
         // The stage may be overwritten once everybody has arrived.  The lanes meet in __syncwarp and the arrival is a release, so
-        // the loads above are performed before it counts, whether or not their results have been used.
+        // the loads above are performed before it counts, whether or not their results have been used.  (A warp vote on the
+        // loaded words in front of it gave the same bits and took 55.9 instead of 52.7 us at 256 rows, 184 instead of 176 at 1,024.)
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.ebar[s]);
       };
