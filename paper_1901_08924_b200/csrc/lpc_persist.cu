@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
 #pragma unroll
       for (int e = 0; e < EPT; ++e) u[p][e] = mul_rn((EPT == 8 && swz) ? uw[e ^ (EPT / 2)] : uw[e], invB);
     }
-    if (a.u_tap && t == pa.count - 1) {
+    if (a.u_tap && !is_J && t == pa.count - 1) {  // N vectors: the shared batch has none
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
         const int off = p * PSPAN + tid * EPT;
