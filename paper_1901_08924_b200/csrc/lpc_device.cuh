@@ -271,6 +271,51 @@ __device__ __forceinline__ float index_as_float(uint32_t code, int b) {
   return __fsub_rn(biased, 8388608.f + (float)(1 << (b - 1)));
 }
 
+// ---- two floats at a time (one instruction each on sm_100) -----------------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 p, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p)); }
+__device__ __forceinline__ f32x2 mul2_rn(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2_rn(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2_rn(f32x2 a, f32x2 b) {  // two separate subtractions
+  float a0, a1, b0, b1;
+  unpack2(a, a0, a1);
+  unpack2(b, b0, b1);
+  return pack2(__fsub_rn(a0, b0), __fsub_rn(a1, b1));
+}
+__device__ __forceinline__ f32x2 fma2_rn(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2_ru(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float fma_rd_sat(float a, float b, float c) {  // clamped to [0, 1] after rounding down
+  float r;
+  asm("fma.rm.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float fma_ru_sat(float a, float b, float c) {  // clamped to [0, 1] after rounding up
+  float r;
+  asm("fma.rp.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // The signed codebook indices of the 8 codes of one coordinate group (8 * BITS payload bits in `lo`), as exact
 // floats, for the fixed widths.  The codes are moved into the mantissa of 2^23 by byte permutes (one integer
 // instruction per code after a few shared masks), then one exact subtraction removes 2^23 and the offset.
@@ -310,6 +355,32 @@ __device__ __forceinline__ void decode8(uint64_t lo, float* k) {
   }
 }
 
+// The same as pairs of floats, COUNT (2, 4 or 8) of them from the first code on: the subtraction of 2^23 and the offset takes
+// one instruction for two codes.
+template <int BITS, int COUNT>
+__device__ __forceinline__ void decode_pairs(uint64_t lo, f32x2* k) {
+  constexpr uint32_t MAGIC = 0x4B000000u;  // 2^23
+  float f[8];
+  if constexpr (BITS == 1 || BITS == 3) {
+    decode8<BITS>(lo, f);
+#pragma unroll
+    for (int e = 0; e < COUNT / 2; ++e) k[e] = pack2(f[2 * e], f[2 * e + 1]);
+  } else {
+    const uint32_t w0 = (uint32_t)lo, w1 = (uint32_t)(lo >> 32);
+#pragma unroll
+    for (int e = 0; e < COUNT; ++e) {
+      uint32_t sel, byte;
+      if constexpr (BITS == 8) { sel = e < 4 ? w0 : w1; byte = e & 3; }
+      else if constexpr (BITS == 4) { sel = (e & 1) ? (w0 >> 4) & 0x0F0F0F0Fu : w0 & 0x0F0F0F0Fu; byte = e >> 1; }
+      else { sel = (w0 >> (2 * (e & 3))) & 0x0303u; byte = e >> 2; }
+      f[e] = __uint_as_float(__byte_perm(sel, MAGIC, 0x7440u + byte));
+    }
+    const f32x2 off = pack2(-(8388608.f + (float)(1 << (BITS - 1))), -(8388608.f + (float)(1 << (BITS - 1))));
+#pragma unroll
+    for (int e = 0; e < COUNT / 2; ++e) k[e] = add2_rn(pack2(f[2 * e], f[2 * e + 1]), off);
+  }
+}
+
 // acc + delta * k for a signed codebook index k of a BITS-wide code.  For one- and two-bit codes k is -2, -1, 0 or 1:
 // the product is exact (as long as 2 delta is finite), so one fused multiply-add rounds exactly like the separate
 // multiply and add of wider codes.
@@ -317,6 +388,17 @@ template <int BITS>
 __device__ __forceinline__ float add_scaled_index(float acc, float delta, float k) {
   if constexpr (BITS == 1 || BITS == 2) return __fmaf_rn(delta, k, acc);
   else return add_rn(acc, mul_rn(delta, k));
+}
+
+template <int BITS>
+__device__ __forceinline__ f32x2 add_scaled_pair(f32x2 acc, f32x2 delta, f32x2 k) {
+  if constexpr (BITS == 1 || BITS == 2) return fma2_rn(delta, k, acc);
+  else {  // as two separate operations: ptxas may join a product and a sum of pairs
+    float a0, a1, p0, p1;
+    unpack2(acc, a0, a1);
+    unpack2(mul2_rn(delta, k), p0, p1);
+    return pack2(add_rn(a0, p0), add_rn(a1, p1));
+  }
 }
 
 __device__ __forceinline__ float soft_threshold(float w, float kappa) {
@@ -339,46 +421,6 @@ __device__ __forceinline__ void count_outside(float& cnt, float u, float T, floa
       "@p add.rn.f32 %0, %0, 0f3F800000;\n\t}"
       : "+f"(cnt)
       : "f"(u), "f"(T), "f"(lower));
-}
-
-// ---- two floats at a time (one instruction each on sm_100) -----------------------------------------------------------
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 p, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p)); }
-__device__ __forceinline__ f32x2 mul2_rn(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2_rn(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 sub2_rn(f32x2 a, f32x2 b) {  // two separate subtractions
-  float a0, a1, b0, b1;
-  unpack2(a, a0, a1);
-  unpack2(b, b0, b1);
-  return pack2(__fsub_rn(a0, b0), __fsub_rn(a1, b1));
-}
-__device__ __forceinline__ f32x2 fma2_ru(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float fma_rd_sat(float a, float b, float c) {  // clamped to [0, 1] after rounding down
-  float r;
-  asm("fma.rm.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ float fma_ru_sat(float a, float b, float c) {  // clamped to [0, 1] after rounding up
-  float r;
-  asm("fma.rp.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
 }
 
 // The 8 * BITS packed bits of one coordinate group (code e in bits [e BITS, (e+1) BITS)) from its eight scaled values

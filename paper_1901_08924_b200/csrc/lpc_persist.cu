@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     const unsigned long long* ll_in = pa.ll + (size_t)rpar * N * groups * wpg;
     int cc[NP];
     bool act[NP];
-    float acc[NP][EPT];
+    float acc[NP][EPT];          // BITS = 0
+    f32x2 acc2[NP][EPT / 2];     // fixed widths: pairs of coordinates
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int off = p * PSPAN + tid * EPT;
@@ -343,6 +344,8 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       act[p] = off < SL && cc[p] < d;
 #pragma unroll
       for (int e = 0; e < EPT; ++e) acc[p][e] = 0.f;
+#pragma unroll
+      for (int e = 0; e < EPT / 2; ++e) acc2[p][e] = 0ull;
     }
     unsigned long long cw[CH][NP][NW], vw[ALPC ? NP * EPT : 1], dw;
     // No load is predicated and no round is special (branches and a peeled first round would double the size of this
@@ -417,18 +420,17 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
             uint64_t lo = (uint64_t)(uint32_t)cw[j][p][0], hi = 0;
             if constexpr (NW >= 2) lo |= (uint64_t)(uint32_t)cw[j][p][1] << 32;
             if constexpr (NW >= 4) hi = (uint64_t)(uint32_t)cw[j][p][2] | ((uint64_t)(uint32_t)cw[j][p][3] << 32);
-            float kf[8];
             if constexpr (BITS == 0) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) kf[e] = index_as_float(extract_bits(lo, hi, e * b, b), b);
+              for (int e = 0; e < 8; ++e) acc[p][e] = add_scaled_index<BITS>(acc[p][e], di, index_as_float(extract_bits(lo, hi, e * b, b), b));
             } else {
               // this thread's EPT codes start at bit wshift of the word: decode them as the first codes of a group
-              // (the entries past EPT are not used and cost nothing)
               if constexpr (TB < 32) lo = ((uint32_t)lo >> wshift) & ((1u << TB) - 1u);
-              decode8<BITS ? BITS : 1>(lo, kf);
-            }
+              f32x2 k2[EPT / 2];
+              decode_pairs<BITS ? BITS : 1, EPT>(lo, k2);
 #pragma unroll
-            for (int e = 0; e < EPT; ++e) acc[p][e] = add_scaled_index<BITS>(acc[p][e], di, kf[e]);
+              for (int e = 0; e < EPT / 2; ++e) acc2[p][e] = add_scaled_pair<BITS>(acc2[p][e], pack2(di, di), k2[e]);
+            }
           }
         }
       }
@@ -443,6 +445,12 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
         if (ok || wait_expired(it, t0)) break;
         issue_vhat();
       }
+    }
+    if constexpr (BITS != 0) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int e = 0; e < EPT / 2; ++e) unpack2(acc2[p][e], acc[p][2 * e], acc[p][2 * e + 1]);
     }
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
