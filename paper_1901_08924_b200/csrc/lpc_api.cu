@@ -93,6 +93,7 @@ struct lpc_ctx {
   unsigned long long* flags = nullptr;    // scale words: 2 x 256, 128 bytes apart, + 1 abort word
   unsigned long long* ll = nullptr;       // code words: 2 x N x dpow2/8 groups x ll_wpg
   unsigned long long* ll_vhat = nullptr;  // second estimator of Algorithm 2: 2 x dpow2
+  unsigned long long* ll_x = nullptr;     // new point of the owned update: 2 x dpow2
   int ll_wpg = 1;                         // words per group of 8 coordinates
   uint32_t ll_tag = 0;                    // tags handed out so far; the buffers start zeroed and tag 0 is never used
   int64_t persist_launches = 0;
@@ -408,13 +409,14 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     pa.row_slots = kind == 0 ? c->pSlots : c->aSlots;
     pa.count = (int)count; pa.eta = kind == 0 ? p[0] : 0.f; pa.lambda_l1 = c->lambda_l1;
     pa.pub = c->flags; pa.abort_flag = reinterpret_cast<unsigned int*>(c->flags + 512 * 16); pa.x_out = c->x;
-    pa.ll = c->ll; pa.ll_vhat = c->ll_vhat; pa.wpg = c->ll_wpg;
+    pa.ll = c->ll; pa.ll_vhat = c->ll_vhat; pa.ll_x = c->ll_x; pa.wpg = c->ll_wpg;
     if ((uint64_t)c->ll_tag + (uint64_t)count >= 0xFFFFFFF0ull) {  // tags would wrap: start over from cleared buffers
       int dp = 32;
       while (dp < c->d) dp <<= 1;
       CU(c, cudaMemsetAsync(c->flags, 0, (512 * 16 + 1) * sizeof(unsigned long long), c->stream));
       CU(c, cudaMemsetAsync(c->ll, 0, sizeof(unsigned long long) * 2 * (size_t)c->N * (size_t)(dp / 8) * c->ll_wpg, c->stream));
       CU(c, cudaMemsetAsync(c->ll_vhat, 0, sizeof(unsigned long long) * 2 * (size_t)dp, c->stream));
+      CU(c, cudaMemsetAsync(c->ll_x, 0, sizeof(unsigned long long) * 2 * (size_t)dp, c->stream));
       c->ll_tag = 0;
     }
     pa.tag_base = c->ll_tag;
@@ -594,6 +596,7 @@ int lpc_init(lpc_ctx** out, const float* X, const float* y, int64_t n, int32_t d
     c->ll_wpg = (b <= 4) ? 1 : (b <= 8) ? 2 : (b <= 16) ? 4 : 8;
     want(&c->ll, 2 * (size_t)N * (size_t)(dp / 8) * c->ll_wpg);
     want(&c->ll_vhat, 2 * (size_t)dp);
+    want(&c->ll_x, 2 * (size_t)dp);
     want(&c->idx_tap, (size_t)(N + 1) * B); want(&c->coef_tap, (size_t)(N + 1) * B);
     want(&c->codes, (size_t)N * (size_t)roundup4(((int64_t)d * b + 31) / 32));  // inner_seg's stride, one segment
     c->dpad = snapshot_dpad(d);

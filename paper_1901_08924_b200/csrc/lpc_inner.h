@@ -50,6 +50,7 @@ struct PersistArgs {
   unsigned long long* pub;   // scale delta: 2 x 256 words, 128 bytes apart, word (worker * CS + rank)
   unsigned long long* ll;    // codes: 2 x N x (CS*SL/8) groups x wpg words
   unsigned long long* ll_vhat;  // Algorithm 2's second estimator: 2 x CS*SL words
+  unsigned long long* ll_x;     // the new point, where its coordinates have owners: 2 x CS*SL words
   uint32_t tag_base;
   int wpg;                   // words per group of 8 coordinates: 1 (b <= 4), 2 (b <= 8), 4 (b <= 16), 8 (b = 32)
   unsigned int* abort_flag;  // zero at launch; set when a bounded wait ran out

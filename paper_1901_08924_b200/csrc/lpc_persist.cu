@@ -47,6 +47,7 @@ constexpr int PT = 256;
 constexpr int PGROUP = PT * 8;
 constexpr int PMAXP = 2;   // passes per CTA: SL <= 4096
 constexpr int PMAXB = 64;
+constexpr int COPIER = PMAXB;  // threads COPIER + a start the row copies
 constexpr int PMAXCS = 8;
 constexpr int PMAXFLAGS = 256;
 constexpr int PMAXN = 64;      // workers in the one-launch loop (a lane carries the scales of PMAXN / 32 of them)
@@ -56,6 +57,9 @@ struct PSmem {
   uint64_t bar[2];
   __align__(16) float coef[PMAXB];
   float wpart[PMAXB * PMAXP * 8];
+  // OWN: scale times index of every worker and owned coordinate (not shared with wpart: no barrier separates the owners' sums
+  // from the margins of a warp that already has its slice of the new point)
+  __align__(16) float prod[PGROUP + 8 * PMAXN];
   // cluster exchange slots, written by the peers through distributed shared memory as tagged words, two
   // step-parity halves: margin partial sums (slot b * PMAXCS + rank) and statistics (max, S1, S2 per rank)
   unsigned long long mx[2][PMAXB * PMAXCS];
@@ -66,6 +70,9 @@ struct PSmem {
   Scale scale;
   __align__(16) uint8_t stage[PT * 16];
 };
+
+// OWN: coordinates of a slice that each worker's CTA owns, whole groups of eight.
+__host__ __device__ constexpr int owned_coords(int SL, int N) { return ((SL + N - 1) / N + 7) & ~7; }
 
 // Tagged 64-bit words (payload | tag << 32): relaxed, device scope, one indivisible access each.
 __device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p) {
@@ -143,8 +150,10 @@ __device__ unsigned long long g_trace[64 * 16];
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && t >= 8 && t < 72)         \
       g_trace[(t - 8) * 16 + (i)] = global_ns();                                            \
   } while (0)
+#define LPC_TRACE_MARK_AT(i, step) do { const int t = (step); LPC_TRACE_MARK(i); } while (0)
 #else
 #define LPC_TRACE_MARK(i) do { } while (0)
+#define LPC_TRACE_MARK_AT(i, step) do { } while (0)
 #endif
 
 // A thread's EPT consecutive row values of a slice from shared memory (zero outside the existing columns).
@@ -190,8 +199,14 @@ __device__ __forceinline__ float tree_ept(const float* v) {
 //      thread of the CTA work, which shortens each serial phase of a step; a group of 8 coordinates (one Philox block,
 //      one tagged code word for b <= 4) is then shared by 8 / EPT neighbouring lanes.  BITS = 0 and NP = 2 use EPT = 8.
 // ALPC: Algorithm 2's step (coupling, double sampling on one more cluster, y/z updates) instead of Algorithm 1's.
-template <int BITS, int NP, int EPT, bool ALPC>
+// OWN: the update of a coordinate is made by one CTA instead of by every cluster.  A slice is divided among the workers' CTAs of
+//      its rank; the owner decodes all workers' codes of its coordinates (a word or two per thread), averages, steps, and sends the
+//      new point to the clusters as tagged words.  That is one more crossing of the chip per step, and N times less to load and
+//      decode: it pays where there are many workers (pays_to_own).
+template <int BITS, int NP, int EPT, bool ALPC, bool OWN>
 __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
+  static_assert(!OWN || NP == 1, "one pass");
+  static_assert(2 * COPIER <= PT && COPIER % 32 == 0, "rows are drawn by the first threads, copied by the next");
   static_assert(EPT == 8 || ((EPT == 4 || EPT == 2) && BITS != 0 && NP == 1), "narrow threads: fixed widths, one pass");
   constexpr int PSPAN = PT * EPT;               // coordinates per pass
   constexpr int LPG = 8 / EPT;                  // lanes that share a group of 8 coordinates
@@ -233,38 +248,39 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   __syncthreads();
 
-  // Thread a < B owns minibatch slot a.  fetch_rows(t, sb, lo, hi) samples step t's row for the slots lo <= a < hi,
-  // starts the bulk copy of this CTA's slice of it into row slot (sb + a) % RS and loads its label and cached
-  // snapshot margin into registers (a step ahead, so these loads never stall the step that issues them).  The
-  // barrier of step t (bar[t & 1]) gets its one arrival from the call that covers the last slot.
+  // Thread a < B owns minibatch slot a: it draws step t's row and loads its label and cached snapshot margin into registers, a
+  // step ahead, so that these loads never stall the step that issues them.  Thread COPIER + a, of a warp that has no serial part
+  // in a step, draws the same row and starts the bulk copy of this CTA's slice of it into row slot (sb + a) % RS: the rows
+  // lo <= a < hi at a time.  The barrier of step t (bar[t & 1]) gets its one arrival with the last of them.
   const int64_t samp_span = (a.sample_global || is_J) ? a.n : a.n / N;  // rows this cluster samples from
   const int64_t samp_lo = (a.sample_global || is_J) ? 0 : (int64_t)worker * samp_span;
+  const int slot_of = tid < COPIER ? tid : tid - COPIER;
   int64_t row_next = 0, row_cur = 0;
   float y_next = 0.f, y_cur = 0.f, ms_next = 0.f, ms_cur = 0.f;
-  auto sample_rows = [&](int t, int lo, int hi) {
-    if (tid >= lo && tid < hi)
+  auto sample_rows = [&](int t) {
+    if (tid < 2 * COPIER && slot_of < B)
       row_next = sample_row_out_of_line(a.seed, is_J ? TAG_BATCH_J : TAG_BATCH, is_J ? 0u : (uint32_t)worker,
-                                        a.k_base + (uint64_t)t, (uint32_t)tid, samp_lo, samp_span);
+                                        a.k_base + (uint64_t)t, (uint32_t)slot_of, samp_lo, samp_span);
   };
-  auto copy_rows = [&](int t, int sb, int lo, int hi) {  // after sample_rows(t, lo, hi)
-    if (hi <= lo) return;
-    uint64_t* bar = &sm.bar[t & 1];
-    if (tid == 0 && width > 0) {
-      const uint32_t bytes = row_bytes * (uint32_t)(hi - lo);
-      if (hi == B) mbar_expect_tx(bar, bytes);  // arrives as well: the phase can now complete
-      else asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-    }
-    if (tid >= lo && tid < hi) {
-      int slot = sb + tid;
-      if (slot >= RS) slot -= RS;
-      if (width > 0) bulk_load(rows + (size_t)slot * SL, a.X + row_next * (int64_t)d + c0, row_bytes, bar);
+  auto load_labels = [&] {  // after sample_rows
+    if (tid < B) {
       y_next = a.y[row_next];
       ms_next = a.margins[row_next];
     }
   };
-  auto fetch_rows = [&](int t, int sb, int lo, int hi) {
-    sample_rows(t, lo, hi);
-    copy_rows(t, sb, lo, hi);
+  auto copy_rows = [&](int t, int sb, int lo, int hi) {  // after sample_rows(t)
+    if (hi <= lo || width <= 0) return;
+    uint64_t* bar = &sm.bar[t & 1];
+    if (tid == COPIER) {
+      const uint32_t bytes = row_bytes * (uint32_t)(hi - lo);
+      if (hi == B) mbar_expect_tx(bar, bytes);  // arrives as well: the phase can now complete
+      else asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+    }
+    if (tid >= COPIER + lo && tid < COPIER + hi) {
+      int slot = sb + slot_of;
+      if (slot >= RS) slot -= RS;
+      bulk_load(rows + (size_t)slot * SL, a.X + row_next * (int64_t)d + c0, row_bytes, bar);
+    }
   };
 
   // this thread's slice of the iterate and of the snapshot gradient stay in registers for the whole loop
@@ -281,7 +297,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
   }
   // Algorithm 2 keeps y, z, the running sum of y and the snapshot in registers too; xr is then the coupled point
   float yr[ALPC ? NP : 1][EPT], zr[ALPC ? NP : 1][EPT], sr[ALPC ? NP : 1][EPT], xtr[ALPC ? NP : 1][EPT];
-  if constexpr (ALPC) {
+  if constexpr (ALPC && !OWN) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int off = p * PSPAN + tid * EPT;
@@ -297,7 +313,37 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
   }
   const float tau3 = __fsub_rn(__fsub_rn(1.0f, pa.tau1), pa.tau2);
   const float kappa_y = mul_rn(pa.inv4L, pa.lambda_l1), kappa_z = mul_rn(pa.alpha, pa.lambda_l1);
-  if (pa.count > 0) fetch_rows(0, 0, 0, B);
+  auto couple = [&](float z, float xt, float y) {  // step 6 of Algorithm 2: x = tau1 z + tau2 x~ + (1 - tau1 - tau2) y
+    return add_rn(add_rn(mul_rn(pa.tau1, z), mul_rn(pa.tau2, xt)), mul_rn(tau3, y));
+  };
+  // OWN: the coordinate whose state this thread keeps, if any
+  const int chunk = OWN ? owned_coords(SL, N) : 0;
+  const int oc = c0 + worker * chunk + tid;
+  const bool owner = OWN && !is_J && tid < chunk && worker * chunk + tid < SL && oc < d;
+  float ox = 0.f, omu = 0.f, oy = 0.f, oz = 0.f, os = 0.f, oxt = 0.f;
+  if constexpr (OWN) {
+    if (owner) {
+      omu = a.mu[oc];
+      if constexpr (ALPC) {
+        oy = pa.y[oc]; oz = pa.z[oc]; os = pa.ysum[oc]; oxt = pa.xt[oc];
+        ox = couple(oz, oxt, oy);
+      } else {
+        ox = a.x[oc];
+      }
+    }
+    if constexpr (ALPC) {  // the first step's coupled point
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) {
+        const int c = c0 + tid * EPT + e;
+        if (tid * EPT + e < width) xr[0][e] = couple(pa.z[c], pa.xt[c], pa.y[c]);
+      }
+    }
+  }
+  if (pa.count > 0) {
+    sample_rows(0);
+    load_labels();
+    copy_rows(0, 0, 0, B);
+  }
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
   // Every spin in this kernel ends: after about two seconds without progress the thread records a timeout and
@@ -474,6 +520,114 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     if constexpr (ALPC) wcur = mul_rn(wcur, pa.theta);  // the next step's snapshot weight (Algorithm 2's last step)
   };
 
+  // OWN: the same update by the owners of the coordinates, then everybody's slice of the new point.
+  auto update_owned = [&](unsigned int target, auto between) {
+    const int rpar = (pa.count - (int)target) & 1;
+    const uint32_t tag = pa.tag_base + target;
+    unsigned long long vw = 0;
+    if (!is_J) {
+      const unsigned long long* vq = pa.ll_vhat + (size_t)rpar * groups * 8 + (owner ? oc : 0);
+      if (ALPC && owner) vw = ld_word(vq);
+      // item i: group i % G of this CTA's coordinates, worker i / G; with all N workers' words of a group in one CTA their
+      // products with the scales go to shared memory and each coordinate's owner adds them in worker order
+      const int G = chunk >> 3;
+      bool first = true;
+#pragma unroll 1
+      for (int i = tid; first || i < G * N; i += PT) {
+        const int j = min(i / G, N - 1), gi = i - (i / G) * G, off = worker * chunk + gi * 8;
+        const bool have = i < G * N && off < SL && c0 + off < d;
+        const unsigned long long* dq = pa.pub + ((size_t)rpar * PMAXFLAGS + j * CS + rank) * PUB_STRIDE;
+        const unsigned long long* q = pa.ll + (((size_t)rpar * N + j) * groups + (have ? (c0 + off) >> 3 : 0)) * wpg;
+        unsigned long long dw = 0, w[WMAX];
+        uint64_t t0 = 0;
+#pragma unroll 1
+        for (uint32_t it = 0;; ++it) {
+          bool ok = true;
+          if (have) {
+            dw = ld_word(dq);
+#pragma unroll
+            for (int k = 0; k < WMAX; ++k) w[k] = (k < wpg) ? ld_word(q + k) : (unsigned long long)tag << 32;
+          }
+          if (first) {
+            between();
+            first = false;
+          }
+          if (have) {
+            ok = word_tag(dw) == tag;
+#pragma unroll
+            for (int k = 0; k < WMAX; ++k) ok = ok && word_tag(w[k]) == tag;
+          }
+          if (ok || wait_expired(it, t0)) break;
+        }
+        if (have) {
+          const float di = __uint_as_float((uint32_t)dw);
+          float pr[8];
+          if (b == 32) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) pr[e] = mul_rn(di, c0 + off + e < d ? __uint_as_float((uint32_t)w[e < WMAX ? e : 0]) : 0.f);
+          } else {
+            uint64_t lo = (uint32_t)w[0], hi = 0;
+            if constexpr (WMAX >= 2) lo |= (uint64_t)(uint32_t)w[1] << 32;
+            if constexpr (WMAX >= 4) hi = (uint64_t)(uint32_t)w[2] | ((uint64_t)(uint32_t)w[3] << 32);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) pr[e] = 0.f;
+            if constexpr (BITS == 0) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) pr[e] = mul_rn(di, index_as_float(extract_bits(lo, hi, e * b, b), b));
+            } else {  // the product of a scale and a one- or two-bit index is exact: adding it later rounds like a multiply-add
+              f32x2 k2[4];
+              decode_pairs<BITS ? BITS : 1, 8>(lo, k2);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) unpack2(mul2_rn(pack2(di, di), k2[e]), pr[2 * e], pr[2 * e + 1]);
+            }
+          }
+          float4* to = reinterpret_cast<float4*>(sm.prod + j * chunk + gi * 8);
+          to[0] = make_float4(pr[0], pr[1], pr[2], pr[3]);
+          to[1] = make_float4(pr[4], pr[5], pr[6], pr[7]);
+        }
+      }
+      __syncthreads();
+      LPC_TRACE_MARK_AT(3, (int)target);
+      if (owner) {
+        float acc = 0.f;
+#pragma unroll 8
+        for (int j = 0; j < N; ++j) acc = add_rn(acc, sm.prod[j * chunk + tid]);
+        const float v = add_rn(mul_rn(acc, invN), omu);
+        if constexpr (ALPC) {
+          uint64_t t0 = 0;
+          for (uint32_t it = 0; word_tag(vw) != tag && !wait_expired(it, t0); ++it) vw = ld_word(vq);
+          oy = mul_rn(soft_threshold(__fsub_rn(ox, mul_rn(pa.inv4L, v)), kappa_y), pa.cy);
+          oz = mul_rn(soft_threshold(__fsub_rn(oz, mul_rn(pa.alpha, __uint_as_float((uint32_t)vw))), kappa_z), pa.cz);
+          os = add_rn(os, mul_rn(wcur, oy));
+          if ((int)target < pa.count) ox = couple(oz, oxt, oy);
+        } else {
+          ox = soft_threshold(__fsub_rn(ox, mul_rn(pa.eta, v)), kappa);
+        }
+        if (pa.v_tap) pa.v_tap[oc] = v;
+        st_word(pa.ll_x + (size_t)rpar * groups * 8 + oc, __float_as_uint(ox), tag);
+      }
+      if constexpr (ALPC) wcur = mul_rn(wcur, pa.theta);
+    } else {
+      between();
+    }
+    if ((int)target == pa.count) return;
+    unsigned long long xw[EPT];
+    uint64_t t0 = 0;
+#pragma unroll 1
+    for (uint32_t it = 0;; ++it) {
+      bool ok = true;
+#pragma unroll
+      for (int e = 0; e < EPT; e += 2) {  // pairs exist or not as a whole; instead of one that does not, the slice's first
+        const int c = c0 + tid * EPT + e;
+        ld_word2(pa.ll_x + (size_t)rpar * groups * 8 + (tid * EPT + e < width ? c : width > 0 ? c0 : 0), xw[e], xw[e + 1]);
+        ok = ok && word_tag(xw[e]) == tag && word_tag(xw[e + 1]) == tag;
+      }
+      if (__all_sync(0xFFFFFFFFu, ok) || __any_sync(0xFFFFFFFFu, wait_expired(it, t0))) break;
+    }
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) xr[0][e] = __uint_as_float((uint32_t)xw[e]);
+  };
+
   int sb = 0;  // first row slot of the current step, (t * B) % RS
 #pragma unroll 1
   for (int t = 0; t <= pa.count; ++t) {  // the pass t = count only applies the last step's update (one copy of that code)
@@ -487,7 +641,6 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     if (sb_next >= RS) sb_next -= RS;
     LPC_TRACE_MARK(0);
     row_cur = row_next; y_cur = y_next; ms_cur = ms_next;
-    // a thread that fetches its row of step t+1 only after u is formed keeps this step's label and margin until then
     const int64_t row_use = row_cur;
     const float y_use = y_cur, ms_use = ms_cur;
 
@@ -511,24 +664,30 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     // fetch they leave a few hundred nanoseconds unused (measured: 5.35 / 5.14 / 4.97 us per step for loads first /
     // fetch first / this order on the least-squares workload).
     const bool more = t + 1 < pa.count;
-    if (more) sample_rows(t + 1, 0, PA);
+    if (more) sample_rows(t + 1);
     LPC_TRACE_MARK(2);
     // The snapshot side of this step's coefficients, l'(m~_a), depends on nothing of this step: the owner of a minibatch
     // slot forms it while the peers' words are on their way (for the logistic loss it is half of the fp64 work).
     float gs_use = 0.f;
     auto ahead = [&] {
-      if (more) copy_rows(t + 1, sb_next, 0, PA);
+      if (more) {
+        load_labels();
+        copy_rows(t + 1, sb_next, 0, PA);
+      }
       if (tid < B && t < pa.count) gs_use = deriv_out_of_line(a.loss, ms_use, y_use);
     };
-    if (t > 0) apply_update((unsigned int)t, ahead);
-    else ahead();
+    if (t > 0) {
+      if constexpr (OWN) update_owned((unsigned int)t, ahead);
+      else apply_update((unsigned int)t, ahead);
+    } else {
+      ahead();
+    }
     if (t == pa.count) break;
-    if constexpr (ALPC) {  // step 6: x = tau1 z + tau2 x~ + (1 - tau1 - tau2) y
+    if constexpr (ALPC && !OWN) {  // step 6
 #pragma unroll
       for (int p = 0; p < NP; ++p)
 #pragma unroll
-        for (int e = 0; e < EPT; ++e)
-          xr[p][e] = add_rn(add_rn(mul_rn(pa.tau1, zr[p][e]), mul_rn(pa.tau2, xtr[p][e])), mul_rn(tau3, yr[p][e]));
+        for (int e = 0; e < EPT; ++e) xr[p][e] = couple(zr[p][e], xtr[p][e], yr[p][e]);
     }
     LPC_TRACE_MARK(4);
 
@@ -733,58 +892,53 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     }
     __syncthreads();  // u is formed everywhere: nobody reads this step's rows any more
     LPC_TRACE_MARK(10);
-    if (t + 1 < pa.count) fetch_rows(t + 1, sb_next, PA, B);  // into the slots this step's rows leave free
+    if (more) copy_rows(t + 1, sb_next, PA, B);  // into the slots this step's rows leave free
     if (is_J) {
       sb = sb_next;
       continue;
     }
-    if (tid == 0) {
-      uint32_t m = 0;
-      for (int w = 0; w < 8; ++w) m = max(m, sm.wmax[w]);
-      float s1 = 0.f, s2 = 0.f;
-      if (a.clip_mode == CLIP_STD) {
-        s1 = tree8(sm.ws1);
-        s2 = tree8(sm.ws2);
-        if (NP == 2) { s1 = add_rn(s1, tree8(sm.ws1 + 8)); s2 = add_rn(s2, tree8(sm.ws2 + 8)); }
+    if (warp == 0) {  // lane 8 k + i, k = 0, 1, 2 for max |u|, S1, S2: the block's from those of warp i, then the rank i's
+      const int k = lane >> 3, i = lane & 7;
+      auto join = [&](uint32_t x, uint32_t y) { return k == 0 ? max(x, y) : __float_as_uint(add_rn(__uint_as_float(x), __uint_as_float(y))); };
+      auto join_lanes = [&](uint32_t v, int count) {  // tree order over a power of two of neighbouring lanes
+        for (int m = 1; m < count; m <<= 1) v = join(v, __shfl_xor_sync(0xFFFFFFFFu, v, m));
+        return v;
+      };
+      const bool sums = a.clip_mode == CLIP_STD;
+      const float* part = k == 1 ? sm.ws1 : sm.ws2;
+      uint32_t v = k == 0 ? sm.wmax[i] : (sums ? __float_as_uint(part[i]) : 0u);
+      v = join_lanes(v, 8);
+      if constexpr (NP == 2) {
+        const uint32_t v2 = join_lanes((k > 0 && sums) ? __float_as_uint(part[8 + i]) : 0u, 8);
+        v = join(v, v2);
       }
       LPC_TRACE_MARK(11);
-      float S1 = s1, S2 = s2;
-      if (CS > 1) {  // the same exchange for the statistics: (max |u|, S1, S2) of every rank
-        for (int q = 0; q < CS; ++q) {
-          st_cluster_word(&sm.sx[xpar][0 * PMAXCS + rank], (uint32_t)q, m, tag);
-          st_cluster_word(&sm.sx[xpar][1 * PMAXCS + rank], (uint32_t)q, __float_as_uint(s1), tag);
-          st_cluster_word(&sm.sx[xpar][2 * PMAXCS + rank], (uint32_t)q, __float_as_uint(s2), tag);
-        }
-        unsigned long long w[3][PMAXCS];
+      if (CS > 1) {
+        const bool mine = k < 3 && i < CS;  // this lane's word to rank i, and the one from there
+        if (mine) st_cluster_word(&sm.sx[xpar][k * PMAXCS + rank], (uint32_t)i, v, tag);
         uint64_t t0 = 0;
         for (uint32_t it = 0;; ++it) {
           bool ok = true;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-#pragma unroll
-            for (int q = 0; q < PMAXCS; ++q) {
-              w[j][q] = ld_shared_word(&sm.sx[xpar][j * PMAXCS + min(q, CS - 1)]);  // past the cluster: the last rank again
-              ok = ok && word_tag(w[j][q]) == tag;
-            }
+          if (mine) {
+            const unsigned long long w = ld_shared_word(&sm.sx[xpar][k * PMAXCS + i]);
+            ok = word_tag(w) == tag;
+            v = (uint32_t)w;
           }
-          if (ok || wait_expired(it, t0)) break;
+          if (__all_sync(0xFFFFFFFFu, ok) || __any_sync(0xFFFFFFFFu, wait_expired(it, t0))) break;
         }
-        float p1[PMAXCS], p2[PMAXCS];
-        m = 0;
-#pragma unroll
-        for (int q = 0; q < PMAXCS; ++q) {
-          m = max(m, (uint32_t)w[0][q]);
-          p1[q] = __uint_as_float((uint32_t)w[1][q]);
-          p2[q] = __uint_as_float((uint32_t)w[2][q]);
-        }
-        if (a.clip_mode == CLIP_STD) { S1 = tree_small(p1, CS); S2 = tree_small(p2, CS); }
+        v = join_lanes(v, CS);
       }
-      sm.scale = scale_out_of_line(m, S1, S2, d, b, a.clip_mode, a.clip_value);
-      // delta travels as a tagged word, one per CTA: the readers of rank r take every worker's rank-r word
-      st_word(pa.pub + ((size_t)wpar * PMAXFLAGS + worker * CS + rank) * PUB_STRIDE, __float_as_uint(sm.scale.delta), tag);
-      if (rank == 0) {
-        if (last) a.delta[worker] = sm.scale.delta;
-        if (sm.scale.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
+      const uint32_t m = __shfl_sync(0xFFFFFFFFu, v, 0);
+      const float S1 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 8)), S2 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 16));
+      const Scale own = scale_out_of_line(m, S1, S2, d, b, a.clip_mode, a.clip_value);
+      if (lane == 0) {
+        sm.scale = own;
+        // delta travels as a tagged word, one per CTA: the readers of rank r take every worker's rank-r word
+        st_word(pa.pub + ((size_t)wpar * PMAXFLAGS + worker * CS + rank) * PUB_STRIDE, __float_as_uint(own.delta), tag);
+        if (rank == 0) {
+          if (last) a.delta[worker] = own.delta;
+          if (own.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
+        }
       }
     }
     __syncthreads();
@@ -904,8 +1058,13 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     sb = sb_next;
   }
 
-  // the slices of the final state go back to memory (worker 0's cluster)
-  if (worker == 0) {
+  // the final state goes back to memory: from the owners, or from worker 0's cluster
+  if constexpr (OWN) {
+    if (owner) {
+      pa.x_out[oc] = ox;  // Algorithm 2: the coupled point of the last step
+      if constexpr (ALPC) { pa.y[oc] = oy; pa.z[oc] = oz; pa.ysum[oc] = os; }
+    }
+  } else if (worker == 0) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int off = p * PSPAN + tid * EPT;
@@ -945,28 +1104,40 @@ void fill_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int cs, int
 using PersistKernel = void (*)(PersistArgs);
 
 template <int BITS, bool ALPC>
-PersistKernel pick_shape(int np, int ept) {
+PersistKernel pick_shape(int np, int ept, bool own) {
   if constexpr (BITS != 0) {
-    if (np == 1 && ept == 4) return persist_kernel<BITS, 1, 4, ALPC>;
-    if (np == 1 && ept == 2) return persist_kernel<BITS, 1, 2, ALPC>;
+    if (np == 1 && ept == 4) return own ? persist_kernel<BITS, 1, 4, ALPC, true> : persist_kernel<BITS, 1, 4, ALPC, false>;
+    if (np == 1 && ept == 2) return own ? persist_kernel<BITS, 1, 2, ALPC, true> : persist_kernel<BITS, 1, 2, ALPC, false>;
   }
-  return np == 2 ? persist_kernel<BITS, 2, 8, ALPC> : persist_kernel<BITS, 1, 8, ALPC>;
+  if (np == 2) return persist_kernel<BITS, 2, 8, ALPC, false>;
+  return own ? persist_kernel<BITS, 1, 8, ALPC, true> : persist_kernel<BITS, 1, 8, ALPC, false>;
 }
 template <bool ALPC>
-PersistKernel pick_width(int b, int np, int ept) {
+PersistKernel pick_width(int b, int np, int ept, bool own) {
   switch (b) {
-    case 1: return pick_shape<1, ALPC>(np, ept);
-    case 2: return pick_shape<2, ALPC>(np, ept);
-    case 4: return pick_shape<4, ALPC>(np, ept);
-    case 8: return pick_shape<8, ALPC>(np, ept);
-    default: return pick_shape<0, ALPC>(np, ept);
+    case 1: return pick_shape<1, ALPC>(np, ept, own);
+    case 2: return pick_shape<2, ALPC>(np, ept, own);
+    case 4: return pick_shape<4, ALPC>(np, ept, own);
+    case 8: return pick_shape<8, ALPC>(np, ept, own);
+    default: return pick_shape<0, ALPC>(np, ept, own);
   }
 }
-// The instantiation for code width b, slice SL and algorithm.
-PersistKernel pick_kernel(int b, int SL, bool alpc) {
+// Whether the update is left to the owners of the coordinates.  With more workers than one round of loads takes (CH in
+// apply_update) the second round alone is as long as the second crossing; the widths known at run time load up to eight words per
+// group and decode slowly.  us per step, everybody / owners: Algorithm 2, d = 8,192, N = 32, b = 2: 9.68 / 8.47, b = 8: 10.2 / 8.7;
+// Algorithm 1, d = 4,096, b = 4: N = 17: 5.84 / 4.86, N = 16: 4.70 / 4.84; d = 1,024, N = 32: 5.22 / 4.81, N = 2: 4.31 / 4.37;
+// b = 3: N = 16, d = 512: 9.27 / 5.78, N = 2: 5.69 / 5.47; b = 32, d = 2,048, N = 16: 10.9 / 5.3, N = 4: 6.5 / 5.6.
+bool pays_to_own(int b, int SL, int N) {
+  const int ept = persist_coords_per_thread(b, SL);
+  if (SL > PT * ept || owned_coords(SL, N) > PT) return false;  // one pass, one owned coordinate per thread
+  return N > 16 || !(b == 1 || b == 2 || b == 4 || b == 8);
+}
+// The instantiation for code width b, slice SL, N workers and algorithm.
+PersistKernel pick_kernel(int b, int SL, int N, bool alpc) {
   const int ept = persist_coords_per_thread(b, SL);
   const int np = (SL > PT * ept) ? 2 : 1;
-  return alpc ? pick_width<true>(b, np, ept) : pick_width<false>(b, np, ept);
+  const bool own = pays_to_own(b, SL, N);
+  return alpc ? pick_width<true>(b, np, ept, own) : pick_width<false>(b, np, ept, own);
 }
 
 int max_clusters(PersistKernel k, int cs, size_t smem) {
@@ -1020,7 +1191,7 @@ bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_sme
     int slots = (int)(((size_t)max_smem - fixed) / one);
     if (slots > 2 * B) slots = 2 * B;
     const size_t smem = fixed + (size_t)slots * one;
-    if (max_clusters(pick_kernel(b, SL, alpc != 0), cs, smem) < clusters) continue;
+    if (max_clusters(pick_kernel(b, SL, N, alpc != 0), cs, smem) < clusters) continue;
     *CS_out = cs; *SL_out = SL; *smem_out = smem; *row_slots_out = slots;
     found = true;
     if (want_cs > 0) break;
@@ -1035,7 +1206,7 @@ bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_sme
 }
 
 cudaError_t launch_persist(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative) {
-  PersistKernel k = pick_kernel(pa.in.b, pa.in.SL, pa.alpc != 0);
+  PersistKernel k = pick_kernel(pa.in.b, pa.in.SL, pa.in.N, pa.alpc != 0);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
