@@ -312,7 +312,7 @@ InnerArgs inner_args(lpc_ctx* c, uint64_t k_base, const uint64_t* k_dev, int has
   InnerArgs a;
   a.X = c->X; a.y = c->y; a.n = c->n; a.d = c->d; a.loss = c->loss;
   a.N = c->N; a.B = c->B; a.b = c->b; a.clip_mode = c->clip_mode; a.clip_value = c->clip_value;
-  a.seed = c->seed; a.sample_global = c->sample_global;
+  a.seed = c->seed; a.sample_global = c->sample_global; a.rule = scale_rule(c->d, c->b);
   a.k_base = k_base; a.k_dev = k_dev;
   a.x = c->x; a.margins = c->margins; a.mu = c->mu; a.has_J = has_J; a.vhat = c->vhat;
   a.codes = c->codes; a.stride_words = c->inner_seg.stride_words; a.pad_words = c->inner_seg.stride_words;

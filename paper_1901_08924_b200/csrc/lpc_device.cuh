@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lpc_scale.h"
 #include "lpc_status.h"
 
 namespace lpc {
@@ -141,8 +142,51 @@ struct Scale {
 
 constexpr int CLIP_NONE = 0, CLIP_LAMBDA = 1, CLIP_STD = 2;
 
+// The c * std threshold, fl32(min(c sqrt(S2 / len - (S1 / len)^2), M)) with every operation rounded to double: the definition.
+static __device__ __noinline__ float std_threshold_double(float S1, float S2, int64_t len, float c, float M) {
+  double mean, ex2;
+  if (len > 0 && (len & (len - 1)) == 0) {
+    // a power-of-two length: multiplying by 2^-log2(len) is the same exact operation as the division
+    const double inv = __longlong_as_double((long long)(1023 - (63 - __clzll(len))) << 52);
+    mean = __dmul_rn((double)S1, inv);
+    ex2 = __dmul_rn((double)S2, inv);
+  } else {
+    mean = __ddiv_rn((double)S1, (double)len);
+    ex2 = __ddiv_rn((double)S2, (double)len);
+  }
+  double var = __dsub_rn(ex2, __dmul_rn(mean, mean));
+  if (var < 0.0) var = 0.0;
+  double t = __dmul_rn((double)c, __dsqrt_rn(var));
+  if (t > (double)M) t = (double)M;
+  return __double2float_rn(t);
+}
+
+// The same bits from single precision.  The chain of doubles, with its root and up to two quotients, takes 0.35 us, and it stands
+// between a step's u and its codes; here every quantity is the sum of two floats (the error of a product by a multiply-add, that
+// of a sum by Dekker's and Knuth's formulas), the root one Newton step from a reciprocal root.  Both this value and the
+// definition's lie within 2^-42 of the true threshold (where the mean takes less than 3/4 of the second moment, and far from
+// the ends of the range), so if everything within 2^-38 of it rounds to one float, that float is the definition's; rounding
+// keeps the order, so min(., M) can come after it.  One scale in 10^4 is left to the doubles.
+__device__ __forceinline__ float std_threshold(float S1, float S2, const ScaleRule& r, float c, float M) {
+  auto sub = [](float a, float b) { return __fsub_rn(a, b); };
+  const float mh = mul_rn(S1, r.inv_len), me = add_rn(__fmaf_rn(S1, r.inv_len, -mh), mul_rn(S1, r.inv_len_low));
+  const float xh = mul_rn(S2, r.inv_len), xe = add_rn(__fmaf_rn(S2, r.inv_len, -xh), mul_rn(S2, r.inv_len_low));
+  const float qh = mul_rn(mh, mh), qe = add_rn(__fmaf_rn(mh, mh, -qh), mul_rn(mul_rn(2.f, mh), me));
+  const float s = sub(xh, qh), bb = sub(s, xh);
+  const float err = add_rn(sub(xh, sub(s, bb)), sub(-qh, bb));
+  const float ve = add_rn(err, sub(xe, qe)), vh = add_rn(s, ve), vl = sub(ve, sub(vh, s));
+  if (vh >= mul_rn(0.25f, xh) && vh >= 1e-25f && vh <= 1e25f && c >= 1e-6f && c <= 1e6f) {
+    const float y = rsqrtf(vh), sh = mul_rn(vh, y);
+    const float sl = mul_rn(add_rn(__fmaf_rn(-sh, sh, vh), vl), mul_rn(0.5f, y));
+    const float th = mul_rn(c, sh), te = add_rn(__fmaf_rn(c, sh, -th), mul_rn(c, sl));
+    const float T = add_rn(th, te), low = sub(te, sub(T, th)), d = mul_rn(T, 3.637978807091713e-12f);  // 2^-38
+    if (add_rn(T, add_rn(low, d)) == T && add_rn(T, sub(low, d)) == T) return fminf(T, M);
+  }
+  return std_threshold_double(S1, S2, r.len, c, M);
+}
+
 // max_bits = max over coordinates of the bit pattern of |u| (monotone in |u|; NaN/Inf >= 0x7F800000).
-__device__ __forceinline__ Scale make_scale(uint32_t max_bits, float S1, float S2, int64_t len, int b,
+__device__ __forceinline__ Scale make_scale(uint32_t max_bits, float S1, float S2, const ScaleRule& rule, int b,
                                             int clip_mode, float clip_value) {
   Scale sc;
   if (max_bits >= 0x7F800000u) {
@@ -152,33 +196,21 @@ __device__ __forceinline__ Scale make_scale(uint32_t max_bits, float S1, float S
   }
   const float M = __uint_as_float(max_bits);
   float T = M;
-  if (clip_mode == CLIP_LAMBDA) {
-    T = mul_rn(clip_value, M);
-  } else if (clip_mode == CLIP_STD) {
-    double mean, ex2;
-    if (len > 0 && (len & (len - 1)) == 0) {
-      // a power-of-two length: multiplying by 2^-log2(len) is the same exact operation as the division
-      const double inv = __longlong_as_double((long long)(1023 - (63 - __clzll(len))) << 52);
-      mean = __dmul_rn((double)S1, inv);
-      ex2 = __dmul_rn((double)S2, inv);
-    } else {
-      mean = __ddiv_rn((double)S1, (double)len);
-      ex2 = __ddiv_rn((double)S2, (double)len);
-    }
-    double var = __dsub_rn(ex2, __dmul_rn(mean, mean));
-    if (var < 0.0) var = 0.0;
-    double t = __dmul_rn((double)clip_value, __dsqrt_rn(var));
-    if (t > (double)M) t = (double)M;
-    T = __double2float_rn(t);
-  }
+  if (clip_mode == CLIP_LAMBDA) T = mul_rn(clip_value, M);
+  else if (clip_mode == CLIP_STD && max_bits != 0u) T = std_threshold(S1, S2, rule, clip_value, M);  // of zeros: T = M = 0
   sc.T = T;
   if (b == 32) {
     sc.delta = 1.f; sc.rdelta = 1.f; sc.lower = -T; sc.flags = 0u;
     return sc;
   }
-  const float Lv = (float)((1 << (b - 1)) - 1);
-  const float delta = (b == 1) ? T : __fdiv_rn(T, Lv);
-  const float rdelta = __fdiv_rn(1.0f, delta);
+  float delta = T;
+  if (b != 1) {
+    // RN(T / levels): a quotient within an ulp and one correction by the rounded reciprocal (Markstein, "Computation of
+    // elementary functions on the IBM RISC System/6000 processor", 1990), away from underflow
+    const float q = mul_rn(T, rule.inv_levels);
+    delta = T >= 1e-30f ? __fmaf_rn(__fmaf_rn(-q, rule.levels, T), rule.inv_levels, q) : __fdiv_rn(T, rule.levels);
+  }
+  const float rdelta = __frcp_rn(delta);
   if (M == 0.f || T == 0.f || delta == 0.f || isinf(rdelta) || isnan(rdelta)) {
     sc.delta = 0.f; sc.rdelta = 0.f; sc.lower = 0.f; sc.flags = 1u;
     return sc;

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lpc_scale.h"
+
 namespace lpc {
 
 struct InnerArgs {
@@ -35,6 +37,7 @@ struct InnerArgs {
   int CS;                  // CTAs per cluster
   int SL;                  // coordinates per CTA slice
   int overlapped;          // 1: may come in while earlier kernels are leaving that write nothing but this step's point
+  ScaleRule rule;          // of vectors of d values in b bits
   int stream_stages;       // 0: the B rows are resident in shared memory; > 0: they stream through that many ring stages
 };
 

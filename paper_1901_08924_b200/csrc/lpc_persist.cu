@@ -122,9 +122,9 @@ __device__ __forceinline__ uint32_t extract_bits(uint64_t lo, uint64_t hi, int p
 
 // Bulky scalar routines that one thread (or B threads) run once per step: kept out of line so that the loop
 // body every warp walks through stays small.
-__device__ __noinline__ Scale scale_out_of_line(uint32_t max_bits, float S1, float S2, int64_t len, int b, int clip_mode,
-                                               float clip_value) {
-  return make_scale(max_bits, S1, S2, len, b, clip_mode, clip_value);
+__device__ __noinline__ Scale scale_out_of_line(uint32_t max_bits, float S1, float S2, ScaleRule rule, int b, int clip_mode,
+                                               float clip_value) {  // by value: a reference would put the arguments into local memory
+  return make_scale(max_bits, S1, S2, rule, b, clip_mode, clip_value);
 }
 __device__ __noinline__ float deriv_out_of_line(int loss, float m, float y) { return loss_deriv(loss, m, y); }
 __device__ __noinline__ int64_t sample_row_out_of_line(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t slot,
@@ -930,7 +930,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       }
       const uint32_t m = __shfl_sync(0xFFFFFFFFu, v, 0);
       const float S1 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 8)), S2 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 16));
-      const Scale own = scale_out_of_line(m, S1, S2, d, b, a.clip_mode, a.clip_value);
+      const Scale own = scale_out_of_line(m, S1, S2, a.rule, b, a.clip_mode, a.clip_value);
       if (lane == 0) {
         sm.scale = own;
         // delta travels as a tagged word, one per CTA: the readers of rank r take every worker's rank-r word

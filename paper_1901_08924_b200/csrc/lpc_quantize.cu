@@ -237,8 +237,8 @@ __device__ __forceinline__ void block_tree_sums(const float* __restrict__ v1, co
 
 // ---- between the passes: Eq. 2 from the tile partials --------------------------------------------------------------
 // The scale record of (segment, worker), the scale for the caller and the cleared count; one thread.
-__device__ __forceinline__ void write_scale(const QuantArgs& a, const SegInfo& s, int seg, int worker, uint32_t m, float S1, float S2) {
-  const Scale sc = make_scale(m, S1, S2, s.len, a.b, a.clip_mode, a.clip_value);
+__device__ __forceinline__ void write_scale(const QuantArgs& a, const SegInfo& s, int seg, int worker, uint32_t m, float S1, float S2, const ScaleRule& rule) {
+  const Scale sc = make_scale(m, S1, S2, rule, a.b, a.clip_mode, a.clip_value);
   ScaleRec r;
   r.delta = sc.delta; r.rdelta = sc.rdelta; r.T = sc.T; r.lower = sc.lower; r.flags = sc.flags;
   r.pad0 = r.pad1 = r.pad2 = 0;
@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
   const int seg = blockIdx.x, worker = blockIdx.y;
   const SegInfo s = a.segs[seg];
   const int64_t base = (int64_t)worker * a.ntiles + s.tile_first;
+  const ScaleRule rule = scale_rule(s.len, a.b);  // its divisions while the partials are on their way
   uint32_t mx = 0;
 #pragma unroll 8
   for (int t = threadIdx.x; t < s.tile_count; t += QT) mx = max(mx, __ldcg(a.pmax + base + t));
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(QT) finish_kernel(QuantArgs a) {
     uint32_t m = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) m = max(m, shm[w]);
-    write_scale(a, s, seg, worker, m, S1, S2);
+    write_scale(a, s, seg, worker, m, S1, S2, rule);
   }
 }
 
@@ -651,6 +652,7 @@ __global__ void __launch_bounds__(QT) quantize_cluster_kernel(QuantArgs a) {
   const float* q = a.U_sub ? a.U_sub + (int64_t)worker * a.ld : nullptr;
   const bool vec = aligned16(p) && (!q || aligned16(q)), al32 = aligned32(p);
   const int len = (int)s.len, j0 = rank * TILE + tid * 8;
+  const ScaleRule rule = scale_rule(len, a.b);
   wait_for_launch_before();
 
   f32x2 v[QITER][4], pr[QITER];
@@ -696,7 +698,7 @@ __global__ void __launch_bounds__(QT) quantize_cluster_kernel(QuantArgs a) {
     uint32_t m = 0;
     for (int c = 0; c < ctas; ++c) m = max(m, sm.pmx[c]);
     const float S1 = NEED_SUMS ? smem_tree_sum(sm.p1, ctas) : 0.f, S2 = NEED_SUMS ? smem_tree_sum(sm.p2, ctas) : 0.f;
-    const Scale sc = make_scale(m, S1, S2, len, a.b, a.clip_mode, a.clip_value);
+    const Scale sc = make_scale(m, S1, S2, rule, a.b, a.clip_mode, a.clip_value);
     sm.sc.delta = sc.delta; sm.sc.rdelta = sc.rdelta; sm.sc.T = sc.T; sm.sc.lower = sc.lower;
     sm.sc.flags = sc.flags | (sc.T >= __uint_as_float(m) ? SCALE_NONE_OUTSIDE : 0u);
     if (rank == 0) {
