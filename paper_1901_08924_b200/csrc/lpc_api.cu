@@ -190,7 +190,7 @@ int layout(int64_t len, int b, const int64_t* seg_offsets, int nseg, std::vector
     g.tile_first = (int32_t)tiles;
     const int64_t tc = (g.len + TILE - 1) / TILE;
     g.tile_count = (int32_t)tc;
-    g.pad_ = 0;
+    g.rule = scale_rule(g.len, b);
     word += g.pad_words;
     block += (g.len + 7) / 8;
     tiles += tc;

@@ -1,4 +1,4 @@
-// The reciprocals that the scale rule (the c * std threshold and Eq. 2) uses, for host and device.
+// The reciprocals that the scale rule (the c * std threshold and Eq. 2) uses, made on the host.
 #pragma once
 #include <stdint.h>
 
@@ -9,7 +9,7 @@ struct ScaleRule {
   float inv_len, inv_len_low;  // 1 / len as the unrounded sum of two floats
   float levels, inv_levels;    // 2^(b-1) - 1 (b = 1, 32: 1) and its reciprocal, rounded
 };
-__host__ __device__ inline ScaleRule scale_rule(int64_t len, int b) {
+inline ScaleRule scale_rule(int64_t len, int b) {
   ScaleRule r;
   r.len = len;
   const double inv = 1.0 / (double)len;
