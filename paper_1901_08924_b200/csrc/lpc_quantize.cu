@@ -191,8 +191,9 @@ __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int wor
 // The second pass goes back from the end, so the tiles worth keeping in L2 are the last ones: those before the last `keep` are
 // read so that they go first.  Quantizer, us, with 40 / 60 / 100 MB kept and without: 8 x 2^24, b = 8 184.4 / 184.0 / 184.6, 190.7;
 // 8 x 2^22 on one scale 52.2 / 53.6 / 55.7, 56.6; 8 x 2^26 690 / 690 / 693, 693.  With a subtrahend, whose second pass takes longer
-// per byte: 8 x 2^23 160.6 / 159.6 / 160.1, 164.0; 62 tensors for 16 workers 447 / 445 / 443, 446.
-constexpr int64_t KEEP_BYTES = 48ll << 20, KEEP_BYTES_SUB = 96ll << 20;
+// per byte: 8 x 2^23 160.6 / 159.6 / 160.1, 164.0.  The loads cost a hundredth of the first pass, and what is saved does not grow with
+// the input: from 1 GB on it is not worth it (62 tensors for 16 workers, 1.5 GB: first pass 218.6 -> 220.7, second 240.2 -> 240.3).
+constexpr int64_t KEEP_BYTES = 48ll << 20, KEEP_BYTES_SUB = 96ll << 20, KEEP_MAX_INPUT = 1ll << 30;
 
 template <bool NEED_SUMS, bool POLICY>
 __global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a, int keep) {
@@ -902,9 +903,10 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
   cudaError_t e = cudaSuccess;
   if (a.ntiles > 0) {
     if (hook) hook(user, 3 /* LPC_KERNEL_QUANT_STATS */, 1);
-    const int keep = (int)(a.U_sub ? KEEP_BYTES_SUB / (2 * TILE * sizeof(float)) : KEEP_BYTES / (TILE * sizeof(float)));
+    const int64_t tile_bytes = (int64_t)TILE * sizeof(float) * (a.U_sub ? 2 : 1), tiles = (int64_t)a.N * a.ntiles;
+    const int keep = (int)((a.U_sub ? KEEP_BYTES_SUB : KEEP_BYTES) / tile_bytes);
     const bool sums = a.clip_mode == CLIP_STD;
-    if ((int64_t)a.N * a.ntiles <= keep) e = sums ? launch(stats_kernel<true, false>, grid, 0) : launch(stats_kernel<false, false>, grid, 0);
+    if (tiles <= keep || tiles * tile_bytes > KEEP_MAX_INPUT) e = sums ? launch(stats_kernel<true, false>, grid, 0) : launch(stats_kernel<false, false>, grid, 0);
     else e = sums ? launch(stats_kernel<true, true>, grid, keep) : launch(stats_kernel<false, true>, grid, keep);
     if (hook) hook(user, 3, 0);
     if (e != cudaSuccess) return e;

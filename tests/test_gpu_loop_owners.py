@@ -1,0 +1,62 @@
+"""The one-launch loop where each coordinate's update belongs to one CTA: worker counts and widths around the rule that takes it,
+slices that the workers do not divide evenly, coordinates that end inside an owner's share, empty slices; bit for bit the
+iterates, codes and estimators of one-step launches."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1901_08924_b200 import lpc, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _same(a, b):
+    return torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("alpc", [False, True])
+@pytest.mark.parametrize("n,d,N,B,b", [
+    (17 * 8, 4096, 17, 3, 4),    # the first count beyond sixteen; shares of 64 coordinates of a slice of 1,024
+    (31 * 8, 8188, 31, 16, 2),   # 31 shares of 72 in slices of 2,048, the last column inside one; rows that do not fit a step ahead
+    (32 * 4, 5000, 32, 2, 8),    # the last CTA of a cluster has few columns
+    (24 * 4, 64, 24, 1, 1),      # more workers than groups of eight coordinates
+    (33 * 4, 2052, 33, 4, 4),    # slices that are half empty
+    (2 * 16, 512, 2, 5, 3),      # widths known at run time: owners whatever the worker count
+    (5 * 16, 1000, 5, 32, 6),
+    (16 * 8, 2048, 16, 8, 32),
+    (64 * 2, 1024, 64, 2, 16),   # the most workers the loop takes
+])
+def test_owned_update_equals_single_steps(n, d, N, B, b, alpc):
+    X, y, _ = synth.linear_problem(n, d, loss="least_squares", sparsity=0.2, noise=0.1, seed=d + N)
+    X, y = X.cuda(), y.cuda()
+    x0 = torch.from_numpy((np.random.default_rng(3).standard_normal(d) * 0.1).astype(np.float32)).cuda()
+    one, many = (lpc.Context(X, y, lpc.LEAST_SQUARES, 1e-5, N, B, b, lpc.CLIP_STD, 2.0, 11) for _ in range(2))
+    count = 9
+    for c in (one, many):
+        c.set_option(lpc.OPT_TAP_U, 1)
+        c.set_iterate(x0)
+        if alpc:
+            c.alpc_begin()
+        c.snapshot_full_grad()
+    one.set_option(lpc.OPT_PERSISTENT, 0)
+    par = (0.4, 0.5, 0.3, 0.2)
+    for k in range(2 * count):
+        if alpc:
+            one.alpc_double_sample_step(*par, k)
+        else:
+            one.inner_step(0.05, k)
+    for k0 in (0, count):  # two launches: the second one's words must not be taken for the first one's
+        if alpc:
+            many.alpc_double_sample_steps(*par, k0, count)
+        else:
+            many.inner_steps(0.05, k0, count)
+    one.sync_status()
+    many.sync_status()
+    if many.query(lpc.INFO_ALPC_LOOP_CLUSTER_SIZE if alpc else lpc.INFO_LOOP_CLUSTER_SIZE):
+        assert many.query(lpc.INFO_LOOP_LAUNCHES) == 2
+    for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_U, lpc.BUF_V, lpc.BUF_CLIPPED] + (
+            [lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_VHAT] if alpc else []):
+        assert _same(one.get_buffer(w), many.get_buffer(w)), w
+    assert torch.isfinite(many.get_iterate()).all()
+    one.close()
+    many.close()
