@@ -190,7 +190,7 @@ int layout(int64_t len, int b, const int64_t* seg_offsets, int nseg, std::vector
     g.tile_first = (int32_t)tiles;
     const int64_t tc = (g.len + TILE - 1) / TILE;
     g.tile_count = (int32_t)tc;
-    g.rule = scale_rule(g.len, b);
+    g.pad_ = 0;
     word += g.pad_words;
     block += (g.len + 7) / 8;
     tiles += tc;
@@ -312,7 +312,7 @@ InnerArgs inner_args(lpc_ctx* c, uint64_t k_base, const uint64_t* k_dev, int has
   InnerArgs a;
   a.X = c->X; a.y = c->y; a.n = c->n; a.d = c->d; a.loss = c->loss;
   a.N = c->N; a.B = c->B; a.b = c->b; a.clip_mode = c->clip_mode; a.clip_value = c->clip_value;
-  a.seed = c->seed; a.sample_global = c->sample_global; a.rule = scale_rule(c->d, c->b);
+  a.seed = c->seed; a.sample_global = c->sample_global;
   a.k_base = k_base; a.k_dev = k_dev;
   a.x = c->x; a.margins = c->margins; a.mu = c->mu; a.has_J = has_J; a.vhat = c->vhat;
   a.codes = c->codes; a.stride_words = c->inner_seg.stride_words; a.pad_words = c->inner_seg.stride_words;
@@ -404,6 +404,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     // the whole loop in one cooperative launch; on a launch refusal fall through to the per-step kernels
     PersistArgs pa;
     pa.in = inner_args(c, k0, nullptr, 0);
+    pa.rule = scale_rule(c->d, c->b);
     pa.in.CS = kind == 0 ? c->pCS : c->aCS;
     pa.in.SL = kind == 0 ? c->pSL : c->aSL;
     pa.row_slots = kind == 0 ? c->pSlots : c->aSlots;

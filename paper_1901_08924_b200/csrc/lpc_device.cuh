@@ -143,7 +143,7 @@ struct Scale {
 constexpr int CLIP_NONE = 0, CLIP_LAMBDA = 1, CLIP_STD = 2;
 
 // The c * std threshold, fl32(min(c sqrt(S2 / len - (S1 / len)^2), M)) with every operation rounded to double: the definition.
-static __device__ __noinline__ float std_threshold_double(float S1, float S2, int64_t len, float c, float M) {
+__device__ __forceinline__ float std_threshold_double(float S1, float S2, int64_t len, float c, float M) {
   double mean, ex2;
   if (len > 0 && (len & (len - 1)) == 0) {
     // a power-of-two length: multiplying by 2^-log2(len) is the same exact operation as the division
@@ -159,6 +159,45 @@ static __device__ __noinline__ float std_threshold_double(float S1, float S2, in
   double t = __dmul_rn((double)c, __dsqrt_rn(var));
   if (t > (double)M) t = (double)M;
   return __double2float_rn(t);
+}
+
+// max_bits = max over coordinates of the bit pattern of |u| (monotone in |u|; NaN/Inf >= 0x7F800000).
+__device__ __forceinline__ Scale make_scale(uint32_t max_bits, float S1, float S2, int64_t len, int b,
+                                            int clip_mode, float clip_value) {
+  Scale sc;
+  if (max_bits >= 0x7F800000u) {
+    sc.delta = __int_as_float(0x7FC00000);
+    sc.rdelta = 0.f; sc.T = 0.f; sc.lower = 0.f; sc.flags = 3u;
+    return sc;
+  }
+  const float M = __uint_as_float(max_bits);
+  float T = M;
+  if (clip_mode == CLIP_LAMBDA) {
+    T = mul_rn(clip_value, M);
+  } else if (clip_mode == CLIP_STD) {
+    T = std_threshold_double(S1, S2, len, clip_value, M);
+  }
+  sc.T = T;
+  if (b == 32) {
+    sc.delta = 1.f; sc.rdelta = 1.f; sc.lower = -T; sc.flags = 0u;
+    return sc;
+  }
+  const float Lv = (float)((1 << (b - 1)) - 1);
+  const float delta = (b == 1) ? T : __fdiv_rn(T, Lv);
+  const float rdelta = __fdiv_rn(1.0f, delta);
+  if (M == 0.f || T == 0.f || delta == 0.f || isinf(rdelta) || isnan(rdelta)) {
+    sc.delta = 0.f; sc.rdelta = 0.f; sc.lower = 0.f; sc.flags = 1u;
+    return sc;
+  }
+  sc.delta = delta;
+  sc.rdelta = rdelta;
+  sc.lower = (b == 1) ? -T : -add_rn(T, delta);
+  sc.flags = 0u;
+  return sc;
+}
+
+static __device__ __noinline__ float std_threshold_rare(float S1, float S2, int64_t len, float c, float M) {  // out of line
+  return std_threshold_double(S1, S2, len, c, M);
 }
 
 // The same bits from single precision.  The chain of doubles, with its root and up to two quotients, takes 0.35 us, and it stands
@@ -182,11 +221,12 @@ __device__ __forceinline__ float std_threshold(float S1, float S2, const ScaleRu
     const float T = add_rn(th, te), low = sub(te, sub(T, th)), d = mul_rn(T, 3.637978807091713e-12f);  // 2^-38
     if (add_rn(T, add_rn(low, d)) == T && add_rn(T, sub(low, d)) == T) return fminf(T, M);
   }
-  return std_threshold_double(S1, S2, r.len, c, M);
+  return std_threshold_rare(S1, S2, r.len, c, M);
 }
 
-// max_bits = max over coordinates of the bit pattern of |u| (monotone in |u|; NaN/Inf >= 0x7F800000).
-__device__ __forceinline__ Scale make_scale(uint32_t max_bits, float S1, float S2, const ScaleRule& rule, int b,
+// make_scale, bit for bit, with a shorter chain and more code: for a loop that runs it every step.  (In kernels that form one scale
+// and end, the code has to be fetched first: 0.1 us more for a streaming step, 0.5 us for a short quantizer call.)
+__device__ __forceinline__ Scale make_scale_in_loop(uint32_t max_bits, float S1, float S2, const ScaleRule& rule, int b,
                                             int clip_mode, float clip_value) {
   Scale sc;
   if (max_bits >= 0x7F800000u) {

@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
     for (int q = 0; q < CS; ++q) m = max(m, sm.maxpart[q]);
     float S1 = 0.f, S2 = 0.f;
     if (a.clip_mode == CLIP_STD) { S1 = smem_tree_sum(sm.s1part, CS); S2 = smem_tree_sum(sm.s2part, CS); }
-    sm.scale = make_scale(m, S1, S2, a.rule, b, a.clip_mode, a.clip_value);
+    sm.scale = make_scale(m, S1, S2, d, b, a.clip_mode, a.clip_value);
     if (rank == 0) {
       a.delta[worker] = sm.scale.delta;
       if (sm.scale.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);

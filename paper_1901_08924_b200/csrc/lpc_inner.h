@@ -37,13 +37,13 @@ struct InnerArgs {
   int CS;                  // CTAs per cluster
   int SL;                  // coordinates per CTA slice
   int overlapped;          // 1: may come in while earlier kernels are leaving that write nothing but this step's point
-  ScaleRule rule;          // of vectors of d values in b bits
   int stream_stages;       // 0: the B rows are resident in shared memory; > 0: they stream through that many ring stages
 };
 
 // Arguments of the persistent inner loop (lpc_persist.cu): `count` steps k_base, k_base+1, ... in one launch.
 struct PersistArgs {
   InnerArgs in;              // in.x = iterate at entry, in.k_dev unused, in.has_J = 0
+  ScaleRule rule;            // of vectors of d values in b bits
   int count;
   float eta;
   float lambda_l1;

@@ -3,8 +3,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "lpc_scale.h"
-
 namespace lpc {
 
 constexpr int TILE = 8192;  // coordinates per CTA tile of the standalone quantizer / aggregator kernels
@@ -34,7 +32,7 @@ struct SegInfo {
   uint32_t block_base; // first Philox block of its rounding stream
   int32_t tile_first;  // first tile index
   int32_t tile_count;
-  ScaleRule rule;      // for the code width of the layout
+  int32_t pad_;
 };
 
 struct ScaleRec {  // result of the scale rule for one (worker, segment)

@@ -19,15 +19,14 @@ namespace {
 using namespace lpc;
 
 // Layout of the fixed working memory (bytes from the start of the array):
-//   [0, 128)                     one SegInfo (the vector as a single segment)
-//   [128, 192)                   status word: the kernels need a place to flag non-finite input; nothing reads it back
+//   [0, 64)                      one SegInfo (the vector as a single segment)
+//   [64, 128)                    status word: the kernels need a place to flag non-finite input; nothing reads it back
 //                                (there is no context to report through), the caller's signal is the NaN delta
 //   [256, 256 + 32*MAX_N)        ScaleRec per worker
 //   then three arrays of MAX_PARTS 32-bit entries: tile maxima, tile sums, tile sums of squares
 constexpr int MAX_N = LPC_STATIC_MAX_WORKERS;
 constexpr int MAX_PARTS = LPC_STATIC_MAX_TILES;  // workers x tiles of 8192 coordinates
-constexpr size_t OFF_SEG = 0, OFF_STATUS = 128, OFF_SCALES = 256;
-static_assert(sizeof(SegInfo) <= OFF_STATUS, "the segment record fits in front of the status word");
+constexpr size_t OFF_SEG = 0, OFF_STATUS = 64, OFF_SCALES = 256;
 constexpr size_t OFF_PMAX = OFF_SCALES + sizeof(ScaleRec) * MAX_N;
 constexpr size_t OFF_PS1 = OFF_PMAX + 4 * (size_t)MAX_PARTS;
 constexpr size_t OFF_PS2 = OFF_PS1 + 4 * (size_t)MAX_PARTS;
@@ -91,7 +90,7 @@ extern "C" int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld,
   SegInfo seg;
   seg.off = 0; seg.len = len; seg.word_off = 0;
   seg.pad_words = (((len * b + 31) / 32) + 3) & ~(int64_t)3;
-  seg.block_base = 0; seg.tile_first = 0; seg.tile_count = (int32_t)ntiles; seg.rule = scale_rule(len, b);
+  seg.block_base = 0; seg.tile_first = 0; seg.tile_count = (int32_t)ntiles; seg.pad_ = 0;
   static_setup_kernel<<<1, 1, 0, st>>>(seg);
   if (cudaGetLastError() != cudaSuccess) return LPC_ERR_CUDA;
 

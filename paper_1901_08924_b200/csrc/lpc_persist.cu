@@ -6,11 +6,11 @@
 // grid stays resident for `count` steps (one cluster per worker, one CTA per SM, launched
 // cooperatively so that co-residency is guaranteed) and the only grid-wide dependency per step is the
 // arrival of the other workers' messages:
-//   - every CTA keeps its slice of x and of mu in REGISTERS across steps;
+//   - every CTA keeps its slice of x and of mu in REGISTERS across steps (x~, y, z of Algorithm 2 as well, unless
+//     coordinates have owners: those keep them);
 //   - the rows of step t+1 do not depend on step t (sampling is counter-based), so they are sampled
-//     and fetched by bulk copies (TMA) into the other half of a double buffer while step t computes;
-//     labels and cached snapshot margins of those rows travel in registers of the thread that owns the
-//     minibatch slot;
+//     and fetched by bulk copies (TMA) into free row slots while step t computes; labels and cached snapshot
+//     margins of those rows travel in registers of the thread that owns the minibatch slot;
 //   - the codes travel between CTAs as self-validating 64-bit words: 32 bits of payload (the codes of 8
 //     coordinates, or part of them) and a 32-bit tag that names the step (unique across launches).  Aligned
 //     64-bit stores are single-copy atomic, so a reader that sees the tag it expects also sees the payload:
@@ -21,6 +21,8 @@
 //     matches, then averages, adds mu and applies the proximal step in registers.  The exchange buffers are
 //     double-buffered by step parity, because a fast CTA may store step t+1 while a slow one still reads
 //     step t (it cannot get further ahead: storing step t+2 needs every reader's step t+1).
+//   - with many workers (pays_to_own) the update of a coordinate belongs to one CTA, which sends the new point as
+//     tagged words too: one crossing of the chip more, and N times less to load and decode per CTA.
 //   - only the last step also writes the packed codes, delta and the second estimator in their documented
 //     layouts, for the caller.
 // Every wait is bounded; when one runs out the thread records a timeout in the status word, raises a global
@@ -124,7 +126,7 @@ __device__ __forceinline__ uint32_t extract_bits(uint64_t lo, uint64_t hi, int p
 // body every warp walks through stays small.
 __device__ __noinline__ Scale scale_out_of_line(uint32_t max_bits, float S1, float S2, ScaleRule rule, int b, int clip_mode,
                                                float clip_value) {  // by value: a reference would put the arguments into local memory
-  return make_scale(max_bits, S1, S2, rule, b, clip_mode, clip_value);
+  return make_scale_in_loop(max_bits, S1, S2, rule, b, clip_mode, clip_value);
 }
 __device__ __noinline__ float deriv_out_of_line(int loss, float m, float y) { return loss_deriv(loss, m, y); }
 __device__ __noinline__ int64_t sample_row_out_of_line(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t slot,
@@ -930,7 +932,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       }
       const uint32_t m = __shfl_sync(0xFFFFFFFFu, v, 0);
       const float S1 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 8)), S2 = __uint_as_float(__shfl_sync(0xFFFFFFFFu, v, 16));
-      const Scale own = scale_out_of_line(m, S1, S2, a.rule, b, a.clip_mode, a.clip_value);
+      const Scale own = scale_out_of_line(m, S1, S2, pa.rule, b, a.clip_mode, a.clip_value);
       if (lane == 0) {
         sm.scale = own;
         // delta travels as a tagged word, one per CTA: the readers of rank r take every worker's rank-r word

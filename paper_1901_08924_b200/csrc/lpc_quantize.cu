@@ -265,7 +265,7 @@ __device__ __forceinline__ void block_tree_sums(const float* __restrict__ v1, co
 // ---- between the passes: Eq. 2 from the tile partials --------------------------------------------------------------
 // The scale record of (segment, worker), the scale for the caller and the cleared count; one thread.
 __device__ __forceinline__ void write_scale(const QuantArgs& a, const SegInfo& s, int seg, int worker, uint32_t m, float S1, float S2) {
-  const Scale sc = make_scale(m, S1, S2, s.rule, a.b, a.clip_mode, a.clip_value);
+  const Scale sc = make_scale(m, S1, S2, s.len, a.b, a.clip_mode, a.clip_value);
   ScaleRec r;
   r.delta = sc.delta; r.rdelta = sc.rdelta; r.T = sc.T; r.lower = sc.lower; r.flags = sc.flags;
   r.pad0 = r.pad1 = r.pad2 = 0;
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(QT) quantize_cluster_kernel(QuantArgs a) {
     uint32_t m = 0;
     for (int c = 0; c < ctas; ++c) m = max(m, sm.pmx[c]);
     const float S1 = NEED_SUMS ? smem_tree_sum(sm.p1, ctas) : 0.f, S2 = NEED_SUMS ? smem_tree_sum(sm.p2, ctas) : 0.f;
-    const Scale sc = make_scale(m, S1, S2, s.rule, a.b, a.clip_mode, a.clip_value);
+    const Scale sc = make_scale(m, S1, S2, len, a.b, a.clip_mode, a.clip_value);
     sm.sc.delta = sc.delta; sm.sc.rdelta = sc.rdelta; sm.sc.T = sc.T; sm.sc.lower = sc.lower;
     sm.sc.flags = sc.flags | (sc.T >= __uint_as_float(m) ? SCALE_NONE_OUTSIDE : 0u);
     if (rank == 0) {

@@ -1,39 +1,49 @@
-"""The c * std scale rule on vectors whose sums, lengths and thresholds cover its branches: the threshold is formed in single
-precision with an interval around it, and by doubles where that interval does not decide; the scale, its reciprocal (through
-the codes) and the counts have to be the oracle's bits either way."""
+"""The scale of the one-launch loop, which is formed in single precision with an interval around the threshold and by doubles where
+that does not decide: bit for bit the scales of one-step launches, which take the doubles.  Gradients from 2^-100 to 2^100, with
+means up to a thousand deviations, with one coordinate that is not zero, constant ones."""
 import numpy as np
 import pytest
 import torch
 
-import oracle as orc
 from paper_1901_08924_b200 import lpc
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("b", [1, 2, 3, 4, 7, 8, 16, 32])
-@pytest.mark.parametrize("length", [1, 3, 64, 1000, 4099])
-def test_scale_of_many_vectors_bit_exact(b, length):
-    # 512 vectors per call: scales over 2^-140 .. 2^120 (second moments underflow and overflow), constant vectors (variance zero
-    # or rounding noise), a mean far above the deviation, one outlier, a single value
-    rng = np.random.default_rng(1000 * b + length)
-    N = 512
-    U = rng.standard_normal((N, length)) * np.exp2(rng.uniform(-140, 60, (N, 1)))
-    U[1::8] += np.abs(U[1::8]).max(axis=1, keepdims=True) * 1000.0
-    U[2::8] = U[2::8, :1]
-    U[3::8] *= 0.0
-    U[3::8, 0] = rng.standard_normal(U[3::8, 0].shape)
-    U[4::8] = rng.standard_normal(U[4::8].shape) * np.exp2(rng.uniform(60, 120, (U[4::8].shape[0], 1)))
-    U = U.astype(np.float32)
-    for value in (0.5, 2.5, 3.0000002):
-        ctx = lpc.Context(None, None, lpc.LOGISTIC, 0.0, N, 1, b, lpc.CLIP_STD, value, 3)
-        codes, delta, clipped = ctx.quantize_pack(torch.from_numpy(U).cuda(), 1)
-        ctx.status()
-        got = delta.cpu().numpy()[:, 0].view(np.uint32)
-        W = orc.packed_words(length, b)
-        words = codes.cpu().numpy().view(np.uint32)[:, :W]
-        for i in range(N):
-            w, dl, cl = orc.quantize_pack(U[i], b, orc.CLIP_STD, value, 3, i, 1)
-            assert got[i] == np.float32(dl).view(np.uint32), (i, value)
-            assert (words[i] == w).all() and int(clipped[i, 0]) == cl, (i, value)
-        ctx.close()
+def _same(a, b):
+    return torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+
+
+@pytest.mark.parametrize("kind", ["gauss", "mean", "single", "constant"])
+@pytest.mark.parametrize("exponent", [-55, -30, -13, 0, 20, 50])
+@pytest.mark.parametrize("b,value", [(1, 0.5), (2, 2.5), (3, 3.0000002), (4, 3.0), (8, 2.0), (32, 1.0)])
+def test_loop_scales_equal_single_steps(kind, exponent, b, value):
+    N, B, d, n, count = 4, 1, 1000, 64, 40
+    rng = np.random.default_rng((exponent + 100) * 7 + b)
+    X = rng.standard_normal((n, d))
+    if kind == "mean":
+        X = X + np.exp2(rng.uniform(-4, 10, (n, 1)))
+    elif kind == "single":
+        X = np.where(np.arange(d) == rng.integers(0, d, (n, 1)), X, 0.0)
+    elif kind == "constant":
+        X = np.repeat(X[:, :1], d, axis=1)
+    # u = (X_a (x - x~)) X_a grows with the square of the rows' scale
+    X = torch.from_numpy((X * np.exp2(exponent)).astype(np.float32)).cuda()
+    y = torch.from_numpy(rng.standard_normal(n).astype(np.float32)).cuda()
+    shift = torch.from_numpy((rng.standard_normal(d) * 0.1).astype(np.float32)).cuda()
+    out = []
+    for persistent in (0, 1):
+        c = lpc.Context(X, y, lpc.LEAST_SQUARES, 0.0, N, B, b, lpc.CLIP_STD, value, 5)
+        c.set_option(lpc.OPT_PERSISTENT, persistent)
+        c.snapshot_full_grad()
+        c.set_iterate(shift)  # away from the snapshot, or the first step's u is zero
+        deltas = []
+        for k in range(0, count, 2):  # two steps per call: the loop leaves the last step's scales
+            c.inner_steps(0.0, k, 2)  # step 0: the iterate stays, every pair of steps sees other rows
+            deltas.append(c.get_buffer(lpc.BUF_DELTA).clone())
+        c.status()
+        assert c.query(lpc.INFO_LOOP_LAUNCHES) == (count // 2 if persistent else 0)
+        out.append((torch.stack(deltas), c.get_buffer(lpc.BUF_CODES), c.get_buffer(lpc.BUF_CLIPPED)))
+        c.close()
+    for a, e in zip(*out):
+        assert _same(a, e)
