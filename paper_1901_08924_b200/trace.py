@@ -25,8 +25,8 @@ import sys
 PHASES = [
     (0, 1, "rounding bits (Philox)"),
     (1, 2, "sampling of the next step's rows"),
-    (2, 3, "loads of all workers' words issued -> all tags valid (the next step's row copies are issued meanwhile)"),
-    (3, 4, "decode + average + proximal step (Algorithm 2: y, z updates and coupling)"),
+    (2, 3, "loads of all workers' words issued -> all tags valid (owned update: -> the owners have all products); row copies meanwhile"),
+    (3, 4, "decode + average + proximal step (Algorithm 2: y, z updates, coupling; owned update: sums, step, -> the new point is there)"),
     (4, 5, "wait for this step's rows"),
     (5, 6, "margins (partial sums, warp reduction, block barrier)"),
     (6, 7, "cluster exchange of the margin partial sums"),
