@@ -87,7 +87,7 @@ struct lpc_ctx {
   SegPlan inner_seg;  // one segment of length d for the aggregator
   // persistent inner loop
   bool persist_ok = false, apersist_ok = false;  // Algorithm 1 loop / Algorithm 2 loop
-  int pCS = 1, pSL = 0, pSlots = 0, aCS = 1, aSL = 0, aSlots = 0;  // cluster size, slice, row slots of the two loops
+  int pCS = 1, pSL = 0, pSlots = 0, pOwn = 0, aCS = 1, aSL = 0, aSlots = 0, aOwn = 0;  // cluster size, slice, row slots, owned update of the two loops
   size_t persistSmem = 0, apersistSmem = 0;
   // exchange buffers of the one-launch loops: tagged 64-bit words (payload | tag << 32), two step-parity halves
   unsigned long long* flags = nullptr;    // scale words: 2 x 256, 128 bytes apart, + 1 abort word
@@ -342,11 +342,11 @@ int replan_inner(lpc_ctx* c) {
   int stages = 0;
   c->inner_ok = inner_plan(c->d, c->B, c->want_cs, c->max_smem, &cs, &sl, &smem, &stages);
   if (c->inner_ok) { c->CS = cs; c->SL = sl; c->innerSmem = smem; c->innerStages = stages; }
-  int slots = 0;
-  c->persist_ok = persist_plan(c->d, c->N, c->B, c->b, 0, c->want_cs, c->max_smem, &cs, &sl, &smem, &slots);
-  if (c->persist_ok) { c->pCS = cs; c->pSL = sl; c->persistSmem = smem; c->pSlots = slots; }
-  c->apersist_ok = persist_plan(c->d, c->N, c->B, c->b, 1, c->want_cs, c->max_smem, &cs, &sl, &smem, &slots);
-  if (c->apersist_ok) { c->aCS = cs; c->aSL = sl; c->apersistSmem = smem; c->aSlots = slots; }
+  int slots = 0, own = 0;
+  c->persist_ok = persist_plan(c->d, c->N, c->B, c->b, 0, c->want_cs, c->max_smem, &cs, &sl, &smem, &slots, &own);
+  if (c->persist_ok) { c->pCS = cs; c->pSL = sl; c->persistSmem = smem; c->pSlots = slots; c->pOwn = own; }
+  c->apersist_ok = persist_plan(c->d, c->N, c->B, c->b, 1, c->want_cs, c->max_smem, &cs, &sl, &smem, &slots, &own);
+  if (c->apersist_ok) { c->aCS = cs; c->aSL = sl; c->apersistSmem = smem; c->aSlots = slots; c->aOwn = own; }
   return LPC_OK;
 }
 
@@ -405,6 +405,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     PersistArgs pa;
     pa.in = inner_args(c, k0, nullptr, 0);
     pa.rule = scale_rule(c->d, c->b);
+    pa.own = kind == 0 ? c->pOwn : c->aOwn;
     pa.in.CS = kind == 0 ? c->pCS : c->aCS;
     pa.in.SL = kind == 0 ? c->pSL : c->aSL;
     pa.row_slots = kind == 0 ? c->pSlots : c->aSlots;

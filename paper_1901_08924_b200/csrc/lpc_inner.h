@@ -44,6 +44,7 @@ struct InnerArgs {
 struct PersistArgs {
   InnerArgs in;              // in.x = iterate at entry, in.k_dev unused, in.has_J = 0
   ScaleRule rule;            // of vectors of d values in b bits
+  int own;                   // 1: the update of a coordinate belongs to one CTA (persist_plan)
   int count;
   float eta;
   float lambda_l1;
@@ -74,7 +75,7 @@ struct PersistArgs {
   float* vhat;
 };
 bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_smem, int* CS_out, int* SL_out,
-                  size_t* smem_out, int* row_slots_out);
+                  size_t* smem_out, int* row_slots_out, int* own_out);
 int persist_coords_per_thread(int b, int SL);
 // cooperative = false drops the launch attribute that makes the driver guarantee co-residency of the grid (the plan has
 // checked that all clusters fit; the kernel's waits are bounded): for profilers that cannot replay cooperative launches.

@@ -59,9 +59,6 @@ struct PSmem {
   uint64_t bar[2];
   __align__(16) float coef[PMAXB];
   float wpart[PMAXB * PMAXP * 8];
-  // OWN: scale times index of every worker and owned coordinate (not shared with wpart: no barrier separates the owners' sums
-  // from the margins of a warp that already has its slice of the new point)
-  __align__(16) float prod[PGROUP + 8 * PMAXN];
   // cluster exchange slots, written by the peers through distributed shared memory as tagged words, two
   // step-parity halves: margin partial sums (slot b * PMAXCS + rank) and statistics (max, S1, S2 per rank)
   unsigned long long mx[2][PMAXB * PMAXCS];
@@ -218,7 +215,10 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PSmem& sm = *reinterpret_cast<PSmem*>(smem_raw);
   const int CS = a.CS, SL = a.SL, B = a.B, d = a.d, N = a.N;
-  float* rows = reinterpret_cast<float*>(smem_raw + ((sizeof(PSmem) + 15) & ~(size_t)15));  // RS row slots of SL floats
+  // OWN: scale times index of every worker and owned coordinate (not shared with wpart: no barrier separates the owners' sums from
+  // the margins of a warp that already has its slice of the new point); then RS row slots of SL floats
+  float* prod = reinterpret_cast<float*>(smem_raw + ((sizeof(PSmem) + 15) & ~(size_t)15));
+  float* rows = prod + (OWN ? N * owned_coords(SL, N) : 0);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool swz = (EPT == 8) && ((lane >> 2) & 1);  // this thread reads the halves of its row values exchanged (row_vals)
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
               for (int e = 0; e < 4; ++e) unpack2(mul2_rn(pack2(di, di), k2[e]), pr[2 * e], pr[2 * e + 1]);
             }
           }
-          float4* to = reinterpret_cast<float4*>(sm.prod + j * chunk + gi * 8);
+          float4* to = reinterpret_cast<float4*>(prod + j * chunk + gi * 8);
           to[0] = make_float4(pr[0], pr[1], pr[2], pr[3]);
           to[1] = make_float4(pr[4], pr[5], pr[6], pr[7]);
         }
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       if (owner) {
         float acc = 0.f;
 #pragma unroll 8
-        for (int j = 0; j < N; ++j) acc = add_rn(acc, sm.prod[j * chunk + tid]);
+        for (int j = 0; j < N; ++j) acc = add_rn(acc, prod[j * chunk + tid]);
         const float v = add_rn(mul_rn(acc, invN), omu);
         if constexpr (ALPC) {
           uint64_t t0 = 0;
@@ -1134,11 +1134,10 @@ bool pays_to_own(int b, int SL, int N) {
   if (SL > PT * ept || owned_coords(SL, N) > PT) return false;  // one pass, one owned coordinate per thread
   return N > 16 || !(b == 1 || b == 2 || b == 4 || b == 8);
 }
-// The instantiation for code width b, slice SL, N workers and algorithm.
-PersistKernel pick_kernel(int b, int SL, int N, bool alpc) {
+// The instantiation for code width b, slice SL, kind of update and algorithm.
+PersistKernel pick_kernel(int b, int SL, bool own, bool alpc) {
   const int ept = persist_coords_per_thread(b, SL);
   const int np = (SL > PT * ept) ? 2 : 1;
-  const bool own = pays_to_own(b, SL, N);
   return alpc ? pick_width<true>(b, np, ept, own) : pick_width<false>(b, np, ept, own);
 }
 
@@ -1174,7 +1173,7 @@ int persist_coords_per_thread(int b, int SL) {
 // soon as u is formed.  Among the sizes that fit, the largest cluster whose slices still keep a CTA busy wins: more
 // CTAs per worker shorten every serial phase of a step.
 bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_smem, int* CS_out, int* SL_out,
-                  size_t* smem_out, int* row_slots_out) {
+                  size_t* smem_out, int* row_slots_out, int* own_out) {
   int P = 1;
   while (P < d) P <<= 1;
   if (P < 32) P = 32;
@@ -1187,14 +1186,17 @@ bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_sme
     if (SL < 32) break;
     if (SL > PGROUP * PMAXP) continue;
     if (clusters * cs > PMAXFLAGS) break;
-    const size_t fixed = (sizeof(PSmem) + 15) & ~(size_t)15;
     const size_t one = (size_t)SL * 4;  // one row slot
+    const size_t base = (sizeof(PSmem) + 15) & ~(size_t)15, products = (size_t)N * owned_coords(SL, N) * 4;
+    // the owners' products must not take the place of a step's rows
+    const bool own = pays_to_own(b, SL, N) && base + products + (size_t)B * one <= (size_t)max_smem;
+    const size_t fixed = base + (own ? products : 0);
     if (fixed + (size_t)B * one > (size_t)max_smem) continue;
     int slots = (int)(((size_t)max_smem - fixed) / one);
     if (slots > 2 * B) slots = 2 * B;
     const size_t smem = fixed + (size_t)slots * one;
-    if (max_clusters(pick_kernel(b, SL, N, alpc != 0), cs, smem) < clusters) continue;
-    *CS_out = cs; *SL_out = SL; *smem_out = smem; *row_slots_out = slots;
+    if (max_clusters(pick_kernel(b, SL, own, alpc != 0), cs, smem) < clusters) continue;
+    *CS_out = cs; *SL_out = SL; *smem_out = smem; *row_slots_out = slots; *own_out = own ? 1 : 0;
     found = true;
     if (want_cs > 0) break;
     // (512 threads per CTA with half the coordinates per thread were tried as well: 5.53 against 4.92 us per step on the
@@ -1208,7 +1210,7 @@ bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_sme
 }
 
 cudaError_t launch_persist(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative) {
-  PersistKernel k = pick_kernel(pa.in.b, pa.in.SL, pa.in.N, pa.alpc != 0);
+  PersistKernel k = pick_kernel(pa.in.b, pa.in.SL, pa.own != 0, pa.alpc != 0);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;

@@ -25,6 +25,9 @@ def _same(a, b):
     (5 * 16, 1000, 5, 32, 6),
     (16 * 8, 2048, 16, 8, 32),
     (64 * 2, 1024, 64, 2, 16),   # the most workers the loop takes
+    (32 * 8, 8192, 32, 25, 2),   # the most rows that leave room for the products (8 KB), and one more
+    (32 * 8, 8192, 32, 26, 2),
+    (32 * 8, 8192, 32, 27, 2),
 ])
 def test_owned_update_equals_single_steps(n, d, N, B, b, alpc):
     X, y, _ = synth.linear_problem(n, d, loss="least_squares", sparsity=0.2, noise=0.1, seed=d + N)
