@@ -628,6 +628,10 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
     }
 #pragma unroll
     for (int e = 0; e < EPT; ++e) xr[0][e] = __uint_as_float((uint32_t)xw[e]);
+    if (width < PSPAN) {  // columns that do not exist stay 0: the margins multiply them by 0, which an infinity would not survive
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) xr[0][e] = tid * EPT + e < width ? xr[0][e] : 0.f;
+    }
   };
 
   int sb = 0;  // first row slot of the current step, (t * B) % RS

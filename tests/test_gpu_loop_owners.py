@@ -63,3 +63,48 @@ def test_owned_update_equals_single_steps(n, d, N, B, b, alpc):
     assert torch.isfinite(many.get_iterate()).all()
     one.close()
     many.close()
+
+
+@pytest.mark.parametrize("alpc", [False, True])
+@pytest.mark.parametrize("n,d,N,b,at", [
+    (17 * 8, 1000, 17, 4, 512),   # the last slice ends early; its first coordinate is the infinite one
+    (33 * 4, 2052, 33, 4, 2048),  # four columns in a slice of 1,024
+    (33 * 4, 2052, 33, 4, 0),     # an empty slice: its threads hold no coordinate, the first one is infinite
+    (4 * 16, 64, 4, 3, 0),        # a slice narrower than a pass
+    (64 * 2, 996, 64, 16, 512),
+])
+def test_columns_outside_a_slice_stay_zero_beside_an_infinite_coordinate(n, d, N, b, at, alpc):
+    # a logistic margin may be infinite, its derivative is not: gradients, scales and codes stay finite as long as
+    # nobody multiplies the infinite coordinate by the zeros that stand for columns that do not exist
+    X, y, _ = synth.linear_problem(n, d, loss="logistic", sparsity=0.2, noise=0.1, seed=d + N)
+    X[:, at] = X[:, at].abs() + 0.5  # 0 * inf in the column itself would be a NaN of its own
+    X, y = X.cuda(), y.cuda()
+    x0 = torch.from_numpy((np.random.default_rng(3).standard_normal(d) * 0.1).astype(np.float32)).cuda()
+    far = x0.clone()
+    far[at] = float("inf")
+    one, many = (lpc.Context(X, y, lpc.LOGISTIC, 1e-5, N, 3, b, lpc.CLIP_STD, 2.0, 11) for _ in range(2))
+    one.set_option(lpc.OPT_PERSISTENT, 0)
+    par, count = (0.4, 0.5, 0.3, 0.2), 4
+    for c in (one, many):
+        c.set_iterate(x0)
+        if alpc:
+            c.alpc_begin()
+        c.snapshot_full_grad()
+        if alpc:
+            c.set_buffer(lpc.BUF_Y, far)
+            c.set_buffer(lpc.BUF_Z, far)
+        else:
+            c.set_iterate(far)
+        if alpc:
+            c.alpc_double_sample_steps(*par, 0, count)
+        else:
+            c.inner_steps(0.05, 0, count)
+        c.sync_status()
+    assert many.query(lpc.INFO_LOOP_LAUNCHES) == 1
+    for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA] + ([lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM] if alpc else []):
+        assert _same(one.get_buffer(w), many.get_buffer(w)), w
+    delta, x = many.get_buffer(lpc.BUF_DELTA), many.get_iterate()
+    assert torch.isfinite(delta).all() and (delta > 0).all()
+    assert x[at] == float("inf") and torch.isfinite(x).sum() == d - 1
+    one.close()
+    many.close()
