@@ -303,6 +303,9 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
                                               on a 16-byte boundary (ld % 4 == 0), for b = 32, and when the call was one launch */
 #define LPC_INFO_QUANT_LAUNCHES 14         /* last lpc_quantize_pack: kernels it launched.  1: a cluster per worker (or an empty vector);
                                               3: statistics, scale, codes; 4: the same and the unified scale */
+#define LPC_INFO_LOOP_OWNED 15             /* one-launch loop: 1 when each coordinate's update is made by one CTA, which sends the new
+                                              point to the others; 0 when every cluster updates its copy, or loop not available */
+#define LPC_INFO_ALPC_LOOP_OWNED 16        /* the same for the loop of Algorithm 2 */
 int lpc_query(const lpc_ctx* ctx, int what, int64_t* out);
 
 /* Per-kernel device time measured with CUDA events on the context's stream while LPC_OPT_PROFILE is

@@ -820,6 +820,8 @@ int lpc_query(const lpc_ctx* c, int what, int64_t* out) {
     case LPC_INFO_ALPC_LOOP_ROW_SLOTS: *out = c->apersist_ok ? c->aSlots : 0; return LPC_OK;
     case LPC_INFO_LOOP_COORDS_PER_THREAD: *out = c->persist_ok ? persist_coords_per_thread(c->b, c->pSL) : 0; return LPC_OK;
     case LPC_INFO_ALPC_LOOP_COORDS_PER_THREAD: *out = c->apersist_ok ? persist_coords_per_thread(c->b, c->aSL) : 0; return LPC_OK;
+    case LPC_INFO_LOOP_OWNED: *out = c->persist_ok ? c->pOwn : 0; return LPC_OK;
+    case LPC_INFO_ALPC_LOOP_OWNED: *out = c->apersist_ok ? c->aOwn : 0; return LPC_OK;
     case LPC_INFO_STEP_RING_STAGES: *out = c->inner_ok ? c->innerStages : 0; return LPC_OK;
     case LPC_INFO_LOOP_LAUNCHES: *out = c->persist_launches; return LPC_OK;
     case LPC_INFO_SNAPSHOT_ROWS_PER_TILE: *out = c->snapR; return LPC_OK;

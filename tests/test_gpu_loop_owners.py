@@ -14,22 +14,27 @@ def _same(a, b):
     return torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
 
 
+OWN = {False: (lpc.INFO_LOOP_CLUSTER_SIZE, lpc.INFO_LOOP_OWNED), True: (lpc.INFO_ALPC_LOOP_CLUSTER_SIZE, lpc.INFO_ALPC_LOOP_OWNED)}
+
+
 @pytest.mark.parametrize("alpc", [False, True])
-@pytest.mark.parametrize("n,d,N,B,b", [
-    (17 * 8, 4096, 17, 3, 4),    # the first count beyond sixteen; shares of 64 coordinates of a slice of 1,024
-    (31 * 8, 8188, 31, 16, 2),   # 31 shares of 72 in slices of 2,048, the last column inside one; rows that do not fit a step ahead
-    (32 * 4, 5000, 32, 2, 8),    # the last CTA of a cluster has few columns
-    (24 * 4, 64, 24, 1, 1),      # more workers than groups of eight coordinates
-    (33 * 4, 2052, 33, 4, 4),    # slices that are half empty
-    (2 * 16, 512, 2, 5, 3),      # widths known at run time: owners whatever the worker count
-    (5 * 16, 1000, 5, 32, 6),
-    (16 * 8, 2048, 16, 8, 32),
-    (64 * 2, 1024, 64, 2, 16),   # the most workers the loop takes
-    (32 * 8, 8192, 32, 25, 2),   # the most rows that leave room for the products (8 KB), and one more
-    (32 * 8, 8192, 32, 26, 2),
-    (32 * 8, 8192, 32, 27, 2),
+@pytest.mark.parametrize("n,d,N,B,b,own", [
+    (17 * 8, 4096, 17, 3, 4, 1),    # the first count beyond sixteen; shares of 64 coordinates of a slice of 1,024
+    (16 * 8, 4096, 16, 3, 4, 0),    # sixteen: every cluster updates its copy
+    (31 * 8, 8188, 31, 16, 2, 1),   # 31 shares of 72 in slices of 2,048, the last column inside one; rows that do not fit a step ahead
+    (32 * 4, 5000, 32, 2, 8, 1),    # the last CTA of a cluster has few columns
+    (24 * 4, 64, 24, 1, 1, 1),      # more workers than groups of eight coordinates
+    (33 * 4, 2052, 33, 4, 4, 1),    # slices that are half empty
+    (2 * 16, 512, 2, 5, 3, 1),      # widths known at run time: owners whatever the worker count
+    (5 * 16, 1000, 5, 32, 6, 1),
+    (16 * 8, 2048, 16, 8, 32, 1),
+    (4 * 16, 512, 1, 5, 3, 0),      # more coordinates to an owner than threads
+    (64 * 2, 1024, 64, 2, 16, 1),   # the most workers the loop takes
+    (32 * 8, 8192, 32, 25, 2, 1),   # the most rows that leave room for the products (8 KB), one more, and too many for the loop
+    (32 * 8, 8192, 32, 26, 2, 0),
+    (32 * 8, 8192, 32, 27, 2, None),
 ])
-def test_owned_update_equals_single_steps(n, d, N, B, b, alpc):
+def test_owned_update_equals_single_steps(n, d, N, B, b, own, alpc):
     X, y, _ = synth.linear_problem(n, d, loss="least_squares", sparsity=0.2, noise=0.1, seed=d + N)
     X, y = X.cuda(), y.cuda()
     x0 = torch.from_numpy((np.random.default_rng(3).standard_normal(d) * 0.1).astype(np.float32)).cuda()
@@ -55,8 +60,9 @@ def test_owned_update_equals_single_steps(n, d, N, B, b, alpc):
             many.inner_steps(0.05, k0, count)
     one.sync_status()
     many.sync_status()
-    if many.query(lpc.INFO_ALPC_LOOP_CLUSTER_SIZE if alpc else lpc.INFO_LOOP_CLUSTER_SIZE):
-        assert many.query(lpc.INFO_LOOP_LAUNCHES) == 2
+    cluster, owned = (many.query(q) for q in OWN[alpc])
+    assert (owned if cluster else None) == own
+    assert many.query(lpc.INFO_LOOP_LAUNCHES) == (2 if cluster else 0)
     for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_U, lpc.BUF_V, lpc.BUF_CLIPPED] + (
             [lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_VHAT] if alpc else []):
         assert _same(one.get_buffer(w), many.get_buffer(w)), w
@@ -100,7 +106,7 @@ def test_columns_outside_a_slice_stay_zero_beside_an_infinite_coordinate(n, d, N
         else:
             c.inner_steps(0.05, 0, count)
         c.sync_status()
-    assert many.query(lpc.INFO_LOOP_LAUNCHES) == 1
+    assert many.query(lpc.INFO_LOOP_LAUNCHES) == 1 and many.query(OWN[alpc][1]) == 1
     for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA] + ([lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM] if alpc else []):
         assert _same(one.get_buffer(w), many.get_buffer(w)), w
     delta, x = many.get_buffer(lpc.BUF_DELTA), many.get_iterate()
