@@ -559,6 +559,9 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
 #pragma unroll
             for (int k = 0; k < WMAX; ++k) ok = ok && word_tag(w[k]) == tag;
           }
+#ifdef LPC_TRACE
+          if (i == 0 && blockIdx.x == 0 && blockIdx.y == 0 && target >= 8 && target < 72) g_trace[(target - 8) * 16 + 15] = it + 1;
+#endif
           if (ok || wait_expired(it, t0)) break;
         }
         if (have) {
