@@ -1131,15 +1131,25 @@ PersistKernel pick_width(int b, int np, int ept, bool own) {
     default: return pick_shape<0, ALPC>(np, ept, own);
   }
 }
-// Whether the update is left to the owners of the coordinates.  With more workers than one round of loads takes (CH in
-// apply_update) the second round alone is as long as the second crossing; the widths known at run time load up to eight words per
-// group and decode slowly.  us per step, everybody / owners: Algorithm 2, d = 8,192, N = 32, b = 2: 9.68 / 8.47, b = 8: 10.2 / 8.7;
-// Algorithm 1, d = 4,096, b = 4: N = 17: 5.84 / 4.86, N = 16: 4.70 / 4.84; d = 1,024, N = 32: 5.22 / 4.81, N = 2: 4.31 / 4.37;
-// b = 3: N = 16, d = 512: 9.27 / 5.78, N = 2: 5.69 / 5.47; b = 32, d = 2,048, N = 16: 10.9 / 5.3, N = 4: 6.5 / 5.6.
-bool pays_to_own(int b, int SL, int N) {
+// Whether the update is left to the owners of the coordinates.  us per step below: everybody / owners.
+// Fixed widths: with more workers than one round of loads takes (CH in apply_update) the second round alone is as long as the second
+// crossing.  N = 16 / 17, b = 4: Algorithm 1, d = 1,024 4.05 / 4.32 and 5.10 / 4.37, d = 8,192 5.03 / 5.13 and 6.47 / 5.65; Algorithm 2,
+// d = 1,024 4.36 / 4.81 and 5.30 / 4.84, d = 8,192 5.68 / 5.89 and 7.13 / 6.40 (N = 4, 8 and 12: owners 4 to 14 % slower).  64 workers,
+// d = 4,096: 8.93 / 5.88 and 9.56 / 6.44.  b = 1, 2 and 8 lie alike (b = 8, d = 8,192, N = 16: 5.30 / 5.20).
+// The widths known at run time load up to eight words per group, those of four workers a round, and decode slowly.  Five workers,
+// d = 2,048: b = 3 6.73 / 5.73 and 7.52 / 6.41, b = 32 7.20 / 5.04 and 7.89 / 5.77.  Up to four the two are close.  Clusters of four CTAs
+// and more without a second round of rows (eight are kept in registers) leave the crossing nothing to hide behind: b = 3, N = 4,
+// d = 2,048: B = 8 5.74 / 5.80 and 6.34 / 6.48, B = 16 6.87 / 6.79 and 7.51 / 7.56, d = 1,024, B = 8 5.51 / 5.47 and 6.07 / 6.05, N = 2,
+// d = 2,048, B = 8 5.58 / 5.45 and 6.18 / 6.06; N = 1, d = 256, B = 4 5.27 / 5.20 and 5.75 / 5.68.  b = 32, whose eight words per group have
+// to be found somewhere: Algorithm 1, N = 4, d = 256 4.35 / 4.31, d = 512 5.09 / 4.31; Algorithm 2, whose estimator adds as many,
+// d = 480 4.89 / 5.04, d = 512 5.32 / 5.07.
+bool pays_to_own(int b, int d, int SL, int CS, int N, int B, bool alpc) {
   const int ept = persist_coords_per_thread(b, SL);
   if (SL > PT * ept || owned_coords(SL, N) > PT) return false;  // one pass, one owned coordinate per thread
-  return N > 16 || !(b == 1 || b == 2 || b == 4 || b == 8);
+  if (b == 1 || b == 2 || b == 4 || b == 8) return N > 16;
+  if (N > 4) return true;
+  if (b == 32) return !alpc || d >= 512;
+  return N < 3 || CS < 4 || B > 8;
 }
 // The instantiation for code width b, slice SL, kind of update and algorithm.
 PersistKernel pick_kernel(int b, int SL, bool own, bool alpc) {
@@ -1196,7 +1206,7 @@ bool persist_plan(int d, int N, int B, int b, int alpc, int want_cs, int max_sme
     const size_t one = (size_t)SL * 4;  // one row slot
     const size_t base = (sizeof(PSmem) + 15) & ~(size_t)15, products = (size_t)N * owned_coords(SL, N) * 4;
     // the owners' products must not take the place of a step's rows
-    const bool own = pays_to_own(b, SL, N) && base + products + (size_t)B * one <= (size_t)max_smem;
+    const bool own = pays_to_own(b, d, SL, cs, N, B, alpc != 0) && base + products + (size_t)B * one <= (size_t)max_smem;
     const size_t fixed = base + (own ? products : 0);
     if (fixed + (size_t)B * one > (size_t)max_smem) continue;
     int slots = (int)(((size_t)max_smem - fixed) / one);

@@ -25,10 +25,17 @@ OWN = {False: (lpc.INFO_LOOP_CLUSTER_SIZE, lpc.INFO_LOOP_OWNED), True: (lpc.INFO
     (32 * 4, 5000, 32, 2, 8, 1),    # the last CTA of a cluster has few columns
     (24 * 4, 64, 24, 1, 1, 1),      # more workers than groups of eight coordinates
     (33 * 4, 2052, 33, 4, 4, 1),    # slices that are half empty
-    (2 * 16, 512, 2, 5, 3, 1),      # widths known at run time: owners whatever the worker count
+    (2 * 16, 512, 2, 5, 3, 1),      # widths known at run time: owners from one worker on
+    (4 * 16, 256, 1, 5, 3, 1),
     (5 * 16, 1000, 5, 32, 6, 1),
     (16 * 8, 2048, 16, 8, 32, 1),
     (4 * 16, 512, 1, 5, 3, 0),      # more coordinates to an owner than threads
+    (4 * 16, 2048, 4, 8, 3, 0),     # but not for three or four in clusters of four CTAs whose rows stay in registers
+    (3 * 16, 2048, 3, 8, 16, 0),
+    (4 * 16, 2048, 4, 9, 3, 1),
+    (5 * 16, 2048, 5, 8, 3, 1),
+    (4 * 16, 512, 4, 4, 32, 1),
+    (4 * 16, 508, 4, 4, 32, (1, 0)),  # Algorithm 1 / Algorithm 2, whose short vectors of whole floats are updated by everybody
     (64 * 2, 1024, 64, 2, 16, 1),   # the most workers the loop takes
     (32 * 8, 8192, 32, 25, 2, 1),   # the most rows that leave room for the products (8 KB), one more, and too many for the loop
     (32 * 8, 8192, 32, 26, 2, 0),
@@ -61,7 +68,7 @@ def test_owned_update_equals_single_steps(n, d, N, B, b, own, alpc):
     one.sync_status()
     many.sync_status()
     cluster, owned = (many.query(q) for q in OWN[alpc])
-    assert (owned if cluster else None) == own
+    assert (owned if cluster else None) == (own[alpc] if isinstance(own, tuple) else own)
     assert many.query(lpc.INFO_LOOP_LAUNCHES) == (2 if cluster else 0)
     for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_U, lpc.BUF_V, lpc.BUF_CLIPPED] + (
             [lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_VHAT] if alpc else []):
