@@ -318,6 +318,8 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
   auto couple = [&](float z, float xt, float y) {  // step 6 of Algorithm 2: x = tau1 z + tau2 x~ + (1 - tau1 - tau2) y
     return add_rn(add_rn(mul_rn(pa.tau1, z), mul_rn(pa.tau2, xt)), mul_rn(tau3, y));
   };
+  // columns that do not exist stay 0: the margins multiply them by 0, which an infinity would not survive
+  const uint32_t keep_lo = tid * EPT < width ? 0xFFFFFFFFu : 0u, keep_hi = tid * EPT + 4 < width ? 0xFFFFFFFFu : 0u;
   // OWN: the coordinate whose state this thread keeps, if any
   const int chunk = OWN ? owned_coords(SL, N) : 0;
   const int oc = c0 + worker * chunk + tid;
@@ -630,11 +632,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       if (__all_sync(0xFFFFFFFFu, ok) || __any_sync(0xFFFFFFFFu, wait_expired(it, t0))) break;
     }
 #pragma unroll
-    for (int e = 0; e < EPT; ++e) xr[0][e] = __uint_as_float((uint32_t)xw[e]);
-    if (width < PSPAN) {  // columns that do not exist stay 0: the margins multiply them by 0, which an infinity would not survive
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) xr[0][e] = tid * EPT + e < width ? xr[0][e] : 0.f;
-    }
+    for (int e = 0; e < EPT; ++e) xr[0][e] = __uint_as_float((uint32_t)xw[e] & (e < 4 ? keep_lo : keep_hi));
   };
 
   int sb = 0;  // first row slot of the current step, (t * B) % RS
