@@ -306,6 +306,8 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
 #define LPC_INFO_LOOP_OWNED 15             /* one-launch loop: 1 when each coordinate's update is made by one CTA, which sends the new
                                               point to the others; 0 when every cluster updates its copy, or loop not available */
 #define LPC_INFO_ALPC_LOOP_OWNED 16        /* the same for the loop of Algorithm 2 */
+#define LPC_INFO_QUANT_KEPT_TILES 17       /* last lpc_quantize_pack: tiles of 8192 values at the end of the input that the first look left in
+                                              L2 for the second while it let the others go; 0: its loads carried no cache policy */
 int lpc_query(const lpc_ctx* ctx, int what, int64_t* out);
 
 /* Per-kernel device time measured with CUDA events on the context's stream while LPC_OPT_PROFILE is

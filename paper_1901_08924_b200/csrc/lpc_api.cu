@@ -32,6 +32,7 @@ struct SegPlan {
   std::vector<int32_t> tile_seg;    // host copy
   SegInfo* d_segs = nullptr;
   int32_t* d_tile_seg = nullptr;    // nullptr when nseg == 1
+  bool offsets_x8 = true;           // every segment's offset is a multiple of 8
   uint64_t msg_bits = 0;            // sum over segments of 32 + b*len_s
   int64_t whole_runs = 0;           // runs of 8 tiles that consist of whole tiles of one segment whose offset keeps 16-byte alignment
 };
@@ -115,7 +116,7 @@ struct lpc_ctx {
   size_t q_scale_cap = 0;
   int loop_cooperative = 1;       // LPC_OPT_LOOP_COOPERATIVE
   int one_launch = 1;             // LPC_OPT_ONE_LAUNCH_QUANTIZE
-  int last_one_launch = 0, last_quant_launches = 0;
+  int last_one_launch = 0, last_quant_launches = 0, last_kept_tiles = 0;
   unsigned long long* coded_host = nullptr;  // pinned: entropy (double) and Huffman length of coded_cap messages each
   size_t coded_cap = 0;
   // graph replay
@@ -131,7 +132,7 @@ struct lpc_ctx {
   int64_t prof_n[LPC_KERNEL_KINDS] = {0};
   // accounting
   uint64_t step1_bits = 0, step2_bits = 0;
-  int sm_count = 148, max_smem = 227 * 1024;
+  int sm_count = 148, max_smem = 227 * 1024, l2_bytes = 0;
   std::string err;
 };
 
@@ -227,6 +228,7 @@ int make_plan(lpc_ctx* c, SegPlan& p, int64_t len, int b, const int64_t* seg_off
   p.offsets[nseg] = len;
   p.segs = segs;
   p.tile_seg = tile_seg;
+  for (const SegInfo& g : p.segs) p.offsets_x8 = p.offsets_x8 && g.off % 8 == 0;
   const int run = quantize_run_tiles();
   for (int t0 = 0; t0 < p.ntiles; t0 += run) {
     const int t1 = std::min(t0 + run, p.ntiles) - 1;
@@ -574,6 +576,7 @@ int lpc_init(lpc_ctx** out, const float* X, const float* y, int64_t n, int32_t d
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, dev);
   int optin = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) { delete c; return LPC_ERR_CUDA; }
@@ -828,6 +831,7 @@ int lpc_query(const lpc_ctx* c, int what, int64_t* out) {
     case LPC_INFO_SNAPSHOT_STAGES: *out = c->snapStages; return LPC_OK;
     case LPC_INFO_QUANT_ONE_LAUNCH: *out = c->last_one_launch; return LPC_OK;
     case LPC_INFO_QUANT_LAUNCHES: *out = c->last_quant_launches; return LPC_OK;
+    case LPC_INFO_QUANT_KEPT_TILES: *out = c->last_kept_tiles; return LPC_OK;
     case LPC_INFO_AGGREGATE_SPLIT: *out = c->last_split; return LPC_OK;
     case LPC_INFO_QUANT_PIPELINED_RUNS: *out = c->last_pipelined_runs; return LPC_OK;
     default: return LPC_ERR_INVALID_ARG;
@@ -888,6 +892,7 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   const bool cluster = c->last_one_launch && quantize_fits_cluster(a, c->sm_count);
   c->last_pipelined_runs = vec && c->b != 32 && !cluster ? p.whole_runs : 0;
   c->last_quant_launches = cluster ? 1 : quantize_pack_launches(a);
+  c->last_kept_tiles = a.kept_tiles = cluster ? 0 : quantize_kept_tiles(a, p.offsets_x8, c->l2_bytes);
   if (cluster) {
     ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
     CU(c, launch_quantize_cluster(a, c->stream));

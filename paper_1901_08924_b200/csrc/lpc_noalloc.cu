@@ -45,9 +45,9 @@ __global__ void static_setup_kernel(SegInfo seg) {
 // is asked for once per device, with that device current.
 std::mutex g_mu;
 unsigned char* g_dev_ptr[64] = {nullptr};
-int g_sm_count[64];
+int g_sm_count[64], g_l2_bytes[64];
 
-int scratch_address(unsigned char** out, int* sm_count) {
+int scratch_address(unsigned char** out, int* sm_count, int* l2_bytes) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LPC_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mu);
@@ -57,11 +57,14 @@ int scratch_address(unsigned char** out, int* sm_count) {
       cudaGetLastError();
       return LPC_ERR_CUDA;
     }
-    if (cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LPC_ERR_CUDA;
+    if (cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&g_l2_bytes[dev], cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+      return LPC_ERR_CUDA;
     g_dev_ptr[dev] = static_cast<unsigned char*>(p);
   }
   *out = g_dev_ptr[dev];
   *sm_count = g_sm_count[dev];
+  *l2_bytes = g_l2_bytes[dev];
   return LPC_OK;
 }
 
@@ -82,8 +85,8 @@ extern "C" int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld,
   if (N > MAX_N || ntiles * N > MAX_PARTS || (len + 7) / 8 > 0xFFFFFFFFll) return LPC_ERR_UNSUPPORTED;
 
   unsigned char* base = nullptr;
-  int sm_count = 0;
-  const int rc = scratch_address(&base, &sm_count);
+  int sm_count = 0, l2_bytes = 0;
+  const int rc = scratch_address(&base, &sm_count, &l2_bytes);
   if (rc != LPC_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
 
@@ -106,5 +109,6 @@ extern "C" int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld,
   a.codes = codes_out; a.stride_words = seg.pad_words;
   a.delta_out = delta_out; a.clipped_out = clipped_out; a.count_clipped = 1; a.shared_scale = 0;
   a.dev_status = reinterpret_cast<unsigned int*>(base + OFF_STATUS);
+  a.kept_tiles = quantize_kept_tiles(a, true, l2_bytes);
   return launch_quantize_pack(a, sm_count, st) == cudaSuccess ? LPC_OK : LPC_ERR_CUDA;
 }

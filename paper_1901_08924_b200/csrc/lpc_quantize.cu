@@ -188,22 +188,17 @@ __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int wor
   }
 }
 
-// The second pass goes back from the end, so the tiles worth keeping in L2 are the last ones: those before the last `keep` are
-// read so that they go first.  Quantizer, us, with 40 / 60 / 100 MB kept and without: 8 x 2^24, b = 8 184.4 / 184.0 / 184.6, 190.7;
-// 8 x 2^22 on one scale 52.2 / 53.6 / 55.7, 56.6; 8 x 2^26 690 / 690 / 693, 693.  With a subtrahend, whose second pass takes longer
-// per byte: 8 x 2^23 160.6 / 159.6 / 160.1, 164.0.  The loads cost a hundredth of the first pass, and what is saved does not grow with
-// the input: from 1 GB on it is not worth it (62 tensors for 16 workers, 1.5 GB: first pass 218.6 -> 220.7, second 240.2 -> 240.3).
-constexpr int64_t KEEP_BYTES = 48ll << 20, KEEP_BYTES_SUB = 96ll << 20, KEEP_MAX_INPUT = 1ll << 30;
-
+// POLICY: the second pass goes back from the end, so the tiles worth keeping in L2 are the last a.kept_tiles ones: those before them
+// are read so that they go first.
 template <bool NEED_SUMS, bool POLICY>
-__global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a, int keep) {
+__global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a) {
   launch_dependents();
   wait_for_launch_before();
   __shared__ float sh1[QITER * 8], sh2[QITER * 8];
   __shared__ uint32_t shm[8];
   uint64_t policy = 0;
   if constexpr (POLICY) {
-    if ((int64_t)blockIdx.y * a.ntiles + blockIdx.x < (int64_t)a.N * a.ntiles - keep)
+    if ((int64_t)blockIdx.y * a.ntiles + blockIdx.x < (int64_t)a.N * a.ntiles - a.kept_tiles)
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     else
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
@@ -854,6 +849,25 @@ __global__ void __launch_bounds__(QT) bypass_kernel(QuantArgs a) {
 
 }  // namespace
 
+// Where the first look's loads carry a cache policy, and how much is kept: three eighths of L2 of each input.  Quantizer, us, on the
+// 126.5 MB of a B200, 8 workers, without / with 24, 36, 47 (three eighths), 60 and 100 MB kept: 134 MB of values, b = 4 54.6 / 51.7, 51.3,
+// 51.8, 52.5, 54.6; 537 MB, b = 8 201.6 / 193.1, 192.8, 193.3, 193.5, 194.5.  With a subtrahend, without / with 48, 72, 95 and 120 MB:
+// 537 MB, b = 4 168.1 / 166.3, 165.8, 165.2, 164.9.
+// From: inputs beyond five eighths of L2 (each).  Shorter ones stay by themselves: 75 MB 34.5 / 34.7, 84 MB 38.0 / 37.8, 92 MB 41.5 / 40.4;
+// with a subtrahend 134 MB together 47.0 / 47.0, 168 MB 57.4 / 56.8.
+// To: what is saved does not grow with the input, while the loads cost a hundredth of the first look: 16 times L2 (2.0 GB 680.6 / 674.9,
+// 2.1 GB 702.3 / 702.3), with a subtrahend 6 times (b = 4 / b = 8 without and with, 738 MB 226.2, 225.4 / 235.7, 234.1; 805 MB 246.3, 249.1 /
+// 260.3, 258.9; 1.1 GB 326.2, 333.7 / 343.9, 345.6).
+// Only where all rows and tensors start on 32-byte boundaries: the shorter loads of the others have no policy to carry (537 MB with
+// every second row off 181.9 / 183.5).
+int quantize_kept_tiles(const QuantArgs& a, bool offsets_aligned, int64_t l2_bytes) {
+  auto aligned = [](const float* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; };
+  if (!offsets_aligned || !aligned(a.U) || !aligned(a.U_sub) || (a.N > 1 && a.ld % 8 != 0)) return 0;
+  const int64_t tile_bytes = (int64_t)TILE * sizeof(float), bytes = (int64_t)a.N * a.ntiles * tile_bytes;  // of each input
+  if (bytes <= l2_bytes / 8 * 5 || bytes * (a.U_sub ? 2 : 1) > l2_bytes * (a.U_sub ? 6 : 16)) return 0;
+  return (int)(l2_bytes / 8 * 3 / tile_bytes);
+}
+
 // One cluster per worker: vectors of one segment and at most CTILES tiles, the fixed widths.  Up to about four CTAs per SM
 // the clusters run side by side; with more of them the two passes over L2 of the other paths are as good.
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count) {
@@ -903,11 +917,9 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
   cudaError_t e = cudaSuccess;
   if (a.ntiles > 0) {
     if (hook) hook(user, 3 /* LPC_KERNEL_QUANT_STATS */, 1);
-    const int64_t tile_bytes = (int64_t)TILE * sizeof(float) * (a.U_sub ? 2 : 1), tiles = (int64_t)a.N * a.ntiles;
-    const int keep = (int)((a.U_sub ? KEEP_BYTES_SUB : KEEP_BYTES) / tile_bytes);
     const bool sums = a.clip_mode == CLIP_STD;
-    if (tiles <= keep || tiles * tile_bytes > KEEP_MAX_INPUT) e = sums ? launch(stats_kernel<true, false>, grid, 0) : launch(stats_kernel<false, false>, grid, 0);
-    else e = sums ? launch(stats_kernel<true, true>, grid, keep) : launch(stats_kernel<false, true>, grid, keep);
+    if (a.kept_tiles > 0) e = sums ? launch(stats_kernel<true, true>, grid) : launch(stats_kernel<false, true>, grid);
+    else e = sums ? launch(stats_kernel<true, false>, grid) : launch(stats_kernel<false, false>, grid);
     if (hook) hook(user, 3, 0);
     if (e != cudaSuccess) return e;
   }
