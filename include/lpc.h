@@ -368,6 +368,16 @@ int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld, int32_t N,
 int lpc_debug_wait_timeout(lpc_ctx* ctx, uint64_t limit_ns);
 
 /*
+ * Inspection aid for the scale rule (Eq. 2 and its c * std form) of the one-launch loops, which forms the threshold in single precision
+ * with an interval around it and leaves what that does not decide to doubles, the definition.  For i < count, from max_bits[i] (the bit
+ * pattern of max |u|), S1[i] and S2[i] (the sums of u and u^2; device) of vectors of len values in b bits: scale_out (device) takes
+ * delta, 1 / delta, the threshold and the hull's lower end, flags_out (device) bit 0 degenerate (zeros are sent), bit 1 not finite,
+ * bit 2 threshold left to the doubles.
+ */
+int lpc_debug_loop_scales(const uint32_t* max_bits, const float* S1, const float* S2, int64_t count, int64_t len, int32_t b,
+                          int clip_mode, float clip_value, float* scale_out, uint32_t* flags_out, void* stream);
+
+/*
  * Inspection aid: writes `count` consecutive 4-word blocks, starting at block `block0`, of the
  * counter-based random stream (tag, worker, k) keyed by `seed` to out (device, 4*count words).
  * The streams are Philox4x32-10 (Salmon et al., SC'11) with counter (block, k_lo, worker | tag<<24,

@@ -1006,6 +1006,16 @@ int lpc_debug_wait_timeout(lpc_ctx* c, uint64_t limit_ns) {
   return LPC_OK;
 }
 
+int lpc_debug_loop_scales(const uint32_t* max_bits, const float* S1, const float* S2, int64_t count, int64_t len, int32_t b, int clip_mode,
+                          float clip_value, float* scale_out, uint32_t* flags_out, void* stream) {
+  if (count < 0 || len < 1 || !valid_b(b) || clip_mode < LPC_CLIP_NONE || clip_mode > LPC_CLIP_STD) return LPC_ERR_INVALID_ARG;
+  if (count == 0) return LPC_OK;
+  if (!max_bits || !S1 || !S2 || !scale_out || !aligned16(scale_out) || !flags_out) return LPC_ERR_INVALID_ARG;
+  const cudaError_t e = launch_loop_scales(max_bits, S1, S2, count, scale_rule(len, b), b, clip_mode, clip_value,
+                                           reinterpret_cast<float4*>(scale_out), flags_out, reinterpret_cast<cudaStream_t>(stream));
+  return e == cudaSuccess ? LPC_OK : LPC_ERR_CUDA;
+}
+
 int lpc_debug_stream_blocks(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t block0, int64_t count,
                             uint32_t* out, void* stream) {
   if (count < 0 || (count > 0 && !out)) return LPC_ERR_INVALID_ARG;

@@ -205,8 +205,8 @@ static __device__ __noinline__ float std_threshold_rare(float S1, float S2, int6
 // of a sum by Dekker's and Knuth's formulas), the root one Newton step from a reciprocal root.  Both this value and the
 // definition's lie within 2^-42 of the true threshold (where the mean takes less than 3/4 of the second moment, and far from
 // the ends of the range), so if everything within 2^-38 of it rounds to one float, that float is the definition's; rounding
-// keeps the order, so min(., M) can come after it.  One scale in 10^4 is left to the doubles.
-__device__ __forceinline__ float std_threshold(float S1, float S2, const ScaleRule& r, float c, float M) {
+// keeps the order, so min(., M) can come after it.  Returns whether that decided T; one scale in 10^4 is left to the doubles.
+__device__ __forceinline__ bool std_threshold_single(float S1, float S2, const ScaleRule& r, float c, float M, float& T) {
   auto sub = [](float a, float b) { return __fsub_rn(a, b); };
   const float mh = mul_rn(S1, r.inv_len), me = add_rn(__fmaf_rn(S1, r.inv_len, -mh), mul_rn(S1, r.inv_len_low));
   const float xh = mul_rn(S2, r.inv_len), xe = add_rn(__fmaf_rn(S2, r.inv_len, -xh), mul_rn(S2, r.inv_len_low));
@@ -218,10 +218,15 @@ __device__ __forceinline__ float std_threshold(float S1, float S2, const ScaleRu
     const float y = rsqrtf(vh), sh = mul_rn(vh, y);
     const float sl = mul_rn(add_rn(__fmaf_rn(-sh, sh, vh), vl), mul_rn(0.5f, y));
     const float th = mul_rn(c, sh), te = add_rn(__fmaf_rn(c, sh, -th), mul_rn(c, sl));
-    const float T = add_rn(th, te), low = sub(te, sub(T, th)), d = mul_rn(T, 3.637978807091713e-12f);  // 2^-38
-    if (add_rn(T, add_rn(low, d)) == T && add_rn(T, sub(low, d)) == T) return fminf(T, M);
+    const float t = add_rn(th, te), low = sub(te, sub(t, th)), d = mul_rn(t, 3.637978807091713e-12f);  // 2^-38
+    T = fminf(t, M);
+    return add_rn(t, add_rn(low, d)) == t && add_rn(t, sub(low, d)) == t;
   }
-  return std_threshold_rare(S1, S2, r.len, c, M);
+  return false;
+}
+__device__ __forceinline__ float std_threshold(float S1, float S2, const ScaleRule& r, float c, float M) {
+  float T;
+  return std_threshold_single(S1, S2, r, c, M, T) ? T : std_threshold_rare(S1, S2, r.len, c, M);
 }
 
 // make_scale, bit for bit, with a shorter chain and more code: for a loop that runs it every step.  (In kernels that form one scale

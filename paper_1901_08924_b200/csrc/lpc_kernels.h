@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lpc_scale.h"
+
 namespace lpc {
 
 constexpr int TILE = 8192;  // coordinates per CTA tile of the standalone quantizer / aggregator kernels
@@ -163,6 +165,8 @@ cudaError_t launch_coded_size(const unsigned long long* hist, int messages, int 
 }  // namespace lpc
 
 namespace lpc {
+cudaError_t launch_loop_scales(const uint32_t* max_bits, const float* S1, const float* S2, int64_t count, const ScaleRule& rule, int b,
+                               int clip_mode, float clip_value, float4* scale_out, uint32_t* flags_out, cudaStream_t st);
 cudaError_t launch_stream_blocks(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t block0,
                                  int64_t count, uint32_t* out, cudaStream_t st);
 }  // namespace lpc

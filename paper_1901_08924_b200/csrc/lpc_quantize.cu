@@ -968,7 +968,28 @@ __global__ void stream_blocks_kernel(uint64_t seed, uint32_t tag, uint32_t worke
     out[4 * i + 0] = r.x; out[4 * i + 1] = r.y; out[4 * i + 2] = r.z; out[4 * i + 3] = r.w;
   }
 }
+
+__global__ void loop_scales_kernel(const uint32_t* __restrict__ max_bits, const float* __restrict__ S1, const float* __restrict__ S2,
+                                   int64_t count, ScaleRule rule, int b, int clip_mode, float clip_value,
+                                   float4* __restrict__ scale_out, uint32_t* __restrict__ flags_out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const uint32_t m = max_bits[i];
+  const Scale sc = make_scale_in_loop(m, S1[i], S2[i], rule, b, clip_mode, clip_value);
+  float T;
+  const bool doubles = clip_mode == CLIP_STD && m != 0u && m < 0x7F800000u &&
+                       !std_threshold_single(S1[i], S2[i], rule, clip_value, __uint_as_float(m), T);
+  scale_out[i] = make_float4(sc.delta, sc.rdelta, sc.T, sc.lower);
+  flags_out[i] = sc.flags | (doubles ? 4u : 0u);
+}
 }  // namespace
+
+cudaError_t launch_loop_scales(const uint32_t* max_bits, const float* S1, const float* S2, int64_t count, const ScaleRule& rule, int b,
+                               int clip_mode, float clip_value, float4* scale_out, uint32_t* flags_out, cudaStream_t st) {
+  loop_scales_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(max_bits, S1, S2, count, rule, b, clip_mode, clip_value, scale_out,
+                                                                     flags_out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_stream_blocks(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t block0,
                                  int64_t count, uint32_t* out, cudaStream_t st) {

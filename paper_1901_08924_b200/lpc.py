@@ -66,6 +66,7 @@ SYMBOLS = [
                                  _f32, _vp, _f64p, _u64p]),
     ("lpc_quantize_pack_static", _int, [_vp, _i64, _i64, _i32, _i32, _int, _f32, _u64, _u64, _vp, _vp, _vp, _vp]),
     ("lpc_debug_wait_timeout", _int, [_vp, _u64]),
+    ("lpc_debug_loop_scales", _int, [_vp, _vp, _vp, _i64, _i64, _i32, _int, _f32, _vp, _vp, _vp]),
     ("lpc_debug_stream_blocks", _int, [_u64, C.c_uint32, C.c_uint32, _u64, C.c_uint32, _i64, _vp, _vp]),
 ]
 
@@ -348,6 +349,21 @@ def svrg_run_host(X, y, loss, lambda_l1, N, B, b, clip_mode, clip_value, seed, S
     if rc != OK:
         raise LpcError(rc, "lpc_svrg_run_host")
     return x, P.value, bits.value
+
+
+def debug_loop_scales(max_bits, S1, S2, length, b, clip_mode, clip_value):
+    """The scale rule of the one-launch loops on CUDA tensors (max_bits int32, sums fp32); see lpc_debug_loop_scales.
+    Returns ((count, 4) fp32: delta, 1 / delta, threshold, lower end; flags int32)."""
+    assert all(t.is_cuda and t.is_contiguous() and t.numel() == S1.numel() for t in (max_bits, S1, S2))
+    assert max_bits.dtype == torch.int32 and S1.dtype == torch.float32 and S2.dtype == torch.float32
+    out = torch.empty((S1.numel(), 4), dtype=torch.float32, device=S1.device)
+    flags = torch.empty(S1.numel(), dtype=torch.int32, device=S1.device)
+    st = torch.cuda.current_stream(S1.device)
+    rc = lib().lpc_debug_loop_scales(_ptr(max_bits), _ptr(S1), _ptr(S2), S1.numel(), length, b, clip_mode, clip_value, _ptr(out),
+                                     _ptr(flags), C.c_void_p(st.cuda_stream))
+    if rc != OK:
+        raise LpcError(rc, "lpc_debug_loop_scales")
+    return out, flags
 
 
 def debug_stream_blocks(seed, tag, worker, k, block0, count, device=None):
