@@ -124,6 +124,32 @@ def test_one_launch_loop_equals_single_steps_with_weights(loss):
     ref.close()
 
 
+@pytest.mark.parametrize("n,d,N,B,b", [(17 * 16, 1000, 17, 3, 4), (32 * 8, 8192, 32, 4, 2), (5 * 32, 516, 5, 2, 3), (8 * 16, 2048, 8, 4, 32)])
+def test_weights_in_the_loop_whose_coordinates_have_owners(n, d, N, B, b):
+    P, ctx = _setup(n, d, "least_squares", N, B, b)
+    ref = lpc.Context(ctx.X, ctx.y, P.loss, P.lambda_l1, P.N, P.B, P.b, P.clip_mode, P.clip_value, P.seed)
+    ref.set_option(lpc.OPT_PERSISTENT, 0)
+    x0 = (np.random.default_rng(5).standard_normal(d) * 0.1).astype(np.float32)
+    for cx in (ctx, ref):
+        cx.set_strong_convexity(0.35)
+        cx.set_iterate(torch.from_numpy(x0).to(DEV))
+        cx.alpc_begin()
+        cx.snapshot_full_grad()
+        for k0, count in ((0, 7), (7, 4)):  # the second call goes on from the seventh weight
+            cx.alpc_double_sample_steps(0.4, 0.5, 0.3, 0.2, k0, count)
+        cx.sync_status()
+    assert ctx.query(lpc.INFO_LOOP_LAUNCHES) == 2 and ctx.query(lpc.INFO_ALPC_LOOP_OWNED) == 1
+    assert ref.query(lpc.INFO_LOOP_LAUNCHES) == 0
+    for w in (lpc.BUF_X, lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_VHAT):
+        assert _same(ctx.get_buffer(w), ref.get_buffer(w)), w
+    for cx in (ctx, ref):
+        cx.alpc_end_epoch(11)
+        cx.sync_status()
+    assert _same(ctx.get_iterate(), ref.get_iterate())
+    ctx.close()
+    ref.close()
+
+
 def test_sigma_zero_is_the_general_convex_path_and_bad_values_are_rejected():
     P, ctx = _setup(256, 128, "least_squares", N=4, B=2, b=4)
     ref = lpc.Context(ctx.X, ctx.y, P.loss, P.lambda_l1, P.N, P.B, P.b, P.clip_mode, P.clip_value, P.seed)

@@ -121,3 +121,38 @@ def test_columns_outside_a_slice_stay_zero_beside_an_infinite_coordinate(n, d, N
     assert x[at] == float("inf") and torch.isfinite(x).sum() == d - 1
     one.close()
     many.close()
+
+
+@pytest.mark.parametrize("alpc", [False, True])
+@pytest.mark.parametrize("n,d,N,b", [(17 * 8, 1000, 17, 4), (33 * 4, 2052, 33, 2), (5 * 16, 512, 5, 3), (4 * 16, 1024, 4, 32)])
+def test_owned_update_with_gradients_that_are_not_finite(n, d, N, b, alpc):
+    # least squares with entries whose products overflow in the rows of one worker: its message is a NaN scale with zero codes (b = 32:
+    # its values), which the proximal step takes to 0, and the loop goes on and ends with the status of single steps
+    X, y, _ = synth.linear_problem(n, d, loss="least_squares", sparsity=0.2, noise=0.1, seed=d + N)
+    rows = n // N
+    X[2 * rows:3 * rows, 5] = 1e25
+    X, y = X.cuda(), y.cuda()
+    x0 = torch.from_numpy((np.random.default_rng(3).standard_normal(d) * 0.1).astype(np.float32)).cuda()
+    count, out = 3, []
+    for persistent in (0, 1):
+        c = lpc.Context(X, y, lpc.LEAST_SQUARES, 1e-5, N, 3, b, lpc.CLIP_STD, 2.0, 11)
+        c.set_option(lpc.OPT_PERSISTENT, persistent)
+        c.set_iterate(x0)
+        if alpc:
+            c.alpc_begin()
+        for w in (lpc.BUF_MARGINS, lpc.BUF_MU):  # the snapshot's own values stay finite
+            c.set_buffer(w, torch.zeros(n if w == lpc.BUF_MARGINS else d, device="cuda"))
+        if alpc:
+            c.alpc_double_sample_steps(0.4, 0.5, 0.3, 0.2, 0, count)
+        else:
+            c.inner_steps(0.05, 0, count)
+        assert c.status() == lpc.ERR_NONFINITE
+        assert c.query(lpc.INFO_LOOP_LAUNCHES) == persistent and (not persistent or c.query(OWN[alpc][1]) == 1)
+        out.append([c.get_buffer(w) for w in (lpc.BUF_X, lpc.BUF_DELTA, lpc.BUF_CODES, lpc.BUF_CLIPPED)])
+        assert c.status() == lpc.OK  # reported once
+        c.close()
+    for a, e in zip(*out):
+        if a.dtype == torch.float32:  # NaNs, and zeros with the sign of one, need not have the same bits
+            assert torch.equal(torch.isnan(a), torch.isnan(e)) and torch.equal(torch.nan_to_num(a, nan=0.0), torch.nan_to_num(e, nan=0.0))
+        else:
+            assert torch.equal(a, e)
