@@ -219,8 +219,10 @@ __device__ __forceinline__ bool std_threshold_single(float S1, float S2, const S
     const float sl = mul_rn(add_rn(__fmaf_rn(-sh, sh, vh), vl), mul_rn(0.5f, y));
     const float th = mul_rn(c, sh), te = add_rn(__fmaf_rn(c, sh, -th), mul_rn(c, sl));
     const float t = add_rn(th, te), low = sub(te, sub(t, th)), d = mul_rn(t, 3.637978807091713e-12f);  // 2^-38
-    T = fminf(t, M);
-    return add_rn(t, add_rn(low, d)) == t && add_rn(t, sub(low, d)) == t;
+    if (add_rn(t, add_rn(low, d)) == t && add_rn(t, sub(low, d)) == t) {
+      T = fminf(t, M);
+      return true;
+    }
   }
   return false;
 }
