@@ -892,12 +892,12 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   const bool cluster = c->last_one_launch && quantize_fits_cluster(a, c->sm_count);
   c->last_pipelined_runs = vec && c->b != 32 && !cluster ? p.whole_runs : 0;
   c->last_quant_launches = cluster ? 1 : quantize_pack_launches(a);
-  c->last_kept_tiles = a.kept_tiles = cluster ? 0 : quantize_kept_tiles(a, p.offsets_x8, c->l2_bytes);
+  c->last_kept_tiles = cluster ? 0 : quantize_kept_tiles(a, p.offsets_x8, c->l2_bytes);
   if (cluster) {
     ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
     CU(c, launch_quantize_cluster(a, c->stream));
   } else {
-    CU(c, launch_quantize_pack(a, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
+    CU(c, launch_quantize_pack(a, c->last_kept_tiles, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
   }
   if (!c->shared_scale) c->step2_bits += p.msg_bits * (uint64_t)c->N * (uint64_t)(c->N - 1);  // scheme (a); the server schemes count in lpc_server_reduce
   return LPC_OK;

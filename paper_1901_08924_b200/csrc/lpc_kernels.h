@@ -69,7 +69,6 @@ struct QuantArgs {
   uint32_t* clipped_out;  // N * nseg, cleared with the scale (never null: internal scratch when the caller gives none)
   int count_clipped;      // 0: skip counting the coordinates outside the hull (the counts stay zero)
   int shared_scale;       // 1: every worker quantizes with delta_t = max_i delta_t^i (schemes (b), (c) of Section 3.2)
-  int kept_tiles;         // tiles at the end that the first look leaves in L2 for the second (quantize_kept_tiles; 0: no cache policy)
   unsigned int* dev_status;
 };
 
@@ -79,9 +78,9 @@ typedef void (*LaunchHook)(void* user, int kind, int begin);
 // segment (the condition, besides 16-byte aligned vectors and a non-degenerate scale, for its pipelined loop).
 int quantize_run_tiles();
 int quantize_pack_launches(const QuantArgs& a);  // kernels that launch_quantize_pack launches
-cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
+cudaError_t launch_quantize_pack(const QuantArgs& a, int kept_tiles, int sm_count, cudaStream_t st, LaunchHook hook = nullptr, void* user = nullptr);
 // The same for short vectors, one cluster per worker and nothing looked at twice.
-// For kept_tiles: offsets_aligned says that every segment's offset is a multiple of 8; l2_bytes is the size of the device's L2.
+// Tiles at the end that the first look leaves in L2 for the second (0: no cache policy).  offsets_aligned says that every segment's offset is a multiple of 8; l2_bytes is the size of the device's L2.
 int quantize_kept_tiles(const QuantArgs& a, bool offsets_aligned, int64_t l2_bytes);
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count);
 cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st);

@@ -109,6 +109,5 @@ extern "C" int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld,
   a.codes = codes_out; a.stride_words = seg.pad_words;
   a.delta_out = delta_out; a.clipped_out = clipped_out; a.count_clipped = 1; a.shared_scale = 0;
   a.dev_status = reinterpret_cast<unsigned int*>(base + OFF_STATUS);
-  a.kept_tiles = quantize_kept_tiles(a, true, l2_bytes);
-  return launch_quantize_pack(a, sm_count, st) == cudaSuccess ? LPC_OK : LPC_ERR_CUDA;
+  return launch_quantize_pack(a, quantize_kept_tiles(a, true, l2_bytes), sm_count, st) == cudaSuccess ? LPC_OK : LPC_ERR_CUDA;
 }

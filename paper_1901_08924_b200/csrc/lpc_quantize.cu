@@ -188,17 +188,17 @@ __device__ __forceinline__ void stats_tile(const QuantArgs& a, int tile, int wor
   }
 }
 
-// POLICY: the second pass goes back from the end, so the tiles worth keeping in L2 are the last a.kept_tiles ones: those before them
+// POLICY: the second pass goes back from the end, so the tiles worth keeping in L2 are the last `keep` ones: those before them
 // are read so that they go first.
 template <bool NEED_SUMS, bool POLICY>
-__global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a) {
+__global__ void __launch_bounds__(QT) stats_kernel(QuantArgs a, int keep) {
   launch_dependents();
   wait_for_launch_before();
   __shared__ float sh1[QITER * 8], sh2[QITER * 8];
   __shared__ uint32_t shm[8];
   uint64_t policy = 0;
   if constexpr (POLICY) {
-    if ((int64_t)blockIdx.y * a.ntiles + blockIdx.x < (int64_t)a.N * a.ntiles - a.kept_tiles)
+    if ((int64_t)blockIdx.y * a.ntiles + blockIdx.x < (int64_t)a.N * a.ntiles - keep)
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     else
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
@@ -910,7 +910,7 @@ int quantize_pack_launches(const QuantArgs& a) {
   return (a.ntiles > 0 ? 3 : 1) + (a.shared_scale ? 1 : 0);  // statistics, scale, codes; nothing but the scale of an empty vector
 }
 
-cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
+cudaError_t launch_quantize_pack(const QuantArgs& a, int kept_tiles, int sm_count, cudaStream_t st, LaunchHook hook, void* user) {
   if (a.N <= 0 || a.nseg <= 0) return cudaSuccess;
   const dim3 grid((unsigned)(a.ntiles > 0 ? a.ntiles : 1), (unsigned)a.N), block(QT);
   auto launch = [&](auto kernel, dim3 g, auto... args) { return launch_overlapped(kernel, g, block, 0, st, a, args...); };
@@ -918,8 +918,8 @@ cudaError_t launch_quantize_pack(const QuantArgs& a, int sm_count, cudaStream_t 
   if (a.ntiles > 0) {
     if (hook) hook(user, 3 /* LPC_KERNEL_QUANT_STATS */, 1);
     const bool sums = a.clip_mode == CLIP_STD;
-    if (a.kept_tiles > 0) e = sums ? launch(stats_kernel<true, true>, grid) : launch(stats_kernel<false, true>, grid);
-    else e = sums ? launch(stats_kernel<true, false>, grid) : launch(stats_kernel<false, false>, grid);
+    if (kept_tiles > 0) e = sums ? launch(stats_kernel<true, true>, grid, kept_tiles) : launch(stats_kernel<false, true>, grid, kept_tiles);
+    else e = sums ? launch(stats_kernel<true, false>, grid, 0) : launch(stats_kernel<false, false>, grid, 0);
     if (hook) hook(user, 3, 0);
     if (e != cudaSuccess) return e;
   }
