@@ -85,7 +85,7 @@ typedef struct lpc_ctx lpc_ctx;
 #define LPC_OPT_SHARED_SCALE 6  /* 1: lpc_quantize_pack gives every worker the unified scale delta_t = max_i delta_t^i of the parameter-server schemes (b), (c) of Section 3.2; needs b in 2..16 */
 #define LPC_OPT_AVERAGE_DIVISOR 7 /* lpc_unpack_average_prox (and only it: the training loops always average over N) divides the decoded sum by this count instead of the context's N (0 = N): the worker count behind a server's sum stream */
 #define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits */
-#define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack may take its short-vector path (one launch where a vector fits a cluster) for inputs of at most LPC_ONE_LAUNCH_BYTES */
+#define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack may take its short-vector path (one launch where a vector fits a cluster) for inputs of at most LPC_ONE_LAUNCH_BYTES, and one launch for many tensors with a subtrahend */
 #define LPC_ONE_LAUNCH_BYTES (48ll << 20)
 #define LPC_OPT_LOOP_COOPERATIVE 9 /* 1 (default): the one-launch loops are cooperative launches (the driver guarantees that all their CTAs are resident together, which they rely on).  0: a plain cluster launch of the same grid, for profilers that cannot replay a cooperative cluster launch; use it only on a GPU that runs nothing else (the launch plan has checked that all clusters fit, and every wait in the kernel is bounded, so a grid that is not resident together ends with LPC_ERR_TIMEOUT instead of hanging) */
 
@@ -183,8 +183,9 @@ int lpc_packed_words(int64_t len, int32_t b, int64_t* words_out); /* ceil(len*b/
  * Vectors longer than L2 are read twice (once for ||u||_inf and the variance, once to quantize) by three launches that overlap;
  * when all N vectors together take at most LPC_ONE_LAUNCH_BYTES the second look is served by L2, and vectors of at most
  * 65,536 values in one segment, with b in {1, 2, 3, 4, 8}, own scales and at most four CTAs per SM in all, take ONE launch, a
- * cluster per worker that keeps the values in registers (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches that off).  Same codes
- * either way; LPC_INFO_QUANT_LAUNCHES says which it was.
+ * cluster per worker that keeps the values in registers.  With U_sub, inputs beyond L2 whose tensors are short against the chip (up to
+ * some 2.4 million values each, on 16-byte boundaries) take ONE launch as well, which reads both inputs once.
+ * (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches both off.)  Same codes either way; LPC_INFO_QUANT_LAUNCHES says which it was.
  * N, b and the clip rule come from the context.
  */
 int lpc_quantize_pack(lpc_ctx* ctx, const float* U, const float* U_sub, int64_t len, int64_t ld,
@@ -301,7 +302,7 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
                                               so took the second pass's software-pipelined loop (unless that worker's scale was
                                               degenerate; short vectors take it in shorter runs); 0 unless every worker's vector starts
                                               on a 16-byte boundary (ld % 4 == 0), for b = 32, and when the call was one launch */
-#define LPC_INFO_QUANT_LAUNCHES 14         /* last lpc_quantize_pack: kernels it launched.  1: a cluster per worker (or an empty vector);
+#define LPC_INFO_QUANT_LAUNCHES 14         /* last lpc_quantize_pack: kernels it launched.  1: a cluster per worker, one look at many tensors (or an empty vector);
                                               3: statistics, scale, codes; 4: the same and the unified scale */
 #define LPC_INFO_LOOP_OWNED 15             /* one-launch loop: 1 when each coordinate's update is made by one CTA, which sends the new
                                               point to the others; 0 when every cluster updates its copy, or loop not available */

@@ -33,6 +33,8 @@ struct SegPlan {
   SegInfo* d_segs = nullptr;
   int32_t* d_tile_seg = nullptr;    // nullptr when nseg == 1
   bool offsets_x8 = true;           // every segment's offset is a multiple of 8
+  bool offsets_x4 = true;           // ... of 4
+  int max_tiles = 0;                // tiles of the longest segment
   uint64_t msg_bits = 0;            // sum over segments of 32 + b*len_s
   int64_t whole_runs = 0;           // runs of 8 tiles that consist of whole tiles of one segment whose offset keeps 16-byte alignment
 };
@@ -114,6 +116,10 @@ struct lpc_ctx {
   ScaleRec* q_scales = nullptr;
   uint32_t* q_clip = nullptr;
   size_t q_scale_cap = 0;
+  ulonglong2* q_partials = nullptr;          // one look at the values: partials of the tiles and, in the same allocation,
+  unsigned long long* q_counts = nullptr;    // the counts of the messages
+  unsigned int* q_epoch = nullptr;           // the call's tag and, behind it, the CTAs that are through
+  size_t q_once_tiles = 0, q_once_messages = 0;
   int loop_cooperative = 1;       // LPC_OPT_LOOP_COOPERATIVE
   int one_launch = 1;             // LPC_OPT_ONE_LAUNCH_QUANTIZE
   int last_one_launch = 0, last_quant_launches = 0, last_kept_tiles = 0;
@@ -228,7 +234,11 @@ int make_plan(lpc_ctx* c, SegPlan& p, int64_t len, int b, const int64_t* seg_off
   p.offsets[nseg] = len;
   p.segs = segs;
   p.tile_seg = tile_seg;
-  for (const SegInfo& g : p.segs) p.offsets_x8 = p.offsets_x8 && g.off % 8 == 0;
+  for (const SegInfo& g : p.segs) {
+    p.offsets_x8 = p.offsets_x8 && g.off % 8 == 0;
+    p.offsets_x4 = p.offsets_x4 && g.off % 4 == 0;
+    p.max_tiles = std::max(p.max_tiles, (int)g.tile_count);
+  }
   const int run = quantize_run_tiles();
   for (int t0 = 0; t0 < p.ntiles; t0 += run) {
     const int t1 = std::min(t0 + run, p.ntiles) - 1;
@@ -258,6 +268,38 @@ int dalloc(lpc_ctx* c, T** p, size_t count) {
   } while (0)
 
 bool has_model(const lpc_ctx* c) { return c->X != nullptr; }
+
+// The scratch of the quantizer's one look: everything starts at zero but the tag, which starts at 1.  False where it cannot be had now: the caller
+// takes the other path (a captured call may need less scratch than the calls before it, but not another kind of it).
+bool once_scratch(lpc_ctx* c, size_t tiles, size_t messages) {
+  if (tiles <= c->q_once_tiles && messages <= c->q_once_messages) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  tiles = std::max(tiles, c->q_once_tiles);
+  messages = std::max(messages, c->q_once_messages);
+  unsigned long long* p = nullptr;
+  if (cudaMalloc(reinterpret_cast<void**>(&p), (tiles * 2 + messages + 1) * 8) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaStreamSynchronize(c->stream);  // the old one may still be in use
+  cudaFree(c->q_partials);
+  c->q_partials = reinterpret_cast<ulonglong2*>(p);
+  c->q_counts = p + tiles * 2;
+  c->q_epoch = reinterpret_cast<unsigned int*>(c->q_counts + messages);
+  c->q_once_tiles = tiles;
+  c->q_once_messages = messages;
+  if (cudaMemsetAsync(p, 0, (tiles * 2 + messages + 1) * 8, c->stream) != cudaSuccess ||
+      cudaMemsetAsync(c->q_epoch, 1, 1, c->stream) != cudaSuccess) {
+    cudaGetLastError();
+    c->q_once_tiles = c->q_once_messages = 0;
+    return false;
+  }
+  return true;
+}
 
 // ---- per-kernel timing ------------------------------------------------------------------------------
 int prof_resolve(lpc_ctx* c) {
@@ -633,7 +675,7 @@ int lpc_destroy(lpc_ctx* c) {
   if (c->graph) cudaGraphExecDestroy(c->graph);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-  void* ptrs[] = {c->arena, c->u_tap, c->q_pmax, c->q_ps1, c->q_ps2, c->q_scales, c->q_clip};
+  void* ptrs[] = {c->arena, c->u_tap, c->q_pmax, c->q_ps1, c->q_ps2, c->q_scales, c->q_clip, c->q_partials};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->coded_host) cudaFreeHost(c->coded_host);
@@ -863,7 +905,13 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
   if (len < 0 || ld < len || nseg < 1) return fail(c, LPC_ERR_INVALID_ARG, "len / ld / nseg");  if (!aligned16(codes_out)) return fail(c, LPC_ERR_INVALID_ARG, "codes_out must be 16-byte aligned");
   TRY(make_plan(c, c->seg, len, c->b, seg_offsets, nseg));
   const SegPlan& p = c->seg;
+  QuantArgs a;
+  a.U = U; a.U_sub = U_sub; a.ld = ld; a.N = c->N; a.b = c->b; a.clip_mode = c->clip_mode; a.clip_value = c->clip_value;
+  a.seed = c->seed; a.k = k; a.segs = p.d_segs; a.tile_seg = p.d_tile_seg; a.nseg = p.nseg; a.ntiles = p.ntiles;
+  a.shared_scale = c->shared_scale;
   const size_t parts = (size_t)c->N * (size_t)std::max(p.ntiles, 1);
+  const bool once = c->one_launch && quantize_takes_one_look(a, len, p.max_tiles, p.offsets_x4, c->sm_count, c->l2_bytes) &&
+                    once_scratch(c, parts, (size_t)c->N * (size_t)nseg);
   if (parts > c->q_part_cap) {
     CU(c, cudaStreamSynchronize(c->stream));
     if (c->q_pmax) { cudaFree(c->q_pmax); cudaFree(c->q_ps1); cudaFree(c->q_ps2); c->q_pmax = nullptr; c->q_ps1 = c->q_ps2 = nullptr; }
@@ -879,23 +927,26 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
     CU(c, cudaMalloc(&c->q_scales, recs * sizeof(ScaleRec))); CU(c, cudaMalloc(&c->q_clip, recs * 4));
     c->q_scale_cap = recs;
   }
-  QuantArgs a;
-  a.U = U; a.U_sub = U_sub; a.ld = ld; a.N = c->N; a.b = c->b; a.clip_mode = c->clip_mode; a.clip_value = c->clip_value;
-  a.seed = c->seed; a.k = k; a.segs = p.d_segs; a.tile_seg = p.d_tile_seg; a.nseg = p.nseg; a.ntiles = p.ntiles;
   a.pmax = c->q_pmax; a.ps1 = c->q_ps1; a.ps2 = c->q_ps2; a.scales = c->q_scales;
   a.codes = codes_out; a.stride_words = p.stride_words; a.delta_out = delta_out;
   a.clipped_out = clipped_out ? clipped_out : c->q_clip; a.count_clipped = clipped_out ? 1 : 0; a.dev_status = c->dev_status;
-  a.shared_scale = c->shared_scale;
   const bool vec = aligned16(U) && (!U_sub || aligned16(U_sub)) && (ld % 4 == 0);
   c->last_one_launch = (c->one_launch && !c->shared_scale && c->b != 32 && p.ntiles > 0 &&
                         (int64_t)c->N * len * 4 * (U_sub ? 2 : 1) <= LPC_ONE_LAUNCH_BYTES) ? 1 : 0;
   const bool cluster = c->last_one_launch && quantize_fits_cluster(a, c->sm_count);
-  c->last_pipelined_runs = vec && c->b != 32 && !cluster ? p.whole_runs : 0;
-  c->last_quant_launches = cluster ? 1 : quantize_pack_launches(a);
-  c->last_kept_tiles = cluster ? 0 : quantize_kept_tiles(a, p.offsets_x8, c->l2_bytes);
+  c->last_pipelined_runs = vec && c->b != 32 && !cluster && !once ? p.whole_runs : 0;
+  c->last_quant_launches = cluster || once ? 1 : quantize_pack_launches(a);
+  c->last_kept_tiles = cluster || once ? 0 : quantize_kept_tiles(a, p.offsets_x8, c->l2_bytes);
   if (cluster) {
     ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
     CU(c, launch_quantize_cluster(a, c->stream));
+  } else if (once) {
+    QuantOnceArgs oa;
+    oa.q = a; oa.partials = c->q_partials; oa.counts = c->q_counts; oa.epoch = c->q_epoch; oa.done = c->q_epoch + 1;
+    const ScaleRule rule = scale_rule(len, c->b);
+    oa.levels = rule.levels; oa.inv_levels = rule.inv_levels;
+    ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
+    CU(c, launch_quantize_once(oa, c->sm_count, c->stream));
   } else {
     CU(c, launch_quantize_pack(a, c->last_kept_tiles, c->sm_count, c->stream, c->profile ? prof_hook : nullptr, c));
   }

@@ -85,6 +85,19 @@ int quantize_kept_tiles(const QuantArgs& a, bool offsets_aligned, int64_t l2_byt
 bool quantize_fits_cluster(const QuantArgs& a, int sm_count);
 cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st);
 
+// One look at the values for many messages with a subtrahend (lpc_quantize_once.cu).
+struct QuantOnceArgs {
+  QuantArgs q;                // pmax, ps1, ps2 and scales are not used
+  ulonglong2* partials;       // one per tile of every worker, zero before the first call: max |u|, S1, S2 and the call's tag
+  unsigned long long* counts; // N * nseg, zero between calls
+  unsigned int* epoch;        // the call's tag: 1 before the first call, moved on by each
+  unsigned int* done;         // zero between calls
+  float levels, inv_levels;   // as in ScaleRule
+};
+// Whether a call takes that path.  max_tiles: tiles of the longest message; offsets_x4: every segment's offset is a multiple of 4.
+bool quantize_takes_one_look(const QuantArgs& a, int64_t len, int max_tiles, bool offsets_x4, int sm_count, int64_t l2_bytes);
+cudaError_t launch_quantize_once(const QuantOnceArgs& oa, int sm_count, cudaStream_t st);
+
 struct AggArgs {
   const uint32_t* codes;
   int64_t stride_words;
