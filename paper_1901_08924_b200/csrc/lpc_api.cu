@@ -444,7 +444,11 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     return kind == 0 ? enqueue_lpc_step(c, p[0], kb, kd, kc, overlapped) : enqueue_alpc_step(c, p[0], p[1], p[2], p[3], kb, kd, kc, overlapped);
   };
   int64_t done = 0;
-  const bool loop_ok = (kind == 0) ? c->persist_ok : c->apersist_ok;
+  // A captured launch is replayed with the tags it was captured with, and would take the words of the replay before for its own: in a
+  // capture of the caller's the steps are plain launches.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
+  const bool loop_ok = ((kind == 0) ? c->persist_ok : c->apersist_ok) && !capturing;
   // the strongly convex ALPC step carries a weight that changes from step to step: plain per-step launches
   const bool weighted = (kind == 1 && c->sigma > 0.f);
   if (c->use_persist && loop_ok && count >= 2 && count <= 0x7FFFFFFF) {
@@ -497,7 +501,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
       if (kind == 0) c->persist_ok = false; else c->apersist_ok = false;
     }
   }
-  if (done < count && c->use_graph && !c->profile && !weighted && count >= GRAPH_STEPS) {
+  if (done < count && c->use_graph && !c->profile && !weighted && !capturing && count >= GRAPH_STEPS) {
     GraphKey key;
     key.kind = kind; key.steps = GRAPH_STEPS; key.tap = c->tap_u; key.cs = c->CS; key.sample_global = c->sample_global;
     for (int i = 0; i < 4; ++i) key.p[i] = p[i];
