@@ -77,14 +77,14 @@ typedef struct lpc_ctx lpc_ctx;
 
 /* options for lpc_set_option */
 #define LPC_OPT_SAMPLE_GLOBAL 0 /* 0 (default): worker i samples its own block of n/N rows; 1: all n rows (the paper's shared-storage setting, Section 2.1) */
-#define LPC_OPT_TAP_U 1         /* 1: inner steps also store u^i and v for inspection (slower) */
+#define LPC_OPT_TAP_U 1         /* 1: inner steps also store u^i and v for inspection (slower; the loop for minibatches of more than 64 rows is off meanwhile) */
 #define LPC_OPT_CLUSTER_SIZE 2  /* thread-block cluster size per worker for the fused step: 0 = automatic, else 1, 2, 4 or 8 */
 #define LPC_OPT_USE_GRAPH 3     /* 1 (default): lpc_inner_steps replays a CUDA graph; 0: plain launches */
-#define LPC_OPT_PROFILE 4       /* 1: record CUDA events around every kernel launch (graph replay is off meanwhile) */
+#define LPC_OPT_PROFILE 4       /* 1: record CUDA events around every kernel launch (graph replay and the loop for minibatches of more than 64 rows are off meanwhile) */
 
 #define LPC_OPT_SHARED_SCALE 6  /* 1: lpc_quantize_pack gives every worker the unified scale delta_t = max_i delta_t^i of the parameter-server schemes (b), (c) of Section 3.2; needs b in 2..16 */
 #define LPC_OPT_AVERAGE_DIVISOR 7 /* lpc_unpack_average_prox (and only it: the training loops always average over N) divides the decoded sum by this count instead of the context's N (0 = N): the worker count behind a server's sum stream */
-#define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits */
+#define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits: rows resident in shared memory (up to 64 per worker), or streaming through it (up to 256) */
 #define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack may take its short-vector path (one launch where a vector fits a cluster) for inputs of at most LPC_ONE_LAUNCH_BYTES, and one launch for many tensors with a subtrahend */
 #define LPC_ONE_LAUNCH_BYTES (48ll << 20)
 #define LPC_OPT_LOOP_COOPERATIVE 9 /* 1 (default): the one-launch loops are cooperative launches (the driver guarantees that all their CTAs are resident together, which they rely on).  0: a plain cluster launch of the same grid, for profilers that cannot replay a cooperative cluster launch; use it only on a GPU that runs nothing else (the launch plan has checked that all clusters fit, and every wait in the kernel is bounded, so a grid that is not resident together ends with LPC_ERR_TIMEOUT instead of hanging) */

@@ -93,6 +93,8 @@ struct lpc_ctx {
   bool persist_ok = false, apersist_ok = false;  // Algorithm 1 loop / Algorithm 2 loop
   int pCS = 1, pSL = 0, pSlots = 0, pOwn = 0, aCS = 1, aSL = 0, aSlots = 0, aOwn = 0;  // cluster size, slice, row slots, owned update of the two loops
   size_t persistSmem = 0, apersistSmem = 0;
+  // the loops whose rows stream: Algorithm 1, Algorithm 2
+  struct StreamLoop { bool planned = false, ok = false; int CS = 1, SL = 0, stages = 0; size_t smem = 0; } sloop[2];
   // exchange buffers of the one-launch loops: tagged 64-bit words (payload | tag << 32), two step-parity halves
   unsigned long long* flags = nullptr;    // scale words: 2 x 256, 128 bytes apart, + 1 abort word
   unsigned long long* ll = nullptr;       // code words: 2 x N x dpow2/8 groups x ll_wpg
@@ -159,6 +161,11 @@ int fail(lpc_ctx* c, int code, const std::string& msg) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 int64_t roundup4(int64_t v) { return (v + 3) & ~(int64_t)3; }
+int loop_coords(int d) {  // coordinates that the loops' exchange buffers cover: slices of a power of two, 128 at least
+  int p = 128;
+  while (p < d) p <<= 1;
+  return p;
+}
 bool valid_b(int b) { return (b >= 1 && b <= 16) || b == 32; }
 
 __global__ void set_u64_kernel(uint64_t* p, uint64_t v) { *p = v; }
@@ -392,6 +399,7 @@ int replan_inner(lpc_ctx* c) {
   if (c->persist_ok) { c->pCS = cs; c->pSL = sl; c->persistSmem = smem; c->pSlots = slots; c->pOwn = own; }
   c->apersist_ok = persist_plan(c->d, c->N, c->B, c->b, 1, c->want_cs, c->max_smem, &cs, &sl, &smem, &slots, &own);
   if (c->apersist_ok) { c->aCS = cs; c->aSL = sl; c->apersistSmem = smem; c->aSlots = slots; c->aOwn = own; }
+  c->sloop[0].planned = c->sloop[1].planned = false;
   return LPC_OK;
 }
 
@@ -444,11 +452,19 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     return kind == 0 ? enqueue_lpc_step(c, p[0], kb, kd, kc, overlapped) : enqueue_alpc_step(c, p[0], p[1], p[2], p[3], kb, kd, kc, overlapped);
   };
   int64_t done = 0;
+  const bool small_ok = (kind == 0) ? c->persist_ok : c->apersist_ok;
+  // large minibatches: where nobody looks at u and v or times the launches of a step one by one
+  lpc_ctx::StreamLoop& sl = c->sloop[kind];
+  if (!small_ok && !sl.planned) {  // planned when it is first needed: few contexts use it, and with one of the algorithms
+    sl.planned = true;
+    sl.ok = c->want_cs == 0 && stream_loop_plan(c->d, c->N, c->B, c->b, kind, c->max_smem, c->sm_count, &sl.CS, &sl.SL, &sl.smem, &sl.stages);
+  }
+  const bool stream_ok = !small_ok && sl.ok && !c->tap_u && !c->profile && count <= (1 << 24);
   // A captured launch is replayed with the tags it was captured with, and would take the words of the replay before for its own: in a
   // capture of the caller's the steps are plain launches.
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
-  const bool loop_ok = ((kind == 0) ? c->persist_ok : c->apersist_ok) && !capturing;
+  const bool loop_ok = (small_ok || stream_ok) && !capturing;
   // the strongly convex ALPC step carries a weight that changes from step to step: plain per-step launches
   const bool weighted = (kind == 1 && c->sigma > 0.f);
   if (c->use_persist && loop_ok && count >= 2 && count <= 0x7FFFFFFF) {
@@ -457,15 +473,15 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     pa.in = inner_args(c, k0, nullptr, 0);
     pa.rule = scale_rule(c->d, c->b);
     pa.own = kind == 0 ? c->pOwn : c->aOwn;
-    pa.in.CS = kind == 0 ? c->pCS : c->aCS;
-    pa.in.SL = kind == 0 ? c->pSL : c->aSL;
+    pa.in.CS = stream_ok ? sl.CS : kind == 0 ? c->pCS : c->aCS;
+    pa.in.SL = stream_ok ? sl.SL : kind == 0 ? c->pSL : c->aSL;
+    pa.in.stream_stages = stream_ok ? sl.stages : 0;
     pa.row_slots = kind == 0 ? c->pSlots : c->aSlots;
     pa.count = (int)count; pa.eta = kind == 0 ? p[0] : 0.f; pa.lambda_l1 = c->lambda_l1;
     pa.pub = c->flags; pa.abort_flag = reinterpret_cast<unsigned int*>(c->flags + 512 * 16); pa.x_out = c->x;
     pa.ll = c->ll; pa.ll_vhat = c->ll_vhat; pa.ll_x = c->ll_x; pa.wpg = c->ll_wpg;
     if ((uint64_t)c->ll_tag + (uint64_t)count >= 0xFFFFFFF0ull) {  // tags would wrap: start over from cleared buffers
-      int dp = 32;
-      while (dp < c->d) dp <<= 1;
+      const int dp = loop_coords(c->d);
       CU(c, cudaMemsetAsync(c->flags, 0, (512 * 16 + 1) * sizeof(unsigned long long), c->stream));
       CU(c, cudaMemsetAsync(c->ll, 0, sizeof(unsigned long long) * 2 * (size_t)c->N * (size_t)(dp / 8) * c->ll_wpg, c->stream));
       CU(c, cudaMemsetAsync(c->ll_vhat, 0, sizeof(unsigned long long) * 2 * (size_t)dp, c->stream));
@@ -484,7 +500,8 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     }
     CU(c, cudaMemsetAsync(pa.abort_flag, 0, sizeof(unsigned long long), c->stream));
     cudaError_t e;
-    { ProfScope ps_(c, LPC_KERNEL_INNER_LOOP); e = launch_persist(pa, kind == 0 ? c->persistSmem : c->apersistSmem, c->stream, c->loop_cooperative != 0); }
+    { ProfScope ps_(c, LPC_KERNEL_INNER_LOOP); e = stream_ok ? launch_stream_loop(pa, sl.smem, c->stream, c->loop_cooperative != 0)
+                    : launch_persist(pa, kind == 0 ? c->persistSmem : c->apersistSmem, c->stream, c->loop_cooperative != 0); }
     if (e == cudaSuccess) {
       done = count;
       if (weighted) {  // the weights the loop went through, and the one the next step starts from
@@ -498,7 +515,9 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
       c->ll_tag += (uint32_t)count;
     } else {
       cudaGetLastError();  // clear the refusal and use the per-step path
-      if (kind == 0) c->persist_ok = false; else c->apersist_ok = false;
+      if (stream_ok) sl.ok = false;
+      else if (kind == 0) c->persist_ok = false;
+      else c->apersist_ok = false;
     }
   }
   if (done < count && c->use_graph && !c->profile && !weighted && !capturing && count >= GRAPH_STEPS) {
@@ -647,8 +666,7 @@ int lpc_init(lpc_ctx** out, const float* X, const float* y, int64_t n, int32_t d
     want(&c->clipped, (size_t)N);
     want(&c->clipped_part, (size_t)N * inner_clipped_stride());
     want(&c->flags, 512 * 16 + 1);
-    int dp = 32;
-    while (dp < d) dp <<= 1;
+    const int dp = loop_coords(d);
     c->ll_wpg = (b <= 4) ? 1 : (b <= 8) ? 2 : (b <= 16) ? 4 : 8;
     want(&c->ll, 2 * (size_t)N * (size_t)(dp / 8) * c->ll_wpg);
     want(&c->ll_vhat, 2 * (size_t)dp);

@@ -80,6 +80,10 @@ int persist_coords_per_thread(int b, int SL);
 // cooperative = false drops the launch attribute that makes the driver guarantee co-residency of the grid (the plan has
 // checked that all clusters fit; the kernel's waits are bounded): for profilers that cannot replay cooperative launches.
 cudaError_t launch_persist(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative = true);
+// The same with rows that stream, up to 256 per worker (lpc_stream_loop.cu): in.CS CTAs per cluster, as many as there are slices of in.SL
+// columns, and in.stream_stages ring stages; own, ll_x, row_slots, v_tap and in.u_tap are not used.
+bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out);
+cudaError_t launch_stream_loop(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative = true);
 // One small kernel whose bounded waits (an mbarrier phase; a tagged word when `word` is given) run out after limit_ns.
 cudaError_t launch_wait_timeout(const unsigned long long* word, unsigned int* abort_flag, unsigned int* dev_status,
                                 uint64_t limit_ns, cudaStream_t st);
