@@ -121,6 +121,7 @@ def stream_table(args, dev, torch, lpc, synth):
                                    device=dev)
     ctx = lpc.Context(X, y, lpc.LOGISTIC, 1e-5, N, B, b, lpc.CLIP_STD, 2.0, 0)
     ctx.snapshot_full_grad()
+    ctx.set_option(lpc.OPT_PERSISTENT, 0)  # the per-step kernel's marks
     ctx.inner_steps(1e-3, 0, 5)
     ctx.set_option(lpc.OPT_PROFILE, 1)
     ctx.inner_steps(1e-3, 5, 10)
