@@ -455,7 +455,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
   const bool small_ok = (kind == 0) ? c->persist_ok : c->apersist_ok;
   // large minibatches: where nobody looks at u and v or times the launches of a step one by one
   lpc_ctx::StreamLoop& sl = c->sloop[kind];
-  if (!small_ok && !sl.planned) {  // planned when it is first needed: few contexts use it, and with one of the algorithms
+  if (!small_ok && !sl.planned && c->use_persist && count >= 2) {  // planned when it is first needed: few contexts use it, and with one of the algorithms
     sl.planned = true;
     sl.ok = c->want_cs == 0 && stream_loop_plan(c->d, c->N, c->B, c->b, kind, c->max_smem, c->sm_count, &sl.CS, &sl.SL, &sl.smem, &sl.stages);
   }
