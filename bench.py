@@ -564,14 +564,15 @@ def quantize_aggregate_bench(dev, peak, log2_len=26, full=True):
     ta = _kernel_ms(q, lambda i: q.unpack_average_prox(codes[i % 2], delta, total, xs[i % 4], 0.1, 0.0, mu=mu, seg_offsets=offs), 20,
                     ("aggregate",))["aggregate"]
     q.sync_status()
-    bq, ba = N * total * (16 + b / 8), total * (N * b / 8 + 16)  # aggregate: codes + mu + x read + x write
+    one_look = q.query(lpc.INFO_QUANT_LAUNCHES) == 1
+    bq, ba = N * total * ((8 if one_look else 16) + b / 8), total * (N * b / 8 + 16)  # aggregate: codes + mu + x read + x write
     res["dnn_62_tensors_N16_b4"] = {
         "quantize_pack": {"ms": round(tq, 4), "bytes": bq, "gbs": round(bq / tq * 1e-6, 1), "frac": round(bq / tq * 1e-6 / peak, 4),
-                          "note": "u = cur - snap formed on the fly: 2 x 8 B read + b/8 B written per element"},
+                          "note": "u = cur - snap formed on the fly: %d x 8 B read + b/8 B written per element" % (1 if one_look else 2)},
         "unpack_average_prox": {"ms": round(ta, 4), "bytes": ba, "gbs": round(ba / ta * 1e-6, 1), "frac": round(ba / ta * 1e-6 / peak, 4)},
         "combined_gbs": round((bq + ba) / (tq + ta) * 1e-6, 1)}
     wl = "62 tensors of an 18-layer residual network, 11.7M parameters, N=16, b=4, clip 2.5 std per tensor"
-    roof.append(roofline_entry("quantize+pack with u = cur - snap (3 launches)", wl, tq * 1e3, bq, peak, short="quantize 62 tensors"))
+    roof.append(roofline_entry("quantize+pack with u = cur - snap (%s)" % ("quantize_once_kernel<4>" if one_look else "3 launches"), wl, tq * 1e3, bq, peak, short="quantize 62 tensors"))
     roof.append(roofline_entry("unpack_average_prox_kernel<4> (+ mu)", wl, ta * 1e3, ba, peak, short="aggregate 62 tensors"))
     q.close()
     res["roofline_kernels"] = roof
