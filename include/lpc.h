@@ -379,6 +379,15 @@ int lpc_debug_loop_scales(const uint32_t* max_bits, const float* S1, const float
                           int clip_mode, float clip_value, float* scale_out, uint32_t* flags_out, void* stream);
 
 /*
+ * Inspection aid for the launch plan of the one-launch loop whose rows stream; it needs no device.  For d features, N workers, B rows each,
+ * Algorithm 2 (alpc != 0) or 1, smem_bytes of shared memory per CTA and sm_count SMs: *ctas_out = CTAs per worker with slices of `slice`
+ * columns (a power of two, 128 .. 2,048), 0 where the plan does not take such slices; *room_out = coordinates that the buffers
+ * through which the loop's CTAs exchange codes and points have room for (a context allocates them for d).
+ */
+int lpc_debug_stream_loop_slices(int32_t d, int32_t N, int32_t B, int32_t alpc, int32_t smem_bytes, int32_t sm_count, int32_t slice,
+                                 int32_t* ctas_out, int32_t* room_out);
+
+/*
  * Inspection aid: writes `count` consecutive 4-word blocks, starting at block `block0`, of the
  * counter-based random stream (tag, worker, k) keyed by `seed` to out (device, 4*count words).
  * The streams are Philox4x32-10 (Salmon et al., SC'11) with counter (block, k_lo, worker | tag<<24,

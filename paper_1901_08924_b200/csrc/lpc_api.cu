@@ -161,11 +161,6 @@ int fail(lpc_ctx* c, int code, const std::string& msg) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 int64_t roundup4(int64_t v) { return (v + 3) & ~(int64_t)3; }
-int loop_coords(int d) {  // coordinates that the loops' exchange buffers cover: slices of a power of two, 128 at least
-  int p = 128;
-  while (p < d) p <<= 1;
-  return p;
-}
 bool valid_b(int b) { return (b >= 1 && b <= 16) || b == 32; }
 
 __global__ void set_u64_kernel(uint64_t* p, uint64_t v) { *p = v; }
@@ -514,10 +509,11 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
       c->clipped_ctas = pa.in.CS;
       c->ll_tag += (uint32_t)count;
     } else {
-      cudaGetLastError();  // clear the refusal and use the per-step path
-      if (stream_ok) sl.ok = false;
-      else if (kind == 0) c->persist_ok = false;
+      cudaGetLastError();  // clear the refusal and use the per-step path, from now on: the loop whose rows stream does not step in for the other one
+      if (kind == 0) c->persist_ok = false;
       else c->apersist_ok = false;
+      sl.planned = true;
+      sl.ok = false;
     }
   }
   if (done < count && c->use_graph && !c->profile && !weighted && !capturing && count >= GRAPH_STEPS) {
@@ -1092,6 +1088,17 @@ int lpc_debug_loop_scales(const uint32_t* max_bits, const float* S1, const float
   const cudaError_t e = launch_loop_scales(max_bits, S1, S2, count, scale_rule(len, b), b, clip_mode, clip_value,
                                            reinterpret_cast<float4*>(scale_out), flags_out, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? LPC_OK : LPC_ERR_CUDA;
+}
+
+int lpc_debug_stream_loop_slices(int32_t d, int32_t N, int32_t B, int32_t alpc, int32_t smem_bytes, int32_t sm_count, int32_t slice, int32_t* ctas_out,
+                                 int32_t* room_out) {
+  if (d < 4 || (d & 3) || N < 1 || B < 1 || smem_bytes < 0 || sm_count < 1 || !ctas_out || !room_out) return LPC_ERR_INVALID_ARG;
+  if (slice < 128 || slice > 2048 || (slice & (slice - 1))) return LPC_ERR_INVALID_ARG;
+  int cs = 0, stages = 0;
+  size_t smem = 0;
+  *ctas_out = stream_loop_slices(d, N, B, alpc ? 1 : 0, smem_bytes, sm_count, slice, &cs, &smem, &stages) ? cs : 0;
+  *room_out = loop_coords(d);
+  return LPC_OK;
 }
 
 int lpc_debug_stream_blocks(uint64_t seed, uint32_t tag, uint32_t worker, uint64_t k, uint32_t block0, int64_t count,

@@ -80,8 +80,16 @@ int persist_coords_per_thread(int b, int SL);
 // cooperative = false drops the launch attribute that makes the driver guarantee co-residency of the grid (the plan has
 // checked that all clusters fit; the kernel's waits are bounded): for profilers that cannot replay cooperative launches.
 cudaError_t launch_persist(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative = true);
+// Coordinates that the loops' exchange buffers have room for: slices of a power of two, 128 at least.
+inline int loop_coords(int d) {
+  int p = 128;
+  while (p < d) p <<= 1;
+  return p;
+}
 // The same with rows that stream, up to 256 per worker (lpc_stream_loop.cu): in.CS CTAs per cluster, as many as there are slices of in.SL
 // columns, and in.stream_stages ring stages; own, ll_x, row_slots, v_tap and in.u_tap are not used.
+// stream_loop_slices is the part of the plan that asks no device: whether slices of SL columns are possible at all.
+bool stream_loop_slices(int d, int N, int B, int alpc, int max_smem, int sm_count, int SL, int* CS_out, size_t* smem_out, int* stages_out);
 bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out);
 cudaError_t launch_stream_loop(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative = true);
 // One small kernel whose bounded waits (an mbarrier phase; a tagged word when `word` is given) run out after limit_ns.

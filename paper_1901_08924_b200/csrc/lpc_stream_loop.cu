@@ -824,21 +824,28 @@ void loop_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int cs, int
 // as there are slices with columns.  us per step with slices of 128, 256, 512, 1,024 and 2,048 columns: d = 752, N = 8, B = 256 9.4, 11.7, 15.9,
 // 25.7, 37.3; d = 128, N = 2, B = 256 8.4, 10.9, 13.9, 22.9, 36.2; d = 1,000, N = 4, B = 100 7.2, 8.4, 10.1, 14.7, 18.6; d = 8,192, N = 8, B = 100 with
 // 1,024 and 2,048 14.5, 19.4.
-bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out) {
+bool stream_loop_slices(int d, int N, int B, int alpc, int max_smem, int sm_count, int SL, int* CS_out, size_t* smem_out, int* stages_out) {
   if (B > LMAXB || N > LMAXN || d > 2048 * LCS) return false;
-  const int clusters = N + (alpc ? 1 : 0);
-  const size_t meta = (size_t)((B + 3) & ~3) * 2 * 16 + sizeof(LSmem);
+  if (SL > loop_coords(d)) return false;  // few rows rule the narrow slices out, but the exchange buffers end where the vector's power of two does
+  const int cs = (d + SL - 1) / SL;
+  if (cs > LCS || (N + (alpc ? 1 : 0)) * cs > std::min(LFLAGS, sm_count)) return false;  // one CTA per SM
+  const LoopShape s = loop_shape(SL);
+  if (B <= 2 * s.rows) return false;  // a step has three groups at least: both sides of the margins and both coefficient warps take part in it
+  const size_t fixed = (size_t)SL * 4 * (alpc ? 5 : 2) + s.part * cs + (size_t)((B + 3) & ~3) * 2 * 16 + sizeof(LSmem);
+  if (fixed + 3 * s.stage > (size_t)max_smem) return false;
+  const int R = (int)(((size_t)max_smem - fixed) / s.stage);
+  // as in the per-step kernel: of a peer's u a CTA is at most 2 R + 3 groups ahead, which has to stay below the exchange slots
+  *stages_out = std::min(R, cs > 1 ? (LSLOTS - 4) / 2 : LMAXR);
+  *CS_out = cs;
+  *smem_out = fixed + (size_t)*stages_out * s.stage;
+  return true;
+}
+
+bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out) {
   for (int SL = 128; SL <= 2048; SL *= 2) {
-    const int cs = (d + SL - 1) / SL;
-    if (cs > LCS || clusters * cs > std::min(LFLAGS, sm_count)) continue;  // one CTA per SM
-    const LoopShape s = loop_shape(SL);
-    if (B <= 2 * s.rows) continue;  // a step has three groups at least: both sides of the margins and both coefficient warps take part in it
-    const size_t fixed = (size_t)SL * 4 * (alpc ? 5 : 2) + s.part * cs + meta;
-    if (fixed + 3 * s.stage > (size_t)max_smem) continue;
-    int R = (int)(((size_t)max_smem - fixed) / s.stage);
-    // as in the per-step kernel: of a peer's u a CTA is at most 2 R + 3 groups ahead, which has to stay below the exchange slots
-    R = std::min(R, cs > 1 ? (LSLOTS - 4) / 2 : LMAXR);
-    const size_t smem = fixed + (size_t)R * s.stage;
+    int cs = 0, R = 0;
+    size_t smem = 0;
+    if (!stream_loop_slices(d, N, B, alpc, max_smem, sm_count, SL, &cs, &smem, &R)) continue;
     LoopKernel k = pick_loop(b, SL, alpc != 0);
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       cudaGetLastError();
@@ -846,13 +853,13 @@ bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    loop_config(&cfg, attr, cs, 1, s.threads, smem, nullptr, false);
+    loop_config(&cfg, attr, cs, 1, loop_shape(SL).threads, smem, nullptr, false);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
-    if (n < clusters) continue;
+    if (n < N + (alpc ? 1 : 0)) continue;
     *CS_out = cs; *SL_out = SL; *smem_out = smem; *stages_out = R;
     return true;
   }

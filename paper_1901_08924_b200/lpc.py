@@ -67,6 +67,7 @@ SYMBOLS = [
     ("lpc_quantize_pack_static", _int, [_vp, _i64, _i64, _i32, _i32, _int, _f32, _u64, _u64, _vp, _vp, _vp, _vp]),
     ("lpc_debug_wait_timeout", _int, [_vp, _u64]),
     ("lpc_debug_loop_scales", _int, [_vp, _vp, _vp, _i64, _i64, _i32, _int, _f32, _vp, _vp, _vp]),
+    ("lpc_debug_stream_loop_slices", _int, [_i32, _i32, _i32, _i32, _i32, _i32, _i32, C.POINTER(_i32), C.POINTER(_i32)]),
     ("lpc_debug_stream_blocks", _int, [_u64, C.c_uint32, C.c_uint32, _u64, C.c_uint32, _i64, _vp, _vp]),
 ]
 
@@ -364,6 +365,16 @@ def debug_loop_scales(max_bits, S1, S2, length, b, clip_mode, clip_value):
     if rc != OK:
         raise LpcError(rc, "lpc_debug_loop_scales")
     return out, flags
+
+
+def debug_stream_loop_slices(d, N, B, alpc, smem_bytes, sm_count, slice_columns):
+    """CTAs per worker that the streaming loop's plan gives slices of this width (0: not taken), and the coordinates that the exchange
+    buffers have room for (see lpc_debug_stream_loop_slices); needs no device."""
+    ctas, room = C.c_int32(0), C.c_int32(0)
+    rc = lib().lpc_debug_stream_loop_slices(d, N, B, alpc, smem_bytes, sm_count, slice_columns, C.byref(ctas), C.byref(room))
+    if rc != OK:
+        raise LpcError(rc)
+    return ctas.value, room.value
 
 
 def debug_stream_blocks(seed, tag, worker, k, block0, count, device=None):
