@@ -72,7 +72,6 @@ struct lpc_ctx {
   uint32_t* codes = nullptr;
   float* delta = nullptr;
   uint32_t *clipped_part = nullptr, *clipped = nullptr;
-  int clipped_ctas = 0;  // CTAs per worker whose counts of the last step are in clipped_part
   int64_t* idx_tap = nullptr;
   float* coef_tap = nullptr;
   uint64_t* k_dev = nullptr;
@@ -405,7 +404,6 @@ constexpr int GRAPH_STEPS = 128;  // inner steps per captured graph
 int enqueue_lpc_step(lpc_ctx* c, float eta, uint64_t k_base, const uint64_t* k_dev, uint64_t* k_counter, bool overlapped) {
   InnerArgs ia = inner_args(c, k_base, k_dev, 0);
   ia.overlapped = overlapped ? 1 : 0;
-  c->clipped_ctas = c->CS;
   { ProfScope ps_(c, LPC_KERNEL_WORKER); CU(c, launch_inner(ia, c->innerSmem, c->stream)); }
   // the training loops always average over the context's N workers (Eq. 3); LPC_OPT_AVERAGE_DIVISOR does not apply
   AggArgs ag = agg_args(c, c->inner_seg, c->codes, c->delta, c->mu, c->x, eta, c->lambda_l1, c->tap_u ? c->v_tap : nullptr, c->N);
@@ -420,7 +418,6 @@ int enqueue_alpc_step(lpc_ctx* c, float tau1, float tau2, float alpha, float inv
   { ProfScope ps_(c, LPC_KERNEL_OTHER); CU(c, launch_coupling(c->zv, c->xt, c->yv, tau1, tau2, c->d, c->x, c->stream)); }
   InnerArgs ia = inner_args(c, k_base, k_dev, 1);
   ia.overlapped = overlapped ? 1 : 0;
-  c->clipped_ctas = c->CS;
   { ProfScope ps_(c, LPC_KERNEL_WORKER); CU(c, launch_inner(ia, c->innerSmem, c->stream)); }
   AggArgs ag = agg_args(c, c->inner_seg, c->codes, c->delta, c->mu, c->x, 0.f, c->lambda_l1, c->tap_u ? c->v_tap : nullptr, c->N);
   ag.k_counter = k_counter; ag.k_step = GRAPH_STEPS;
@@ -506,7 +503,6 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
         }
       }
       c->persist_launches += 1;
-      c->clipped_ctas = pa.in.CS;
       c->ll_tag += (uint32_t)count;
     } else {
       cudaGetLastError();  // clear the refusal and use the per-step path, from now on: the loop whose rows stream does not step in for the other one
@@ -542,8 +538,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
     }
     set_u64_kernel<<<1, 1, 0, c->stream>>>(c->k_dev, k0);
     CU(c, cudaGetLastError());
-    c->clipped_ctas = c->CS;
-    while (count - done >= GRAPH_STEPS) {
+      while (count - done >= GRAPH_STEPS) {
       CU(c, cudaGraphLaunch(c->graph, c->stream));
       done += GRAPH_STEPS;
     }
@@ -763,7 +758,7 @@ int lpc_get_buffer(lpc_ctx* c, int which, void* dst, size_t bytes) {
   if (!has_model(c)) return fail(c, LPC_ERR_UNSUPPORTED, "quantizer-only context");
   void* p = nullptr;
   size_t cap = 0;
-  if (which == LPC_BUF_CLIPPED) CU(c, launch_clipped_sum(c->clipped_part, c->N, c->clipped_ctas, c->clipped, c->stream));
+  if (which == LPC_BUF_CLIPPED) CU(c, launch_clipped_sum(c->clipped_part, c->N, c->clipped, c->stream));
   const int rc = buffer_of(c, which, &p, &cap);
   if (rc != LPC_OK) return fail(c, rc, "buffer not available");
   if (bytes > cap) return fail(c, LPC_ERR_INVALID_ARG, "bytes exceed the buffer");

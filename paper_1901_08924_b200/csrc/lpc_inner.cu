@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
   if (tid == 0) {
     uint32_t t = 0;
     for (int w = 0; w < 8; ++w) t += sm.wclip[w];
-    a.clipped_part[worker * MAXCS + rank] = t;
+    put_clipped<MAXCS>(a.clipped_part + worker * MAXCS, rank, CS, t);
   }
   LPC_PHASE_MARK(7);
   wait_to_leave();
@@ -838,11 +838,11 @@ cudaError_t launch_t(const InnerArgs& a, size_t smem, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, inner_kernel<BITS, STREAM>, a);
 }
 
-__global__ void clipped_sum_kernel(const uint32_t* __restrict__ part, int N, int ctas, uint32_t* __restrict__ out) {
+__global__ void clipped_sum_kernel(const uint32_t* __restrict__ part, int N, uint32_t* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) {
     uint32_t t = 0;
-    for (int q = 0; q < ctas; ++q) t += part[i * MAXCS + q];
+    for (int q = 0; q < MAXCS; ++q) t += part[i * MAXCS + q];
     out[i] = t;
   }
 }
@@ -932,8 +932,8 @@ cudaError_t read_stream_trace(unsigned long long* host_out) {  // TRACE_CTAS x 8
 }
 #endif
 
-cudaError_t launch_clipped_sum(const uint32_t* part, int N, int ctas, uint32_t* out, cudaStream_t st) {
-  clipped_sum_kernel<<<(N + 127) / 128, 128, 0, st>>>(part, N, ctas, out);
+cudaError_t launch_clipped_sum(const uint32_t* part, int N, uint32_t* out, cudaStream_t st) {
+  clipped_sum_kernel<<<(N + 127) / 128, 128, 0, st>>>(part, N, out);
   return cudaGetLastError();
 }
 

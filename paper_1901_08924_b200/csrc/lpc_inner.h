@@ -100,7 +100,7 @@ int inner_max_b();
 int inner_clipped_stride();
 bool inner_plan(int d, int B, int want_cs, int max_smem, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out);
 cudaError_t launch_inner(const InnerArgs& a, size_t smem, cudaStream_t st);
-cudaError_t launch_clipped_sum(const uint32_t* part, int N, int ctas, uint32_t* out, cudaStream_t st);
+cudaError_t launch_clipped_sum(const uint32_t* part, int N, uint32_t* out, cudaStream_t st);
 cudaError_t launch_coupling(const float* z, const float* xt, const float* y, float tau1, float tau2, int d, float* x,
                             cudaStream_t st);
 cudaError_t launch_mean_y(float* ysum, float inv_m, int d, float* x, cudaStream_t st);
