@@ -369,6 +369,13 @@ int lpc_quantize_pack_static(const float* U, int64_t len, int64_t ld, int32_t N,
 int lpc_debug_wait_timeout(lpc_ctx* ctx, uint64_t limit_ns);
 
 /*
+ * Inspection aid for the same path inside lpc_quantize_pack's one look at many tensors: in the next such launch of the context the first CTA
+ * goes no further than `tiles` of its tiles, as after a wait that ran out.  That call's outputs are incomplete and the next lpc_sync_status
+ * returns LPC_ERR_TIMEOUT; the calls after it are as good as ever.  Calls that take another path leave the request standing.
+ */
+int lpc_debug_one_look_stop(lpc_ctx* ctx, int32_t tiles);
+
+/*
  * Inspection aid for the scale rule (Eq. 2 and its c * std form) of the one-launch loops, which forms the threshold in single precision
  * with an interval around it and leaves what that does not decide to doubles, the definition.  For i < count, from max_bits[i] (the bit
  * pattern of max |u|), S1[i] and S2[i] (the sums of u and u^2; device) of vectors of len values in b bits: scale_out (device) takes

@@ -122,6 +122,7 @@ struct lpc_ctx {
   unsigned long long* q_counts = nullptr;    // the counts of the messages
   unsigned int* q_epoch = nullptr;           // the call's tag and, behind it, the CTAs that are through
   size_t q_once_tiles = 0, q_once_messages = 0;
+  int q_once_stop = -1;                      // lpc_debug_one_look_stop, for the next launch
   int loop_cooperative = 1;       // LPC_OPT_LOOP_COOPERATIVE
   int one_launch = 1;             // LPC_OPT_ONE_LAUNCH_QUANTIZE
   int last_one_launch = 0, last_quant_launches = 0, last_kept_tiles = 0;
@@ -963,6 +964,8 @@ int lpc_quantize_pack(lpc_ctx* c, const float* U, const float* U_sub, int64_t le
     oa.q = a; oa.partials = c->q_partials; oa.counts = c->q_counts; oa.epoch = c->q_epoch; oa.done = c->q_epoch + 1;
     const ScaleRule rule = scale_rule(len, c->b);
     oa.levels = rule.levels; oa.inv_levels = rule.inv_levels;
+    oa.stop_at = c->q_once_stop;
+    c->q_once_stop = -1;
     ProfScope ps_(c, LPC_KERNEL_QUANT_FUSED);
     CU(c, launch_quantize_once(oa, c->sm_count, c->stream));
   } else {
@@ -1072,6 +1075,13 @@ int lpc_debug_wait_timeout(lpc_ctx* c, uint64_t limit_ns) {
   unsigned int* abort_flag = c->flags ? reinterpret_cast<unsigned int*>(c->flags + 512 * 16) : nullptr;
   if (abort_flag) CU(c, cudaMemsetAsync(abort_flag, 0, sizeof(unsigned long long), c->stream));
   CU(c, launch_wait_timeout(c->flags, abort_flag, c->dev_status, limit_ns, c->stream));
+  return LPC_OK;
+}
+
+int lpc_debug_one_look_stop(lpc_ctx* c, int32_t tiles) {
+  if (!c) return LPC_ERR_INVALID_ARG;
+  if (tiles < 0) return fail(c, LPC_ERR_INVALID_ARG, "tiles < 0");
+  c->q_once_stop = tiles;
   return LPC_OK;
 }
 

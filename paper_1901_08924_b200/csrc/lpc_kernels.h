@@ -93,6 +93,7 @@ struct QuantOnceArgs {
   unsigned int* epoch;        // the call's tag: 1 before the first call, moved on by each
   unsigned int* done;         // zero between calls
   float levels, inv_levels;   // as in ScaleRule
+  int stop_at;                // -1; else CTA 0 goes no further than this many tiles, as after a wait that ran out
 };
 // Whether a call takes that path.  max_tiles: tiles of the longest message; offsets_x4: every segment's offset is a multiple of 4.
 bool quantize_takes_one_look(const QuantArgs& a, int64_t len, int max_tiles, bool offsets_x4, int sm_count, int64_t l2_bytes);

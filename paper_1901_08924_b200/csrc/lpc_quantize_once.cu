@@ -134,12 +134,20 @@ __device__ __noinline__ ulonglong2 zero_group(int b, int valid) {  // a group of
   for (int e = min(8, valid) - 1; e >= 0 && b > 1; --e) push_code(lo, hi, 1u << (b - 1), b);
   return make_ulonglong2(lo, hi);
 }
-// Out of line, so that the code that every warp walks through stays small.  After one wait ran out nobody waits any more (the status word
-// says so).
-__device__ __noinline__ void slow_wait(uint64_t* bar, uint32_t parity, volatile int* failed, unsigned int* dev_status) {
-  if (*failed || mbar_wait(bar, parity)) return;
+__device__ __forceinline__ void give_up(volatile int* failed, unsigned int* dev_status) {
   atomicOr(dev_status, DEV_TIMEOUT);
+  __threadfence();  // the CTA that ends the launch sees it: it counts this one among those that are through
   *failed = 1;
+}
+// Out of line, so that the code that every warp walks through stays small.  False: this wait or another one of the CTA ran out (the status
+// word says so).  Whoever gets that goes no further: what it waited for, pointers among it, may never have been written.
+__device__ __noinline__ bool slow_wait(uint64_t* bar, uint32_t parity, volatile int* failed, unsigned int* dev_status) {
+  for (int i = 0; i < 200; ++i) {  // two seconds; the CTA's other waits end within a hundredth of one
+    if (*failed) return false;
+    if (mbar_wait(bar, parity, 10000000ull)) return true;
+  }
+  give_up(failed, dev_status);
+  return false;
 }
 
 __device__ __forceinline__ void lds_pairs(const float* s, f32x2& a, f32x2& b) {
@@ -179,8 +187,12 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
   }
   __syncthreads();
   const uint32_t tag = sm.tag;
-  auto wait_on = [&](uint64_t* bar, uint32_t parity) {
-    if (!mbar_test(bar, parity)) slow_wait(bar, parity, &sm.failed, a.dev_status);
+  auto lane_waits = [&](uint64_t* bar, uint32_t parity) {  // one thread
+    return mbar_test(bar, parity) || slow_wait(bar, parity, &sm.failed, a.dev_status);
+  };
+  auto warp_waits = [&](uint64_t* bar, uint32_t parity) {  // a whole warp, which goes on together or not at all
+    if (__all_sync(0xFFFFFFFFu, mbar_test(bar, parity))) return true;
+    return (bool)__all_sync(0xFFFFFFFFu, slow_wait(bar, parity, &sm.failed, a.dev_status));
   };
   auto parity_of = [](int i) { return (uint32_t)((i / SLOTS) & 1); };
 
@@ -205,7 +217,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
     auto statistics = [&](const Place& at) {
       const int s = at.s, own = at.part * UNIT + lane * 8;  // this thread's groups: `own` and own + 256
       float* slot = slots + (size_t)s * TILE;
-      wait_on(&sm.known[s], at.parity);
+      if (!warp_waits(&sm.known[s], at.parity)) return false;
       const int valid = sm.info[s].valid;
       f32x2 qv[2][4];
       const float* q = sm.info[s].q;
@@ -217,7 +229,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
           ldg_pairs(q + j + (4 - first), qv[h][2], qv[h][3]);
         }
       }
-      wait_on(&sm.full[s], at.parity);
+      if (!warp_waits(&sm.full[s], at.parity)) return false;
       float mx = 0.f;
       f32x2 pr[2];
 #pragma unroll
@@ -255,11 +267,12 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
       if (lane == 0) sm.mx[s][at.part] = m;
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.summed[s]);
+      return true;
     };
     auto codes = [&](const Place& at) {
       const int s = at.s, own = at.part * UNIT + lane * 8;
       float* slot = slots + (size_t)s * TILE;
-      wait_on(&sm.scaled[s], at.parity);
+      if (!warp_waits(&sm.scaled[s], at.parity)) return false;
       const TileInfo& t = sm.info[s];
       const ScaleRec sc = sm.scale[s];
       const int valid = t.valid, words = t.words, b = BITS ? BITS : a.b;
@@ -330,19 +343,20 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
         if (nclip) atomicAdd(&sm.clip[s], nclip);
         mbar_arrive(&sm.coded[s]);
       }
+      return true;
     };
     Place now = {warp / UNITS, warp % UNITS, warp / UNITS, 0u}, then = now;
     int behind = LAG;
 #pragma unroll 1
     while (then.i < n) {
       if (now.i < n) {
-        statistics(now);
+        if (!statistics(now)) break;
         now.advance();
       }
       if (behind > 0) {
         --behind;
       } else {
-        codes(then);
+        if (!codes(then)) break;
         then.advance();
       }
     }
@@ -372,6 +386,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
         return t;
       };
       TileInfo next = describe();
+      int issued = 0;
 #pragma unroll 1
       for (int i = 0; i < n; ++i) {
         const int s = i % SLOTS;
@@ -380,20 +395,20 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
           w.advance(G, a.ntiles);
           next = describe();
         }
-        if (i >= SLOTS) wait_on(&sm.empty[s], parity_of(i - SLOTS));
-        if (*(volatile int*)&sm.failed) break;
+        if (i == oa.stop_at && blockIdx.x == 0) {  // inspection of what follows a wait that ran out
+          give_up(&sm.failed, a.dev_status);
+          break;
+        }
+        if (i >= SLOTS && !lane_waits(&sm.empty[s], parity_of(i - SLOTS))) break;
         sm.info[s] = t;
         mbar_arrive(&sm.known[s]);
         const uint32_t bytes = (uint32_t)(t.valid & ~3) * 4u;  // a ragged end of less than 16 bytes is read by whoever needs it
         mbar_expect_tx(&sm.full[s], bytes);
         if (bytes) bulk_load(slots + (size_t)s * TILE, t.p, bytes, &sm.full[s]);
+        issued = i + 1;
       }
-      if (*(volatile int*)&sm.failed) {  // the copies on their way get a bounded chance to land before this CTA leaves
-        const int issued = min(n, SLOTS);
-        for (int s = 0; s < issued; ++s) mbar_wait(&sm.full[s], 0u, 10000000ull);
-        const uint64_t t0 = global_ns();
-        while (global_ns() - t0 < 1000000ull) __nanosleep(1000);
-      }
+      // no CTA leaves with copies on their way: they have all landed where nothing failed, and get a bounded chance where something did
+      for (int i = max(0, issued - SLOTS); i < issued; ++i) mbar_wait(&sm.full[i % SLOTS], parity_of(i), 100000000ull);
     }
   } else if (warp == W_PUBLISH) {
     // ---- a tile's partials to whoever needs them ---------------------------------------------------------------------
@@ -408,7 +423,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int s = i % SLOTS;
-      wait_on(&sm.summed[s], parity_of(i));
+      if (!warp_waits(&sm.summed[s], parity_of(i))) break;
       float s1 = SUMS ? sm.s1[s][lane & (UNITS - 1)] : 0.f, s2 = SUMS ? sm.s2[s][lane & (UNITS - 1)] : 0.f;
       const uint32_t m = warp_max_u32(sm.mx[s][lane & (UNITS - 1)]);
       if constexpr (SUMS) {
@@ -440,7 +455,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
         const ulonglong2* from = oa.partials + (int64_t)w.worker * a.ntiles + g.tile_first;
         // Nobody looks at other CTAs' partials before this CTA's are out, nor at all of them before the last tile's are there: looks that
         // come too early keep L2 busy.
-        wait_on(&sm.summed[s], parity_of(i));
+        if (!warp_waits(&sm.summed[s], parity_of(i))) break;
         {
           uint64_t since = 0;
 #pragma unroll 1
@@ -521,7 +536,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
           if (sc.flags & 2u) atomicOr(a.dev_status, DEV_NONFINITE);
         }
       }
-      wait_on(&sm.known[s], parity_of(i));  // the slot is this tile's: nobody reads the scale of the one before any more
+      if (!warp_waits(&sm.known[s], parity_of(i))) break;  // the slot is this tile's: nobody reads the scale of the one before any more
       if (lane == 0) {
         sm.scale[s] = rec;
         mbar_arrive(&sm.scaled[s]);
@@ -545,7 +560,7 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int s = i % SLOTS;
-      wait_on(&sm.coded[s], parity_of(i));
+      if (!lane_waits(&sm.coded[s], parity_of(i))) break;
       const int m = sm.info[s].msg, t = sm.info[s].tiles;
       const uint32_t c = sm.clip[s];
       sm.clip[s] = 0u;

@@ -66,6 +66,7 @@ SYMBOLS = [
                                  _f32, _vp, _f64p, _u64p]),
     ("lpc_quantize_pack_static", _int, [_vp, _i64, _i64, _i32, _i32, _int, _f32, _u64, _u64, _vp, _vp, _vp, _vp]),
     ("lpc_debug_wait_timeout", _int, [_vp, _u64]),
+    ("lpc_debug_one_look_stop", _int, [_vp, _i32]),
     ("lpc_debug_loop_scales", _int, [_vp, _vp, _vp, _i64, _i64, _i32, _int, _f32, _vp, _vp, _vp]),
     ("lpc_debug_stream_loop_slices", _int, [_i32, _i32, _i32, _i32, _i32, _i32, _i32, C.POINTER(_i32), C.POINTER(_i32)]),
     ("lpc_debug_stream_blocks", _int, [_u64, C.c_uint32, C.c_uint32, _u64, C.c_uint32, _i64, _vp, _vp]),
@@ -331,6 +332,10 @@ class Context:
     def debug_wait_timeout(self, limit_ns):
         """Enqueues a kernel whose bounded waits run out after limit_ns (see lpc_debug_wait_timeout)."""
         self._ck(lib().lpc_debug_wait_timeout(self._h, limit_ns))
+
+    def debug_one_look_stop(self, tiles):
+        """The next one-look launch stops short in its first CTA (see lpc_debug_one_look_stop)."""
+        self._ck(lib().lpc_debug_one_look_stop(self._h, tiles))
 
     def comm_bits(self):
         a, b = C.c_uint64(0), C.c_uint64(0)
