@@ -89,7 +89,7 @@ cudaError_t launch_quantize_cluster(const QuantArgs& a, cudaStream_t st);
 struct QuantOnceArgs {
   QuantArgs q;                // pmax, ps1, ps2 and scales are not used
   ulonglong2* partials;       // one per tile of every worker, zero before the first call: max |u|, S1, S2 and the call's tag
-  unsigned long long* counts; // N * nseg, zero between calls
+  unsigned long long* counts; // N * nseg, zero between calls (also after one whose waits ran out)
   unsigned int* epoch;        // the call's tag: 1 before the first call, moved on by each
   unsigned int* done;         // zero between calls
   float levels, inv_levels;   // as in ScaleRule

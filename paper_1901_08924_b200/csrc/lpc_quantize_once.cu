@@ -575,7 +575,13 @@ __global__ void __launch_bounds__(OT, 1) quantize_once_kernel(QuantOnceArgs oa) 
     flush();
     // the last CTA of the grid moves the tag on
     __threadfence();
-    if (atomicInc(oa.done, (unsigned)G - 1u) == (unsigned)G - 1u) *oa.epoch = tag == 0xFFFFFFFFu ? 1u : tag + 1u;
+    if (atomicInc(oa.done, (unsigned)G - 1u) == (unsigned)G - 1u) {
+      __threadfence();
+      // where a wait ran out tiles are missing from some messages' counters, which the next call would go on from
+      if (*(volatile unsigned int*)a.dev_status & DEV_TIMEOUT)
+        for (int m = 0; m < a.N * a.nseg; ++m) oa.counts[m] = 0ull;
+      *oa.epoch = tag == 0xFFFFFFFFu ? 1u : tag + 1u;
+    }
   }
 }
 
