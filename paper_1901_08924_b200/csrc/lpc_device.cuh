@@ -731,13 +731,9 @@ __device__ __forceinline__ int64_t next_pow2_i64(int64_t n) {
   return p;
 }
 
-// The count of clipped coordinates of CTA `rank` of a worker's `ctas`, in the worker's SLOTS places.  The sum takes all of them, so the places
-// that a launch has no CTA for are cleared by the launch itself: a host variable would follow what was enqueued or captured, not what ran.
-template <int SLOTS>
-__device__ __forceinline__ void put_clipped(uint32_t* places, int rank, int ctas, uint32_t count) {
-  places[rank] = count;
-  for (int q = rank + ctas; q < SLOTS; q += ctas) places[q] = 0u;
-}
+// A CTA's count of clipped coordinates, and above it how many CTAs its worker has in this launch: the sum takes that many.  (A host variable
+// would follow what was enqueued or captured, not what ran.)
+__device__ __forceinline__ uint32_t clipped_word(uint32_t count, int ctas) { return count | ((uint32_t)ctas << 24); }
 
 // ---- losses ----------------------------------------------------------------------------------------------
 constexpr int LOSS_LOGISTIC = 0, LOSS_LEAST_SQUARES = 1;

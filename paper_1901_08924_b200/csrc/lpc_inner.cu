@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(STREAM ? SNT : IT) inner_kernel(InnerArgs a) {
   if (tid == 0) {
     uint32_t t = 0;
     for (int w = 0; w < 8; ++w) t += sm.wclip[w];
-    put_clipped<MAXCS>(a.clipped_part + worker * MAXCS, rank, CS, t);
+    a.clipped_part[worker * MAXCS + rank] = clipped_word(t, CS);
   }
   LPC_PHASE_MARK(7);
   wait_to_leave();
@@ -842,7 +842,8 @@ __global__ void clipped_sum_kernel(const uint32_t* __restrict__ part, int N, uin
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) {
     uint32_t t = 0;
-    for (int q = 0; q < MAXCS; ++q) t += part[i * MAXCS + q];
+    const int ctas = (int)(part[i * MAXCS] >> 24);  // 0 before the first step
+    for (int q = 0; q < ctas; ++q) t += part[i * MAXCS + q] & 0xFFFFFFu;
     out[i] = t;
   }
 }

@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(PT, 1) persist_kernel(PersistArgs pa) {
       if (tid == 0) {
         uint32_t tc = 0;
         for (int w = 0; w < 8; ++w) tc += sm.wclip[w];
-        put_clipped<PMAXCS>(a.clipped_part + worker * PMAXCS, rank, CS, tc);
+        a.clipped_part[worker * PMAXCS + rank] = clipped_word(tc, CS);
       }
     }
     LPC_TRACE_MARK(14);

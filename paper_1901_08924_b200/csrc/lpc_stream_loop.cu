@@ -275,7 +275,7 @@ __device__ __forceinline__ void end_of_step(const PersistArgs& pa, float* ring, 
       if (tu == 0) {
         uint32_t n = 0;
         for (int w = 0; w < DW; ++w) n += sm.wclip[w];
-        put_clipped<LCS>(a.clipped_part + worker * LCS, rank, CW, n);
+        a.clipped_part[worker * LCS + rank] = clipped_word(n, CW);
       }
     }
   }
