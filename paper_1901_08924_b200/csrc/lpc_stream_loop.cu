@@ -107,7 +107,6 @@ __device__ __forceinline__ void end_of_step(const PersistArgs& pa, float* ring, 
   const float invN = __fdiv_rn(1.0f, (float)N), invB = __fdiv_rn(1.0f, (float)a.B);
   const float kappa = mul_rn(pa.eta, pa.lambda_l1), kappa_y = mul_rn(pa.inv4L, pa.lambda_l1), kappa_z = mul_rn(pa.alpha, pa.lambda_l1);
   constexpr int WPG = BITS == 0 ? 8 : (BITS == 8 ? 2 : 1);  // tagged words per group of 8 coordinates, at most
-  constexpr int CH = BITS == 0 ? 4 : 16 / WPG;              // workers per round of loads
   const int wpg = BITS == 0 ? pa.wpg : WPG;
   const size_t groups = (size_t)(CW * SL) >> 3;
   auto expired = [&](uint32_t it, uint64_t& t0) -> bool {
@@ -295,57 +294,73 @@ __device__ __forceinline__ void end_of_step(const PersistArgs& pa, float* ring, 
   }
   const unsigned long long* dwords = pa.pub + ((size_t)wpar * LFLAGS + rank) * LPUB;
   const unsigned long long* from = pa.ll + ((size_t)wpar * N * groups + (mine ? (size_t)(c >> 3) : (size_t)(c0 >> 3))) * wpg;
-  const unsigned long long good = (unsigned long long)tag << 32;
+  // one round: the words of `CHW` workers, W each, and their scales in flight together; add(worker of the round, its scale, its words)
+  auto rounds = [&](auto words, auto per_round, auto&& add) {
+    constexpr int W = decltype(words)::value, CHW = decltype(per_round)::value;
 #pragma unroll 1
-  for (int i0 = 0; i0 < N; i0 += CH) {
-    unsigned long long cw[CH][WPG], dw;
-    uint64_t t0 = 0;
-    const int his = i0 + (lane & (CH - 1));  // the worker whose scale this lane fetches
+    for (int i0 = 0; i0 < N; i0 += CHW) {
+      unsigned long long cw[CHW][W], dw;
+      uint64_t t0 = 0;
+      const int his = i0 + (lane & (CHW - 1));  // the worker whose scale this lane fetches
 #pragma unroll 1
-    for (uint32_t it = 0;; ++it) {
-      dw = ld_word(dwords + (size_t)min(his, N - 1) * CW * LPUB);
-      bool ok = word_tag(dw) == tag;
+      for (uint32_t it = 0;; ++it) {
+        dw = ld_word(dwords + (size_t)min(his, N - 1) * CW * LPUB);
+        bool ok = word_tag(dw) == tag;
 #pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        const unsigned long long* q = from + (size_t)min(i0 + j, N - 1) * groups * wpg;
-        if constexpr (BITS == 8) {
-          ld_word2(q, cw[j][0], cw[j][1]);
-        } else {
+        for (int j = 0; j < CHW; ++j) ld_words<W>(from + (size_t)min(i0 + j, N - 1) * groups * W, cw[j]);
 #pragma unroll
-          for (int w = 0; w < WPG; ++w) cw[j][w] = w < wpg ? ld_word(q + w) : good;
-        }
+        for (int j = 0; j < CHW; ++j)
+#pragma unroll
+          for (int w = 0; w < W; ++w) ok = ok && word_tag(cw[j][w]) == tag;
+        if (__all_sync(0xFFFFFFFFu, ok) || __any_sync(0xFFFFFFFFu, expired(it, t0))) break;
       }
+      const uint32_t dmine = his < N ? (uint32_t)dw : 0u;
 #pragma unroll
-      for (int j = 0; j < CH; ++j)
-#pragma unroll
-        for (int w = 0; w < WPG; ++w) ok = ok && word_tag(cw[j][w]) == tag;
-      if (__all_sync(0xFFFFFFFFu, ok) || __any_sync(0xFFFFFFFFu, expired(it, t0))) break;
+      for (int j = 0; j < CHW; ++j) {
+        const float di = __uint_as_float(__shfl_sync(0xFFFFFFFFu, dmine, j));
+        if (i0 + j < N) add(di, cw[j]);
+      }
     }
-    const uint32_t dmine = his < N ? (uint32_t)dw : 0u;
+  };
+  if constexpr (BITS != 0) {
+    rounds(std::integral_constant<int, WPG>(), std::integral_constant<int, 16 / WPG>(), [&](float di, const unsigned long long (&cw)[WPG]) {
+      uint64_t l = (uint32_t)cw[0];
+      if constexpr (WPG >= 2) l |= (uint64_t)(uint32_t)cw[1] << 32;
+      f32x2 k2[4];
+      decode_pairs<BITS ? BITS : 1, 8>(l, k2);
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      const float di = __uint_as_float(__shfl_sync(0xFFFFFFFFu, dmine, j));
-      if (b == 32) {
-        if (i0 + j < N) {
+      for (int e = 0; e < 4; ++e) acc2[e] = add_scaled_pair<BITS>(acc2[e], pack2(di, di), k2[e]);
+    });
+  } else {
+    // The width decides how many words a group has.  One loop for all widths fetched eight words of four workers one by one: every sector came
+    // once per word, and values spilled.  Sixteen words a round in whole accesses, us per step before / after: b = 12, 32 workers, d = 2,432,
+    // B = 128 43.7 / 36.7; b = 16, 16 workers, d = 4,896, B = 100 30.8 / 26.6; b = 32, 16 workers, d = 5,156, B = 200 53.0 / 40.7; b = 32, 32 workers,
+    // d = 4,000, B = 66 40.5 / 26.5.  Tried: the step's end as a function of its own (1.17 to 1.33 times as long), the snapshot gradient and the old
+    // point read after the rounds (fewer spills, 0.95 to 1.05 times).
+    const uint32_t mask = b < 32 ? (1u << b) - 1u : 0u;
+    auto add_index = [&](int e, float di, uint32_t code) { acc[e] = add_scaled_index<0>(acc[e], di, index_as_float(code, b)); };
+    if (wpg == 1) {
+      rounds(std::integral_constant<int, 1>(), std::integral_constant<int, 16>(), [&](float di, const unsigned long long (&cw)[1]) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] = add_rn(acc[e], mul_rn(di, c + e < d ? __uint_as_float((uint32_t)cw[j][e < WPG ? e : 0]) : 0.f));
-        }
-      } else {
-        uint64_t l = (uint32_t)cw[j][0], h = 0;
-        if constexpr (WPG >= 2) l |= (uint64_t)(uint32_t)cw[j][1] << 32;
-        if constexpr (WPG >= 4) h = (uint64_t)(uint32_t)cw[j][2] | ((uint64_t)(uint32_t)cw[j][3] << 32);
-        if constexpr (BITS == 0) {
-          if (i0 + j < N) {
+        for (int e = 0; e < 8; ++e) add_index(e, di, ((uint32_t)cw[0] >> (e * b)) & mask);
+      });
+    } else if (wpg == 2) {
+      rounds(std::integral_constant<int, 2>(), std::integral_constant<int, 8>(), [&](float di, const unsigned long long (&cw)[2]) {
+        const uint64_t l = (uint32_t)cw[0] | (uint64_t)(uint32_t)cw[1] << 32;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = add_scaled_index<0>(acc[e], di, index_as_float(extract_bits(l, h, e * b, b), b));
-          }
-        } else if (i0 + j < N) {
-          f32x2 k2[4];
-          decode_pairs<BITS ? BITS : 1, 8>(l, k2);
+        for (int e = 0; e < 8; ++e) add_index(e, di, (uint32_t)(l >> (e * b)) & mask);
+      });
+    } else if (wpg == 4) {
+      rounds(std::integral_constant<int, 4>(), std::integral_constant<int, 4>(), [&](float di, const unsigned long long (&cw)[4]) {
+        const uint64_t l = (uint32_t)cw[0] | (uint64_t)(uint32_t)cw[1] << 32, h = (uint32_t)cw[2] | (uint64_t)(uint32_t)cw[3] << 32;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc2[e] = add_scaled_pair<BITS>(acc2[e], pack2(di, di), k2[e]);
-        }
-      }
+        for (int e = 0; e < 8; ++e) add_index(e, di, extract_bits(l, h, e * b, b));
+      });
+    } else {
+      rounds(std::integral_constant<int, 8>(), std::integral_constant<int, 2>(), [&](float di, const unsigned long long (&cw)[8]) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = add_rn(acc[e], mul_rn(di, c + e < d ? __uint_as_float((uint32_t)cw[e]) : 0.f));
+      });
     }
   }
   if constexpr (BITS != 0) {

@@ -20,6 +20,21 @@ __device__ __forceinline__ uint32_t word_tag(unsigned long long w) { return (uin
 __device__ __forceinline__ void ld_word2(const unsigned long long* p, unsigned long long& w0, unsigned long long& w1) {
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
 }
+// W words from p on (8 W bytes, up to 32 at a time; p aligned to them): words of one thread that are fetched one by one touch each sector once
+// per word.
+template <int W>
+__device__ __forceinline__ void ld_words(const unsigned long long* p, unsigned long long (&w)[W]) {
+  static_assert(W == 1 || W == 2 || W == 4 || W == 8, "whole accesses");
+  if constexpr (W == 1) {
+    w[0] = ld_word(p);
+  } else if constexpr (W == 2) {
+    ld_word2(p, w[0], w[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < W; i += 4)
+      asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(w[i]), "=l"(w[i + 1]), "=l"(w[i + 2]), "=l"(w[i + 3]) : "l"(p + i) : "memory");
+  }
+}
 __device__ __forceinline__ void st_word2(unsigned long long* p, uint32_t payload0, uint32_t payload1, uint32_t tag) {
   const unsigned long long v0 = (unsigned long long)payload0 | ((unsigned long long)tag << 32);
   const unsigned long long v1 = (unsigned long long)payload1 | ((unsigned long long)tag << 32);
