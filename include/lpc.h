@@ -309,6 +309,9 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
 #define LPC_INFO_ALPC_LOOP_OWNED 16        /* the same for the loop of Algorithm 2 */
 #define LPC_INFO_QUANT_KEPT_TILES 17       /* last lpc_quantize_pack: tiles of 8192 values at the end of the input that the first look left in
                                               L2 for the second while it let the others go; 0: its loads carried no cache policy */
+#define LPC_INFO_STREAM_LOOP_SLICE 18      /* the one-launch loop whose rows stream: columns per CTA (CTAs per worker: d over that, rounded up); 0 where the loop is not
+                                              available and before the first call that could use it, which plans it */
+#define LPC_INFO_ALPC_STREAM_LOOP_SLICE 19 /* the same for the loop of Algorithm 2 */
 int lpc_query(const lpc_ctx* ctx, int what, int64_t* out);
 
 /* Per-kernel device time measured with CUDA events on the context's stream while LPC_OPT_PROFILE is

@@ -450,7 +450,9 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
   lpc_ctx::StreamLoop& sl = c->sloop[kind];
   if (!small_ok && !sl.planned && c->use_persist && count >= 2) {  // planned when it is first needed: few contexts use it, and with one of the algorithms
     sl.planned = true;
-    sl.ok = c->want_cs == 0 && stream_loop_plan(c->d, c->N, c->B, c->b, kind, c->max_smem, c->sm_count, &sl.CS, &sl.SL, &sl.smem, &sl.stages);
+    const int at_once = inner_clusters_at_once(c->CS, c->innerSmem, c->innerStages, c->max_smem), clusters = c->N + kind;
+    sl.ok = c->want_cs == 0 && stream_loop_plan(c->d, c->N, c->B, c->b, kind, c->max_smem, c->sm_count, c->innerStages == 0,
+                                                at_once > 0 ? (clusters + at_once - 1) / at_once : 1, &sl.CS, &sl.SL, &sl.smem, &sl.stages);
   }
   const bool stream_ok = !small_ok && sl.ok && !c->tap_u && !c->profile && count <= (1 << 24);
   // A captured launch is replayed with the tags it was captured with, and would take the words of the replay before for its own: in a
@@ -886,6 +888,8 @@ int lpc_query(const lpc_ctx* c, int what, int64_t* out) {
     case LPC_INFO_ALPC_LOOP_COORDS_PER_THREAD: *out = c->apersist_ok ? persist_coords_per_thread(c->b, c->aSL) : 0; return LPC_OK;
     case LPC_INFO_LOOP_OWNED: *out = c->persist_ok ? c->pOwn : 0; return LPC_OK;
     case LPC_INFO_ALPC_LOOP_OWNED: *out = c->apersist_ok ? c->aOwn : 0; return LPC_OK;
+    case LPC_INFO_STREAM_LOOP_SLICE: *out = c->sloop[0].planned && c->sloop[0].ok ? c->sloop[0].SL : 0; return LPC_OK;
+    case LPC_INFO_ALPC_STREAM_LOOP_SLICE: *out = c->sloop[1].planned && c->sloop[1].ok ? c->sloop[1].SL : 0; return LPC_OK;
     case LPC_INFO_STEP_RING_STAGES: *out = c->inner_ok ? c->innerStages : 0; return LPC_OK;
     case LPC_INFO_LOOP_LAUNCHES: *out = c->persist_launches; return LPC_OK;
     case LPC_INFO_SNAPSHOT_ROWS_PER_TILE: *out = c->snapR; return LPC_OK;

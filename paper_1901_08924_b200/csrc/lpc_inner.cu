@@ -923,6 +923,28 @@ cudaError_t launch_s(const InnerArgs& a, size_t smem, cudaStream_t st) {
   }
 }
 
+int inner_clusters_at_once(int CS, size_t smem, int stages, int max_smem) {  // any width stands for all: shared memory and threads decide
+  auto* k = stages > 0 ? inner_kernel<4, true> : inner_kernel<4, false>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)CS, 1, 1);
+  cfg.blockDim = dim3(stages > 0 ? SNT : IT, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)CS;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  // up to the most that a plan uses: launch_t counts on an attribute that is never lowered
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 cudaError_t launch_inner(const InnerArgs& a, size_t smem, cudaStream_t st) {
   return a.stream_stages > 0 ? launch_s<true>(a, smem, st) : launch_s<false>(a, smem, st);
 }

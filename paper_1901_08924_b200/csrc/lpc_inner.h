@@ -90,7 +90,10 @@ inline int loop_coords(int d) {
 // columns, and in.stream_stages ring stages; own, ll_x, row_slots, v_tap and in.u_tap are not used.
 // stream_loop_slices is the part of the plan that asks no device: whether slices of SL columns are possible at all.
 bool stream_loop_slices(int d, int N, int B, int alpc, int max_smem, int sm_count, int SL, int* CS_out, size_t* smem_out, int* stages_out);
-bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out);
+// single_resident, single_waves: whether the per-step kernel keeps the rows resident, and how many times its clusters fill the device.
+bool stream_loop_pays(int b, int N, int B, int alpc, int CS, int SL, bool single_resident, int single_waves);
+bool stream_loop_plan(int d, int N, int B, int b, int alpc, int max_smem, int sm_count, bool single_resident, int single_waves, int* CS_out, int* SL_out,
+                      size_t* smem_out, int* stages_out);
 cudaError_t launch_stream_loop(const PersistArgs& pa, size_t smem, cudaStream_t st, bool cooperative = true);
 // One small kernel whose bounded waits (an mbarrier phase; a tagged word when `word` is given) run out after limit_ns.
 cudaError_t launch_wait_timeout(const unsigned long long* word, unsigned int* abort_flag, unsigned int* dev_status,
@@ -100,6 +103,7 @@ int inner_max_b();
 int inner_clipped_stride();
 bool inner_plan(int d, int B, int want_cs, int max_smem, int* CS_out, int* SL_out, size_t* smem_out, int* stages_out);
 cudaError_t launch_inner(const InnerArgs& a, size_t smem, cudaStream_t st);
+int inner_clusters_at_once(int CS, size_t smem, int stages, int max_smem);  // clusters of that kernel that fit on the device together; 0: not known
 cudaError_t launch_clipped_sum(const uint32_t* part, int N, uint32_t* out, cudaStream_t st);
 cudaError_t launch_coupling(const float* z, const float* xt, const float* y, float tau1, float tau2, int d, float* x,
                             cudaStream_t st);

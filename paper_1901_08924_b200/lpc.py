@@ -26,7 +26,7 @@ SCHEME_BROADCAST, SCHEME_SERVER_SUM, SCHEME_SERVER_REQUANTIZE = 0, 1, 2
  INFO_ALPC_LOOP_CLUSTER_SIZE, INFO_LOOP_ROW_SLOTS, INFO_ALPC_LOOP_ROW_SLOTS, INFO_STEP_RING_STAGES,
  INFO_AGGREGATE_SPLIT, INFO_QUANT_PIPELINED_RUNS, INFO_LOOP_COORDS_PER_THREAD, INFO_ALPC_LOOP_COORDS_PER_THREAD,
  INFO_QUANT_ONE_LAUNCH, INFO_QUANT_LAUNCHES, INFO_LOOP_OWNED, INFO_ALPC_LOOP_OWNED,
- INFO_QUANT_KEPT_TILES) = range(18)
+ INFO_QUANT_KEPT_TILES, INFO_STREAM_LOOP_SLICE, INFO_ALPC_STREAM_LOOP_SLICE) = range(20)
 KERNEL_NAMES = ["snapshot", "worker", "aggregate", "quant_stats", "quant_pack", "other", "inner_loop", "quant_fused"]
 
 # every symbol that include/lpc.h declares: (name, restype, argtypes)

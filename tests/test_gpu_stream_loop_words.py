@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-def _pair(n, d, N, B, b, alpc, clip=lpc.CLIP_STD, value=2.0):
+def _pair(n, d, N, B, b, alpc, clip=lpc.CLIP_STD, value=2.0, want_slice=0):
     X, y, _ = synth.linear_problem(n, d, loss="logistic", sparsity=0.2, noise=0.1, seed=d + B, device=DEV)
     g = torch.Generator(device=DEV).manual_seed(d + B)
     x0 = 0.1 * torch.randn(d, generator=g, device=DEV)
@@ -34,6 +34,8 @@ def _pair(n, d, N, B, b, alpc, clip=lpc.CLIP_STD, value=2.0):
     one.sync_status()
     many.sync_status()
     assert many.query(lpc.INFO_LOOP_LAUNCHES) == 1
+    if want_slice:
+        assert many.query(lpc.INFO_ALPC_STREAM_LOOP_SLICE if alpc else lpc.INFO_STREAM_LOOP_SLICE) == want_slice
     for w in [lpc.BUF_X, lpc.BUF_CODES, lpc.BUF_DELTA, lpc.BUF_CLIPPED] + ([lpc.BUF_Y, lpc.BUF_Z, lpc.BUF_YSUM, lpc.BUF_VHAT] if alpc else []):
         assert torch.equal(one.get_buffer(w).view(torch.int32), many.get_buffer(w).view(torch.int32)), w
     one.close()
@@ -47,11 +49,34 @@ def test_every_width(N, d, b, alpc):
     _pair(510 // N * N, d, N, 70, b, alpc)
 
 
-# by the plan's arithmetic on 148 SMs: slices of 512 columns, whose groups have sixteen rows in four row parts; the last slice of 4, 512 and 440
+# slices of 512 columns, whose groups have sixteen rows in four row parts; the last slice of 4, 512 and 440
 @pytest.mark.parametrize("alpc", [False, True])
 @pytest.mark.parametrize("b", [1, 2, 4, 8, 3, 6, 9, 32])
 @pytest.mark.parametrize("d,N,B", [(2052, 4, 70), (4096, 8, 256), (3000, 16, 77)])
 def test_slices_of_512_columns(d, N, B, b, alpc):
-    assert lpc.debug_stream_loop_slices(d, N, B, alpc, 231424, 148, 256)[0] == 0
-    assert lpc.debug_stream_loop_slices(d, N, B, alpc, 231424, 148, 512)[0] == (d + 511) // 512
-    _pair(512, d, N, B, b, alpc, clip=lpc.CLIP_LAMBDA if b == 2 else lpc.CLIP_STD, value=0.5 if b == 2 else 2.0)
+    _pair(512, d, N, B, b, alpc, clip=lpc.CLIP_LAMBDA if b == 2 else lpc.CLIP_STD, value=0.5 if b == 2 else 2.0, want_slice=512)
+
+
+@pytest.mark.parametrize("N,d,B,b,alpc,loops", [
+    (16, 8192, 256, 4, False, 1), (64, 2552, 65, 4, True, 1),     # a fixed width always takes the loop
+    (16, 8000, 256, 5, False, 0), (32, 8192, 256, 3, False, 0),   # clusters of eight with 128 CTAs; slices of 2,048 columns
+    (8, 8192, 256, 3, False, 1), (32, 4000, 66, 32, False, 1),    # 64 CTAs; 128 of them in clusters of four
+    (64, 2000, 100, 32, False, 0), (4, 10000, 100, 32, False, 0),
+    (3, 10000, 100, 9, False, 1), (3, 10000, 100, 9, True, 0), (3, 10000, 64, 9, True, 1),
+    (64, 900, 256, 7, True, 1), (33, 1000, 100, 32, True, 1),     # slices of 512 columns and narrower ones
+])
+def test_lines_of_the_rule(N, d, B, b, alpc, loops):
+    X, y, _ = synth.linear_problem(N * 16, d, loss="logistic", sparsity=0.2, noise=0.1, seed=1, device=DEV)
+    c = lpc.Context(X, y, lpc.LOGISTIC, 1e-4, N, B, b, lpc.CLIP_STD, 2.0, 7)
+    c.set_iterate(torch.zeros(d, device=DEV))
+    if alpc:
+        c.alpc_begin()
+    c.snapshot_full_grad()
+    if alpc:
+        c.alpc_double_sample_steps(0.4, 0.5, 0.3, 0.2, 0, 2)
+    else:
+        c.inner_steps(0.05, 0, 2)
+    c.sync_status()
+    assert c.query(lpc.INFO_LOOP_LAUNCHES) == loops
+    assert (c.query(lpc.INFO_ALPC_STREAM_LOOP_SLICE if alpc else lpc.INFO_STREAM_LOOP_SLICE) > 0) == bool(loops)
+    c.close()
