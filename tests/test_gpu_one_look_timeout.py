@@ -33,3 +33,36 @@ def test_calls_after_a_wait_that_ran_out(b, clip, value):
         ctx.debug_one_look_stop(-1)
     ctx.close()
     ref.close()
+
+
+@pytest.mark.parametrize("b,clip,value", [(4, lpc.CLIP_STD, 1.0), (3, lpc.CLIP_LAMBDA, 0.5), (8, lpc.CLIP_STD, 3.0)])
+def test_tiles_that_never_come_are_looked_at_by_those_who_need_them(b, clip, value):
+    # the first CTA does nothing: the scales of all messages that it has a tile of need that tile's maximum and sums from somebody else.  With one tile
+    # more per worker than there are CTAs its tiles walk down from the end, through second tiles of short tensors with ragged ends
+    tile, sms, N = 8192, torch.cuda.get_device_properties(0).multi_processor_count, 32
+    ends = [8188, 12, 4100, 4, 1064, 8192, 8, 8184, 516, 5]
+    sizes = [(sms + 1 - 2 * len(ends)) * tile] + [tile + e for e in ends]
+    offs = [sum(sizes[:i]) for i in range(len(sizes) + 1)]
+    tiles = [-(-s // tile) for s in sizes]
+    first = [sum(tiles[:i]) for i in range(len(tiles))]
+    assert sum(tiles) == sms + 1
+    g = torch.Generator(device=DEV).manual_seed(b)
+    ld = (offs[-1] + 3) // 4 * 4
+    U, S = (torch.randn((N, ld), generator=g, device=DEV)[:, :offs[-1]] for _ in range(2))
+    ctx, ref = (lpc.Context(None, None, lpc.LOGISTIC, 0.0, N, 1, b, clip, value, 3) for _ in range(2))
+    ref.set_option(lpc.OPT_ONE_LAUNCH_QUANTIZE, 0)
+    want = ref.quantize_pack(U, 7, U_sub=S, seg_offsets=offs)[1]
+    ref.sync_status()
+    ctx.debug_one_look_stop(0)
+    got = ctx.quantize_pack(U, 7, U_sub=S, seg_offsets=offs, delta_out=torch.full((N, len(sizes)), -1.0, device=DEV))[1]
+    assert ctx.query(lpc.INFO_QUANT_LAUNCHES) == 1 and ctx.status() == lpc.ERR_TIMEOUT
+    ragged = 0
+    for i in range(N):
+        for s, t0 in enumerate(first):
+            mine = [t for t in range(tiles[s]) if (i * sum(tiles) + t0 + t) % sms == 0]
+            if mine and mine[0] > 0:  # whoever has a message's first tile reports its scale
+                ragged += s > 0
+                assert got[i, s].item() == want[i, s].item(), (i, s)
+    assert ragged >= 8
+    ctx.close()
+    ref.close()
