@@ -77,14 +77,14 @@ typedef struct lpc_ctx lpc_ctx;
 
 /* options for lpc_set_option */
 #define LPC_OPT_SAMPLE_GLOBAL 0 /* 0 (default): worker i samples its own block of n/N rows; 1: all n rows (the paper's shared-storage setting, Section 2.1) */
-#define LPC_OPT_TAP_U 1         /* 1: inner steps also store u^i and v for inspection (slower; the loop for minibatches of more than 64 rows is off meanwhile) */
-#define LPC_OPT_CLUSTER_SIZE 2  /* thread-block cluster size per worker for the fused step: 0 = automatic, else 1, 2, 4 or 8 */
+#define LPC_OPT_TAP_U 1         /* 1: inner steps also store u^i and v for inspection (slower; the one-launch loop whose rows stream, whatever the number of rows, is off meanwhile: single launches take its place) */
+#define LPC_OPT_CLUSTER_SIZE 2  /* thread-block cluster size per worker for the fused step: 0 = automatic, else 1, 2, 4 or 8 (a fixed size also keeps minibatches whose rows stream on single launches) */
 #define LPC_OPT_USE_GRAPH 3     /* 1 (default): lpc_inner_steps replays a CUDA graph; 0: plain launches */
-#define LPC_OPT_PROFILE 4       /* 1: record CUDA events around every kernel launch (graph replay and the loop for minibatches of more than 64 rows are off meanwhile) */
+#define LPC_OPT_PROFILE 4       /* 1: record CUDA events around every kernel launch (graph replay and the one-launch loop whose rows stream are off meanwhile, so that what is timed for such minibatches are the kernels of single steps and not the loop that runs without it) */
 
 #define LPC_OPT_SHARED_SCALE 6  /* 1: lpc_quantize_pack gives every worker the unified scale delta_t = max_i delta_t^i of the parameter-server schemes (b), (c) of Section 3.2; needs b in 2..16 */
 #define LPC_OPT_AVERAGE_DIVISOR 7 /* lpc_unpack_average_prox (and only it: the training loops always average over N) divides the decoded sum by this count instead of the context's N (0 = N): the worker count behind a server's sum stream */
-#define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits: rows resident in shared memory (up to 64 per worker), or streaming through it (up to 256) */
+#define LPC_OPT_PERSISTENT 5    /* 1 (default): lpc_inner_steps runs the whole loop in one cooperative launch when it fits: rows resident in shared memory (up to 64 per worker), or, where they have no room, streaming through it (up to 256; code widths other than 1, 2, 4 and 8 only where that is faster than single steps).  Steps that the caller captures into a graph are single launches */
 #define LPC_OPT_ONE_LAUNCH_QUANTIZE 8 /* 1 (default): lpc_quantize_pack may take its short-vector path (one launch where a vector fits a cluster) for inputs of at most LPC_ONE_LAUNCH_BYTES, and one launch for many tensors with a subtrahend */
 #define LPC_ONE_LAUNCH_BYTES (48ll << 20)
 #define LPC_OPT_LOOP_COOPERATIVE 9 /* 1 (default): the one-launch loops are cooperative launches (the driver guarantees that all their CTAs are resident together, which they rely on).  0: a plain cluster launch of the same grid, for profilers that cannot replay a cooperative cluster launch; use it only on a GPU that runs nothing else (the launch plan has checked that all clusters fit, and every wait in the kernel is bounded, so a grid that is not resident together ends with LPC_ERR_TIMEOUT instead of hanging) */
@@ -110,8 +110,8 @@ typedef struct lpc_ctx lpc_ctx;
  *   n        rows; must be a multiple of N.  Worker i owns rows [i*n/N, (i+1)*n/N).
  *   d        features, multiple of 4, at most 16384
  *   N        simulated workers, 1..1024;  B minibatch size per worker, 1..1024 (up to 64 rows per worker stay
- *            resident on chip; the one-launch loops are available for N <= 64 and B <= 64 when all worker
- *            clusters fit on the device together; larger minibatches stream through the per-step kernel)
+ *            resident on chip; the one-launch loops are available for N <= 64 and B <= 256 when all worker
+ *            clusters fit on the device together, see LPC_OPT_PERSISTENT; other minibatches take the per-step kernel)
  *   b        bits per coordinate: 1..16 or 32 (32 = full precision, the codes are the floats)
  *   seed     key of every random stream (minibatches, shared batch J, stochastic rounding)
  *   stream   cudaStream_t (NULL = default stream)
@@ -156,7 +156,7 @@ int lpc_snapshot_full_grad(lpc_ctx* ctx, float* mu_out, double* f_snapshot);
  * Counts (32 + b*d)*N*(N-1) step-2 bits (Table 1, broadcast).
  */
 int lpc_inner_step(lpc_ctx* ctx, float eta, uint64_t k);
-/* `count` consecutive inner steps k0, k0+1, ... replayed from a captured CUDA graph. */
+/* `count` consecutive inner steps k0, k0+1, ...: a one-launch loop where there is one (LPC_OPT_PERSISTENT), else replayed from a captured CUDA graph. */
 int lpc_inner_steps(lpc_ctx* ctx, float eta, uint64_t k0, int64_t count);
 
 /*
@@ -183,8 +183,8 @@ int lpc_packed_words(int64_t len, int32_t b, int64_t* words_out); /* ceil(len*b/
  * Vectors longer than L2 are read twice (once for ||u||_inf and the variance, once to quantize) by three launches that overlap;
  * when all N vectors together take at most LPC_ONE_LAUNCH_BYTES the second look is served by L2, and vectors of at most
  * 65,536 values in one segment, with b in {1, 2, 3, 4, 8}, own scales and at most four CTAs per SM in all, take ONE launch, a
- * cluster per worker that keeps the values in registers.  With U_sub, inputs beyond L2 whose tensors are short against the chip (up to
- * some 2.4 million values each, on 16-byte boundaries) take ONE launch as well, which reads both inputs once.
+ * cluster per worker that keeps the values in registers.  With U_sub, inputs of more than three quarters of L2 each whose tensors are short against the chip (up to
+ * some 2.4 million values each, on 16-byte boundaries, their tiles of 8,192 values full to seven eighths on average) take ONE launch as well, which reads both inputs once.
  * (LPC_OPT_ONE_LAUNCH_QUANTIZE = 0 switches both off.)  Same codes either way; LPC_INFO_QUANT_LAUNCHES says which it was.
  * N, b and the clip rule come from the context.
  */
@@ -284,17 +284,17 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
 
 /* Launch-plan facts of a context (host scalars): what = LPC_INFO_*. */
 #define LPC_INFO_STEP_CLUSTER_SIZE 0       /* CTAs per worker cluster of the per-step kernel (0: d too large) */
-#define LPC_INFO_LOOP_CLUSTER_SIZE 1       /* CTAs per worker cluster of the one-launch inner loop (0: not available) */
-#define LPC_INFO_LOOP_LAUNCHES 2           /* lpc_inner_steps calls served by the one-launch inner loop so far */
+#define LPC_INFO_LOOP_CLUSTER_SIZE 1       /* CTAs per worker cluster of the one-launch inner loop with resident rows (0: not available; the loop whose rows stream may still be: LPC_INFO_STREAM_LOOP_SLICE) */
+#define LPC_INFO_LOOP_LAUNCHES 2           /* lpc_inner_steps calls served by a one-launch inner loop so far, rows resident or streaming */
 #define LPC_INFO_SNAPSHOT_ROWS_PER_TILE 3  /* rows per shared-memory stage of the snapshot pass */
 #define LPC_INFO_SNAPSHOT_STAGES 4         /* shared-memory stages of the snapshot pass */
 #define LPC_INFO_ALPC_LOOP_CLUSTER_SIZE 5  /* as LOOP_CLUSTER_SIZE, for the one-launch loop of Algorithm 2 */
-#define LPC_INFO_LOOP_ROW_SLOTS 6          /* shared-memory slots for sampled-row slices per CTA of the one-launch loop: between B
+#define LPC_INFO_LOOP_ROW_SLOTS 6          /* shared-memory slots for sampled-row slices per CTA of the loop with resident rows: between B
                                               (a step's rows are fetched once the step before has formed its u) and 2B (all of them
                                               are fetched a whole step ahead); 0: loop not available */
 #define LPC_INFO_ALPC_LOOP_ROW_SLOTS 7     /* the same for the loop of Algorithm 2 */
 #define LPC_INFO_STEP_RING_STAGES 8        /* per-step kernel: 0 = minibatch rows resident on chip, else ring stages they stream through */
-#define LPC_INFO_LOOP_COORDS_PER_THREAD 11  /* one-launch loop: consecutive coordinates a thread owns (8, 4 or 2; 0: not available) */
+#define LPC_INFO_LOOP_COORDS_PER_THREAD 11  /* loop with resident rows: consecutive coordinates a thread owns (8, 4 or 2; 0: not available) */
 #define LPC_INFO_ALPC_LOOP_COORDS_PER_THREAD 12
 #define LPC_INFO_QUANT_ONE_LAUNCH 13        /* last lpc_quantize_pack: 1 when the input was short enough (LPC_ONE_LAUNCH_BYTES) for the short-vector path and LPC_OPT_ONE_LAUNCH_QUANTIZE allowed it */
 #define LPC_INFO_AGGREGATE_SPLIT 9         /* last lpc_unpack_average_prox: CTAs that shared one tile of 8192 coordinates (1, 2 or 4) */
@@ -304,7 +304,7 @@ int lpc_objective(lpc_ctx* ctx, const float* x, double* P_out);
                                               on a 16-byte boundary (ld % 4 == 0), for b = 32, and when the call was one launch */
 #define LPC_INFO_QUANT_LAUNCHES 14         /* last lpc_quantize_pack: kernels it launched.  1: a cluster per worker, one look at many tensors (or an empty vector);
                                               3: statistics, scale, codes; 4: the same and the unified scale */
-#define LPC_INFO_LOOP_OWNED 15             /* one-launch loop: 1 when each coordinate's update is made by one CTA, which sends the new
+#define LPC_INFO_LOOP_OWNED 15             /* loop with resident rows: 1 when each coordinate's update is made by one CTA, which sends the new
                                               point to the others; 0 when every cluster updates its copy, or loop not available */
 #define LPC_INFO_ALPC_LOOP_OWNED 16        /* the same for the loop of Algorithm 2 */
 #define LPC_INFO_QUANT_KEPT_TILES 17       /* last lpc_quantize_pack: tiles of 8192 values at the end of the input that the first look left in
@@ -374,7 +374,8 @@ int lpc_debug_wait_timeout(lpc_ctx* ctx, uint64_t limit_ns);
 /*
  * Inspection aid for the same path inside lpc_quantize_pack's one look at many tensors: in the next such launch of the context the first CTA
  * goes no further than `tiles` of its tiles, as after a wait that ran out.  That call's outputs are incomplete and the next lpc_sync_status
- * returns LPC_ERR_TIMEOUT; the calls after it are as good as ever.  Calls that take another path leave the request standing.
+ * returns LPC_ERR_TIMEOUT; the calls after it are as good as ever.  Calls that take another path leave the request standing; a captured launch
+ * keeps it in each replay.
  */
 int lpc_debug_one_look_stop(lpc_ctx* ctx, int32_t tiles);
 

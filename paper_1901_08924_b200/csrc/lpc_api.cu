@@ -446,7 +446,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
   };
   int64_t done = 0;
   const bool small_ok = (kind == 0) ? c->persist_ok : c->apersist_ok;
-  // large minibatches: where nobody looks at u and v or times the launches of a step one by one
+  // rows that stream: where nobody looks at u and v or times the launches of a step one by one
   lpc_ctx::StreamLoop& sl = c->sloop[kind];
   if (!small_ok && !sl.planned && c->use_persist && count >= 2) {  // planned when it is first needed: few contexts use it, and with one of the algorithms
     sl.planned = true;
@@ -460,7 +460,7 @@ int run_steps(lpc_ctx* c, int kind, const float* p, uint64_t k0, int64_t count) 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
   const bool loop_ok = (small_ok || stream_ok) && !capturing;
-  // the strongly convex ALPC step carries a weight that changes from step to step: plain per-step launches
+  // the strongly convex ALPC step carries a weight that changes from step to step: the loops form it, a captured graph of steps cannot
   const bool weighted = (kind == 1 && c->sigma > 0.f);
   if (c->use_persist && loop_ok && count >= 2 && count <= 0x7FFFFFFF) {
     // the whole loop in one cooperative launch; on a launch refusal fall through to the per-step kernels

@@ -16,6 +16,8 @@
 // chain of a group and the ring; 8 workers, d = 752, B = 256 47.2 / 9.4, eight groups and the end of a step (4); 4 workers, d = 64, B = 100
 // 22.5 / 6.6; 16 workers, d = 8,216, B = 16 23.4 / 9.0.  Tried: the end of a step by the warps of u (44 to 130 us at the first shape: spilled
 // registers), rows two groups ahead in registers (55.3: the same), the next rows prefetched to L2 while a step ends (48.0 to 49.3).
+// 96 registers per thread do not hold this form's values either: 24 to 132 bytes of spill stores per thread with fixed widths (76 in the kernel of the first
+// shape), 114 to 166 with the others.
 //
 // Arithmetic, operation for operation, is that of the per-step kernels.
 #include <algorithm>
