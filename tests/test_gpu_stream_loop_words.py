@@ -63,6 +63,7 @@ def test_slices_of_512_columns(d, N, B, b, alpc):
     (8, 8192, 256, 3, False, 1), (32, 4000, 66, 32, False, 1),    # 64 CTAs; 128 of them in clusters of four
     (64, 2000, 100, 32, False, 0), (4, 10000, 100, 32, False, 0),
     (3, 10000, 100, 9, False, 1), (3, 10000, 100, 9, True, 0), (3, 10000, 64, 9, True, 1),
+    (20, 10000, 100, 9, False, 1), (32, 5000, 33, 32, False, 1),  # single steps need two rounds of clusters; keep their rows resident
     (64, 900, 256, 7, True, 1), (33, 1000, 100, 32, True, 1),     # slices of 512 columns and narrower ones
 ])
 def test_lines_of_the_rule(N, d, B, b, alpc, loops):
